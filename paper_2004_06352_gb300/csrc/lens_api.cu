@@ -143,10 +143,11 @@ int CallScratch::alloc(size_t n) {
   return LENS_OK;
 }
 
-CallScratch::~CallScratch() {
+void CallScratch::release() {
   if (!p) return;
   cudaFreeAsync(p, st);
   ctx->used -= std::min(ctx->used, bytes);
+  p = nullptr;
 }
 
 int check_grid(const lens_grid *g) {
@@ -281,6 +282,14 @@ int build_model(lens_ctx *ctx, const lens_halo *h, int32_t n, Model **out) {
     m->koff[k] = c;
   }
   m->koff[4] = m->n_light;
+  // shapes (q = (1 - eps) / (1 + eps); SIS and point mass: round, no core)
+  double iq = 0.0;
+  for (int32_t i : light) iq += h[i].type == LENS_DPIE ? (1.0 + h[i].eps) / (1.0 - h[i].eps) : 1.0;
+  m->invq_light = light.empty() ? 1.0 : iq / (double)light.size();
+  for (int32_t i : heavy) {
+    const bool d = h[i].type == LENS_DPIE;
+    m->heavy_shape.push_back({d ? (1.0 - h[i].eps) / (1.0 + h[i].eps) : 1.0, d ? h[i].rcore * (1.0 + h[i].eps) : 0.0});
+  }
   const size_t nl = (size_t)m->n_light, nh = (size_t)m->n_heavy, na = (size_t)n;
   // records (built on the device), then the staged halo table and slots
   const size_t sizes[9] = {nl * REC32 * sizeof(float),  nl * 4 * sizeof(double),     nl * 4 * sizeof(float),
@@ -544,7 +553,17 @@ static int map_common(lens_ctx *ctx, lens_model_t model, const lens_grid *grid, 
   cudaSetDevice(ctx->device);
   cudaStream_t st = (cudaStream_t)stream;
   StreamMark mark(ctx, st);
-  if (precision == LENS_MIXED) return launch_map_mixed(ctx, m, grid, dls_ds, hess, d_out, st);
+  if (precision == LENS_MIXED) {
+    FarPlan plan = plan_far(ctx, m, grid, hess);
+    // the repair list first: without it there is no map, without room for
+    // the coarse level's values there is the direct kernel
+    CallScratch list(ctx, st), far(ctx, st);
+    if (plan.use && ctx->repair_ratio > 0.0 && m->n_light > 0 && (rc = list.alloc(map_repair_bytes(grid)))) return rc;
+    if (plan.use && plan.ct && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
+    if (plan.use && (rc = launch_far_coarse(m, grid, plan, hess, far.p, st))) return rc;
+    return launch_map_mixed(ctx, m, grid, dls_ds, hess, d_out, st, 0, -1, true, list.p, plan.use ? &plan : nullptr,
+                            far.p);
+  }
   if (precision == LENS_FP64) return launch_map_fp64(ctx, m, grid, dls_ds, hess, d_out, st);
   return fail(LENS_EINVAL, "precision must be LENS_FP64 or LENS_MIXED");
 }
@@ -592,7 +611,9 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   if ((uintptr_t)h_out % esize) return fail(LENS_EINVAL, "h_out must be aligned to its element size");
   const int planes = hess ? 6 : 2, nx = grid->nx, ny = grid->ny;
   // about 8 bands, each a whole number of tiles
-  const int tile = map_tile_rows(hess);
+  FarPlan plan;
+  if (precision == LENS_MIXED) plan = plan_far(ctx, m, grid, hess);
+  const int tile = plan.use ? FAR_TILE_ROWS : map_tile_rows(hess);
   int rows = (ny + 7) / 8;
   rows = std::max(tile, (rows + tile - 1) / tile * tile);
   const size_t band_bytes = (size_t)rows * nx * planes * esize;
@@ -618,6 +639,18 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   StreamMark mark(ctx, st);  // st joins the band streams at the end
   LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, st));
   for (int k = 0; k < 2; ++k) LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[k], ctx->pipe_start, 0));
+  // the interpolated form's coarse level, of the whole grid, before the bands
+  CallScratch far(ctx, ctx->pipe_cs[0]);
+  if (plan.use && plan.ct) {
+    const bool room = !ctx->budget || ctx->used + plan.bytes + map_repair_bytes(grid, rows) <= ctx->budget;
+    if (!room || far.alloc(plan.bytes) != LENS_OK) {
+      plan = FarPlan();  // no room beside the bands' repair lists: the direct kernel, whose tiles divide the bands too
+    } else {
+      if ((rc = launch_far_coarse(m, grid, plan, hess, far.p, ctx->pipe_cs[0]))) return rc;
+      LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[0]));
+      LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[1], ctx->pipe_start, 0));
+    }
+  }
   char *host = (char *)h_out;
   const size_t host_plane = (size_t)nx * ny * esize;
   for (int row0 = 0, b = 0; row0 < ny; row0 += rows, ++b) {
@@ -626,7 +659,8 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
     cudaStream_t cs = ctx->pipe_cs[k];
     // the buffer's previous band (this call's or an earlier call's) has left
     LENS_CUDA_TRY(cudaStreamWaitEvent(cs, ctx->pipe_copied[k], 0));
-    rc = precision == LENS_MIXED ? launch_map_mixed(ctx, m, grid, dls_ds, hess, buf, cs, row0, r)
+    rc = precision == LENS_MIXED ? launch_map_mixed(ctx, m, grid, dls_ds, hess, buf, cs, row0, r, true, nullptr,
+                                                    plan.use ? &plan : nullptr, far.p)
                                  : launch_map_fp64(ctx, m, grid, dls_ds, hess, buf, cs, row0, r);
     if (rc) return rc;
     LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_done[k], cs));
@@ -637,6 +671,14 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
     LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_copied[k], ctx->pipe_cp));
   }
   for (int k = 0; k < 2; ++k) LENS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->pipe_copied[k], 0));
+  if (far.p) {
+    // the coarse level goes once both band streams have read it; st joins
+    LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[1]));
+    LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[0], ctx->pipe_start, 0));
+    far.release();
+    LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[0]));
+    LENS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->pipe_start, 0));
+  }
   return LENS_OK;
 }
 

@@ -1,0 +1,880 @@
+// LENS_MIXED maps with the far potentials interpolated (Sec. 4.1, Eq. 10;
+// Sec. 2.4, Eqs. 7-9).
+//
+// What bounds a map when every node evaluates every potential is the FP32
+// pipe (k_map_mixed in lens_maps.cu: 65 operations per pair, 4.2e9 pairs for
+// 2048^2 nodes x 1000 potentials), but most potentials are far from any one
+// tile of the map and smooth over it.  A potential's deflection, Hessian and
+// lensing potential are analytic in the node's position out to the complex
+// displacement at which psi^2 = q^2 (s^2 + x^2) + y^2 vanishes, whose length
+// is at least the real psi there (|t|^2 = psi^2 / (q^2 cos^2 + sin^2) along
+// any direction), so on a tile of half-diagonal R polynomial interpolation
+// at P x P Chebyshev nodes converges like rho^-P with rho growing with
+// psi / R (Trefethen, "Approximation Theory and Approximation Practice",
+// ch. 8).  Measured over random dPIE terms at the worst place psi = K R of
+// the tile's centre: P = 10, K = 3 gives 1.2e-8 of the term's own deflection,
+// P = 12, K = 2.5 gives 4e-9 -- below the 1e-7 an FP32 term carries -- and
+// the error falls as psi^-P beyond.
+//
+// Two levels.  k_far_coarse: per coarse tile (ct x ct nodes, ct = 64..512),
+// the potentials with psi >= KC R are summed at 12 x 12 nodes; the others'
+// bits are set in the tile's mask.  k_far_map: per 32 x 32 tile, the
+// potentials left by the coarse tile (all of them without a coarse level)
+// with psi >= KF R are summed at 10 x 10 nodes, the coarse tile's
+// interpolant is added there, and every map node then takes the near
+// potentials one by one plus the interpolant.  Cluster-scale potentials go
+// through the same levels in double-float, with wider margins.
+//
+// Precision.  A potential's terms at the nodes are the FP32 terms the direct
+// kernel would sum, with the same compensated accumulation; the node sums
+// are kept in double-float, a plane (slopes of 8 significant bits, so that
+// its products with node offsets are exact) is taken out of them, and only
+// the remainder is interpolated in FP32.  The map node's value is the plane
+// plus the remainder plus the near sum in double-float, scaled by D_ls/D_s
+// and rounded once.  The magnitude sum that decides the double-float repair
+// is interpolated as well (a few percent off where a far term changes sign).
+#include <algorithm>
+#include <cmath>
+
+#include "lens_device.cuh"
+
+namespace lens {
+namespace {
+
+constexpr int FT = 32;   // nodes a side of a fine tile
+constexpr int FP = 10;   // its interpolation nodes per axis
+constexpr int CP = 12;   // a coarse tile's
+constexpr int FF_THREADS = 256, FF_WARPS = FF_THREADS / 32;
+constexpr int FF_CH = 64;            // potentials per staged chunk
+constexpr int REC_STRIDE4 = REC32 / 4 + 1;  // float4 slots per staged record (the pad spreads the records a warp reads)
+constexpr int FF_SUB = 16;           // partial sums folded every FF_SUB potentials
+constexpr double DET_TERM_ERR = 2e-7, DET_REPAIR_ABS = 1e-5;  // as in lens_maps.cu
+constexpr int CT_MIN = 64, CT_MAX = 512;
+
+enum FarMode : int { FAR_GRAD = 0, FAR_HESS = 1, FAR_POT = 2 };
+// interpolated values: deflection (2), kappa, gamma1, gamma2 (HESS) or the
+// potential alone, then the magnitude sum (not POT)
+__host__ __device__ constexpr int nval(int mode) { return mode == FAR_HESS ? 5 : mode == FAR_GRAD ? 2 : 1; }
+__host__ __device__ constexpr int ncmp(int mode) { return nval(mode) + (mode == FAR_POT ? 0 : 1); }
+__host__ __device__ constexpr int ncmp2(int mode) { return (ncmp(mode) + 1) / 2; }
+
+// Chebyshev nodes of the fine tile in units of 1/64 grid step about the
+// tile's centre (half-width 15.5 steps), of the coarse tile in units of its
+// half-width / 512.
+constexpr int XI64[FP] = {980, 884, 701, 450, 155, -155, -450, -701, -884, -980};
+constexpr int ZC512[CP] = {508, 473, 406, 312, 196, 67, -67, -196, -312, -406, -473, -508};
+__device__ const float D_XI[FP] = {980 / 64.f, 884 / 64.f, 701 / 64.f, 450 / 64.f, 155 / 64.f,
+                                   -155 / 64.f, -450 / 64.f, -701 / 64.f, -884 / 64.f, -980 / 64.f};
+__device__ const float D_ZC[CP] = {508 / 512.f, 473 / 512.f, 406 / 512.f, 312 / 512.f, 196 / 512.f, 67 / 512.f,
+                                   -67 / 512.f, -196 / 512.f, -312 / 512.f, -406 / 512.f, -473 / 512.f, -508 / 512.f};
+
+// Lagrange weights, formed in FP64 at compile time.
+struct FineTab {
+  float w[FT][FP];  // at map node m - 15.5 steps
+};
+constexpr FineTab fine_tab() {
+  FineTab t{};
+  for (int m = 0; m < FT; ++m)
+    for (int i = 0; i < FP; ++i) {
+      double v = 1.0;
+      for (int k = 0; k < FP; ++k)
+        if (k != i) v *= ((m - 15.5) * 64.0 - XI64[k]) / (double)(XI64[i] - XI64[k]);
+      t.w[m][i] = (float)v;
+    }
+  return t;
+}
+__device__ const FineTab D_FINE = fine_tab();
+// the coarse basis at the fine tile's nodes: fine tile c of CT / 32 along an
+// axis, node i, coarse node k
+template <int SUBT>
+struct CoarseTab {
+  float w[SUBT][FP][CP];
+};
+template <int SUBT>
+constexpr CoarseTab<SUBT> coarse_tab() {
+  CoarseTab<SUBT> t{};
+  const double half = 16.0 * SUBT;  // half-width in steps
+  for (int c = 0; c < SUBT; ++c)
+    for (int i = 0; i < FP; ++i)
+      for (int k = 0; k < CP; ++k) {
+        const double x = (32.0 * c + 16.0 - half + XI64[i] / 64.0) / half * 512.0;
+        double v = 1.0;
+        for (int l = 0; l < CP; ++l)
+          if (l != k) v *= (x - ZC512[l]) / (double)(ZC512[k] - ZC512[l]);
+        t.w[c][i][k] = (float)v;
+      }
+  return t;
+}
+__device__ const CoarseTab<2> D_CO2 = coarse_tab<2>();
+__device__ const CoarseTab<4> D_CO4 = coarse_tab<4>();
+__device__ const CoarseTab<8> D_CO8 = coarse_tab<8>();
+__device__ const CoarseTab<16> D_CO16 = coarse_tab<16>();
+
+struct FarArgs {
+  const float *rec32;
+  const float4 *cen32;
+  int n_light;
+  const double *heavy;
+  const float2 *heavydf;
+  int n_heavy;
+  int nwl, nw;       // mask words of the FP32 potentials / of all (the cluster-scale ones start at word nwl)
+  double xmin, ymin, dx, dy;
+  int nx, ny;        // ny: rows of this launch
+  int row0;
+  double dls;
+  float thr_c, thr_ch, thr_f, thr_fh;  // squared psi beyond which a potential is far: coarse / fine, FP32 / cluster-scale
+  // coarse level: tile (0, 0) covers the grid's first nodes
+  int ct, nct;       // nodes a side (0: no coarse level), tiles per row
+  float *cval;       // per coarse tile: remainders [ncmp][CP * CP], planes [nval][4], light kappa and gamma bounds [4]
+  unsigned *cmask;   // per coarse tile: nw words, bit set = left to the fine level
+  float *out;
+  double *out64;
+  long long plane;
+  int tau;
+  double bx, by;
+  float repair_f;    // 2 * ratio, 0: no repair
+  int *rep_count, *rep_list;
+};
+
+__host__ __device__ constexpr int coarse_floats(int mode) { return ncmp(mode) * CP * CP + nval(mode) * 4 + 4; }
+
+// Is the potential far from a tile centred at (dx, dy) from it?
+__device__ __forceinline__ bool far32(const float4 *r4, float dX, float dY, float thr) {
+  const float4 A = r4[0];
+  const int kind = __float_as_int(r4[7].x);
+  if (kind == K32_SIS || kind == K32_POINT) return fmaf(dX, dX, dY * dY) >= thr;
+  const float x = fmaf(A.x, dX, A.y * dY), y = fmaf(A.x, dY, -A.y * dX);
+  return fmaf(A.z, x * x, fmaf(y, y, r4[1].x)) >= thr;
+}
+__device__ __forceinline__ bool far_df(const float2 *r, float dX, float dY, float thr) {
+  if (r[F_U2].x < 0.f) return fmaf(dX, dX, dY * dY) >= thr;
+  const float c = r[F_C].x, s = r[F_S].x, x = fmaf(c, dX, s * dY), y = fmaf(c, dY, -s * dX);
+  return fmaf(r[F_Q2].x, x * x, fmaf(y, y, r[F_KC].x)) >= thr;
+}
+
+// One cluster-scale potential in double-float at (X, Y), added to sum
+// (out of line: it is large and taken rarely).
+template <int MODE>
+__device__ __noinline__ void add_heavy(const float2 *rdf, const double *r64, df X, df Y, df *sum) {
+  const double Xd = df_to_double(X), Yd = df_to_double(Y);
+  if constexpr (MODE == FAR_POT)
+    sum[0] = df_add(sum[0], df_from_double(pot64(r64, Xd, Yd)));
+  else
+    add_potential_dfs<MODE == FAR_HESS>(rdf, 1, r64, Xd, Yd, X, Y, sum);
+}
+
+// The FP32 potentials h0, h0 + step, ... < cnt of a staged chunk at one
+// point pair of the tile: offsets (ox) shared, (oy) per point, from the
+// tile's centre as hi/lo pairs.
+template <int MODE>
+struct Sums {
+  Acc2<MODE == FAR_HESS, 1> tot, cmp, part;
+  int seen;
+  __device__ __forceinline__ void zero() {
+    tot.zero();
+    cmp.zero();
+    part.zero();
+    seen = 0;
+  }
+  __device__ __forceinline__ void fold() {
+    if constexpr (MODE == FAR_POT)
+      fold2_pot(tot, cmp, part);
+    else
+      fold2(tot, cmp, part);
+    seen = 0;
+  }
+  __device__ __forceinline__ void sweep(const float4 *s_rec, const float4 *s_off, int h0, int cnt, int step, float2 ox,
+                                        float2 oyh, float2 oyl) {
+    constexpr bool HESS = MODE == FAR_HESS, POT = MODE == FAR_POT;
+    for (int h = h0; h < cnt; h += step) {
+      const float4 *r4 = s_rec + h * REC_STRIDE4;
+      const float4 o = s_off[h];
+      const float dX = (o.x + ox.x) + (o.y + ox.y);
+      const float2 dY[1] = {add2(add2(dup2(o.z), oyh), add2(dup2(o.w), oyl))};
+      const int kind = __float_as_int(r4[7].x);
+      if (kind == K32_DPIE)
+        dpie32x2<HESS, 1, false, !POT, false, POT>(r4, dX, dY, part);
+      else if (kind == K32_DPIE_SERIES)
+        dpie32x2<HESS, 1, true, !POT, false, POT>(r4, dX, dY, part);
+      else if (kind == K32_SIS)
+        circ32x2<HESS, 1, false, !POT, POT>(r4, dX, dY, part);
+      else
+        circ32x2<HESS, 1, true, !POT, POT>(r4, dX, dY, part);
+      if (++seen == FF_SUB) fold();
+    }
+  }
+  // value c of point h as a double-float number
+  __device__ __forceinline__ df value(int c, int h) const {
+    const float2 *t, *m;
+    if constexpr (MODE == FAR_POT) {
+      t = tot.k;
+      m = cmp.k;
+    } else {
+      t = c == 0 ? tot.ax : c == 1 ? tot.ay : c == 2 ? tot.k : c == 3 ? tot.g1 : tot.g2;
+      m = c == 0 ? cmp.ax : c == 1 ? cmp.ay : c == 2 ? cmp.k : c == 3 ? cmp.g1 : cmp.g2;
+    }
+    return df{part2(t[0], h), -part2(m[0], h)};
+  }
+  __device__ __forceinline__ float mag(int h) const { return part2(tot.mag[0], h); }
+};
+
+// Potential idx of the list (FP32) into staging slot h: its record, and the
+// tile centre's offset from its centre as hi/lo pairs.
+__device__ __forceinline__ void stage_chunk(const FarArgs &a, const unsigned short *list, int cnt, df Tx, df Ty,
+                                            float4 *s_rec, float4 *s_off) {
+  const float4 *g_rec = reinterpret_cast<const float4 *>(a.rec32);
+  for (int q = threadIdx.x; q < cnt * (REC32 / 4); q += FF_THREADS)
+    s_rec[(q >> 3) * REC_STRIDE4 + (q & 7)] = __ldg(g_rec + (size_t)list[q >> 3] * (REC32 / 4) + (q & 7));
+  if (threadIdx.x < cnt) {
+    const float4 c = __ldg(a.cen32 + list[threadIdx.x]);
+    const df ox = df_sub(Tx, df{c.x, c.z}), oy = df_sub(Ty, df{c.y, c.w});
+    s_off[threadIdx.x] = make_float4(ox.hi, ox.lo, oy.hi, oy.lo);
+  }
+}
+
+// Classify the potentials whose bit is set in `in` (NULL: all) as far from
+// the tile or near, and list the far ones then the near ones, each in index
+// order.  s_far / s_near: nw words each.  cnt: far FP32, far cluster-scale,
+// near FP32, near cluster-scale.  Ends synchronised.
+__device__ __forceinline__ void classify(const FarArgs &a, const unsigned *in, df Tx, df Ty, float thr, float thr_h,
+                                         unsigned *s_far, unsigned *s_near, unsigned short *s_list, int *s_cnt) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float4 *g_rec = reinterpret_cast<const float4 *>(a.rec32);
+  for (int w = warp; w < a.nw; w += FF_WARPS) {
+    const bool hv = w >= a.nwl;
+    const int i = (hv ? w - a.nwl : w) * 32 + lane;
+    bool mine = i < (hv ? a.n_heavy : a.n_light);
+    if (in) mine = mine && (in[w] >> lane & 1u);
+    bool far = false;
+    if (mine) {
+      if (hv) {
+        const float2 *r = a.heavydf + (size_t)i * RECDF;
+        far = far_df(r, df_sub(Tx, df{r[F_X0].x, r[F_X0].y}).hi, df_sub(Ty, df{r[F_Y0].x, r[F_Y0].y}).hi, thr_h);
+      } else {
+        const float4 c = __ldg(a.cen32 + i);
+        far = far32(g_rec + (size_t)i * (REC32 / 4), df_sub(Tx, df{c.x, c.z}).hi, df_sub(Ty, df{c.y, c.w}).hi, thr);
+      }
+    }
+    const unsigned f = __ballot_sync(0xffffffffu, mine && far), n = __ballot_sync(0xffffffffu, mine && !far);
+    if (lane == 0) {
+      s_far[w] = f;
+      s_near[w] = n;
+    }
+  }
+  __syncthreads();
+  // positions: warp 0 scans the words' populations, the far words first
+  int *pos = reinterpret_cast<int *>(s_near + a.nw);  // [2 nw]
+  if (warp == 0) {
+    int base = 0;
+    for (int w0 = 0; w0 < 2 * a.nw; w0 += 32) {
+      const int w = w0 + lane;
+      const int c = w < 2 * a.nw ? __popc(w < a.nw ? s_far[w] : s_near[w - a.nw]) : 0;
+      int s = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += t;
+      }
+      if (w < 2 * a.nw) pos[w] = base + s - c;
+      base += __shfl_sync(0xffffffffu, s, 31);
+    }
+    __syncwarp();
+    if (lane == 0) {
+      const int fl = a.nwl < a.nw ? pos[a.nwl] : pos[a.nw], fa = pos[a.nw];
+      const int nl = a.nwl < a.nw ? pos[a.nw + a.nwl] : base;
+      s_cnt[0] = fl;
+      s_cnt[1] = fa - fl;
+      s_cnt[2] = nl - fa;
+      s_cnt[3] = base - nl;
+    }
+  }
+  __syncthreads();
+  for (int w = warp; w < 2 * a.nw; w += FF_WARPS) {
+    const int wi = w < a.nw ? w : w - a.nw;
+    const unsigned m = w < a.nw ? s_far[wi] : s_near[wi];
+    const int i = (wi >= a.nwl ? wi - a.nwl : wi) * 32 + lane;
+    if (m >> lane & 1u) s_list[pos[w] + __popc(m & ((1u << lane) - 1u))] = (unsigned short)i;
+  }
+  __syncthreads();
+}
+
+// Slope with 8 significant bits: its products with node offsets (up to 15
+// bits) are exact in FP32.
+__device__ __forceinline__ float slope8(float v) { return __int_as_float(__float_as_int(v) & 0xffff0000); }
+
+// P x P node sums of the far potentials of one tile: s_val[c][node] in
+// double-float (node = y index * P + x index).  Ends synchronised.
+// kb: the FP32 potentials' largest |kappa|, |gamma1|, |gamma2| at the nodes
+// (HESS), added to what is there.
+template <int MODE, int P>
+__device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short *list, int n_far, int n_far_h,
+                                          df Tx, df Ty, const float2 *s_nx, const float2 *s_ny, float4 *s_rec,
+                                          float4 *s_off, float2 *s_part, float2 *s_val, float *s_kb) {
+  constexpr int NODES = P * P, PAIRS = NODES / 2, SPLITS = FF_THREADS / PAIRS, NC = ncmp(MODE), NV = nval(MODE);
+  const int tid = threadIdx.x, split = tid / PAIRS, pr = tid % PAIRS, ix = pr % P, jy = 2 * (pr / P);
+  const bool active = split < SPLITS;
+  Sums<MODE> S;
+  S.zero();
+  const float2 ox = s_nx[ix], y0 = s_ny[jy], y1 = s_ny[jy + 1];
+  for (int c0 = 0; c0 < n_far; c0 += FF_CH) {
+    const int cnt = min(FF_CH, n_far - c0);
+    if (c0) __syncthreads();  // the previous chunk has been used
+    stage_chunk(a, list + c0, cnt, Tx, Ty, s_rec, s_off);
+    __syncthreads();
+    if (active)
+      S.sweep(s_rec, s_off, split, cnt, SPLITS, ox, make_float2(y0.x, y1.x), make_float2(y0.y, y1.y));
+  }
+  S.fold();
+  if (active) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      float2 *o = s_part + ((size_t)split * NODES + (jy + h) * P + ix) * NC;
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        const df v = S.value(c, h);
+        o[c] = make_float2(v.hi, v.lo);
+      }
+      if (MODE != FAR_POT) o[NV] = make_float2(S.mag(h), 0.f);
+    }
+  }
+  __syncthreads();
+  for (int q = tid; q < NODES * NC; q += FF_THREADS) {
+    df v = {s_part[q].x, s_part[q].y};
+    for (int s = 1; s < SPLITS; ++s) {
+      const float2 t = s_part[(size_t)s * NODES * NC + q];
+      v = df_add(v, df{t.x, t.y});
+    }
+    const int node = q / NC, c = q % NC;
+    s_val[c * NODES + node] = make_float2(v.hi, v.lo);
+    if (MODE == FAR_HESS && c >= 2 && c < 5)
+      atomicMax(reinterpret_cast<int *>(s_kb) + c - 2, __float_as_int(fabsf(v.hi)));
+  }
+  __syncthreads();
+  if (n_far_h > 0) {
+    for (int node = tid; node < NODES; node += FF_THREADS) {
+      const float2 nx = s_nx[node % P], ny = s_ny[node / P];
+      const df X = df_add(Tx, df{nx.x, nx.y}), Y = df_add(Ty, df{ny.x, ny.y});
+      df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+      for (int k = 0; k < n_far_h; ++k) {
+        const int h = list[n_far + k];
+        add_heavy<MODE>(a.heavydf + (size_t)h * RECDF, a.heavy + (size_t)h * REC64, X, Y, sum);
+      }
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        float2 &o = s_val[c * NODES + node];
+        const df v = df_add(df{o.x, o.y}, sum[c]);
+        o = make_float2(v.hi, v.lo);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Plane of value c: the middle node's value and slopes (per grid step)
+// between the outermost nodes of the middle row and column.
+template <int P>
+__device__ __forceinline__ float4 plane_of(const float2 *v, float span) {
+  const int m = P / 2;
+  return make_float4(v[m * P + m].x, slope8((v[m * P].x - v[m * P + P - 1].x) / span),
+                     slope8((v[m].x - v[(P - 1) * P + m].x) / span), 0.f);
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(FF_THREADS, 2) k_far_coarse(const FarArgs a) {
+  constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), SPLITS = FF_THREADS / (NODES / 2);
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);
+  float4 *s_off = s_rec + FF_CH * REC_STRIDE4;
+  float2 *s_part = reinterpret_cast<float2 *>(s_off + FF_CH);
+  float2 *s_val = s_part + SPLITS * NODES * NC;
+  unsigned *s_far = reinterpret_cast<unsigned *>(s_val + NODES * NC);
+  unsigned *s_near = s_far + a.nw;
+  unsigned short *s_list = reinterpret_cast<unsigned short *>(s_near + 3 * a.nw);
+  __shared__ float2 s_nx[CP], s_ny[CP];
+  __shared__ float s_kb[4];
+  __shared__ float4 s_plane[NV];
+  __shared__ int s_cnt[4];
+  const int tid = threadIdx.x, tile = blockIdx.y * a.nct + blockIdx.x;
+  const double half = 0.5 * a.ct;
+  // centre of the tile: half a step past its middle node pair's first
+  const df Tx = df_from_double(a.xmin + (blockIdx.x * (double)a.ct + half - 0.5) * a.dx);
+  const df Ty = df_from_double(a.ymin + (blockIdx.y * (double)a.ct + half - 0.5) * a.dy);
+  if (tid < CP) {
+    // the coarse basis is laid out about the centre of the tile's fine
+    // tiles, each 32 steps wide about its own centre: the same point
+    const df ox = df_from_double(D_ZC[tid] * half * a.dx), oy = df_from_double(D_ZC[tid] * half * a.dy);
+    s_nx[tid] = make_float2(ox.hi, ox.lo);
+    s_ny[tid] = make_float2(oy.hi, oy.lo);
+  }
+  if (tid < 4) s_kb[tid] = 0.f;
+  classify(a, nullptr, Tx, Ty, a.thr_c, a.thr_ch, s_far, s_near, s_list, s_cnt);
+  for (int w = tid; w < a.nw; w += FF_THREADS) a.cmask[(size_t)tile * a.nw + w] = s_near[w];
+  node_sums<MODE, CP>(a, s_list, s_cnt[0], s_cnt[1], Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
+  if (tid < NV) s_plane[tid] = plane_of<CP>(s_val + tid * NODES, (D_ZC[0] - D_ZC[CP - 1]) * (float)half);
+  __syncthreads();
+  float *o = a.cval + (size_t)tile * coarse_floats(MODE);
+  for (int q = tid; q < NODES * NC; q += FF_THREADS) {
+    const int c = q / NODES, node = q % NODES;
+    const float2 v = s_val[q];
+    float r = v.x;
+    if (c < NV) {
+      const float4 p = s_plane[c];
+      const float zx = D_ZC[node % CP] * (float)half, zy = D_ZC[node / CP] * (float)half;
+      df d = df_sub(df{v.x, v.y}, df{p.x, 0.f});
+      d = df_sub(d, df{p.y * zx, 0.f});
+      d = df_sub(d, df{p.z * zy, 0.f});
+      r = d.hi + d.lo;
+    }
+    o[q] = r;
+  }
+  if (tid < NV * 4) o[NC * NODES + tid] = reinterpret_cast<const float *>(s_plane)[tid];
+  if (tid < 4) o[NC * NODES + NV * 4 + tid] = s_kb[tid];
+}
+
+// 1 / (hi + lo), one Newton step on the MUFU reciprocal
+__device__ __forceinline__ float rcp_dff(float hi, float lo) {
+  const float r = rcp_a(hi);
+  const float e = fmaf(-lo, r, fmaf(-hi, r, 1.f));
+  return fabsf(e) < 1e-3f ? fmaf(r, e, r) : 1.f / hi;
+}
+
+template <int MODE>
+__global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
+  constexpr bool HESS = MODE == FAR_HESS, POT = MODE == FAR_POT;
+  constexpr int NODES = FP * FP, NC = ncmp(MODE), NV = nval(MODE), NC2 = ncmp2(MODE), SPLITS = FF_THREADS / (NODES / 2);
+  extern __shared__ __align__(16) unsigned char s_dyn[];
+  float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);                      // [FF_CH][REC_STRIDE4]
+  float4 *s_off = s_rec + FF_CH * REC_STRIDE4;                            // [FF_CH]
+  float4 *s_c = s_off + FF_CH;                                            // [FT / 2][FP][NC2]: row-pair coefficients
+  float2 *s_part = reinterpret_cast<float2 *>(s_c + (FT / 2) * FP * NC2);  // [SPLITS][NODES][NC]
+  float2 *s_val = s_part + SPLITS * NODES * NC;                           // [NC][NODES]
+  unsigned *s_far = reinterpret_cast<unsigned *>(s_val + NODES * NC);
+  unsigned *s_near = s_far + a.nw;
+  unsigned short *s_list = reinterpret_cast<unsigned short *>(s_near + 3 * a.nw);
+  float *s_tmp = reinterpret_cast<float *>(s_part);  // coarse level: [NC][CP * CP] values, [NC][FP][CP] (after node_sums)
+  float *s_rem = s_tmp;                              // then the remainders [NC][NODES]
+  __shared__ float2 s_nx[FP], s_ny[FP];
+  __shared__ float s_L[FT][FP];
+  __shared__ float s_kb[4];
+  __shared__ float4 s_plane[NV];
+  __shared__ int s_cnt[4];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int i0 = blockIdx.x * FT, j0 = a.row0 + blockIdx.y * FT;  // grid column and row of the tile's first node
+  const df Tx = df_from_double(a.xmin + (i0 + 15.5) * a.dx), Ty = df_from_double(a.ymin + (j0 + 15.5) * a.dy);
+  if (tid < FP) {
+    const df ox = df_from_double(D_XI[tid] * a.dx), oy = df_from_double(D_XI[tid] * a.dy);
+    s_nx[tid] = make_float2(ox.hi, ox.lo);
+    s_ny[tid] = make_float2(oy.hi, oy.lo);
+  }
+  if (tid < 4) s_kb[tid] = 0.f;
+  for (int q = tid; q < FT * FP; q += FF_THREADS) (&s_L[0][0])[q] = (&D_FINE.w[0][0])[q];
+  const int ctile = a.ct ? (j0 / a.ct) * a.nct + i0 / a.ct : 0;
+  classify(a, a.ct ? a.cmask + (size_t)ctile * a.nw : nullptr, Tx, Ty, a.thr_f, a.thr_fh, s_far, s_near, s_list, s_cnt);
+  const int n_far = s_cnt[0], n_far_h = s_cnt[1], n_near = s_cnt[2], n_near_h = s_cnt[3];
+  node_sums<MODE, FP>(a, s_list, n_far, n_far_h, Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
+  if (a.ct) {
+    // the coarse tile's interpolant at this tile's nodes: rows of the tensor
+    // product, then columns; its plane (exact products) in double-float
+    const float *cv = a.cval + (size_t)ctile * coarse_floats(MODE);
+    const int sub = a.ct / FT, cx = (i0 % a.ct) / FT, cy = (j0 % a.ct) / FT;
+    const float *W = sub == 2 ? &D_CO2.w[0][0][0] : sub == 4 ? &D_CO4.w[0][0][0] : sub == 8 ? &D_CO8.w[0][0][0] : &D_CO16.w[0][0][0];
+    const float *Wx = W + cx * FP * CP, *Wy = W + cy * FP * CP;
+    float *s_t1 = s_tmp + NC * CP * CP;
+    for (int q = tid; q < NC * CP * CP; q += FF_THREADS) s_tmp[q] = cv[q];
+    __syncthreads();
+    for (int q = tid; q < NC * CP * FP; q += FF_THREADS) {  // (c, coarse row, fine column)
+      const int i = q % FP, cr = q / FP;
+      const float *f = s_tmp + cr * CP;
+      float v = 0.f;
+#pragma unroll
+      for (int k = 0; k < CP; ++k) v = fmaf(Wx[i * CP + k], f[k], v);
+      s_t1[q] = v;
+    }
+    __syncthreads();
+    const float bx0 = 32.f * cx + 16.f - 16.f * sub, by0 = 32.f * cy + 16.f - 16.f * sub;
+    for (int q = tid; q < NC * NODES; q += FF_THREADS) {
+      const int c = q / NODES, node = q % NODES, i = node % FP, j = node / FP;
+      float v = 0.f;
+#pragma unroll
+      for (int k = 0; k < CP; ++k) v = fmaf(Wy[j * CP + k], s_t1[(c * CP + k) * FP + i], v);
+      df d = {s_val[q].x, s_val[q].y};
+      d = df_add(d, df{v, 0.f});
+      if (c < NV) {
+        const float *p = cv + NC * CP * CP + c * 4;
+        d = df_add(d, df{p[0], 0.f});
+        d = df_add(d, df{p[1] * (bx0 + D_XI[i]), 0.f});
+        d = df_add(d, df{p[2] * (by0 + D_XI[j]), 0.f});
+      }
+      s_val[q] = make_float2(d.hi, d.lo);
+    }
+    if (HESS && tid < 3) s_kb[tid] += cv[NC * CP * CP + NV * 4 + tid];
+    __syncthreads();
+  }
+  if (tid < NV) s_plane[tid] = plane_of<FP>(s_val + tid * NODES, D_XI[0] - D_XI[FP - 1]);
+  __syncthreads();
+  for (int q = tid; q < NC * NODES; q += FF_THREADS) {
+    const int c = q / NODES, node = q % NODES;
+    const float2 v = s_val[q];
+    float r = v.x;
+    if (c < NV) {
+      const float4 p = s_plane[c];
+      df d = df_sub(df{v.x, v.y}, df{p.x, 0.f});
+      d = df_sub(d, df{p.y * D_XI[node % FP], 0.f});
+      d = df_sub(d, df{p.z * D_XI[node / FP], 0.f});
+      r = d.hi + d.lo;
+    }
+    s_rem[q] = r;
+  }
+  __syncthreads();
+  // coefficients of every row pair: the remainders interpolated in y at the
+  // tile's rows, one float4 = two values at two rows
+  for (int q = tid; q < (FT / 2) * FP * NC2 * 2; q += FF_THREADS) {
+    const int c = q % (2 * NC2), i = q / (2 * NC2) % FP, rp = q / (2 * NC2 * FP);
+    float u = 0.f, v = 0.f;
+    if (c < NC) {
+#pragma unroll
+      for (int j = 0; j < FP; ++j) {
+        const float f = s_rem[c * NODES + j * FP + i];
+        u = fmaf(s_L[2 * rp][j], f, u);
+        v = fmaf(s_L[2 * rp + 1][j], f, v);
+      }
+    }
+    reinterpret_cast<float2 *>(s_c)[q] = make_float2(u, v);
+  }
+  // the near potentials and the interpolant at the map nodes: lane = column,
+  // a warp takes row pairs warp, warp + FF_WARPS
+  const float mx = lane - 15.5f;
+  const double lx = mx * a.dx;
+  const float lxh = (float)lx;
+  const float2 ox = make_float2(lxh, (float)(lx - (double)lxh));
+  const int i = i0 + lane;
+  float Lx[FP];
+  bool staged = false;
+#pragma unroll 1
+  for (int rp = warp; rp < FT / 2; rp += FF_WARPS) {
+    float2 oyh, oyl;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const double ly = (2 * rp + h - 15.5) * a.dy;
+      const float f = (float)ly;
+      part2(oyh, h) = f;
+      part2(oyl, h) = (float)(ly - (double)f);
+    }
+    Sums<MODE> S;
+    S.zero();
+    for (int c0 = 0; c0 < n_near || (c0 == 0 && !staged); c0 += FF_CH) {
+      const int cnt = min(FF_CH, n_near - c0);
+      if (n_near > FF_CH || !staged) {
+        __syncthreads();
+        stage_chunk(a, s_list + n_far + n_far_h + c0, cnt, Tx, Ty, s_rec, s_off);
+        __syncthreads();
+        staged = true;
+      }
+      S.sweep(s_rec, s_off, 0, cnt, 1, ox, oyh, oyl);
+    }
+    S.fold();
+#pragma unroll
+    for (int k = 0; k < FP; ++k) Lx[k] = s_L[lane][k];
+    float2 v[2 * NC2];
+#pragma unroll
+    for (int c = 0; c < 2 * NC2; ++c) v[c] = make_float2(0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < FP; ++k)
+#pragma unroll
+      for (int c = 0; c < NC2; ++c) {
+        const float4 t = s_c[(rp * FP + k) * NC2 + c];
+        v[2 * c] = fma2(dup2(Lx[k]), make_float2(t.x, t.y), v[2 * c]);
+        v[2 * c + 1] = fma2(dup2(Lx[k]), make_float2(t.z, t.w), v[2 * c + 1]);
+      }
+    // plane + near + remainder, per value and point pair, in double-float
+    const float2 my = make_float2(2 * rp - 15.5f, 2 * rp - 14.5f);
+    float2 vh[NV], vl[NV];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+      const float4 p = s_plane[c];
+      const df x = two_sum(p.x, p.y * mx);
+      const df2 y = two_sum2(dup2(x.hi), mul2(dup2(p.z), my));
+      const df n0 = S.value(c, 0), n1 = S.value(c, 1);
+      const df2 z = two_sum2(y.hi, make_float2(n0.hi, n1.hi));
+      float2 lo = add2(add2(y.lo, dup2(x.lo)), add2(z.lo, make_float2(n0.lo, n1.lo)));
+      lo = add2(lo, v[c]);
+      const df2 r = two_sum2(z.hi, lo);
+      vh[c] = r.hi;
+      vl[c] = r.lo;
+    }
+    if (n_near_h > 0) {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        const df X = df_add(Tx, df{ox.x, ox.y}), Y = df_add(Ty, df{h ? oyh.y : oyh.x, h ? oyl.y : oyl.x});
+        df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+        for (int k = 0; k < n_near_h; ++k) {
+          const int hh = s_list[n_far + n_far_h + n_near + k];
+          add_heavy<MODE>(a.heavydf + (size_t)hh * RECDF, a.heavy + (size_t)hh * REC64, X, Y, sum);
+        }
+#pragma unroll
+        for (int c = 0; c < NV; ++c) {
+          const df t = df_add(df{h ? vh[c].y : vh[c].x, h ? vl[c].y : vl[c].x}, sum[c]);
+          if (h) {
+            vh[c].y = t.hi;
+            vl[c].y = t.lo;
+          } else {
+            vh[c].x = t.hi;
+            vl[c].x = t.lo;
+          }
+        }
+      }
+    }
+    const int jl = blockIdx.y * FT + 2 * rp;  // row of the launch
+    if constexpr (POT) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int j = jl + h;
+        if (i < a.nx && j < a.ny) {
+          const long long o = (long long)j * a.nx + i;
+          const double phi = a.dls * ((double)part2(vh[0], h) + (double)part2(vl[0], h));
+          a.out64[o] = phi;
+          if (a.tau) {
+            const double X = a.xmin + i * a.dx - a.bx, Y = a.ymin + (a.row0 + j) * a.dy - a.by;
+            a.out64[a.plane + o] = 0.5 * (X * X + Y * Y) - phi;
+          }
+        }
+      }
+    } else {
+      const float dh = (float)a.dls, dl = (float)(a.dls - (double)dh);
+      // which nodes the double-float repair recomputes (see k_map_mixed);
+      // the far potentials' kappa and gamma enter by their bounds on the tile
+      if (a.repair_f > 0.f) {
+        bool rep[2], rep_h[2] = {false, false};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const bool in = i < a.nx && jl + h < a.ny;
+          const float m = a.repair_f * (part2(v[NV], h) + S.mag(h)), fx = part2(vh[0], h), fy = part2(vh[1], h);
+          rep[h] = in && fmaf(fx, fx, fy * fy) < m * m;
+          if (HESS) {
+            const float kl = dh * (fabsf(S.value(2, h).hi) + s_kb[0]);
+            const float g1l = dh * (fabsf(S.value(3, h).hi) + s_kb[1]), g2l = dh * (fabsf(S.value(4, h).hi) + s_kb[2]);
+            const float kap = dh * part2(vh[NV > 2 ? 2 : 0], h), g1 = dh * part2(vh[NV > 3 ? 3 : 0], h),
+                        g2 = dh * part2(vh[NV > 4 ? 4 : 0], h);
+            const float gm = sqrtf(fmaf(g1, g1, g2 * g2)), gl = sqrtf(fmaf(g1l, g1l, g2l * g2l));
+            rep_h[h] = in && (float)(2.0 * DET_TERM_ERR) * (fabsf(1.f - kap) * kl + gm * (kl + gl)) > (float)DET_REPAIR_ABS;
+          }
+        }
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const unsigned mask = __ballot_sync(0xffffffffu, rep[h] || rep_h[h]);
+          if (mask) {
+            int first = 0;
+            if (lane == __ffs(mask) - 1) first = atomicAdd(a.rep_count, __popc(mask));
+            first = __shfl_sync(0xffffffffu, first, __ffs(mask) - 1);
+            if (rep[h] || rep_h[h])
+              a.rep_list[first + __popc(mask & ((1u << lane) - 1u))] =
+                  ((jl + h) * a.nx + i) | (rep_h[h] ? (int)0x80000000u : 0);
+          }
+        }
+      }
+      // scaled by D_ls/D_s in double-float, rounded once
+#pragma unroll
+      for (int c = 0; c < NV; ++c) {
+        const float2 p = mul2(vh[c], dup2(dh));
+        const float2 e = fma2(vl[c], dup2(dh), fma2(vh[c], dup2(dl), fma2(vh[c], dup2(dh), neg2(p))));
+        vh[c] = add2(p, e);
+        vl[c] = sub2(e, sub2(vh[c], p));
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int j = jl + h;
+        if (i >= a.nx || j >= a.ny) continue;
+        float *o = a.out + (long long)j * a.nx + i;
+        o[0] = part2(vh[0], h);
+        o[a.plane] = part2(vh[1], h);
+        if constexpr (HESS) {
+          const float kh = part2(vh[2], h), kl = part2(vl[2], h), g1 = part2(vh[3], h), g1l = part2(vl[3], h),
+                      g2 = part2(vh[4], h), g2l = part2(vl[4], h);
+          // det = (1 - kappa)^2 - gamma1^2 - gamma2^2 with the products' errors
+          df om = two_sum(1.f, -kh);
+          om = fast_two_sum(om.hi, om.lo - kl);
+          const float p0 = __fmul_rn(om.hi, om.hi), p1 = __fmul_rn(g1, g1), p2 = __fmul_rn(g2, g2);
+          const float e0 = fmaf(2.f * om.hi, om.lo, fmaf(om.hi, om.hi, -p0));
+          const float e1 = fmaf(2.f * g1, g1l, fmaf(g1, g1, -p1)), e2 = fmaf(2.f * g2, g2l, fmaf(g2, g2, -p2));
+          const df d0 = two_sum(p0, -p1), d1 = two_sum(d0.hi, -p2);
+          const df det = fast_two_sum(d1.hi, (d0.lo + d1.lo) + (e0 - (e1 + e2)));
+          o[2 * a.plane] = kh;
+          o[3 * a.plane] = g1;
+          o[4 * a.plane] = g2;
+          o[5 * a.plane] = rcp_dff(det.hi, det.lo);
+        }
+      }
+    }
+  }
+}
+
+size_t far_smem(int mode, bool coarse, int nw, int n) {
+  const int nodes = coarse ? CP * CP : FP * FP, splits = FF_THREADS / (nodes / 2), nc = ncmp(mode);
+  size_t b = sizeof(float4) * (FF_CH * REC_STRIDE4 + FF_CH);
+  if (!coarse) b += sizeof(float4) * (FT / 2) * FP * ncmp2(mode);
+  // the partial sums' space also holds the coarse tile's values (fine kernel)
+  const size_t part = std::max(sizeof(float2) * splits * nodes * nc, coarse ? 0 : sizeof(float) * nc * (CP * CP + CP * FP));
+  b += (part + 15) / 16 * 16 + sizeof(float2) * nodes * nc;
+  b += sizeof(unsigned) * 4 * (size_t)nw + sizeof(unsigned short) * (size_t)n;
+  return (b + 15) / 16 * 16;
+}
+
+// Margins: squared psi (K R)^2 of the tile's half-diagonal R beyond which a
+// potential is far.  The FP32 potentials' interpolation error stays below
+// 1.2e-8 of the term; the cluster-scale ones', whose deflection is ten times
+// the rest, below 1e-9.
+constexpr double KF = 3.0, KF_H = 3.5, KC = 2.5, KC_H = 3.0;
+constexpr int FAR_MAX_N = 16384;  // potentials (two bytes each of shared memory)
+
+// Fraction of the map's nodes within psi < r of a potential of axis ratio q
+// and core s: the area of the ellipse q^2 (s^2 + x^2) + y^2 < r^2.
+double near_frac(double r, double q, double s, double area) {
+  const double r2 = r * r - q * q * s * s;
+  return r2 <= 0.0 ? 0.0 : std::min(1.0, M_PI * r2 / (q * area));
+}
+
+// The lists' and masks' words, and what a launch of this size needs.
+int far_words(const Model *m) { return (m->n_light + 31) / 32 + (m->n_heavy + 31) / 32; }
+
+}  // namespace
+
+// Expected cost per map node of the direct kernel and of the interpolated
+// one with each coarse level, in evaluations of one FP32 potential (HV of
+// them for a cluster-scale potential in double-float), idle SMs of small
+// grids included.
+FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode) {
+  (void)ctx;
+  FarPlan p;
+  if (m->n > FAR_MAX_N || m->n < 1) return p;
+  const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
+  const double area = (g->xmax - g->xmin) * (g->ymax - g->ymin), nodes = (double)g->nx * g->ny;
+  const double HV = mode == FAR_HESS ? 20.0 : 10.0, step = std::max(dx, dy);
+  const double Rf = std::sqrt(2.0) * 15.5 * step;
+  auto light = [&](double r) { return m->n_light * near_frac(r, 1.0 / m->invq_light, 0.0, area); };
+  auto heavy = [&](double r) {
+    double s = 0.0;
+    for (const auto &h : m->heavy_shape) s += near_frac(r, h.first, h.second, area);
+    return s;
+  };
+  const double direct = (m->n_light + HV * m->n_heavy + 2.0) * std::max(1.0, 608.0 * 256.0 / nodes);
+  const double tiles = std::ceil(g->nx / (double)FT) * std::ceil(g->ny / (double)FT);
+  const double near = light(KF * Rf) + HV * heavy(KF_H * Rf);
+  double best = 0.85 * direct;
+  for (int ct = 0; ct <= CT_MAX; ct = ct ? 2 * ct : CT_MIN) {
+    if (ct && ct >= 2 * std::max(g->nx, g->ny)) break;
+    double mid = m->n_light, mid_h = m->n_heavy, coarse = 0.0;
+    if (ct) {
+      const double Rc = std::sqrt(2.0) * 0.5 * ct * step;
+      const double ctiles = std::ceil(g->nx / (double)ct) * std::ceil(g->ny / (double)ct);
+      coarse = (m->n_light + 2.0 * HV * m->n_heavy) * 170.0 * ctiles / nodes * std::max(1.0, 152.0 / ctiles);
+      mid = light(KC * Rc);
+      mid_h = heavy(KC_H * Rc);
+    }
+    const double fine = (mid + 2.5 * HV * mid_h) * (FP * FP) / (double)(FT * FT);
+    const double c = coarse + (6.0 + fine + near) * tiles * FT * FT / nodes * std::max(1.0, 304.0 / tiles);
+    if (c < best) {
+      best = c;
+      p.use = true;
+      p.ct = ct;
+      p.cost = c;
+    }
+  }
+  if (p.use && p.ct) {
+    p.nct = (g->nx + p.ct - 1) / p.ct;
+    p.ncr = (g->ny + p.ct - 1) / p.ct;
+    const size_t t = (size_t)p.nct * p.ncr;
+    p.val_bytes = (t * coarse_floats(mode) * sizeof(float) + 255) & ~(size_t)255;
+    p.bytes = p.val_bytes + t * far_words(m) * sizeof(unsigned);
+  }
+  return p;
+}
+
+static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem) {
+  FarArgs a;
+  a.rec32 = m->rec32;
+  a.cen32 = (const float4 *)m->cen32;
+  a.n_light = m->n_light;
+  a.heavy = m->heavy;
+  a.heavydf = m->heavydf;
+  a.n_heavy = m->n_heavy;
+  a.nwl = (m->n_light + 31) / 32;
+  a.nw = far_words(m);
+  a.xmin = g->xmin;
+  a.ymin = g->ymin;
+  a.dx = (g->xmax - g->xmin) / (g->nx - 1);
+  a.dy = (g->ymax - g->ymin) / (g->ny - 1);
+  a.nx = g->nx;
+  a.ny = g->ny;
+  a.row0 = 0;
+  a.dls = 1.0;
+  const double step = std::sqrt(2.0) * std::max(a.dx, a.dy), rf = 15.5 * step, rc = 0.5 * p.ct * step;
+  auto sq = [](double v) { return (float)(v * v); };
+  a.thr_c = sq(KC * rc);
+  a.thr_ch = sq(KC_H * rc);
+  a.thr_f = sq(KF * rf);
+  a.thr_fh = sq(KF_H * rf);
+  a.ct = p.ct;
+  a.nct = p.nct;
+  a.cval = (float *)mem;
+  a.cmask = (unsigned *)((char *)mem + p.val_bytes);
+  a.out = nullptr;
+  a.out64 = nullptr;
+  a.plane = 0;
+  a.tau = 0;
+  a.bx = a.by = 0.0;
+  a.repair_f = 0.f;
+  a.rep_count = a.rep_list = nullptr;
+  return a;
+}
+
+template <int MODE>
+static int coarse_launch(const FarArgs &a, const FarPlan &p, int n, cudaStream_t st) {
+  const size_t smem = far_smem(MODE, true, a.nw, n);
+  cudaFuncSetAttribute(k_far_coarse<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_far_coarse<MODE><<<dim3(p.nct, p.ncr), FF_THREADS, smem, st>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LENS_ECUDA, "coarse map level launch: %s", cudaGetErrorString(e));
+  return LENS_OK;
+}
+
+template <int MODE>
+static int fine_launch(const FarArgs &a, int n, cudaStream_t st) {
+  const size_t smem = far_smem(MODE, false, a.nw, n);
+  cudaFuncSetAttribute(k_far_map<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_far_map<MODE><<<dim3((a.nx + FT - 1) / FT, (a.ny + FT - 1) / FT), FF_THREADS, smem, st>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LENS_ECUDA, "interpolated map launch: %s", cudaGetErrorString(e));
+  return LENS_OK;
+}
+
+int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st) {
+  if (!p.ct) return LENS_OK;
+  const FarArgs a = far_args(m, g, p, mode, mem);
+  return mode == FAR_HESS   ? coarse_launch<FAR_HESS>(a, p, m->n, st)
+         : mode == FAR_GRAD ? coarse_launch<FAR_GRAD>(a, p, m->n, st)
+                            : coarse_launch<FAR_POT>(a, p, m->n, st);
+}
+
+int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, double dls, void *out,
+                   int row0, int rows, double repair, int *rep_count, int *rep_list, const double *beta,
+                   cudaStream_t st) {
+  FarArgs a = far_args(m, g, p, mode, mem);
+  a.ny = rows;
+  a.row0 = row0;
+  a.dls = dls;
+  a.plane = (long long)g->nx * rows;
+  a.repair_f = (float)(2.0 * repair);
+  a.rep_count = rep_count;
+  a.rep_list = rep_list;
+  if (mode == FAR_POT) {
+    a.out64 = (double *)out;
+    a.tau = beta != nullptr;
+    a.bx = beta ? beta[0] : 0.0;
+    a.by = beta ? beta[1] : 0.0;
+    return fine_launch<FAR_POT>(a, m->n, st);
+  }
+  a.out = (float *)out;
+  return mode == FAR_HESS ? fine_launch<FAR_HESS>(a, m->n, st) : fine_launch<FAR_GRAD>(a, m->n, st);
+}
+
+}  // namespace lens

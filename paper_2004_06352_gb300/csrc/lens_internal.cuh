@@ -229,6 +229,10 @@ struct Model {
   float2 *heavydf = nullptr;  // [n_heavy][RECDF] double-float records of the heavy potentials (image refinement)
   std::vector<lens_halo> host;
   size_t bytes = 0;
+  // for the map kernels' choice: mean 1/q of the FP32 potentials, axis ratio
+  // and core of each cluster-scale one
+  double invq_light = 1.0;
+  std::vector<std::pair<double, double>> heavy_shape;
 };
 
 struct GridCache {
@@ -343,7 +347,8 @@ struct CallScratch {
   size_t bytes = 0;
   CallScratch(lens_ctx *c, cudaStream_t s) : ctx(c), st(s) {}
   int alloc(size_t n);
-  ~CallScratch();
+  void release();  // freed on st now
+  ~CallScratch() { release(); }
   CallScratch(const CallScratch &) = delete;
   CallScratch &operator=(const CallScratch &) = delete;
 };
@@ -366,15 +371,31 @@ int check_grid(const lens_grid *g);
 // image search's static deflection, which must allocate nothing there).
 // repair_mem: memory for the repair list (map_repair_bytes), else working
 // memory of the call.
+// far, far_mem: the interpolated form (lens_far.cu) with this plan, whose
+// coarse level has been computed into far_mem; NULL: direct.
+struct FarPlan {
+  bool use = false;
+  int ct = 0, nct = 0, ncr = 0;  // coarse tile (0: no coarse level), coarse tiles per row and column
+  size_t val_bytes = 0, bytes = 0;
+  double cost = 0.0;             // expected cost per node in evaluations of one FP32 potential
+};
 int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
-                     cudaStream_t st, int row0 = 0, int rows = -1, bool repair = true, void *repair_mem = nullptr);
+                     cudaStream_t st, int row0 = 0, int rows = -1, bool repair = true, void *repair_mem = nullptr,
+                     const FarPlan *far = nullptr, void *far_mem = nullptr);
+// modes of the interpolated maps: 0 deflection, 1 deflection + Hessian, 2 potential
+constexpr int FAR_TILE_ROWS = 32;  // rows of a band must be a multiple of this
+FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode);
+int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st);
+int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, double dls, void *out,
+                   int row0, int rows, double repair, int *rep_count, int *rep_list, const double *beta,
+                   cudaStream_t st);
 size_t map_repair_bytes(const lens_grid *g, int rows = -1);
 int launch_map_fp64(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
                     cudaStream_t st, int row0 = 0, int rows = -1);
 int map_tile_rows(bool hess);  // rows per CTA tile of the mixed map kernel
 // potential map (and, when beta is not NULL, the Fermat potential about beta)
 int launch_pot_map(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, int32_t precision,
-                   const double *beta, void *out, cudaStream_t st);
+                   const double *beta, void *out, cudaStream_t st);  // (LENS_MIXED: interpolated where that is cheaper)
 int launch_wait_selftest(lens_ctx *ctx, unsigned polls, cudaStream_t st);
 int launch_math_selftest(const double *x, int n, double *out, cudaStream_t st);
 int launch_mcmc_step(lens_ctx *ctx, const Model *m, const CSet *c, double *d_params, double *d_chi2, int32_t W,

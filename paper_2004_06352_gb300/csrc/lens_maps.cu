@@ -655,7 +655,8 @@ size_t map_repair_bytes(const lens_grid *g, int rows) {
 }
 
 int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
-                     cudaStream_t st, int row0, int rows, bool repair, void *repair_mem) {
+                     cudaStream_t st, int row0, int rows, bool repair, void *repair_mem, const FarPlan *far,
+                     void *far_mem) {
   if (rows < 0) rows = g->ny - row0;
   const long long nodes = (long long)g->nx * rows;
   if (nodes > INT32_MAX) return fail(LENS_EINVAL, "map launch of more than 2^31 points");
@@ -700,7 +701,11 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
   a.rep_count = repair ? (int *)repair_mem : nullptr;
   a.rep_list = repair ? (int *)repair_mem + 1 : nullptr;
   constexpr int KPG = LENS_KP_GRAD, KPH = LENS_KP_HESS;
-  if (hess) {
+  if (far) {
+    const int rc = launch_far_map(m, g, *far, hess, far_mem, dls, out, row0, rows, a.repair, a.rep_count, a.rep_list,
+                                  nullptr, st);
+    if (rc) return rc;
+  } else if (hess) {
     const int th = map_tile_rows(true);
     dim3 grid((g->nx + 31) / 32, (rows + th - 1) / th);
     k_map_mixed<MAP_HESS, KPH><<<grid, map_threads(true), 0, st>>>(a);
@@ -770,6 +775,13 @@ int launch_pot_map(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls
                                                  (double *)out, plane, beta != nullptr, beta ? beta[0] : 0.0,
                                                  beta ? beta[1] : 0.0);
   } else {
+    FarPlan plan = plan_far(ctx, m, g, 2);
+    CallScratch far(ctx, st);  // the coarse level's values
+    if (plan.use && plan.ct && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
+    if (plan.use) {
+      const int rc = launch_far_coarse(m, g, plan, 2, far.p, st);
+      return rc ? rc : launch_far_map(m, g, plan, 2, far.p, dls, out, 0, rows, 0.0, nullptr, nullptr, beta, st);
+    }
     MapArgs a;
     a.rec32 = m->rec32;
     a.pos64 = m->pos64;

@@ -87,6 +87,7 @@ struct Req {
   std::vector<double> params;
   size_t out_bytes = 0, in_bytes = 0, scratch_bytes = 0, total = 0, off = 0;
   int32_t batch = 0;
+  FarPlan far;  // maps: the interpolated form's plan, its coarse level after the repair list
   double t_submit = 0, t_admit = 0;
   double cost_ms = 0;  // expected GPU time
   int skips = 0;
@@ -143,9 +144,13 @@ static int launch_req(lens_server *s, Slot &sl, Req *q) {
     if (!m) return fail(LENS_ENOTFOUND, "model released while its request was queued");
     if (r.precision == LENS_FP64)
       rc = launch_map_fp64(ctx, m, &r.grid, r.dls_ds, r.hessian != 0, base, st);
-    else  // the repair list in the request's own arena memory, after its output
-      rc = launch_map_mixed(ctx, m, &r.grid, r.dls_ds, r.hessian != 0, base, st, 0, -1, true,
-                            base + up(q->out_bytes));
+    else {  // the repair list and the coarse level in the request's own arena memory, after its output
+      char *list = base + up(q->out_bytes), *far_mem = list + up(map_repair_bytes(&r.grid));
+      if (q->far.use) rc = launch_far_coarse(m, &r.grid, q->far, r.hessian != 0, far_mem, st);
+      if (!rc)
+        rc = launch_map_mixed(ctx, m, &r.grid, r.dls_ds, r.hessian != 0, base, st, 0, -1, true, list,
+                              q->far.use ? &q->far : nullptr, far_mem);
+    }
   } else {
     CSet *c = find_cset(ctx, r.handle);
     Model *m = c ? find_model(ctx, c->model) : nullptr;
@@ -230,7 +235,15 @@ int lens_server_submit(lens_server *s, const lens_request *r, int64_t *ticket) {
     } else if (!(std::isfinite(r->dls_ds) && r->dls_ds > 0)) rc = fail(LENS_EINVAL, "dls_ds must be > 0");
     else if (r->precision != LENS_FP64 && r->precision != LENS_MIXED) rc = fail(LENS_EINVAL, "bad precision");
     q->out_bytes = map_out_bytes(*r);
-    if (r->precision == LENS_MIXED) q->scratch_bytes = map_repair_bytes(&r->grid);
+    if (!rc && r->precision == LENS_MIXED) {
+      q->scratch_bytes = map_repair_bytes(&r->grid);
+      q->far = plan_far(ctx, find_model(ctx, r->handle), &r->grid, r->hessian != 0);
+      const size_t with = up(q->scratch_bytes) + up(q->far.bytes);
+      if (up(q->out_bytes) + with <= s->pool_bytes)
+        q->scratch_bytes = with;
+      else if (q->far.bytes)
+        q->far = FarPlan();  // only the direct kernel fits the pool
+    }
   } else if (r->kind == LENS_REQ_CHI2_SOURCE || r->kind == LENS_REQ_CHI2_IMAGE) {
     CSet *c = find_cset(ctx, r->handle);
     if (!c) rc = fail(LENS_ENOTFOUND, "constraint set %lld not found", (long long)r->handle);
