@@ -20,14 +20,7 @@
 // The two varying potentials are evaluated in double-float (FP32 pipe,
 // ~1e-13 relative), FP64 only where that fails; the static cache itself is
 // FP64.
-// The double-float division as a called function in this file's kernels:
-// smaller code for the source-plane kernel, whose warps stall on
-// instruction fetch (4096 sets: 0.373 -> 0.359 ms); the image-plane and map
-// kernels keep it inlined (slower called: 12.56 -> 12.68 ms, 10.035 -> 10.055 ms).
-#ifndef LENS_DF_NOINLINE_DIV
-#define LENS_DF_NOINLINE_DIV 1
-#endif
-#include "lens_device.cuh"
+#include "lens_chi2_df.cuh"
 
 namespace lens {
 namespace {
@@ -69,7 +62,7 @@ struct Chi2SrcArgs {
   double *chi2;
 };
 
-// Parameter sets whose varying potentials' records one warp builds at a
+// Parameter sets whose varying potentials' records two warps build at a
 // time (one thread per record: the FP64 record arithmetic runs 32 lanes wide
 // instead of on two threads per set).
 constexpr int SRC_BATCH = 16;
@@ -80,13 +73,27 @@ constexpr int SRC_BATCH = 16;
 #ifndef LENS_SRC_WARPS
 #define LENS_SRC_WARPS 0
 #endif
-// both records of varying potential v of a parameter set, out of line
-__device__ __noinline__ bool var_recs_cold(const double *q, int type0, int type1, int v, double *s_rec,
-                                           float2 *s_rdf) {
+// the varying potentials' evaluator
+struct EvalChi2 {
+  template <bool HESS>
+  static __device__ __forceinline__ bool dpie(const float2 *r, df X, df Y, df &ax, df &ay, df *h) {
+    return dpie_df3<HESS, true>(r, X, Y, ax, ay, h);
+  }
+  template <bool HESS>
+  static __device__ __forceinline__ void circ(const float2 *r, df X, df Y, df &ax, df &ay, df *h) {
+    circ_df3<HESS>(r, X, Y, ax, ay, h);
+  }
+};
+// The FP64 record (kind 0; returns whether the parameters are inside the
+// domain) or the double-float record (kind 1) of varying potential v of a
+// parameter set, out of line.
+__device__ __noinline__ bool var_rec_cold(const double *q, int type0, int type1, int v, int kind, double *s_rec,
+                                          float2 *s_rdf) {
+  if (kind == 0) return load_var_rec64(q, type0, type1, v, s_rec);
   const double *w = q + 7 * v;
-  const bool ok = load_var_rec64(q, type0, type1, v, s_rec);
   make_recdf(v == 0 ? type0 : type1, w[0], w[1], w[3], w[2], w[4], w[5], w[6], s_rdf + v * RECDF);
-  return ok;
+  record_uw(s_rdf + v * RECDF);
+  return true;
 }
 
 // One kernel per Hessian mode (LENS_SRC_SPLIT): HESS = 1 for the variants
@@ -98,7 +105,7 @@ __device__ __noinline__ bool var_recs_cold(const double *q, int type0, int type1
 #endif
 template <int THREADS, int HESS = -1>
 __global__ void __launch_bounds__(THREADS, LENS_SRC_WARPS * 32 / THREADS) k_chi2_source(const Chi2SrcArgs a) {
-  static_assert(THREADS >= 2 * SRC_BATCH, "one thread per record of a batch");
+  static_assert(THREADS >= 4 * SRC_BATCH, "one thread per record of a batch");
   extern __shared__ double sm[];
   double *s_beta = sm;                   // [nimg][2]
   double *s_m = s_beta + 2 * a.nimg;     // [nimg][3]: r hxx, r hyy, r hxy
@@ -110,18 +117,12 @@ __global__ void __launch_bounds__(THREADS, LENS_SRC_WARPS * 32 / THREADS) k_chi2
   // this CTA's sets are p = blockIdx.x + j gridDim.x, taken SRC_BATCH at a time
   for (long long p0 = blockIdx.x; p0 < a.P; p0 += (long long)gridDim.x * SRC_BATCH) {
     __syncthreads();  // the previous batch's records are no longer read
-    if (threadIdx.x < 2 * SRC_BATCH) {
-      const int k = threadIdx.x >> 1, v = threadIdx.x & 1;
+    if (threadIdx.x < 4 * SRC_BATCH) {  // one warp builds the FP64 records, the next the double-float ones
+      const int kind = threadIdx.x / (2 * SRC_BATCH), k = threadIdx.x % (2 * SRC_BATCH) >> 1, v = threadIdx.x & 1;
       const long long p = p0 + (long long)k * gridDim.x;
       if (p < a.P) {
-        const double *q = a.params + p * a.pstride;
-        const double *w = q + 7 * v;  // x0, y0, eps, theta, rcore, rcut, b0
-        if (LENS_COLD_CALLS) {
-          s_ok[k][v] = var_recs_cold(q, a.type0, a.type1, v, s_rec[k], s_rdf[k]);
-        } else {
-          s_ok[k][v] = load_var_rec64(q, a.type0, a.type1, v, s_rec[k]);
-          make_recdf(v == 0 ? a.type0 : a.type1, w[0], w[1], w[3], w[2], w[4], w[5], w[6], s_rdf[k] + v * RECDF);
-        }
+        const bool ok = var_rec_cold(a.params + p * a.pstride, a.type0, a.type1, v, kind, s_rec[k], s_rdf[k]);
+        if (kind == 0) s_ok[k][v] = ok;
       }
     }
     __syncthreads();
@@ -133,7 +134,7 @@ __global__ void __launch_bounds__(THREADS, LENS_SRC_WARPS * 32 / THREADS) k_chi2
         continue;
       }
       const bool hess = HESS < 0 ? a.variant != LENS_CHI2_SRC_PLAIN : HESS == 1;
-      backtrace_set<THREADS, HESS>(a.stat + p * a.stat_stride, a.x, a.y, a.ratio, a.src_of, a.img_off, a.nimg,
+      backtrace_set<THREADS, HESS, EvalChi2>(a.stat + p * a.stat_stride, a.x, a.y, a.ratio, a.src_of, a.img_off, a.nimg,
                                    a.nsrc, s_rec[k], s_rdf[k], s_beta, hess ? s_m : nullptr, s_bary);
       double acc[1] = {0.0};
       for (int j = threadIdx.x; j < a.nimg; j += THREADS) {
@@ -329,7 +330,10 @@ __global__ void __launch_bounds__(CACHE_THREADS) k_static_scaled(const float2 *_
     df ax, ay, hh[3];
     bool ok = true;
     if (g[F_U2 * n].x < 0.f) {
-      circ_df<true>(g, n, Xd, Yd, ax, ay, hh);
+      float2 r[RECDF];
+#pragma unroll
+      for (int k = 0; k < RECDF; ++k) r[k] = g[k * n];
+      circ_df3<true>(r, Xd, Yd, ax, ay, hh);
     } else {
       float2 r[RECDF];
 #pragma unroll
@@ -348,7 +352,7 @@ __global__ void __launch_bounds__(CACHE_THREADS) k_static_scaled(const float2 *_
       put(F_DT0, df_mul(D(F_DT0), f2));
       put(F_U2ST2, df_mul(D(F_U2ST2), f2));
       put(F_KTC, df_mul(q2ds, ss));
-      ok = dpie_df<true, true>(r, 1, Xd, Yd, ax, ay, hh);
+      ok = dpie_df3<true, false>(r, Xd, Yd, ax, ay, hh);
     }
     if (ok) {
       sum[0] = df_add(sum[0], ax);

@@ -159,14 +159,15 @@ __host__ __device__ inline bool halo_params_ok(int type, double x0, double y0, d
 }
 
 // ---------------------------------------------------------------- objects
-// Double-float record of one potential: 16 (hi, lo) float pairs.
+// Double-float record of one potential: (hi, lo) float pairs.
 enum RecDF : int {
   F_X0 = 0, F_Y0, F_C, F_S, F_Q2, F_U2, F_KC, F_KT, F_SC, F_ST, F_Q2SC, F_Q2ST, F_Q2SS, F_Q2DS, F_SS, F_BQ,
   // Hessian: cos 2theta, sin 2theta, (1+q^2) s^2 and u^2 s^2 of both terms,
   // q^2 (st^2 - sc^2), b q / 2
-  F_C2, F_S2, F_DC0, F_DT0, F_U2SC2, F_U2ST2, F_KTC, F_HB
+  F_C2, F_S2, F_DC0, F_DT0, F_U2SC2, F_U2ST2, F_KTC, F_HB,
+  F_DS, F_U, F_BU  // st - sc, u, b q / u (0 for u = 0)
 };
-constexpr int RECDF = 24;
+constexpr int RECDF = 27;
 // SIS and point-mass records carry F_U2 = -1 and -2 (never negative for a
 // dPIE) and b, theta_E^2 in F_BQ.
 
@@ -208,6 +209,9 @@ __host__ __device__ inline void make_recdf(int type, double x0, double y0, doubl
     v[F_U2ST2] = u * u * st * st;
     v[F_KTC] = q2 * (st - sc) * (st + sc);
     v[F_HB] = 0.5 * v[F_BQ];
+    v[F_DS] = st - sc;
+    v[F_U] = u;
+    v[F_BU] = u > 0.0 ? v[F_BQ] / u : 0.0;
   }
   for (int k = 0; k < RECDF; ++k) {
     const float h = (float)v[k];
