@@ -613,7 +613,7 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   // about 8 bands, each a whole number of tiles
   FarPlan plan;
   if (precision == LENS_MIXED) plan = plan_far(ctx, m, grid, hess);
-  const int tile = plan.use ? FAR_TILE_ROWS : map_tile_rows(hess);
+  const int tile = plan.use ? plan.ft : map_tile_rows(hess);
   int rows = (ny + 7) / 8;
   rows = std::max(tile, (rows + tile - 1) / tile * tile);
   const size_t band_bytes = (size_t)rows * nx * planes * esize;

@@ -18,7 +18,7 @@
 //
 // Two levels.  k_far_coarse: per coarse tile (ct x ct nodes, ct = 64..512),
 // the potentials with psi >= KC R are summed at 12 x 12 nodes; the others'
-// bits are set in the tile's mask.  k_far_map: per 32 x 32 tile, the
+// bits are set in the tile's mask.  k_far_map: per 32 x 32 or 64 x 64 tile, the
 // potentials left by the coarse tile (all of them without a coarse level)
 // with psi >= KF R are summed at 10 x 10 nodes, the coarse tile's
 // interpolant is added there, and every map node then takes the near
@@ -41,7 +41,6 @@
 namespace lens {
 namespace {
 
-constexpr int FT = 32;   // nodes a side of a fine tile
 constexpr int FP = 10;   // its interpolation nodes per axis
 constexpr int CP = 12;   // a coarse tile's
 constexpr int FF_THREADS = 256, FF_WARPS = FF_THREADS / 32;
@@ -49,7 +48,7 @@ constexpr int FF_CH = 64;            // potentials per staged chunk
 constexpr int REC_STRIDE4 = REC32 / 4 + 1;  // float4 slots per staged record (the pad spreads the records a warp reads)
 constexpr int FF_SUB = 16;           // partial sums folded every FF_SUB potentials
 constexpr double DET_TERM_ERR = 2e-7, DET_REPAIR_ABS = 1e-5;  // as in lens_maps.cu
-constexpr int CT_MIN = 64, CT_MAX = 512;
+constexpr int CT_MAX = 512;
 
 enum FarMode : int { FAR_GRAD = 0, FAR_HESS = 1, FAR_POT = 2 };
 // interpolated values: deflection (2), kappa, gamma1, gamma2 (HESS) or the
@@ -58,46 +57,57 @@ __host__ __device__ constexpr int nval(int mode) { return mode == FAR_HESS ? 5 :
 __host__ __device__ constexpr int ncmp(int mode) { return nval(mode) + (mode == FAR_POT ? 0 : 1); }
 __host__ __device__ constexpr int ncmp2(int mode) { return (ncmp(mode) + 1) / 2; }
 
-// Chebyshev nodes of the fine tile in units of 1/64 grid step about the
-// tile's centre (half-width 15.5 steps), of the coarse tile in units of its
-// half-width / 512.
-constexpr int XI64[FP] = {980, 884, 701, 450, 155, -155, -450, -701, -884, -980};
+// Chebyshev nodes of a fine tile of FT x FT map nodes (FT = 32 or 64), in
+// units of 1/64 grid step about its centre, and of the coarse tile in units
+// of its half-width / 512.
+template <int FT>
+struct XiTab {
+  static constexpr int v[FP] = {980, 884, 701, 450, 155, -155, -450, -701, -884, -980};
+};
+template <>
+struct XiTab<64> {
+  static constexpr int v[FP] = {1991, 1796, 1426, 915, 315, -315, -915, -1426, -1796, -1991};
+};
 constexpr int ZC512[CP] = {508, 473, 406, 312, 196, 67, -67, -196, -312, -406, -473, -508};
-__device__ const float D_XI[FP] = {980 / 64.f, 884 / 64.f, 701 / 64.f, 450 / 64.f, 155 / 64.f,
-                                   -155 / 64.f, -450 / 64.f, -701 / 64.f, -884 / 64.f, -980 / 64.f};
 __device__ const float D_ZC[CP] = {508 / 512.f, 473 / 512.f, 406 / 512.f, 312 / 512.f, 196 / 512.f, 67 / 512.f,
                                    -67 / 512.f, -196 / 512.f, -312 / 512.f, -406 / 512.f, -473 / 512.f, -508 / 512.f};
 
-// Lagrange weights, formed in FP64 at compile time.
+// A fine tile's nodes in steps and the Lagrange weights at its map nodes,
+// formed in FP64 at compile time.
+template <int FT>
 struct FineTab {
-  float w[FT][FP];  // at map node m - 15.5 steps
+  float w[FT][FP];  // at map node m - (FT - 1) / 2 steps
+  float xi[FP];
 };
-constexpr FineTab fine_tab() {
-  FineTab t{};
+template <int FT>
+constexpr FineTab<FT> fine_tab() {
+  FineTab<FT> t{};
+  for (int i = 0; i < FP; ++i) t.xi[i] = (float)(XiTab<FT>::v[i] / 64.0);
   for (int m = 0; m < FT; ++m)
     for (int i = 0; i < FP; ++i) {
       double v = 1.0;
       for (int k = 0; k < FP; ++k)
-        if (k != i) v *= ((m - 15.5) * 64.0 - XI64[k]) / (double)(XI64[i] - XI64[k]);
+        if (k != i) v *= ((m - 0.5 * (FT - 1)) * 64.0 - XiTab<FT>::v[k]) / (double)(XiTab<FT>::v[i] - XiTab<FT>::v[k]);
       t.w[m][i] = (float)v;
     }
   return t;
 }
-__device__ const FineTab D_FINE = fine_tab();
-// the coarse basis at the fine tile's nodes: fine tile c of CT / 32 along an
+__device__ const FineTab<32> D_FINE32 = fine_tab<32>();
+__device__ const FineTab<64> D_FINE64 = fine_tab<64>();
+// the coarse basis at the fine tile's nodes: fine tile c of SUBT along an
 // axis, node i, coarse node k
 template <int SUBT>
 struct CoarseTab {
   float w[SUBT][FP][CP];
 };
-template <int SUBT>
+template <int FT, int SUBT>
 constexpr CoarseTab<SUBT> coarse_tab() {
   CoarseTab<SUBT> t{};
-  const double half = 16.0 * SUBT;  // half-width in steps
+  const double half = 0.5 * FT * SUBT;  // half-width in steps
   for (int c = 0; c < SUBT; ++c)
     for (int i = 0; i < FP; ++i)
       for (int k = 0; k < CP; ++k) {
-        const double x = (32.0 * c + 16.0 - half + XI64[i] / 64.0) / half * 512.0;
+        const double x = (FT * (c + 0.5) - half + XiTab<FT>::v[i] / 64.0) / half * 512.0;
         double v = 1.0;
         for (int l = 0; l < CP; ++l)
           if (l != k) v *= (x - ZC512[l]) / (double)(ZC512[k] - ZC512[l]);
@@ -105,10 +115,23 @@ constexpr CoarseTab<SUBT> coarse_tab() {
       }
   return t;
 }
-__device__ const CoarseTab<2> D_CO2 = coarse_tab<2>();
-__device__ const CoarseTab<4> D_CO4 = coarse_tab<4>();
-__device__ const CoarseTab<8> D_CO8 = coarse_tab<8>();
-__device__ const CoarseTab<16> D_CO16 = coarse_tab<16>();
+__device__ const CoarseTab<2> D_CO32_2 = coarse_tab<32, 2>(), D_CO64_2 = coarse_tab<64, 2>();
+__device__ const CoarseTab<4> D_CO32_4 = coarse_tab<32, 4>(), D_CO64_4 = coarse_tab<64, 4>();
+__device__ const CoarseTab<8> D_CO32_8 = coarse_tab<32, 8>(), D_CO64_8 = coarse_tab<64, 8>();
+__device__ const CoarseTab<16> D_CO32_16 = coarse_tab<32, 16>();
+template <int FT>
+__device__ __forceinline__ const FineTab<FT> &fine_table();
+template <>
+__device__ __forceinline__ const FineTab<32> &fine_table<32>() { return D_FINE32; }
+template <>
+__device__ __forceinline__ const FineTab<64> &fine_table<64>() { return D_FINE64; }
+template <int FT>
+__device__ __forceinline__ const float *coarse_weights(int sub) {
+  if (FT == 32)
+    return sub == 2 ? &D_CO32_2.w[0][0][0] : sub == 4 ? &D_CO32_4.w[0][0][0] : sub == 8 ? &D_CO32_8.w[0][0][0]
+                                                                                       : &D_CO32_16.w[0][0][0];
+  return sub == 2 ? &D_CO64_2.w[0][0][0] : sub == 4 ? &D_CO64_4.w[0][0][0] : &D_CO64_8.w[0][0][0];
+}
 
 struct FarArgs {
   const float *rec32;
@@ -122,6 +145,7 @@ struct FarArgs {
   int nx, ny;        // ny: rows of this launch
   int row0;
   double dls;
+  float dls_h, dls_l;  // as a float pair
   float thr_c, thr_ch, thr_f, thr_fh;  // squared psi beyond which a potential is far: coarse / fine, FP32 / cluster-scale
   // coarse level: tile (0, 0) covers the grid's first nodes
   int ct, nct;       // nodes a side (0: no coarse level), tiles per row
@@ -438,7 +462,7 @@ __device__ __forceinline__ float rcp_dff(float hi, float lo) {
   return fabsf(e) < 1e-3f ? fmaf(r, e, r) : 1.f / hi;
 }
 
-template <int MODE>
+template <int MODE, int FT>
 __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   constexpr bool HESS = MODE == FAR_HESS, POT = MODE == FAR_POT;
   constexpr int NODES = FP * FP, NC = ncmp(MODE), NV = nval(MODE), NC2 = ncmp2(MODE), SPLITS = FF_THREADS / (NODES / 2);
@@ -454,20 +478,39 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   float *s_tmp = reinterpret_cast<float *>(s_part);  // coarse level: [NC][CP * CP] values, [NC][FP][CP] (after node_sums)
   float *s_rem = s_tmp;                              // then the remainders [NC][NODES]
   __shared__ float2 s_nx[FP], s_ny[FP];
-  __shared__ float s_L[FT][FP];
+  __shared__ float2 s_cx[FT], s_ry[FT];  // offsets of the tile's columns and rows from its centre, hi/lo
+  __shared__ float s_L[FT][FP + 1], s_xi[FP];  // (odd stride: lanes read a column each)
+  __shared__ float4 s_T;                 // the centre, hi/lo
+  __shared__ double s_tau[POT ? 2 : 1][POT ? FT : 1];  // half the squared offsets from beta
   __shared__ float s_kb[4];
   __shared__ float4 s_plane[NV];
   __shared__ int s_cnt[4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int i0 = blockIdx.x * FT, j0 = a.row0 + blockIdx.y * FT;  // grid column and row of the tile's first node
-  const df Tx = df_from_double(a.xmin + (i0 + 15.5) * a.dx), Ty = df_from_double(a.ymin + (j0 + 15.5) * a.dy);
-  if (tid < FP) {
-    const df ox = df_from_double(D_XI[tid] * a.dx), oy = df_from_double(D_XI[tid] * a.dy);
-    s_nx[tid] = make_float2(ox.hi, ox.lo);
-    s_ny[tid] = make_float2(oy.hi, oy.lo);
+  // the few FP64 operations once per tile
+  constexpr double HALF = 0.5 * (FT - 1);
+  if (tid < 2) {
+    const df t = df_from_double(tid == 0 ? a.xmin + (i0 + HALF) * a.dx : a.ymin + (j0 + HALF) * a.dy);
+    reinterpret_cast<float2 *>(&s_T)[tid] = make_float2(t.hi, t.lo);
+  } else if (tid >= 32 && tid < 32 + 2 * FP) {
+    const int k = (tid - 32) % FP;
+    const df o = df_from_double(fine_table<FT>().xi[k] * (tid < 32 + FP ? a.dx : a.dy));
+    (tid < 32 + FP ? s_nx : s_ny)[k] = make_float2(o.hi, o.lo);
+  } else if (tid >= 64 && tid < 64 + 2 * FT) {
+    const int k = (tid - 64) % FT;
+    const df o = df_from_double((k - HALF) * (tid < 64 + FT ? a.dx : a.dy));
+    (tid < 64 + FT ? s_cx : s_ry)[k] = make_float2(o.hi, o.lo);
+    if (POT && a.tau) {
+      const double d = tid < 64 + FT ? a.xmin + (i0 + k) * a.dx - a.bx : a.ymin + (j0 + k) * a.dy - a.by;
+      s_tau[POT && tid >= 64 + FT][POT ? k : 0] = 0.5 * d * d;
+    }
+  } else if (tid < 6) {
+    s_kb[tid - 2] = 0.f;
   }
-  if (tid < 4) s_kb[tid] = 0.f;
-  for (int q = tid; q < FT * FP; q += FF_THREADS) (&s_L[0][0])[q] = (&D_FINE.w[0][0])[q];
+  if (tid >= 256 - FP) s_xi[tid - (256 - FP)] = fine_table<FT>().xi[tid - (256 - FP)];
+  for (int q = tid; q < FT * FP; q += FF_THREADS) s_L[q / FP][q % FP] = (&fine_table<FT>().w[0][0])[q];
+  __syncthreads();
+  const df Tx = {s_T.x, s_T.y}, Ty = {s_T.z, s_T.w};
   const int ctile = a.ct ? (j0 / a.ct) * a.nct + i0 / a.ct : 0;
   classify(a, a.ct ? a.cmask + (size_t)ctile * a.nw : nullptr, Tx, Ty, a.thr_f, a.thr_fh, s_far, s_near, s_list, s_cnt);
   const int n_far = s_cnt[0], n_far_h = s_cnt[1], n_near = s_cnt[2], n_near_h = s_cnt[3];
@@ -477,7 +520,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     // product, then columns; its plane (exact products) in double-float
     const float *cv = a.cval + (size_t)ctile * coarse_floats(MODE);
     const int sub = a.ct / FT, cx = (i0 % a.ct) / FT, cy = (j0 % a.ct) / FT;
-    const float *W = sub == 2 ? &D_CO2.w[0][0][0] : sub == 4 ? &D_CO4.w[0][0][0] : sub == 8 ? &D_CO8.w[0][0][0] : &D_CO16.w[0][0][0];
+    const float *W = coarse_weights<FT>(sub);
     const float *Wx = W + cx * FP * CP, *Wy = W + cy * FP * CP;
     float *s_t1 = s_tmp + NC * CP * CP;
     for (int q = tid; q < NC * CP * CP; q += FF_THREADS) s_tmp[q] = cv[q];
@@ -491,7 +534,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
       s_t1[q] = v;
     }
     __syncthreads();
-    const float bx0 = 32.f * cx + 16.f - 16.f * sub, by0 = 32.f * cy + 16.f - 16.f * sub;
+    const float bx0 = FT * (cx + 0.5f) - 0.5f * a.ct, by0 = FT * (cy + 0.5f) - 0.5f * a.ct;
     for (int q = tid; q < NC * NODES; q += FF_THREADS) {
       const int c = q / NODES, node = q % NODES, i = node % FP, j = node / FP;
       float v = 0.f;
@@ -502,15 +545,15 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
       if (c < NV) {
         const float *p = cv + NC * CP * CP + c * 4;
         d = df_add(d, df{p[0], 0.f});
-        d = df_add(d, df{p[1] * (bx0 + D_XI[i]), 0.f});
-        d = df_add(d, df{p[2] * (by0 + D_XI[j]), 0.f});
+        d = df_add(d, df{p[1] * (bx0 + s_xi[i]), 0.f});
+        d = df_add(d, df{p[2] * (by0 + s_xi[j]), 0.f});
       }
       s_val[q] = make_float2(d.hi, d.lo);
     }
     if (HESS && tid < 3) s_kb[tid] += cv[NC * CP * CP + NV * 4 + tid];
     __syncthreads();
   }
-  if (tid < NV) s_plane[tid] = plane_of<FP>(s_val + tid * NODES, D_XI[0] - D_XI[FP - 1]);
+  if (tid < NV) s_plane[tid] = plane_of<FP>(s_val + tid * NODES, s_xi[0] - s_xi[FP - 1]);
   __syncthreads();
   for (int q = tid; q < NC * NODES; q += FF_THREADS) {
     const int c = q / NODES, node = q % NODES;
@@ -519,8 +562,8 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     if (c < NV) {
       const float4 p = s_plane[c];
       df d = df_sub(df{v.x, v.y}, df{p.x, 0.f});
-      d = df_sub(d, df{p.y * D_XI[node % FP], 0.f});
-      d = df_sub(d, df{p.z * D_XI[node / FP], 0.f});
+      d = df_sub(d, df{p.y * s_xi[node % FP], 0.f});
+      d = df_sub(d, df{p.z * s_xi[node / FP], 0.f});
       r = d.hi + d.lo;
     }
     s_rem[q] = r;
@@ -543,23 +586,13 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   }
   // the near potentials and the interpolant at the map nodes: lane = column,
   // a warp takes row pairs warp, warp + FF_WARPS
-  const float mx = lane - 15.5f;
-  const double lx = mx * a.dx;
-  const float lxh = (float)lx;
-  const float2 ox = make_float2(lxh, (float)(lx - (double)lxh));
-  const int i = i0 + lane;
-  float Lx[FP];
   bool staged = false;
 #pragma unroll 1
-  for (int rp = warp; rp < FT / 2; rp += FF_WARPS) {
-    float2 oyh, oyl;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const double ly = (2 * rp + h - 15.5) * a.dy;
-      const float f = (float)ly;
-      part2(oyh, h) = f;
-      part2(oyl, h) = (float)(ly - (double)f);
-    }
+  for (int task = warp; task < (FT / 2) * (FT / 32); task += FF_WARPS) {
+    const int rp = task % (FT / 2), m = task / (FT / 2) * 32 + lane, i = i0 + m;
+    const float mx = m - (float)HALF;
+    const float2 ox = s_cx[m], r0 = s_ry[2 * rp], r1 = s_ry[2 * rp + 1];
+    const float2 oyh = make_float2(r0.x, r1.x), oyl = make_float2(r0.y, r1.y);
     Sums<MODE> S;
     S.zero();
     for (int c0 = 0; c0 < n_near || (c0 == 0 && !staged); c0 += FF_CH) {
@@ -573,21 +606,21 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
       S.sweep(s_rec, s_off, 0, cnt, 1, ox, oyh, oyl);
     }
     S.fold();
-#pragma unroll
-    for (int k = 0; k < FP; ++k) Lx[k] = s_L[lane][k];
     float2 v[2 * NC2];
 #pragma unroll
     for (int c = 0; c < 2 * NC2; ++c) v[c] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int k = 0; k < FP; ++k)
+    for (int k = 0; k < FP; ++k) {
+      const float2 L = dup2(s_L[m][k]);
 #pragma unroll
       for (int c = 0; c < NC2; ++c) {
         const float4 t = s_c[(rp * FP + k) * NC2 + c];
-        v[2 * c] = fma2(dup2(Lx[k]), make_float2(t.x, t.y), v[2 * c]);
-        v[2 * c + 1] = fma2(dup2(Lx[k]), make_float2(t.z, t.w), v[2 * c + 1]);
+        v[2 * c] = fma2(L, make_float2(t.x, t.y), v[2 * c]);
+        v[2 * c + 1] = fma2(L, make_float2(t.z, t.w), v[2 * c + 1]);
       }
+    }
     // plane + near + remainder, per value and point pair, in double-float
-    const float2 my = make_float2(2 * rp - 15.5f, 2 * rp - 14.5f);
+    const float2 my = make_float2(2 * rp - (float)HALF, 2 * rp + 1 - (float)HALF);
     float2 vh[NV], vl[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
@@ -633,14 +666,11 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
           const long long o = (long long)j * a.nx + i;
           const double phi = a.dls * ((double)part2(vh[0], h) + (double)part2(vl[0], h));
           a.out64[o] = phi;
-          if (a.tau) {
-            const double X = a.xmin + i * a.dx - a.bx, Y = a.ymin + (a.row0 + j) * a.dy - a.by;
-            a.out64[a.plane + o] = 0.5 * (X * X + Y * Y) - phi;
-          }
+          if (a.tau) a.out64[a.plane + o] = s_tau[0][m] + s_tau[1][2 * rp + h] - phi;
         }
       }
     } else {
-      const float dh = (float)a.dls, dl = (float)(a.dls - (double)dh);
+      const float dh = a.dls_h, dl = a.dls_l;
       // which nodes the double-float repair recomputes (see k_map_mixed);
       // the far potentials' kappa and gamma enter by their bounds on the tile
       if (a.repair_f > 0.f) {
@@ -708,10 +738,12 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   }
 }
 
-size_t far_smem(int mode, bool coarse, int nw, int n) {
+// ft = 0: the coarse kernel
+size_t far_smem(int mode, int ft, int nw, int n) {
+  const bool coarse = ft == 0;
   const int nodes = coarse ? CP * CP : FP * FP, splits = FF_THREADS / (nodes / 2), nc = ncmp(mode);
   size_t b = sizeof(float4) * (FF_CH * REC_STRIDE4 + FF_CH);
-  if (!coarse) b += sizeof(float4) * (FT / 2) * FP * ncmp2(mode);
+  if (!coarse) b += sizeof(float4) * (ft / 2) * FP * ncmp2(mode);
   // the partial sums' space also holds the coarse tile's values (fine kernel)
   const size_t part = std::max(sizeof(float2) * splits * nodes * nc, coarse ? 0 : sizeof(float) * nc * (CP * CP + CP * FP));
   b += (part + 15) / 16 * 16 + sizeof(float2) * nodes * nc;
@@ -724,6 +756,8 @@ size_t far_smem(int mode, bool coarse, int nw, int n) {
 // 1.2e-8 of the term; the cluster-scale ones', whose deflection is ten times
 // the rest, below 1e-9.
 constexpr double KF = 3.0, KF_H = 3.5, KC = 2.5, KC_H = 3.0;
+// fixed work in evaluations of one FP32 potential: per fine tile, per map node
+constexpr double TILE_COST = 4000.0, NODE_COST = 3.0;
 constexpr int FAR_MAX_N = 16384;  // potentials (two bytes each of shared memory)
 
 // Fraction of the map's nodes within psi < r of a potential of axis ratio q
@@ -749,34 +783,36 @@ FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mo
   const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
   const double area = (g->xmax - g->xmin) * (g->ymax - g->ymin), nodes = (double)g->nx * g->ny;
   const double HV = mode == FAR_HESS ? 20.0 : 10.0, step = std::max(dx, dy);
-  const double Rf = std::sqrt(2.0) * 15.5 * step;
   auto light = [&](double r) { return m->n_light * near_frac(r, 1.0 / m->invq_light, 0.0, area); };
   auto heavy = [&](double r) {
     double s = 0.0;
     for (const auto &h : m->heavy_shape) s += near_frac(r, h.first, h.second, area);
     return s;
   };
-  const double direct = (m->n_light + HV * m->n_heavy + 2.0) * std::max(1.0, 608.0 * 256.0 / nodes);
-  const double tiles = std::ceil(g->nx / (double)FT) * std::ceil(g->ny / (double)FT);
-  const double near = light(KF * Rf) + HV * heavy(KF_H * Rf);
-  double best = 0.85 * direct;
-  for (int ct = 0; ct <= CT_MAX; ct = ct ? 2 * ct : CT_MIN) {
-    if (ct && ct >= 2 * std::max(g->nx, g->ny)) break;
-    double mid = m->n_light, mid_h = m->n_heavy, coarse = 0.0;
-    if (ct) {
-      const double Rc = std::sqrt(2.0) * 0.5 * ct * step;
-      const double ctiles = std::ceil(g->nx / (double)ct) * std::ceil(g->ny / (double)ct);
-      coarse = (m->n_light + 2.0 * HV * m->n_heavy) * 170.0 * ctiles / nodes * std::max(1.0, 152.0 / ctiles);
-      mid = light(KC * Rc);
-      mid_h = heavy(KC_H * Rc);
-    }
-    const double fine = (mid + 2.5 * HV * mid_h) * (FP * FP) / (double)(FT * FT);
-    const double c = coarse + (6.0 + fine + near) * tiles * FT * FT / nodes * std::max(1.0, 304.0 / tiles);
-    if (c < best) {
-      best = c;
-      p.use = true;
-      p.ct = ct;
-      p.cost = c;
+  double best = 0.85 * (m->n_light + HV * m->n_heavy + 2.0) * std::max(1.0, 608.0 * 256.0 / nodes);
+  for (int ft = 32; ft <= 64; ft *= 2) {
+    const double tiles = std::ceil(g->nx / (double)ft) * std::ceil(g->ny / (double)ft);
+    const double Rf = std::sqrt(2.0) * 0.5 * (ft - 1) * step;
+    const double near = light(KF * Rf) + HV * heavy(KF_H * Rf);
+    for (int ct = 0; ct <= CT_MAX; ct = ct ? 2 * ct : 2 * ft) {
+      if (ct && ct >= 2 * std::max(g->nx, g->ny)) break;
+      double mid = m->n_light, mid_h = m->n_heavy, coarse = 0.0;
+      if (ct) {
+        const double Rc = std::sqrt(2.0) * 0.5 * ct * step;
+        const double ctiles = std::ceil(g->nx / (double)ct) * std::ceil(g->ny / (double)ct);
+        coarse = (m->n_light + 2.0 * HV * m->n_heavy) * 170.0 * ctiles / nodes * std::max(1.0, 152.0 / ctiles);
+        mid = light(KC * Rc);
+        mid_h = heavy(KC_H * Rc);
+      }
+      const double fine = (TILE_COST + (mid + 2.5 * HV * mid_h) * (FP * FP)) / (double)(ft * ft);
+      const double c = coarse + (NODE_COST + fine + near) * tiles * ft * ft / nodes * std::max(1.0, 304.0 / tiles);
+      if (c < best) {
+        best = c;
+        p.use = true;
+        p.ft = ft;
+        p.ct = ct;
+        p.cost = c;
+      }
     }
   }
   if (p.use && p.ct) {
@@ -807,7 +843,9 @@ static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, in
   a.ny = g->ny;
   a.row0 = 0;
   a.dls = 1.0;
-  const double step = std::sqrt(2.0) * std::max(a.dx, a.dy), rf = 15.5 * step, rc = 0.5 * p.ct * step;
+  a.dls_h = 1.f;
+  a.dls_l = 0.f;
+  const double step = std::sqrt(2.0) * std::max(a.dx, a.dy), rf = 0.5 * (p.ft - 1) * step, rc = 0.5 * p.ct * step;
   auto sq = [](double v) { return (float)(v * v); };
   a.thr_c = sq(KC * rc);
   a.thr_ch = sq(KC_H * rc);
@@ -829,7 +867,7 @@ static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, in
 
 template <int MODE>
 static int coarse_launch(const FarArgs &a, const FarPlan &p, int n, cudaStream_t st) {
-  const size_t smem = far_smem(MODE, true, a.nw, n);
+  const size_t smem = far_smem(MODE, 0, a.nw, n);
   cudaFuncSetAttribute(k_far_coarse<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   k_far_coarse<MODE><<<dim3(p.nct, p.ncr), FF_THREADS, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
@@ -837,11 +875,11 @@ static int coarse_launch(const FarArgs &a, const FarPlan &p, int n, cudaStream_t
   return LENS_OK;
 }
 
-template <int MODE>
+template <int MODE, int FT>
 static int fine_launch(const FarArgs &a, int n, cudaStream_t st) {
-  const size_t smem = far_smem(MODE, false, a.nw, n);
-  cudaFuncSetAttribute(k_far_map<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_far_map<MODE><<<dim3((a.nx + FT - 1) / FT, (a.ny + FT - 1) / FT), FF_THREADS, smem, st>>>(a);
+  const size_t smem = far_smem(MODE, FT, a.nw, n);
+  cudaFuncSetAttribute(k_far_map<MODE, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_far_map<MODE, FT><<<dim3((a.nx + FT - 1) / FT, (a.ny + FT - 1) / FT), FF_THREADS, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "interpolated map launch: %s", cudaGetErrorString(e));
   return LENS_OK;
@@ -862,6 +900,8 @@ int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mod
   a.ny = rows;
   a.row0 = row0;
   a.dls = dls;
+  a.dls_h = (float)dls;
+  a.dls_l = (float)(dls - (double)a.dls_h);
   a.plane = (long long)g->nx * rows;
   a.repair_f = (float)(2.0 * repair);
   a.rep_count = rep_count;
@@ -871,10 +911,11 @@ int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mod
     a.tau = beta != nullptr;
     a.bx = beta ? beta[0] : 0.0;
     a.by = beta ? beta[1] : 0.0;
-    return fine_launch<FAR_POT>(a, m->n, st);
+    return p.ft == 32 ? fine_launch<FAR_POT, 32>(a, m->n, st) : fine_launch<FAR_POT, 64>(a, m->n, st);
   }
   a.out = (float *)out;
-  return mode == FAR_HESS ? fine_launch<FAR_HESS>(a, m->n, st) : fine_launch<FAR_GRAD>(a, m->n, st);
+  if (mode == FAR_HESS) return p.ft == 32 ? fine_launch<FAR_HESS, 32>(a, m->n, st) : fine_launch<FAR_HESS, 64>(a, m->n, st);
+  return p.ft == 32 ? fine_launch<FAR_GRAD, 32>(a, m->n, st) : fine_launch<FAR_GRAD, 64>(a, m->n, st);
 }
 
 }  // namespace lens

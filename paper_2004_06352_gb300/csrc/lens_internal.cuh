@@ -379,6 +379,7 @@ int check_grid(const lens_grid *g);
 // coarse level has been computed into far_mem; NULL: direct.
 struct FarPlan {
   bool use = false;
+  int ft = 32;                   // fine tile, nodes a side (32 or 64)
   int ct = 0, nct = 0, ncr = 0;  // coarse tile (0: no coarse level), coarse tiles per row and column
   size_t val_bytes = 0, bytes = 0;
   double cost = 0.0;             // expected cost per node in evaluations of one FP32 potential
@@ -387,7 +388,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
                      cudaStream_t st, int row0 = 0, int rows = -1, bool repair = true, void *repair_mem = nullptr,
                      const FarPlan *far = nullptr, void *far_mem = nullptr);
 // modes of the interpolated maps: 0 deflection, 1 deflection + Hessian, 2 potential
-constexpr int FAR_TILE_ROWS = 32;  // rows of a band must be a multiple of this
+// (rows of a band must be a multiple of the plan's fine tile)
 FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode);
 int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st);
 int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, double dls, void *out,
