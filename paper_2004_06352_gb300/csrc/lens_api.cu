@@ -559,10 +559,10 @@ static int map_common(lens_ctx *ctx, lens_model_t model, const lens_grid *grid, 
     // the coarse level's values there is the direct kernel
     CallScratch list(ctx, st), far(ctx, st);
     if (plan.use && ctx->repair_ratio > 0.0 && m->n_light > 0 && (rc = list.alloc(map_repair_bytes(grid)))) return rc;
-    if (plan.use && plan.ct && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
+    if (plan.use && plan.bytes && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
     if (plan.use && (rc = launch_far_coarse(m, grid, plan, hess, far.p, st))) return rc;
     return launch_map_mixed(ctx, m, grid, dls_ds, hess, d_out, st, 0, -1, true, list.p, plan.use ? &plan : nullptr,
-                            far.p);
+                            far.p, plan.rep_bytes ? (char *)far.p + plan.bytes - plan.rep_bytes : nullptr);
   }
   if (precision == LENS_FP64) return launch_map_fp64(ctx, m, grid, dls_ds, hess, d_out, st);
   return fail(LENS_EINVAL, "precision must be LENS_FP64 or LENS_MIXED");
@@ -641,9 +641,10 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   for (int k = 0; k < 2; ++k) LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[k], ctx->pipe_start, 0));
   // the interpolated form's coarse level, of the whole grid, before the bands
   CallScratch far(ctx, ctx->pipe_cs[0]);
-  if (plan.use && plan.ct) {
-    const bool room = !ctx->budget || ctx->used + plan.bytes + map_repair_bytes(grid, rows) <= ctx->budget;
-    if (!room || far.alloc(plan.bytes) != LENS_OK) {
+  const size_t far_bytes = plan.bytes + plan.rep_bytes;  // the dense tiles' arrays for each band stream
+  if (plan.use && far_bytes) {
+    const bool room = !ctx->budget || ctx->used + far_bytes + map_repair_bytes(grid, rows) <= ctx->budget;
+    if (!room || far.alloc(far_bytes) != LENS_OK) {
       plan = FarPlan();  // no room beside the bands' repair lists: the direct kernel, whose tiles divide the bands too
     } else {
       if ((rc = launch_far_coarse(m, grid, plan, hess, far.p, ctx->pipe_cs[0]))) return rc;
@@ -660,7 +661,8 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
     // the buffer's previous band (this call's or an earlier call's) has left
     LENS_CUDA_TRY(cudaStreamWaitEvent(cs, ctx->pipe_copied[k], 0));
     rc = precision == LENS_MIXED ? launch_map_mixed(ctx, m, grid, dls_ds, hess, buf, cs, row0, r, true, nullptr,
-                                                    plan.use ? &plan : nullptr, far.p)
+                                                    plan.use ? &plan : nullptr, far.p,
+                                                    plan.rep_bytes ? (char *)far.p + plan.bytes - (1 - k) * plan.rep_bytes : nullptr)
                                  : launch_map_fp64(ctx, m, grid, dls_ds, hess, buf, cs, row0, r);
     if (rc) return rc;
     LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_done[k], cs));

@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(CACHE_THREADS) k_static_df(const float2 *__res
   const int img = blockIdx.x;
   stat += (size_t)blockIdx.y * gridDim.x * 5;
   const double X = x[img], Y = y[img];
-  const df Xd = df_from_double(X), Yd = df_from_double(Y);
+  const df Xd = df_kept(X), Yd = df_kept(Y);
   double v[5] = {0, 0, 0, 0, 0};
   // per-thread sums in double-float, converted once (FP64 only for the
   // potentials whose double-float evaluation fails)
@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(CACHE_THREADS) k_static_scaled(const float2 *_
   stat += (size_t)blockIdx.y * gridDim.x * 5;
   const double fb = params[(size_t)blockIdx.y * 16 + 14], ft = params[(size_t)blockIdx.y * 16 + 15];
   const double X = x[img], Y = y[img];
-  const df Xd = df_from_double(X), Yd = df_from_double(Y), fd = df_from_double(ft), f2 = df_mul(fd, fd);
+  const df Xd = df_kept(X), Yd = df_kept(Y), fd = df_kept(ft), f2 = df_mul(fd, fd);
   double v[5] = {0, 0, 0, 0, 0};
   df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
   bool bad = !(fb > 0.0 && ft > 0.0 && isfinite(fb) && isfinite(ft));

@@ -41,7 +41,7 @@
 namespace lens {
 namespace {
 
-constexpr int FP = 10;   // its interpolation nodes per axis
+constexpr int FP = FAR_P;  // interpolation nodes per axis of a fine tile
 constexpr int CP = 12;   // a coarse tile's
 constexpr int FF_THREADS = 256, FF_WARPS = FF_THREADS / 32;
 constexpr int FF_CH = 64;            // potentials per staged chunk
@@ -76,7 +76,8 @@ __device__ const float D_ZC[CP] = {508 / 512.f, 473 / 512.f, 406 / 512.f, 312 / 
 // formed in FP64 at compile time.
 template <int FT>
 struct FineTab {
-  float w[FT][FP];  // at map node m - (FT - 1) / 2 steps
+  float w[FT][FP];    // at map node m - (FT - 1) / 2 steps
+  float wlo[FT][FP];  // w + wlo: in double-float (repair)
   float xi[FP];
 };
 template <int FT>
@@ -89,6 +90,7 @@ constexpr FineTab<FT> fine_tab() {
       for (int k = 0; k < FP; ++k)
         if (k != i) v *= ((m - 0.5 * (FT - 1)) * 64.0 - XiTab<FT>::v[k]) / (double)(XiTab<FT>::v[i] - XiTab<FT>::v[k]);
       t.w[m][i] = (float)v;
+      t.wlo[m][i] = (float)(v - (double)t.w[m][i]);
     }
   return t;
 }
@@ -158,6 +160,8 @@ struct FarArgs {
   double bx, by;
   float repair_f;    // 2 * ratio, 0: no repair
   int *rep_count, *rep_list;
+  DenseRepair dense;
+  int dense_min;     // listed nodes from which a tile is dense
 };
 
 __host__ __device__ constexpr int coarse_floats(int mode) { return ncmp(mode) * CP * CP + nval(mode) * 4 + 4; }
@@ -481,6 +485,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   __shared__ float2 s_cx[FT], s_ry[FT];  // offsets of the tile's columns and rows from its centre, hi/lo
   __shared__ float s_L[FT][FP + 1], s_xi[FP];  // (odd stride: lanes read a column each)
   __shared__ float4 s_T;                 // the centre, hi/lo
+  __shared__ unsigned s_m[FT * FT / 32], s_mh[HESS ? FT * FT / 32 : 1];  // nodes to recompute: deflection alone / all planes
   __shared__ double s_tau[POT ? 2 : 1][POT ? FT : 1];  // half the squared offsets from beta
   __shared__ float s_kb[4];
   __shared__ float4 s_plane[NV];
@@ -678,8 +683,8 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const bool in = i < a.nx && jl + h < a.ny;
-          const float m = a.repair_f * (part2(v[NV], h) + S.mag(h)), fx = part2(vh[0], h), fy = part2(vh[1], h);
-          rep[h] = in && fmaf(fx, fx, fy * fy) < m * m;
+          const float mg = a.repair_f * (part2(v[NV], h) + S.mag(h)), fx = part2(vh[0], h), fy = part2(vh[1], h);
+          rep[h] = in && fmaf(fx, fx, fy * fy) < mg * mg;
           if (HESS) {
             const float kl = dh * (fabsf(S.value(2, h).hi) + s_kb[0]);
             const float g1l = dh * (fabsf(S.value(3, h).hi) + s_kb[1]), g2l = dh * (fabsf(S.value(4, h).hi) + s_kb[2]);
@@ -691,14 +696,10 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
         }
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
-          const unsigned mask = __ballot_sync(0xffffffffu, rep[h] || rep_h[h]);
-          if (mask) {
-            int first = 0;
-            if (lane == __ffs(mask) - 1) first = atomicAdd(a.rep_count, __popc(mask));
-            first = __shfl_sync(0xffffffffu, first, __ffs(mask) - 1);
-            if (rep[h] || rep_h[h])
-              a.rep_list[first + __popc(mask & ((1u << lane) - 1u))] =
-                  ((jl + h) * a.nx + i) | (rep_h[h] ? (int)0x80000000u : 0);
+          const unsigned mh = __ballot_sync(0xffffffffu, rep_h[h]), m1 = __ballot_sync(0xffffffffu, rep[h] && !rep_h[h]);
+          if (lane == 0) {
+            s_m[(2 * rp + h) * (FT / 32) + m / 32] = m1;
+            if (HESS) s_mh[(2 * rp + h) * (FT / 32) + m / 32] = mh;
           }
         }
       }
@@ -736,6 +737,171 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
       }
     }
   }
+  if (POT || !(a.repair_f > 0.f)) return;
+  // the nodes to recompute: a tile with many of them that need the
+  // deflection alone goes to the dense tiles, the others' nodes to the list
+  constexpr int NW = FT * FT / 32;
+  __shared__ int s_pos[2 * NW], s_to[3];  // list positions; list base, dense slot (or -1), listed words
+  __syncthreads();
+  if (warp == 0) {
+    int n1 = 0, nh = 0;
+    for (int w = lane; w < NW; w += 32) {
+      n1 += __popc(s_m[w]);
+      if (HESS) nh += __popc(s_mh[w]);
+    }
+    n1 = __reduce_add_sync(0xffffffffu, n1);
+    nh = __reduce_add_sync(0xffffffffu, nh);
+    int slot = -1;
+    if (lane == 0 && a.dense.cap && n1 >= a.dense_min) {
+      slot = atomicAdd(a.dense.count, 1);
+      if (slot >= a.dense.cap) slot = -1;
+    }
+    slot = __shfl_sync(0xffffffffu, slot, 0);
+    const int nl = nh + (slot < 0 ? n1 : 0);
+    int base = 0;
+    if (lane == 0 && nl) base = atomicAdd(a.rep_count, nl);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    for (int w0 = 0; w0 < 2 * NW && nl; w0 += 32) {  // all-plane words, then the others
+      const int w = w0 + lane;
+      const int c = __popc(w < NW ? (HESS ? s_mh[HESS ? w : 0] : 0u) : slot < 0 ? s_m[w - NW] : 0u);
+      int sum = c;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, sum, o);
+        if (lane >= o) sum += t;
+      }
+      s_pos[w] = base + sum - c;
+      base += __shfl_sync(0xffffffffu, sum, 31);
+    }
+    if (lane == 0) {
+      s_to[0] = nl;
+      s_to[1] = slot;
+      if (slot >= 0) a.dense.tile[slot] = blockIdx.y * gridDim.x + blockIdx.x;
+    }
+  }
+  __syncthreads();
+  const int nl = s_to[0], slot = s_to[1];
+  if (slot >= 0)
+    for (int w = tid; w < NW; w += FF_THREADS) a.dense.mask[(size_t)slot * NW + w] = s_m[w];
+  if (nl)
+    for (int w = warp; w < 2 * NW; w += FF_WARPS) {
+      const int wi = w % NW;
+      const unsigned mask = w < NW ? (HESS ? s_mh[HESS ? wi : 0] : 0u) : slot < 0 ? s_m[wi] : 0u;
+      const int j = blockIdx.y * FT + wi / (FT / 32), i = i0 + wi % (FT / 32) * 32 + lane;
+      if (mask >> lane & 1u)
+        a.rep_list[s_pos[w] + __popc(mask & ((1u << lane) - 1u))] = (j * a.nx + i) | (w < NW ? (int)0x80000000u : 0);
+    }
+}
+
+// The listed nodes of the densely listed tiles: a CTA takes 128 of a tile's
+// nodes, one per thread; the near potentials (those the interpolation nodes
+// left out) one by one in double-float, their records staged, then the far
+// ones' deflection interpolated in double-float (weights and values as
+// pairs: the FP32 weights' 6e-8 of a far sum of tens of arcsec would show
+// where the deflection is near zero).  8192^2 x 2000: the repair spends its
+// time on 100 instead of up to 4096 evaluations of every potential per tile.
+constexpr int FR_THREADS = 128;
+struct FarRepairArgs {
+  const float2 *recdf;
+  const double *all64;
+  int n;
+  double xmin, ymin, dx, dy;
+  int nx, row0;
+  double dls;
+  float *out;
+  long long plane;
+  DenseRepair dense;
+};
+
+template <int FT>
+__global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a) {
+  constexpr int NW = FT * FT / 32, PARTS = FT * FT / FR_THREADS, NODES = FP * FP;
+  __shared__ unsigned s_w[NW];
+  __shared__ int s_pos[NW + 1], s_near[FR_THREADS], s_nn[FR_THREADS / 32];
+  __shared__ float2 s_val[2][NODES];
+  __shared__ float2 s_rdf[RECDF][FR_THREADS];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int nh = min(*a.dense.count, a.dense.cap);
+  for (long long item = blockIdx.x; item < (long long)nh * PARTS; item += gridDim.x) {
+    const int slot = (int)(item / PARTS), part = (int)(item % PARTS);
+    __syncthreads();  // the previous item's shared data has been used
+    for (int w = tid; w < NW; w += FR_THREADS) s_w[w] = a.dense.mask[(size_t)slot * NW + w];
+    for (int q = tid; q < 2 * NODES; q += FR_THREADS) (&s_val[0][0])[q] = a.dense.val[(size_t)slot * 2 * NODES + q];
+    __syncthreads();
+    if (warp == 0) {
+      int base = 0;
+      for (int w0 = 0; w0 < NW; w0 += 32) {
+        const int c = __popc(s_w[w0 + lane]);
+        int sum = c;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int t = __shfl_up_sync(0xffffffffu, sum, o);
+          if (lane >= o) sum += t;
+        }
+        s_pos[w0 + lane] = base + sum - c;
+        base += __shfl_sync(0xffffffffu, sum, 31);
+      }
+      if (lane == 0) s_pos[NW] = base;
+    }
+    __syncthreads();
+    const int listed = s_pos[NW];
+    if (part * FR_THREADS >= listed) continue;  // uniform over the CTA
+    // this thread's node: the (part * 128 + tid)-th listed one
+    const int rank = min(part * FR_THREADS + tid, listed - 1);
+    const bool mine = part * FR_THREADS + tid < listed;
+    int lo = 0, hi = NW;  // s_pos[lo] <= rank < s_pos[hi]
+    while (hi - lo > 1) {
+      const int mid = (lo + hi) / 2;
+      if (s_pos[mid] <= rank)
+        lo = mid;
+      else
+        hi = mid;
+    }
+    unsigned bits = s_w[lo];
+    for (int k = rank - s_pos[lo]; k > 0; --k) bits &= bits - 1u;
+    const int jr = lo / (FT / 32), ic = lo % (FT / 32) * 32 + __ffs(bits) - 1;
+    const int tile = a.dense.tile[slot], i0 = tile % a.dense.tpr * FT, j0 = tile / a.dense.tpr * FT;
+    const df Cx = tile_centre(a.xmin, (double)i0, FT, a.dx), Cy = tile_centre(a.ymin, (double)(a.row0 + j0), FT, a.dy);
+    const double X = a.xmin + (i0 + ic) * a.dx, Y = a.ymin + (a.row0 + j0 + jr) * a.dy;
+    const df Xd = df_kept(X), Yd = df_kept(Y);
+    df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+    for (int h0 = 0; h0 < a.n; h0 += FR_THREADS) {
+      const int h = h0 + tid;
+      const bool near = h < a.n && !repair_far(a.recdf + h, a.n, Cx, Cy, a.dense.thr, a.dense.thr_h);
+      const unsigned b = __ballot_sync(0xffffffffu, near);
+      __syncthreads();  // the previous chunk's records have been used
+      if (lane == 0) s_nn[warp] = __popc(b);
+      __syncthreads();
+      int base = 0, nn = 0;
+      for (int w = 0; w < FR_THREADS / 32; ++w) {
+        if (w < warp) base += s_nn[w];
+        nn += s_nn[w];
+      }
+      if (near) s_near[base + __popc(b & ((1u << lane) - 1u))] = h;
+      __syncthreads();
+      for (int q = tid; q < RECDF * nn; q += FR_THREADS) s_rdf[q / nn][q % nn] = a.recdf[(size_t)(q / nn) * a.n + s_near[q % nn]];
+      __syncthreads();
+      for (int k = 0; k < nn; ++k)
+        add_potential_dfs<false>(&s_rdf[0][k], FR_THREADS, a.all64 + (size_t)s_near[k] * REC64, X, Y, Xd, Yd, sum);
+    }
+    // the far potentials: rows of the tensor product, then the column
+    const FineTab<FT> &t = fine_table<FT>();
+#pragma unroll 1
+    for (int c = 0; c < 2; ++c) {
+      df v = sum[c];
+#pragma unroll 1
+      for (int j = 0; j < FP; ++j) {
+        df r = {0.f, 0.f};
+#pragma unroll
+        for (int i = 0; i < FP; ++i) {
+          const float2 f = s_val[c][j * FP + i];
+          r = df_add(r, df_mul(df{t.w[ic][i], t.wlo[ic][i]}, df{f.x, f.y}));
+        }
+        v = df_add(v, df_mul(df{t.w[jr][j], t.wlo[jr][j]}, r));
+      }
+      if (mine) a.out[c * a.plane + (long long)(j0 + jr) * a.nx + i0 + ic] = (float)(a.dls * df_to_double(v));
+    }
+  }
 }
 
 // ft = 0: the coarse kernel
@@ -758,6 +924,14 @@ size_t far_smem(int mode, int ft, int nw, int n) {
 constexpr double KF = 3.0, KF_H = 3.5, KC = 2.5, KC_H = 3.0;
 // fixed work in evaluations of one FP32 potential: per fine tile, per map node
 constexpr double TILE_COST = 4000.0, NODE_COST = 3.0;
+// densely listed tiles of the repair: from this many nodes, on maps of at
+// least this many nodes and potentials (below, the extra launch costs more
+// than the repair) and at most this many tiles (2.1 KB each)
+constexpr int DENSE_MIN = 150, DENSE_NODES = 1 << 19, DENSE_N = 64;
+constexpr long long DENSE_TILES = 65536;
+// margins of the repair: interpolation error below 4e-11 of a potential's own
+// deflection at the edge of its far region (4e-14 for the strong ones)
+constexpr double KR = 5.0, KR_H = 8.0;
 constexpr int FAR_MAX_N = 16384;  // potentials (two bytes each of shared memory)
 
 // Fraction of the map's nodes within psi < r of a potential of axis ratio q
@@ -777,7 +951,6 @@ int far_words(const Model *m) { return (m->n_light + 31) / 32 + (m->n_heavy + 31
 // them for a cluster-scale potential in double-float), idle SMs of small
 // grids included.
 FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode) {
-  (void)ctx;
   FarPlan p;
   if (m->n > FAR_MAX_N || m->n < 1) return p;
   const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
@@ -820,9 +993,60 @@ FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mo
     p.ncr = (g->ny + p.ct - 1) / p.ct;
     const size_t t = (size_t)p.nct * p.ncr;
     p.val_bytes = (t * coarse_floats(mode) * sizeof(float) + 255) & ~(size_t)255;
-    p.bytes = p.val_bytes + t * far_words(m) * sizeof(unsigned);
+    p.bytes = (p.val_bytes + t * far_words(m) * sizeof(unsigned) + 255) & ~(size_t)255;
+  }
+  if (p.use && mode != FAR_POT && ctx->repair_ratio > 0.0 && nodes >= DENSE_NODES && m->n >= DENSE_N && m->n_light > 0) {
+    const long long tiles = (long long)((g->nx + p.ft - 1) / p.ft) * ((g->ny + p.ft - 1) / p.ft);
+    p.rep_cap = tiles <= DENSE_TILES ? (int)tiles : 0;
+    p.rep_bytes = ((size_t)p.rep_cap * (sizeof(float2) * 2 * FP * FP + sizeof(int) + (size_t)p.ft * p.ft / 8) + 255) & ~(size_t)255;
+    p.bytes += p.rep_bytes;
   }
   return p;
+}
+
+DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, void *mem, int *count) {
+  DenseRepair d;
+  if (!mem || !p.rep_cap) return d;
+  d.count = count;
+  d.cap = p.rep_cap;
+  d.ft = p.ft;
+  d.tpr = (g->nx + p.ft - 1) / p.ft;
+  d.val = (float2 *)mem;
+  d.tile = (int *)(d.val + (size_t)p.rep_cap * 2 * FP * FP);
+  d.mask = (unsigned *)(d.tile + p.rep_cap);
+  const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
+  const double R = std::sqrt(2.0) * 0.5 * (p.ft - 1) * std::max(dx, dy);
+  d.thr = (float)(KR * R * KR * R);
+  d.thr_h = (float)(KR_H * R * KR_H * R);
+  for (int k = 0; k < FP; ++k) d.xi[k] = (float)((p.ft == 32 ? XiTab<32>::v[k] : XiTab<64>::v[k]) / 64.0);
+  return d;
+}
+
+int launch_far_repair(const Model *m, const lens_grid *g, const DenseRepair &dense, double dls, void *out, int row0,
+                      int rows, int device, cudaStream_t st) {
+  FarRepairArgs a;
+  a.recdf = m->recdf;
+  a.all64 = m->all64;
+  a.n = m->n;
+  a.xmin = g->xmin;
+  a.ymin = g->ymin;
+  a.dx = (g->xmax - g->xmin) / (g->nx - 1);
+  a.dy = (g->ymax - g->ymin) / (g->ny - 1);
+  a.nx = g->nx;
+  a.row0 = row0;
+  a.dls = dls;
+  a.out = (float *)out;
+  a.plane = (long long)g->nx * rows;
+  a.dense = dense;
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
+  if (dense.ft == 32)
+    k_far_repair<32><<<4 * nsm, FR_THREADS, 0, st>>>(a);
+  else
+    k_far_repair<64><<<4 * nsm, FR_THREADS, 0, st>>>(a);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LENS_ECUDA, "dense map repair launch: %s", cudaGetErrorString(e));
+  return LENS_OK;
 }
 
 static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem) {
@@ -862,6 +1086,7 @@ static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, in
   a.bx = a.by = 0.0;
   a.repair_f = 0.f;
   a.rep_count = a.rep_list = nullptr;
+  a.dense_min = DENSE_MIN;
   return a;
 }
 
@@ -894,8 +1119,8 @@ int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int 
 }
 
 int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, double dls, void *out,
-                   int row0, int rows, double repair, int *rep_count, int *rep_list, const double *beta,
-                   cudaStream_t st) {
+                   int row0, int rows, double repair, int *rep_count, int *rep_list, const DenseRepair &dense,
+                   const double *beta, cudaStream_t st) {
   FarArgs a = far_args(m, g, p, mode, mem);
   a.ny = rows;
   a.row0 = row0;
@@ -906,6 +1131,7 @@ int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mod
   a.repair_f = (float)(2.0 * repair);
   a.rep_count = rep_count;
   a.rep_list = rep_list;
+  a.dense = dense;
   if (mode == FAR_POT) {
     a.out64 = (double *)out;
     a.tau = beta != nullptr;

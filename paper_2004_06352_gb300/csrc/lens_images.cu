@@ -1800,7 +1800,7 @@ __global__ void __launch_bounds__(NW_THREADS, LENS_POLISH_MINB) k_img_polish(con
       // double-float; the rest (cores: |w|^2 >= 0.16, SIS, point masses)
       // queued and evaluated 32 at a time, so the warp stays converged, by
       // the double-float reductions of atan/atanh (FP64 only if those fail)
-      const df X = df_from_double(tx), Y = df_from_double(ty);
+      const df X = df_kept(tx), Y = df_kept(ty);
       df fx = {0.f, 0.f}, fy = {0.f, 0.f};
       double sx = 0.0, sy = 0.0;
       int nq = 0;

@@ -376,24 +376,49 @@ int check_grid(const lens_grid *g);
 // repair_mem: memory for the repair list (map_repair_bytes), else working
 // memory of the call.
 // far, far_mem: the interpolated form (lens_far.cu) with this plan, whose
-// coarse level has been computed into far_mem; NULL: direct.
+// coarse level has been computed into far_mem; NULL: direct.  dense_mem: the
+// plan's rep_bytes for this launch alone (NULL: every node to recompute is
+// listed).
 struct FarPlan {
   bool use = false;
   int ft = 32;                   // fine tile, nodes a side (32 or 64)
   int ct = 0, nct = 0, ncr = 0;  // coarse tile (0: no coarse level), coarse tiles per row and column
   size_t val_bytes = 0, bytes = 0;
   double cost = 0.0;             // expected cost per node in evaluations of one FP32 potential
+  // repair of densely listed tiles: slots (0: none) and bytes of one launch's
+  // DenseRepair arrays, which lie at byte `bytes - rep_bytes` of the plan's memory
+  int rep_cap = 0;
+  size_t rep_bytes = 0;
+};
+// Tiles of the interpolated maps in which so many nodes are to be recomputed
+// in double-float that the far potentials are evaluated at the tile's FAR_P x
+// FAR_P interpolation nodes instead of at each of them.
+constexpr int FAR_P = 10;
+constexpr float REPAIR_STRONG_BQ = 4.f;  // b q above which a potential takes the wider margin
+struct DenseRepair {
+  int *count = nullptr;      // tiles (may exceed cap: the rest are listed node by node)
+  int cap = 0, ft = 0, tpr = 0;
+  int *tile = nullptr;       // [cap] tile index
+  unsigned *mask = nullptr;  // [cap][ft * ft / 32] nodes to recompute, row-major
+  float2 *val = nullptr;     // [cap][2][FAR_P * FAR_P] the far potentials' deflection at the nodes
+  float thr = 0.f, thr_h = 0.f;  // squared psi beyond which a potential is far
+  float xi[FAR_P];           // the nodes, in grid steps about the tile's centre
 };
 int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
                      cudaStream_t st, int row0 = 0, int rows = -1, bool repair = true, void *repair_mem = nullptr,
-                     const FarPlan *far = nullptr, void *far_mem = nullptr);
+                     const FarPlan *far = nullptr, void *far_mem = nullptr, void *dense_mem = nullptr);
 // modes of the interpolated maps: 0 deflection, 1 deflection + Hessian, 2 potential
 // (rows of a band must be a multiple of the plan's fine tile)
 FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode);
 int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st);
 int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, double dls, void *out,
-                   int row0, int rows, double repair, int *rep_count, int *rep_list, const double *beta,
-                   cudaStream_t st);
+                   int row0, int rows, double repair, int *rep_count, int *rep_list, const DenseRepair &dense,
+                   const double *beta, cudaStream_t st);
+// the plan's DenseRepair arrays at mem, counting in *count; cap = 0 when mem is NULL
+DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, void *mem, int *count);
+// the listed nodes of the dense tiles, after the far potentials' values
+int launch_far_repair(const Model *m, const lens_grid *g, const DenseRepair &dense, double dls, void *out, int row0,
+                      int rows, int device, cudaStream_t st);
 size_t map_repair_bytes(const lens_grid *g, int rows = -1);
 int launch_map_fp64(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
                     cudaStream_t st, int row0 = 0, int rows = -1);

@@ -186,11 +186,11 @@ __global__ void __launch_bounds__(map_threads(MODE == MAP_HESS), MODE == MAP_HES
     if constexpr (!POT) {
       if (a.heavy_df) {
         // in double-float on the FP32 pipe (FP64 where that fails)
-        const df Xd = df_from_double(X);
+        const df Xd = df_kept(X);
 #pragma unroll 1
         for (int k = 0; k < KP; ++k) {
           const double Y = a.ymin + (a.row0 + j0 + warp * KP + k) * a.dy;
-          const df Yd = df_from_double(Y);
+          const df Yd = df_kept(Y);
           df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
           for (int h = 0; h < a.n_heavy; ++h)
             add_potential_dfs<HESS>(a.heavydf + (size_t)h * RECDF, 1, a.heavy + (size_t)h * REC64, X, Y, Xd, Yd,
@@ -482,34 +482,44 @@ struct RepairArgs {
   float *out;
   long long plane;
   const int *count, *list;
+  DenseRepair dense;  // densely listed tiles: the far potentials at their interpolation nodes
 };
 
-// LENS_REPAIR_DFSUM: each lane sums its terms in double-float and converts
-// once (0: every term converted and added in FP64, 20 FP64-pipe operations
-// per term with the Hessian)
-#ifndef LENS_REPAIR_DFSUM
-#define LENS_REPAIR_DFSUM 1
-#endif
 constexpr int REP_WARPS = 8, REP_THREADS = 32 * REP_WARPS, REP_CH = 32;  // potentials per staged chunk (one per lane)
 
+// Each lane sums its terms in double-float and converts once (adding every
+// term in FP64 takes 20 FP64-pipe operations per term with the Hessian).
+// After the listed nodes come the interpolation nodes of the densely listed
+// tiles (lens_far.cu): there the far potentials' deflection goes to
+// dense.val.
 template <bool HESS>
 __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) {
   __shared__ float2 s_rdf[RECDF][REP_CH];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int total = *a.count;
-  for (int e0 = blockIdx.x * REP_WARPS; e0 < total; e0 += gridDim.x * REP_WARPS) {  // uniform over the CTA
+  constexpr int NODES = FAR_P * FAR_P;
+  const int all = total + (a.dense.cap ? min(*a.dense.count, a.dense.cap) * NODES : 0);
+  for (int e0 = blockIdx.x * REP_WARPS; e0 < all; e0 += gridDim.x * REP_WARPS) {  // uniform over the CTA
     const int e = e0 + warp;
-    const bool have = e < total;
-    const int entry = have ? a.list[e] : 0;
+    const bool have = e < all, node = e >= total;  // node: an interpolation node
+    const int entry = have && !node ? a.list[e] : 0;
     const int o = entry & 0x7fffffff;
     const bool full = HESS && entry < 0;  // warp-uniform
-    const int i = o % a.nx, j = o / a.nx;
-    const double X = a.xmin + i * a.dx, Y = a.ymin + (a.row0 + j) * a.dy;
-#if LENS_REPAIR_DFSUM
-    const df Xd = df_from_double(X), Yd = df_from_double(Y);
+    const int slot = node ? (e - total) / NODES : 0, q = node ? (e - total) % NODES : 0;
+    double X, Y;
+    df Cx = {0.f, 0.f}, Cy = {0.f, 0.f};
+    if (have && node) {
+      const int tile = a.dense.tile[slot];
+      Cx = tile_centre(a.xmin, (double)(tile % a.dense.tpr * a.dense.ft), a.dense.ft, a.dx);
+      Cy = tile_centre(a.ymin, (double)(a.row0 + tile / a.dense.tpr * a.dense.ft), a.dense.ft, a.dy);
+      X = df_to_double(Cx) + a.dense.xi[q % FAR_P] * a.dx;
+      Y = df_to_double(Cy) + a.dense.xi[q / FAR_P] * a.dy;
+    } else {
+      X = a.xmin + (o % a.nx) * a.dx;
+      Y = a.ymin + (a.row0 + o / a.nx) * a.dy;
+    }
+    const df Xd = df_kept(X), Yd = df_kept(Y);
     df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-#endif
-    double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     for (int h0 = 0; h0 < a.n; h0 += REP_CH) {
       __syncthreads();  // the previous chunk has been used
       for (int t = threadIdx.x; t < RECDF * REP_CH; t += REP_THREADS) {
@@ -518,29 +528,28 @@ __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) 
       }
       __syncthreads();
       const int h = h0 + lane;
-      if (have && h < a.n) {
-#if LENS_REPAIR_DFSUM
+      if (have && h < a.n &&
+          (!node || repair_far(&s_rdf[0][lane], REP_CH, Cx, Cy, a.dense.thr, a.dense.thr_h))) {
         if (full)
           add_potential_dfs<true>(&s_rdf[0][lane], REP_CH, a.all64 + (size_t)h * REC64, X, Y, Xd, Yd, sum);
         else
           add_potential_dfs<false>(&s_rdf[0][lane], REP_CH, a.all64 + (size_t)h * REC64, X, Y, Xd, Yd, sum);
-#else
-        if (full)
-          add_potential_df<true>(&s_rdf[0][lane], REP_CH, a.all64 + (size_t)h * REC64, X, Y, acc);
-        else
-          add_potential_df<false>(&s_rdf[0][lane], REP_CH, a.all64 + (size_t)h * REC64, X, Y, acc);
-#endif
       }
     }
-#if LENS_REPAIR_DFSUM
+    double acc[5];
 #pragma unroll
     for (int c = 0; c < 5; ++c) acc[c] = df_to_double(sum[c]);
-#endif
 #pragma unroll
     for (int c = 0; c < (HESS ? 5 : 2); ++c)
 #pragma unroll
       for (int off = 16; off; off >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], off);
-    if (have && lane == 0) {
+    if (have && lane == 0 && node) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const df v = df_from_double(acc[c]);
+        a.dense.val[((size_t)slot * 2 + c) * NODES + q] = make_float2(v.hi, v.lo);
+      }
+    } else if (have && lane == 0) {
       a.out[o] = (float)(a.dls * acc[0]);
       a.out[a.plane + o] = (float)(a.dls * acc[1]);
       if (full) {
@@ -650,18 +659,20 @@ static int heavy_in_df(const Model *m) {
 
 int map_tile_rows(bool hess) { return map_threads(hess) / 32 * (hess ? LENS_KP_HESS : LENS_KP_GRAD); }
 
+// the list after the counts of listed nodes and of densely listed tiles
+constexpr int REP_HEADER = 4;
 size_t map_repair_bytes(const lens_grid *g, int rows) {
-  return sizeof(int) * ((size_t)g->nx * (size_t)(rows < 0 ? g->ny : rows) + 1);
+  return sizeof(int) * ((size_t)g->nx * (size_t)(rows < 0 ? g->ny : rows) + REP_HEADER);
 }
 
 int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
                      cudaStream_t st, int row0, int rows, bool repair, void *repair_mem, const FarPlan *far,
-                     void *far_mem) {
+                     void *far_mem, void *dense_mem) {
   if (rows < 0) rows = g->ny - row0;
   const long long nodes = (long long)g->nx * rows;
   if (nodes > INT32_MAX) return fail(LENS_EINVAL, "map launch of more than 2^31 points");
   repair = repair && ctx->repair_ratio > 0.0 && m->n_light > 0;
-  CallScratch rs(ctx, st);  // repair list: a count and up to one entry per node
+  CallScratch rs(ctx, st);  // repair list: the counts and up to one entry per node
   if (repair) {
     if (repair_mem) {
       rs.p = nullptr;  // the caller's memory (the request loop's arena)
@@ -670,7 +681,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
       if (rc) return rc;
       repair_mem = rs.p;
     }
-    if (cudaMemsetAsync(repair_mem, 0, sizeof(int), st) != cudaSuccess)
+    if (cudaMemsetAsync(repair_mem, 0, REP_HEADER * sizeof(int), st) != cudaSuccess)
       return fail(LENS_ECUDA, "cudaMemsetAsync failed");
   }
   MapArgs a;
@@ -699,11 +710,13 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
   a.repair = repair ? ctx->repair_ratio : 0.0;
   a.repair_f = (float)(2.0 * a.repair);
   a.rep_count = repair ? (int *)repair_mem : nullptr;
-  a.rep_list = repair ? (int *)repair_mem + 1 : nullptr;
+  a.rep_list = repair ? (int *)repair_mem + REP_HEADER : nullptr;
   constexpr int KPG = LENS_KP_GRAD, KPH = LENS_KP_HESS;
+  DenseRepair dense;
   if (far) {
+    if (repair && dense_mem) dense = dense_repair(g, *far, dense_mem, a.rep_count + 1);
     const int rc = launch_far_map(m, g, *far, hess, far_mem, dls, out, row0, rows, a.repair, a.rep_count, a.rep_list,
-                                  nullptr, st);
+                                  dense, nullptr, st);
     if (rc) return rc;
   } else if (hess) {
     const int th = map_tile_rows(true);
@@ -732,6 +745,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
     r.plane = a.plane;
     r.count = a.rep_count;
     r.list = a.rep_list;
+    r.dense = dense;
     int nsm = 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device);
     const int blocks = std::max(1, 4 * nsm);  // CTAs loop over the list: any count covers it
@@ -741,6 +755,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
       k_map_repair<false><<<blocks, REP_THREADS, 0, st>>>(r);
     e = cudaGetLastError();
     if (e != cudaSuccess) return fail(LENS_ECUDA, "map repair launch: %s", cudaGetErrorString(e));
+    if (dense.cap) return launch_far_repair(m, g, dense, dls, out, row0, rows, ctx->device, st);
   }
   return LENS_OK;
 }
@@ -780,7 +795,7 @@ int launch_pot_map(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls
     if (plan.use && plan.ct && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
     if (plan.use) {
       const int rc = launch_far_coarse(m, g, plan, 2, far.p, st);
-      return rc ? rc : launch_far_map(m, g, plan, 2, far.p, dls, out, 0, rows, 0.0, nullptr, nullptr, beta, st);
+      return rc ? rc : launch_far_map(m, g, plan, 2, far.p, dls, out, 0, rows, 0.0, nullptr, nullptr, DenseRepair(), beta, st);
     }
     MapArgs a;
     a.rec32 = m->rec32;

@@ -149,7 +149,8 @@ static int launch_req(lens_server *s, Slot &sl, Req *q) {
       if (q->far.use) rc = launch_far_coarse(m, &r.grid, q->far, r.hessian != 0, far_mem, st);
       if (!rc)
         rc = launch_map_mixed(ctx, m, &r.grid, r.dls_ds, r.hessian != 0, base, st, 0, -1, true, list,
-                              q->far.use ? &q->far : nullptr, far_mem);
+                              q->far.use ? &q->far : nullptr, far_mem,
+                              q->far.rep_bytes ? far_mem + q->far.bytes - q->far.rep_bytes : nullptr);
     }
   } else {
     CSet *c = find_cset(ctx, r.handle);
