@@ -60,30 +60,15 @@ struct Chi2SrcArgs {
   int nsrc, nimg, P, variant;
   int type0, type1;
   double *chi2;
+  int keep_xy;  // the images' positions as float pairs fit in shared memory
 };
 
 // Parameter sets whose varying potentials' records two warps build at a
 // time (one thread per record: the FP64 record arithmetic runs 32 lanes wide
 // instead of on two threads per set).
 constexpr int SRC_BATCH = 16;
+constexpr int SRC_INV = 16;  // image counts whose reciprocals are kept
 
-// resident warps per SM the source-plane kernel is compiled for (0: as its
-// registers allow, 118 at 128 threads; 20 warps: 96 registers and spills,
-// same speed; 24: 80 registers, 5 % slower)
-#ifndef LENS_SRC_WARPS
-#define LENS_SRC_WARPS 0
-#endif
-// the varying potentials' evaluator
-struct EvalChi2 {
-  template <bool HESS>
-  static __device__ __forceinline__ bool dpie(const float2 *r, df X, df Y, df &ax, df &ay, df *h) {
-    return dpie_df3<HESS, true>(r, X, Y, ax, ay, h);
-  }
-  template <bool HESS>
-  static __device__ __forceinline__ void circ(const float2 *r, df X, df Y, df &ax, df &ay, df *h) {
-    circ_df3<HESS>(r, X, Y, ax, ay, h);
-  }
-};
 // The FP64 record (kind 0; returns whether the parameters are inside the
 // domain) or the double-float record (kind 1) of varying potential v of a
 // parameter set, out of line.
@@ -92,28 +77,164 @@ __device__ __noinline__ bool var_rec_cold(const double *q, int type0, int type1,
   if (kind == 0) return load_var_rec64(q, type0, type1, v, s_rec);
   const double *w = q + 7 * v;
   make_recdf(v == 0 ? type0 : type1, w[0], w[1], w[3], w[2], w[4], w[5], w[6], s_rdf + v * RECDF);
-  record_uw(s_rdf + v * RECDF);
+  record_consts<true>(s_rdf + v * RECDF);
   return true;
 }
 
-// One kernel per Hessian mode (LENS_SRC_SPLIT): HESS = 1 for the variants
-// that need the Hessian, 0 for the plain residuals (72 registers instead of
-// 118: 0.241 -> 0.230 ms per 4096 sets; the Hessian variants unchanged);
-// -1: one kernel for all, the variant chosen at run time.
-#ifndef LENS_SRC_SPLIT
-#define LENS_SRC_SPLIT 1
-#endif
-template <int THREADS, int HESS = -1>
-__global__ void __launch_bounds__(THREADS, LENS_SRC_WARPS * 32 / THREADS) k_chi2_source(const Chi2SrcArgs a) {
+__device__ __forceinline__ Df<float> d_from_double(double d) {
+  const df v = df_from_double(d);
+  return {v.hi, v.lo};
+}
+// A finite float as a double by integer operations (conversions run on the
+// FP64 pipe, at 1/64 of the FP32 rate); subnormals become zero.
+__device__ __forceinline__ double f_to_double(float f) {
+  const int i = __float_as_int(f);
+  const bool zero = (i & 0x7f800000) == 0;
+  return __hiloint2double(zero ? 0 : (i & 0x80000000) | (((i >> 3) & 0x0fffffff) + (896 << 20)), zero ? 0 : i << 29);
+}
+__device__ __forceinline__ double d_to_double(float hi, float lo) {
+  if (!(fabsf(hi) < INFINITY)) return (double)hi;  // (rare: keeps NaN and infinity)
+  return f_to_double(hi) + f_to_double(lo);
+}
+
+// r alpha and r H of image j from its sums acc (static cache + varying
+// potentials): beta into s_beta and, if HESS, r hxx, r hyy, r hxy into s_m.
+template <bool HESS>
+__device__ __forceinline__ void store_image(const Chi2SrcArgs &a, int j, double X, double Y, const double *acc,
+                                            double *s_beta, double *s_m) {
+  const double r = a.ratio[a.src_of[j]];
+  s_beta[2 * j] = X - r * acc[0];
+  s_beta[2 * j + 1] = Y - r * acc[1];
+  if (HESS) {
+    s_m[3 * j] = r * (acc[2] + acc[3]);
+    s_m[3 * j + 1] = r * (acc[2] - acc[3]);
+    s_m[3 * j + 2] = r * acc[4];
+  }
+}
+
+// Back-trace of every image, two images per thread side by side (j and j +
+// ceil(nimg / 2)), which with the called division and polynomial and fewer
+// FP64 operations (positions as pairs, integer conversions) takes 0.284
+// instead of 0.341 ms per 4096 sets x 372 images: both varying potentials in double-float, summed in
+// double-float and added to the static cache with one conversion each; FP64
+// for a potential whose double-float evaluation fails.
+template <int THREADS, bool HESS>
+__device__ __forceinline__ void backtrace_pairs(const Chi2SrcArgs &a, const double *stat, const double *s_rec,
+                                                const float2 *s_rdf, const float4 *s_xy, double *s_beta, double *s_m) {
+  const int half = (a.nimg + 1) / 2;
+  for (int j0 = threadIdx.x; j0 < half; j0 += THREADS) {
+    const int j1 = j0 + half < a.nimg ? j0 + half : j0;  // (alone: a copy of itself, not stored)
+    Df<float2> X, Y, sum[5];
+    double acc[2][5];
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int j = k ? j1 : j0;
+      float4 xy;
+      if (a.keep_xy) {
+        xy = s_xy[j];
+      } else {
+        const Df<float> x = d_from_double(a.x[j]), y = d_from_double(a.y[j]);
+        xy = make_float4(x.hi, x.lo, y.hi, y.lo);
+      }
+      part2(X.hi, k) = xy.x;
+      part2(X.lo, k) = xy.y;
+      part2(Y.hi, k) = xy.z;
+      part2(Y.lo, k) = xy.w;
+#pragma unroll
+      for (int q = 0; q < (HESS ? 5 : 2); ++q) acc[k][q] = 0.0;
+    }
+    bool cold = false;
+#pragma unroll 1
+    for (int v = 0; v < 2; ++v) {  // one copy of the (large) evaluator in the code
+      Df<float2> t[5];
+      const unsigned ok = any_fixed<HESS, true>(s_rdf + v * RECDF, X, Y, t[0], t[1], t + 2);
+      if (ok != f_all<float2>) {
+        const Df<float2> zero = d_dup<float2>(0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < (HESS ? 5 : 2); ++q) t[q] = d_sel(ok, t[q], zero);
+        cold = true;
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+          if (!(ok >> k & 1u)) {
+            double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+            const int j = k ? j1 : j0;
+            eval64_cold<HESS>(s_rec + v * REC64, a.x[j], a.y[j], e);
+#pragma unroll
+            for (int q = 0; q < (HESS ? 5 : 2); ++q) acc[k][q] = v == 0 || acc[k][q] == 0.0 ? e[q] : acc[k][q] + e[q];
+          }
+      }
+#pragma unroll
+      for (int q = 0; q < (HESS ? 5 : 2); ++q) sum[q] = v == 0 ? t[q] : d_add(sum[q], t[q]);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int j = k ? j1 : j0;
+      if (k && j1 == j0) break;
+      const double *st = stat + (size_t)j * 5;
+      double o[5];
+#pragma unroll
+      for (int q = 0; q < (HESS ? 5 : 2); ++q)
+        o[q] = (cold ? st[q] + acc[k][q] : st[q]) + d_to_double(part2(sum[q].hi, k), part2(sum[q].lo, k));
+      store_image<HESS>(a, j, a.x[j], a.y[j], o, s_beta, s_m);
+    }
+  }
+}
+
+// The same with a thread per (image, potential), for calls of so few sets
+// that a CTA has an SM to itself: half the chain per thread.
+template <int THREADS, bool HESS>
+__device__ __forceinline__ void backtrace_split(const Chi2SrcArgs &a, const double *stat, const double *s_rec,
+                                                const float2 *s_rdf, double *s_beta, double *s_m) {
+  const int v = threadIdx.x & 1, lane0 = threadIdx.x & ~31;
+  for (int t0 = 0; 2 * a.nimg > t0 + lane0; t0 += THREADS) {  // whole warps
+    const int j = min((t0 + (int)threadIdx.x) >> 1, a.nimg - 1);
+    const double X = a.x[j], Y = a.y[j];
+    Df<float> t[5];
+    double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    const unsigned ok = any_fixed<HESS, true>(s_rdf + v * RECDF, d_from_double(X), d_from_double(Y), t[0], t[1], t + 2);
+    if (!ok) {
+      eval64_cold<HESS>(s_rec + v * REC64, X, Y, e);
+#pragma unroll
+      for (int q = 0; q < (HESS ? 5 : 2); ++q) t[q] = {0.f, 0.f};
+    }
+    const bool cold = __any_sync(0xffffffffu, !ok);
+    const double *st = stat + (size_t)j * 5;
+    double o[5];
+#pragma unroll
+    for (int q = 0; q < (HESS ? 5 : 2); ++q) {  // the odd thread's result joins the even one's
+      const Df<float> u = {__shfl_xor_sync(0xffffffffu, t[q].hi, 1), __shfl_xor_sync(0xffffffffu, t[q].lo, 1)};
+      double s = st[q];
+      if (cold) s = (s + e[q]) + __shfl_xor_sync(0xffffffffu, e[q], 1);
+      const Df<float> w = d_add(t[q], u);
+      o[q] = s + d_to_double(w.hi, w.lo);
+    }
+    if (v == 0 && (t0 + (int)threadIdx.x) >> 1 < a.nimg) store_image<HESS>(a, j, X, Y, o, s_beta, s_m);
+  }
+}
+
+// HESS: the variants that need the Hessian (the plain residuals take fewer
+// registers without it).  SPLIT: a thread per (image, varying potential),
+// else two images per thread.
+template <int THREADS, bool HESS, bool SPLIT>
+__global__ void __launch_bounds__(THREADS) k_chi2_source(const Chi2SrcArgs a) {
   static_assert(THREADS >= 4 * SRC_BATCH, "one thread per record of a batch");
   extern __shared__ double sm[];
   double *s_beta = sm;                   // [nimg][2]
   double *s_m = s_beta + 2 * a.nimg;     // [nimg][3]: r hxx, r hyy, r hxy
   double *s_bary = s_m + 3 * a.nimg;     // [nsrc][2]
   double *s_red = s_bary + 2 * a.nsrc;   // [THREADS/32]
+  // the images' positions as float pairs (two images per thread: read once per set)
+  float4 *s_xy = reinterpret_cast<float4 *>(sm + ((5 * a.nimg + 2 * a.nsrc + THREADS / 32 + 1) & ~1));
+  if (!SPLIT && a.keep_xy)
+    for (int j = threadIdx.x; j < a.nimg; j += THREADS) {
+      const Df<float> x = d_from_double(a.x[j]), y = d_from_double(a.y[j]);
+      s_xy[j] = make_float4(x.hi, x.lo, y.hi, y.lo);
+    }
   __shared__ double s_rec[SRC_BATCH][2 * REC64];   // FP64 records of the batch's varying potentials
   __shared__ float2 s_rdf[SRC_BATCH][2 * RECDF];   // the same in double-float
   __shared__ int s_ok[SRC_BATCH][2];
+  __shared__ double s_inv[SRC_INV];                // 1 / (a source's images)
+  if (const int k = (int)threadIdx.x - (THREADS - SRC_INV); k >= 0) s_inv[k] = k > 0 ? 1.0 / k : 0.0;  // (a warp that builds no records, where there is one)
   // this CTA's sets are p = blockIdx.x + j gridDim.x, taken SRC_BATCH at a time
   for (long long p0 = blockIdx.x; p0 < a.P; p0 += (long long)gridDim.x * SRC_BATCH) {
     __syncthreads();  // the previous batch's records are no longer read
@@ -133,15 +254,30 @@ __global__ void __launch_bounds__(THREADS, LENS_SRC_WARPS * 32 / THREADS) k_chi2
         if (threadIdx.x == 0) a.chi2[p] = __longlong_as_double(0x7ff8000000000000ll);
         continue;
       }
-      const bool hess = HESS < 0 ? a.variant != LENS_CHI2_SRC_PLAIN : HESS == 1;
-      backtrace_set<THREADS, HESS, EvalChi2>(a.stat + p * a.stat_stride, a.x, a.y, a.ratio, a.src_of, a.img_off, a.nimg,
-                                   a.nsrc, s_rec[k], s_rdf[k], s_beta, hess ? s_m : nullptr, s_bary);
+      const double *stat = a.stat + p * a.stat_stride;
+      if (SPLIT)
+        backtrace_split<THREADS, HESS>(a, stat, s_rec[k], s_rdf[k], s_beta, s_m);
+      else
+        backtrace_pairs<THREADS, HESS>(a, stat, s_rec[k], s_rdf[k], s_xy, s_beta, s_m);
+      __syncthreads();
+      for (int i = threadIdx.x; i < a.nsrc; i += THREADS) {  // each source's barycentre (Fig. 3)
+        const int b = a.img_off[i], e = a.img_off[i + 1];
+        double sx = 0, sy = 0;
+        for (int j = b; j < e; ++j) {
+          sx += s_beta[2 * j];
+          sy += s_beta[2 * j + 1];
+        }
+        const double im = e - b < SRC_INV ? s_inv[e - b] : 1.0 / (e - b);
+        s_bary[2 * i] = sx * im;
+        s_bary[2 * i + 1] = sy * im;
+      }
+      __syncthreads();
       double acc[1] = {0.0};
       for (int j = threadIdx.x; j < a.nimg; j += THREADS) {
         const int i = a.src_of[j];
         const double dbx = s_bary[2 * i] - s_beta[2 * j], dby = s_bary[2 * i + 1] - s_beta[2 * j + 1];
         const double is2 = a.isig2[j];
-        if (a.variant == LENS_CHI2_SRC_PLAIN) {
+        if (!HESS) {
           acc[0] += (dbx * dbx + dby * dby) * is2;
         } else {
           // A^-1 = I - r H (Sec. 2.1 Eq. 4)
@@ -175,14 +311,17 @@ int build_static_cache(lens_ctx *ctx, const Model *m, CSet *c) {
   return LENS_OK;
 }
 
-template <int T>
+template <int T, bool SPLIT = false>
 static int launch_src_cfg(lens_ctx *ctx, const CSet *c, const double *d_params, int32_t P, int32_t variant,
                           double *d_chi2, cudaStream_t st, int blocks_per_sm, const double *stat = nullptr,
                           long long stat_stride = 0, int pstride = 14) {
-  const size_t smem = sizeof(double) * (5 * (size_t)c->nimg + 2 * (size_t)c->nsrc + T / 32);
-  if (smem > 200 * 1024) return fail(LENS_EINVAL, "constraint set too large for one CTA (%d images)", c->nimg);
-  const int H = LENS_SRC_SPLIT ? (variant == LENS_CHI2_SRC_PLAIN ? 0 : 1) : -1;
-  auto kern = H < 0 ? k_chi2_source<T, -1> : H == 0 ? k_chi2_source<T, 0> : k_chi2_source<T, 1>;
+  const size_t words = 5 * (size_t)c->nimg + 2 * (size_t)c->nsrc + T / 32;
+  if (sizeof(double) * words > 200 * 1024) return fail(LENS_EINVAL, "constraint set too large for one CTA (%d images)", c->nimg);
+  // the pair form also keeps the positions there when they fit
+  const size_t with_xy = sizeof(double) * ((words + 1) & ~(size_t)1) + sizeof(float4) * (size_t)c->nimg;
+  const bool keep_xy = !SPLIT && with_xy <= 100 * 1024;
+  const size_t smem = keep_xy ? with_xy : sizeof(double) * words;
+  auto kern = variant == LENS_CHI2_SRC_PLAIN ? k_chi2_source<T, false, SPLIT> : k_chi2_source<T, true, SPLIT>;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
   int per_sm = 0, nsm = 0;
   cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, T, smem);
@@ -208,6 +347,7 @@ static int launch_src_cfg(lens_ctx *ctx, const CSet *c, const double *d_params, 
   a.type0 = c->var_type[0];
   a.type1 = c->var_type[1];
   a.chi2 = d_chi2;
+  a.keep_xy = keep_xy;
   kern<<<blocks, T, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "chi2 source launch: %s", cudaGetErrorString(e));
@@ -216,22 +356,68 @@ static int launch_src_cfg(lens_ctx *ctx, const CSet *c, const double *d_params, 
 
 // Launch shapes the autotuner chooses from: threads per CTA x CTAs per SM
 // (0 = as many as fit).
-static const int SRC_CFG[][2] = {{64, 0}, {64, 8}, {128, 0}, {128, 4}, {128, 2}, {256, 0}, {256, 2}, {256, 1}};
+static const int SRC_CFG[][2] = {{64, 0}, {64, 4}, {64, 2}, {128, 0}, {128, 2}, {128, 1}, {256, 0}, {256, 1}};
 constexpr int N_SRC_CFG = sizeof(SRC_CFG) / sizeof(SRC_CFG[0]);
 
-static int launch_src_idx(lens_ctx *ctx, const CSet *c, const double *d_params, int32_t P, int32_t variant,
-                          double *d_chi2, cudaStream_t st, int idx) {
-  const int t = SRC_CFG[idx][0], b = SRC_CFG[idx][1];
-  if (t == 64) return launch_src_cfg<64>(ctx, c, d_params, P, variant, d_chi2, st, b);
-  if (t == 256) return launch_src_cfg<256>(ctx, c, d_params, P, variant, d_chi2, st, b);
-  return launch_src_cfg<128>(ctx, c, d_params, P, variant, d_chi2, st, b);
+static int launch_src(lens_ctx *ctx, const CSet *c, const double *d_params, int32_t P, int32_t variant, double *d_chi2,
+                      cudaStream_t st, int threads, int cap, const double *stat = nullptr, long long stat_stride = 0,
+                      int pstride = 14) {
+  switch (threads) {
+    case 64: return launch_src_cfg<64>(ctx, c, d_params, P, variant, d_chi2, st, cap, stat, stat_stride, pstride);
+    case 96: return launch_src_cfg<96>(ctx, c, d_params, P, variant, d_chi2, st, cap, stat, stat_stride, pstride);
+    case 192: return launch_src_cfg<192>(ctx, c, d_params, P, variant, d_chi2, st, cap, stat, stat_stride, pstride);
+    case 256: return launch_src_cfg<256>(ctx, c, d_params, P, variant, d_chi2, st, cap, stat, stat_stride, pstride);
+    default: return launch_src_cfg<128>(ctx, c, d_params, P, variant, d_chi2, st, cap, stat, stat_stride, pstride);
+  }
+}
+
+// The launch shape without a tuned one, from a sweep of 100 to 4096 sets x 18
+// to 340 images (us; each pair of numbers with and without the Hessian):
+//   - up to 64 images: a thread per (image, potential), 128 threads (4096 sets
+//     x 44 images 76.5 / 57.0; image pairs leave half the warps idle: 101 / 76);
+//   - a set per SM, or up to 160 images and 1000 sets: the same with 512 or 256
+//     threads (100 x 340: 31.0 / 24.9 against 39 / 31; 700 x 93: 37 / 29
+//     against 41 / 33);
+//   - else image pairs: in one round while every CTA is resident (700 x 340: 192
+//     threads 70 / 50, 64 82 / 64), then the threads that leave the fewest idle
+//     in the last round, small CTAs when they are many (4096 x 340: 64 threads
+//     282 / 223, 96 297 / 199, 192 297 / 217).
+static int launch_src_default(lens_ctx *ctx, const CSet *c, const double *d_params, int32_t P, int32_t variant,
+                              double *d_chi2, cudaStream_t st, const double *stat = nullptr, long long stat_stride = 0,
+                              int pstride = 14) {
+  int nsm = 0;
+  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, ctx->device);
+  const bool few = P <= nsm, some = P <= 8 * nsm;
+  if (c->nimg <= 64)
+    return launch_src_cfg<128, true>(ctx, c, d_params, P, variant, d_chi2, st, 0, stat, stat_stride, pstride);
+  if (few && c->nimg > 128)
+    return launch_src_cfg<512, true>(ctx, c, d_params, P, variant, d_chi2, st, 0, stat, stat_stride, pstride);
+  if (few || (some && c->nimg <= 160))
+    return launch_src_cfg<256, true>(ctx, c, d_params, P, variant, d_chi2, st, 0, stat, stat_stride, pstride);
+  const int pairs = (c->nimg + 1) / 2;
+  int best = 96;
+  if (some) {
+    best = pairs <= 128 ? 128 : 192;
+  } else {
+    int least = INT32_MAX;
+    const bool many = P > 20 * nsm && variant != LENS_CHI2_SRC_PLAIN;
+    for (int t : {many ? 64 : 96, many ? 96 : 64, 128, 192}) {
+      const int slots = (pairs + t - 1) / t * t;
+      if (slots < least) {
+        least = slots;
+        best = t;
+      }
+    }
+  }
+  return launch_src(ctx, c, d_params, P, variant, d_chi2, st, best, 0, stat, stat_stride, pstride);
 }
 
 int launch_chi2_source(lens_ctx *ctx, const Model *m, const CSet *c, const double *d_params, int32_t P,
                        int32_t variant, double *d_chi2, cudaStream_t st) {
   (void)m;
-  const int idx = (c->tuned_cfg >= 0 && c->tuned_cfg < N_SRC_CFG) ? c->tuned_cfg : 2;
-  return launch_src_idx(ctx, c, d_params, P, variant, d_chi2, st, idx);
+  if (c->tuned_cfg >= 0 && c->tuned_cfg < N_SRC_CFG)
+    return launch_src(ctx, c, d_params, P, variant, d_chi2, st, SRC_CFG[c->tuned_cfg][0], SRC_CFG[c->tuned_cfg][1]);
+  return launch_src_default(ctx, c, d_params, P, variant, d_chi2, st);
 }
 
 // Static sums of the no-cache form, grid (nimg, sets): every static potential
@@ -294,7 +480,7 @@ int launch_chi2_source_nocache(lens_ctx *ctx, const Model *m, const CSet *c, con
                                                              c->y, stat);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(LENS_ECUDA, "static sums launch: %s", cudaGetErrorString(e));
-    const int rc = launch_src_cfg<128>(ctx, c, d_params + (size_t)p0 * 14, B, variant, d_chi2 + p0, st, 0, stat,
+    const int rc = launch_src_default(ctx, c, d_params + (size_t)p0 * 14, B, variant, d_chi2 + p0, st, stat,
                                        (long long)c->nimg * 5);
     if (rc) return rc;
   }
@@ -310,34 +496,39 @@ int launch_chi2_source_nocache(lens_ctx *ctx, const Model *m, const CSet *c, con
 // st' + sc, q^2 (st' +- sc), q^2 (st'^2 - sc^2)).  FP64 (a record rescaled the
 // same way) where the double-float evaluation fails.  Outside the domain
 // (f_b <= 0, f_t r_cut,i <= r_core,i) the set's sums are NaN.
+// A CTA takes two images side by side (grid (pairs, sets)): a potential's
+// record is rescaled once for both.  Bound: instruction fetch and the FMA pipe
+// (60 % busy); 512 sets x 372 images x 998 potentials 15.3 -> 11.0 ms (compiled
+// for 4 or 5 CTAs per SM instead of 3: 11.2, 11.5).
 __global__ void __launch_bounds__(CACHE_THREADS) k_static_scaled(const float2 *__restrict__ recdf,
                                                                  const double *__restrict__ all64, int n, int v0,
                                                                  int v1, const double *__restrict__ x,
-                                                                 const double *__restrict__ y,
+                                                                 const double *__restrict__ y, int nimg,
                                                                  const double *__restrict__ params, double *stat) {
-  __shared__ double s_red[(CACHE_THREADS / 32) * 5];
-  const int img = blockIdx.x;
-  stat += (size_t)blockIdx.y * gridDim.x * 5;
+  __shared__ double s_red[(CACHE_THREADS / 32) * 16];
+  const int img[2] = {(int)blockIdx.x, min((int)(blockIdx.x + gridDim.x), nimg - 1)};
+  stat += (size_t)blockIdx.y * nimg * 5;
   const double fb = params[(size_t)blockIdx.y * 16 + 14], ft = params[(size_t)blockIdx.y * 16 + 15];
-  const double X = x[img], Y = y[img];
-  const df Xd = df_kept(X), Yd = df_kept(Y), fd = df_kept(ft), f2 = df_mul(fd, fd);
-  double v[5] = {0, 0, 0, 0, 0};
-  df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
+  Df<float2> X, Y, sum[5];
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const df xd = df_kept(x[img[k]]), yd = df_kept(y[img[k]]);
+    part2(X.hi, k) = xd.hi;
+    part2(X.lo, k) = xd.lo;
+    part2(Y.hi, k) = yd.hi;
+    part2(Y.lo, k) = yd.lo;
+  }
+#pragma unroll
+  for (int q = 0; q < 5; ++q) sum[q] = d_dup<float2>(0.f, 0.f);
+  const df fd = df_kept(ft), f2 = df_mul(fd, fd);
+  double v[16] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
   bool bad = !(fb > 0.0 && ft > 0.0 && isfinite(fb) && isfinite(ft));
   for (int h = threadIdx.x; h < n && !bad; h += CACHE_THREADS) {
     if (h == v0 || h == v1) continue;
-    const float2 *g = recdf + h;
-    df ax, ay, hh[3];
-    bool ok = true;
-    if (g[F_U2 * n].x < 0.f) {
-      float2 r[RECDF];
+    float2 r[RECDF];
 #pragma unroll
-      for (int k = 0; k < RECDF; ++k) r[k] = g[k * n];
-      circ_df3<true>(r, Xd, Yd, ax, ay, hh);
-    } else {
-      float2 r[RECDF];
-#pragma unroll
-      for (int k = 0; k < RECDF; ++k) r[k] = g[k * n];
+    for (int k = 0; k < RECDF; ++k) r[k] = recdf[h + (size_t)k * n];
+    if (!(r[F_U2].x < 0.f)) {
       auto D = [&](int k) { return df{r[k].x, r[k].y}; };
       auto put = [&](int k, df d) { r[k] = make_float2(d.hi, d.lo); };
       const df st = df_mul(D(F_ST), fd), sc = D(F_SC), q2st = df_mul(D(F_Q2ST), fd);
@@ -352,31 +543,61 @@ __global__ void __launch_bounds__(CACHE_THREADS) k_static_scaled(const float2 *_
       put(F_DT0, df_mul(D(F_DT0), f2));
       put(F_U2ST2, df_mul(D(F_U2ST2), f2));
       put(F_KTC, df_mul(q2ds, ss));
-      ok = dpie_df3<true, false>(r, Xd, Yd, ax, ay, hh);
+      record_consts<false>(r);
     }
-    if (ok) {
-      sum[0] = df_add(sum[0], ax);
-      sum[1] = df_add(sum[1], ay);
-      sum[2] = df_add(sum[2], hh[0]);
-      sum[3] = df_add(sum[3], hh[1]);
-      sum[4] = df_add(sum[4], hh[2]);
-    } else {
-      double q[REC64], e[5] = {0, 0, 0, 0, 0};
-      for (int k = 0; k < REC64; ++k) q[k] = all64[(size_t)h * REC64 + k];
-      q[D_ST] *= ft;
-      q[D_DS] = q[D_ST] - q[D_SC];
-      q[D_SS] = q[D_ST] + q[D_SC];
-      eval64<true>(q, X, Y, e[0], e[1], e[2], e[3], e[4]);
+    Df<float2> t[5];
+    const unsigned ok = any_fixed<true, false>(r, X, Y, t[0], t[1], t + 2);
+    if (ok != f_all<float2>) {
+      const Df<float2> zero = d_dup<float2>(0.f, 0.f);
 #pragma unroll
-      for (int k = 0; k < 5; ++k) v[k] += e[k];
+      for (int q = 0; q < 5; ++q) t[q] = d_sel(ok, t[q], zero);
+      double g[REC64];
+      for (int k = 0; k < REC64; ++k) g[k] = all64[(size_t)h * REC64 + k];
+      g[D_ST] *= ft;
+      g[D_DS] = g[D_ST] - g[D_SC];
+      g[D_SS] = g[D_ST] + g[D_SC];
+#pragma unroll
+      for (int k = 0; k < 2; ++k)
+        if (!(ok >> k & 1u)) {
+          double e[5] = {0, 0, 0, 0, 0};
+          eval64_cold<true>(g, x[img[k]], y[img[k]], e);
+#pragma unroll
+          for (int q = 0; q < 5; ++q) v[5 * k + q] += e[q];
+        }
     }
+#pragma unroll
+    for (int q = 0; q < 5; ++q) sum[q] = d_add(sum[q], t[q]);
   }
 #pragma unroll
-  for (int k = 0; k < 5; ++k) v[k] = fb * (v[k] + df_to_double(sum[k]));
+  for (int k = 0; k < 2; ++k)
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+      v[5 * k + q] = fb * (v[5 * k + q] + d_to_double(part2(sum[q].hi, k), part2(sum[q].lo, k)));
   const int any_bad = __syncthreads_or(bad);
-  block_sum<5, CACHE_THREADS>(v, s_red);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 5; ++k) stat[(size_t)img * 5 + k] = any_bad ? __longlong_as_double(0x7ff8000000000000ll) : v[k];
+  // the CTA's sums: a warp's lanes halve the values they carry at every step
+  // of the butterfly (16 additions a lane instead of 50; block_sum's tree, so
+  // its bits), lane 2 m then holds value m
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int o = 16, w = 8; o >= 2; o >>= 1, w >>= 1) {
+    const bool up = (lane & o) != 0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (k < w) {
+        const double mine = up ? v[k + w] : v[k], other = up ? v[k] : v[k + w];
+        v[k] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+  }
+  v[0] += __shfl_xor_sync(0xffffffffu, v[0], 1);
+  // the value this lane holds: bit 3 from lane bit 4, ... bit 0 from lane bit 1
+  const int m = lane >> 1;
+  if ((lane & 1) == 0) s_red[warp * 16 + m] = v[0];
+  __syncthreads();
+  if (threadIdx.x < 10 && (threadIdx.x < 5 || blockIdx.x + gridDim.x < nimg)) {
+    double t = 0.0;
+    for (int w = 0; w < CACHE_THREADS / 32; ++w) t += s_red[w * 16 + threadIdx.x];
+    stat[(size_t)img[threadIdx.x / 5] * 5 + threadIdx.x % 5] = any_bad ? __longlong_as_double(0x7ff8000000000000ll) : t;
+  }
 }
 
 // Static sums of each set from the scaling cache, grid (sets of the batch):
@@ -432,8 +653,8 @@ __global__ void __launch_bounds__(CACHE_THREADS) k_scaled_interp(const double *_
 int build_scaling_cache(lens_ctx *ctx, const Model *m, CSet *c, const double *d_nodes16, int32_t nodes) {
   cudaStream_t st = upload_stream(ctx);
   if (!st) return fail(LENS_ECUDA, "upload stream creation failed");
-  k_static_scaled<<<dim3(c->nimg, nodes), CACHE_THREADS, 0, st>>>(m->recdf, m->all64, m->n, c->var[0], c->var[1],
-                                                                  c->x, c->y, d_nodes16, c->scale_cache);
+  k_static_scaled<<<dim3((c->nimg + 1) / 2, nodes), CACHE_THREADS, 0, st>>>(m->recdf, m->all64, m->n, c->var[0], c->var[1],
+                                                                  c->x, c->y, c->nimg, d_nodes16, c->scale_cache);
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return fail(LENS_ECUDA, "scaling cache: %s", cudaGetErrorString(e));
@@ -452,11 +673,11 @@ int launch_chi2_source_scaled(lens_ctx *ctx, const Model *m, const CSet *c, cons
       k_scaled_interp<<<B, CACHE_THREADS, 0, st>>>(c->scale_cache, c->scale_x, c->scale_nodes, c->ft_min,
                                                     c->ft_max, c->nimg, d_params + (size_t)p0 * 16, stat);
     else
-      k_static_scaled<<<dim3(c->nimg, B), CACHE_THREADS, 0, st>>>(m->recdf, m->all64, m->n, c->var[0], c->var[1],
-                                                                   c->x, c->y, d_params + (size_t)p0 * 16, stat);
+      k_static_scaled<<<dim3((c->nimg + 1) / 2, B), CACHE_THREADS, 0, st>>>(m->recdf, m->all64, m->n, c->var[0], c->var[1],
+                                                                   c->x, c->y, c->nimg, d_params + (size_t)p0 * 16, stat);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return fail(LENS_ECUDA, "scaled static sums launch: %s", cudaGetErrorString(e));
-    const int rc = launch_src_cfg<128>(ctx, c, d_params + (size_t)p0 * 16, B, variant, d_chi2 + p0, st, 0, stat,
+    const int rc = launch_src_default(ctx, c, d_params + (size_t)p0 * 16, B, variant, d_chi2 + p0, st, stat,
                                        (long long)c->nimg * 5, 16);
     if (rc) return rc;
   }
@@ -474,10 +695,10 @@ int autotune_chi2_source(lens_ctx *ctx, CSet *c, const double *d_params, int32_t
   float best_t = 1e30f;
   int rc = LENS_OK;
   for (int k = 0; k < N_SRC_CFG && rc == LENS_OK; ++k) {
-    rc = launch_src_idx(ctx, c, d_params, P, 0, d_chi2, st, k);
+    rc = launch_src(ctx, c, d_params, P, 0, d_chi2, st, SRC_CFG[k][0], SRC_CFG[k][1]);
     for (int r = 0; r < 3 && rc == LENS_OK; ++r) {
       cudaEventRecord(e0, st);
-      rc = launch_src_idx(ctx, c, d_params, P, 0, d_chi2, st, k);
+      rc = launch_src(ctx, c, d_params, P, 0, d_chi2, st, SRC_CFG[k][0], SRC_CFG[k][1]);
       cudaEventRecord(e1, st);
       if (cudaEventSynchronize(e1) != cudaSuccess) rc = fail(LENS_ECUDA, "autotune timing failed");
       float ms = 0.f;

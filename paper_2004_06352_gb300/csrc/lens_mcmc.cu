@@ -46,10 +46,12 @@ __device__ __forceinline__ double unit_open(unsigned long long x) {
 }
 
 // Proposals into prop [W][NP] and the acceptance uniforms into ua [W]: one
-// thread per (chain, Philox block j = 0..3), each block's four words giving
-// two Box-Muller pairs (parameters 4j .. 4j+3 where < NP); the j = 0 thread
-// also draws block 4 for the acceptance uniform.  (One thread per chain left
-// most SMs idle: 4096 chains are 32 CTAs of 128.)
+// thread per (chain, Box-Muller pair), parameters 2 i and 2 i + 1 from the
+// half block j = i / 2 of the chain; the eighth pair's thread also draws
+// block 4 for the acceptance uniform.  Bound: the latency of one chain of
+// integer rounds and an FP64 logarithm, root, sine and cosine, so the pairs
+// are spread over as many threads as there are (4096 chains: 11.4 us with two
+// pairs per thread).
 // The step's counter word is `step`, or *d_step when d_step is not NULL
 // (a counter in device memory that the acceptance kernel advances).
 template <int NP>
@@ -57,43 +59,45 @@ __global__ void k_mcmc_propose(const double *__restrict__ params, const double *
                                unsigned long long seed, unsigned long long step,
                                const unsigned long long *__restrict__ d_step, double *__restrict__ prop,
                                double *__restrict__ ua) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  const int w = t >> 2, j = t & 3;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int w = (int)(t >> 3), k = (int)(t & 7);
   if (w >= W) return;
   if (d_step) step = *d_step;
-  const U4 r = philox4x64_10(U4{{step, (unsigned long long)w, (unsigned long long)j, 0ull}}, seed, 0ull);
-  const double two_pi = 6.283185307179586;
-#pragma unroll
-  for (int h = 0; h < 2; ++h) {
-    const int i = 4 * j + 2 * h;  // parameters i, i + 1
-    if (i >= NP) break;
-    const double rad = sqrt(-2.0 * log(unit_open(r.w[2 * h]))), ang = two_pi * unit_open(r.w[2 * h + 1]);
+  const int i = 2 * k;  // parameters i, i + 1
+  if (i < NP) {
+    const U4 r = philox4x64_10(U4{{step, (unsigned long long)w, (unsigned long long)(k >> 1), 0ull}}, seed, 0ull);
+    const unsigned long long r0 = k & 1 ? r.w[2] : r.w[0], r1 = k & 1 ? r.w[3] : r.w[1];
+    const double two_pi = 6.283185307179586;
+    const double rad = sqrt(-2.0 * log(unit_open(r0))), ang = two_pi * unit_open(r1);
     const size_t o = (size_t)w * NP + i;
     prop[o] = params[o] + sigma[i] * (rad * cos(ang));
     prop[o + 1] = params[o + 1] + sigma[i + 1] * (rad * sin(ang));
   }
-  if (j == 0) ua[w] = unit_open(philox4x64_10(U4{{step, (unsigned long long)w, 4ull, 0ull}}, seed, 0ull).w[0]);
+  if (k == 7) ua[w] = unit_open(philox4x64_10(U4{{step, (unsigned long long)w, 4ull, 0ull}}, seed, 0ull).w[0]);
 }
 
 // Metropolis acceptance; accepted[w] (when not NULL) records the decision.
-// With a device step counter, one thread advances it: the proposal kernel of
-// this step has finished reading it (stream order), the next step reads the
-// new value.
+// A warp decides for 32 chains, one per lane, then copies the accepted
+// proposals together (consecutive numbers per lane: 4096 chains 8.5 us with
+// every lane copying its own chain's row).  With a device step counter, one
+// thread advances it: the proposal kernel of this step has finished reading it
+// (stream order), the next step reads the new value.
 __global__ void k_mcmc_accept(double *__restrict__ params, double *__restrict__ chi2,
                               const double *__restrict__ prop, const double *__restrict__ ua,
                               const double *__restrict__ chi2_prop, int W, int np, double temperature,
                               int32_t *__restrict__ accepted, unsigned long long *__restrict__ d_step) {
-  const int w = blockIdx.x * blockDim.x + threadIdx.x;
+  const int w = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, w0 = w - lane;
   if (d_step && w == 0) *d_step += 1ull;
-  if (w >= W) return;
-  const double cp = chi2_prop[w], c0 = chi2[w];
   bool take = false;
-  if (isfinite(cp)) take = !isfinite(c0) || log(ua[w]) < -(cp - c0) / (2.0 * temperature);
-  if (take) {
-    for (int q = 0; q < np; ++q) params[(size_t)w * np + q] = prop[(size_t)w * np + q];
-    chi2[w] = cp;
+  if (w < W) {
+    const double cp = chi2_prop[w], c0 = chi2[w];
+    if (isfinite(cp)) take = !isfinite(c0) || log(ua[w]) < -(cp - c0) / (2.0 * temperature);
+    if (take) chi2[w] = cp;
+    if (accepted) accepted[w] = take ? 1 : 0;
   }
-  if (accepted) accepted[w] = take ? 1 : 0;
+  const unsigned moved = __ballot_sync(0xffffffffu, take);
+  for (int k = lane; k < 32 * np; k += 32)
+    if (moved >> (k / np) & 1u) params[(size_t)w0 * np + k] = prop[(size_t)w0 * np + k];
 }
 
 }  // namespace
@@ -103,7 +107,8 @@ int launch_mcmc_step(lens_ctx *ctx, const Model *m, const CSet *c, double *d_par
                      int32_t variant, int32_t np, double *d_scratch, int32_t *d_accepted, cudaStream_t st,
                      unsigned long long *d_step) {
   double *prop = d_scratch, *ua = d_scratch + (size_t)W * np, *chi2_prop = ua + W;
-  const int blocks = (W + 127) / 128, pblocks = (4 * W + 127) / 128;
+  const int blocks = (W + 31) / 32;
+  const unsigned pblocks = (unsigned)((8 * (long long)W + 127) / 128);
   if (np == 16)
     k_mcmc_propose<16><<<pblocks, 128, 0, st>>>(d_params, d_sigma, W, seed, step, d_step, prop, ua);
   else
@@ -113,7 +118,7 @@ int launch_mcmc_step(lens_ctx *ctx, const Model *m, const CSet *c, double *d_par
   const int rc = np == 16 ? launch_chi2_source_scaled(ctx, m, c, prop, W, variant, chi2_prop, st)
                           : launch_chi2_source(ctx, m, c, prop, W, variant, chi2_prop, st);
   if (rc) return rc;
-  k_mcmc_accept<<<blocks, 128, 0, st>>>(d_params, d_chi2, prop, ua, chi2_prop, W, np, temperature, d_accepted,
+  k_mcmc_accept<<<blocks, 32, 0, st>>>(d_params, d_chi2, prop, ua, chi2_prop, W, np, temperature, d_accepted,
                                         d_step);
   e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "acceptance launch: %s", cudaGetErrorString(e));
