@@ -738,10 +738,10 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     }
   }
   if (POT || !(a.repair_f > 0.f)) return;
-  // the nodes to recompute: a tile with many of them that need the
-  // deflection alone goes to the dense tiles, the others' nodes to the list
+  // the nodes to recompute: a tile with many of them goes to the dense tiles
+  // (all planes' nodes with it where they are many), the others' to the list
   constexpr int NW = FT * FT / 32;
-  __shared__ int s_pos[2 * NW], s_to[3];  // list positions; list base, dense slot (or -1), listed words
+  __shared__ int s_pos[2 * NW], s_to[3];  // list positions; listed nodes, dense slot (or -1), its all-planes flag
   __syncthreads();
   if (warp == 0) {
     int n1 = 0, nh = 0;
@@ -752,18 +752,20 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     n1 = __reduce_add_sync(0xffffffffu, n1);
     nh = __reduce_add_sync(0xffffffffu, nh);
     int slot = -1;
-    if (lane == 0 && a.dense.cap && n1 >= a.dense_min) {
+    const bool full = HESS && nh >= a.dense_min;
+    if (lane == 0 && a.dense.cap && (full || n1 >= a.dense_min)) {
       slot = atomicAdd(a.dense.count, 1);
       if (slot >= a.dense.cap) slot = -1;
     }
     slot = __shfl_sync(0xffffffffu, slot, 0);
-    const int nl = nh + (slot < 0 ? n1 : 0);
+    const bool list_h = slot < 0 || !full;
+    const int nl = (list_h ? nh : 0) + (slot < 0 ? n1 : 0);
     int base = 0;
     if (lane == 0 && nl) base = atomicAdd(a.rep_count, nl);
     base = __shfl_sync(0xffffffffu, base, 0);
     for (int w0 = 0; w0 < 2 * NW && nl; w0 += 32) {  // all-plane words, then the others
       const int w = w0 + lane;
-      const int c = __popc(w < NW ? (HESS ? s_mh[HESS ? w : 0] : 0u) : slot < 0 ? s_m[w - NW] : 0u);
+      const int c = __popc(w < NW ? (HESS && list_h ? s_mh[HESS ? w : 0] : 0u) : slot < 0 ? s_m[w - NW] : 0u);
       int sum = c;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -776,17 +778,23 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     if (lane == 0) {
       s_to[0] = nl;
       s_to[1] = slot;
-      if (slot >= 0) a.dense.tile[slot] = blockIdx.y * gridDim.x + blockIdx.x;
+      s_to[2] = full;
+      if (slot >= 0) a.dense.tile[slot] = (blockIdx.y * gridDim.x + blockIdx.x) | (full ? (int)0x80000000u : 0);
     }
   }
   __syncthreads();
   const int nl = s_to[0], slot = s_to[1];
+  const bool full = s_to[2] != 0, list_h = slot < 0 || !full;
   if (slot >= 0)
-    for (int w = tid; w < NW; w += FF_THREADS) a.dense.mask[(size_t)slot * NW + w] = s_m[w];
+    for (int w = tid; w < NW; w += FF_THREADS) {
+      unsigned *m = a.dense.mask + (size_t)slot * (HESS ? 2 : 1) * NW + w;
+      m[0] = s_m[w];
+      if (HESS) m[NW] = full ? s_mh[HESS ? w : 0] : 0u;
+    }
   if (nl)
     for (int w = warp; w < 2 * NW; w += FF_WARPS) {
       const int wi = w % NW;
-      const unsigned mask = w < NW ? (HESS ? s_mh[HESS ? wi : 0] : 0u) : slot < 0 ? s_m[wi] : 0u;
+      const unsigned mask = w < NW ? (HESS && list_h ? s_mh[HESS ? wi : 0] : 0u) : slot < 0 ? s_m[wi] : 0u;
       const int j = blockIdx.y * FT + wi / (FT / 32), i = i0 + wi % (FT / 32) * 32 + lane;
       if (mask >> lane & 1u)
         a.rep_list[s_pos[w] + __popc(mask & ((1u << lane) - 1u))] = (j * a.nx + i) | (w < NW ? (int)0x80000000u : 0);
@@ -813,20 +821,27 @@ struct FarRepairArgs {
   DenseRepair dense;
 };
 
-template <int FT>
+template <int FT, bool HESS>
 __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a) {
-  constexpr int NW = FT * FT / 32, PARTS = FT * FT / FR_THREADS, NODES = FP * FP;
-  __shared__ unsigned s_w[NW];
+  constexpr int NW = FT * FT / 32, PARTS = FT * FT / FR_THREADS, NODES = FP * FP, NV = HESS ? 5 : 2, NM = HESS ? 2 : 1;
+  __shared__ unsigned s_w[NW], s_wh[HESS ? NW : 1];
   __shared__ int s_pos[NW + 1], s_near[FR_THREADS], s_nn[FR_THREADS / 32];
-  __shared__ float2 s_val[2][NODES];
+  __shared__ float2 s_val[NV][NODES];
   __shared__ float2 s_rdf[RECDF][FR_THREADS];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nh = min(*a.dense.count, a.dense.cap);
   for (long long item = blockIdx.x; item < (long long)nh * PARTS; item += gridDim.x) {
     const int slot = (int)(item / PARTS), part = (int)(item % PARTS);
     __syncthreads();  // the previous item's shared data has been used
-    for (int w = tid; w < NW; w += FR_THREADS) s_w[w] = a.dense.mask[(size_t)slot * NW + w];
-    for (int q = tid; q < 2 * NODES; q += FR_THREADS) (&s_val[0][0])[q] = a.dense.val[(size_t)slot * 2 * NODES + q];
+    const int entry = a.dense.tile[slot], tile = entry & 0x7fffffff;
+    const bool full = HESS && entry < 0;  // the tile's Hessian values are there too
+    for (int w = tid; w < NW; w += FR_THREADS) {
+      const unsigned *m = a.dense.mask + (size_t)slot * NM * NW + w;
+      const unsigned mh = HESS ? m[HESS ? NW : 0] : 0u;
+      s_w[w] = m[0] | mh;
+      if (HESS) s_wh[HESS ? w : 0] = mh;
+    }
+    for (int q = tid; q < (full ? NV : 2) * NODES; q += FR_THREADS) (&s_val[0][0])[q] = a.dense.val[(size_t)slot * NV * NODES + q];
     __syncthreads();
     if (warp == 0) {
       int base = 0;
@@ -860,7 +875,8 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
     unsigned bits = s_w[lo];
     for (int k = rank - s_pos[lo]; k > 0; --k) bits &= bits - 1u;
     const int jr = lo / (FT / 32), ic = lo % (FT / 32) * 32 + __ffs(bits) - 1;
-    const int tile = a.dense.tile[slot], i0 = tile % a.dense.tpr * FT, j0 = tile / a.dense.tpr * FT;
+    const bool all = HESS && mine && (s_wh[HESS ? lo : 0] >> (__ffs(bits) - 1) & 1u);  // every plane of this node
+    const int i0 = tile % a.dense.tpr * FT, j0 = tile / a.dense.tpr * FT;
     const df Cx = tile_centre(a.xmin, (double)i0, FT, a.dx), Cy = tile_centre(a.ymin, (double)(a.row0 + j0), FT, a.dy);
     const double X = a.xmin + (i0 + ic) * a.dx, Y = a.ymin + (a.row0 + j0 + jr) * a.dy;
     const df Xd = df_kept(X), Yd = df_kept(Y);
@@ -882,12 +898,17 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
       for (int q = tid; q < RECDF * nn; q += FR_THREADS) s_rdf[q / nn][q % nn] = a.recdf[(size_t)(q / nn) * a.n + s_near[q % nn]];
       __syncthreads();
       for (int k = 0; k < nn; ++k)
-        add_potential_dfs<false>(&s_rdf[0][k], FR_THREADS, a.all64 + (size_t)s_near[k] * REC64, X, Y, Xd, Yd, sum);
+        if (HESS && full)
+          add_potential_dfs<true>(&s_rdf[0][k], FR_THREADS, a.all64 + (size_t)s_near[k] * REC64, X, Y, Xd, Yd, sum);
+        else
+          add_potential_dfs<false>(&s_rdf[0][k], FR_THREADS, a.all64 + (size_t)s_near[k] * REC64, X, Y, Xd, Yd, sum);
     }
     // the far potentials: rows of the tensor product, then the column
     const FineTab<FT> &t = fine_table<FT>();
-#pragma unroll 1
-    for (int c = 0; c < 2; ++c) {
+    double val[NV];
+#pragma unroll
+    for (int c = 0; c < NV; ++c) {
+      if (c >= 2 && !full) break;
       df v = sum[c];
 #pragma unroll 1
       for (int j = 0; j < FP; ++j) {
@@ -899,7 +920,22 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
         }
         v = df_add(v, df_mul(df{t.w[jr][j], t.wlo[jr][j]}, r));
       }
-      if (mine) a.out[c * a.plane + (long long)(j0 + jr) * a.nx + i0 + ic] = (float)(a.dls * df_to_double(v));
+      val[c] = a.dls * df_to_double(v);
+    }
+    float *o = a.out + (long long)(j0 + jr) * a.nx + i0 + ic;
+    if (mine) {
+      o[0] = (float)val[0];
+      o[a.plane] = (float)val[1];
+    }
+    if constexpr (HESS) {
+      if (all) {
+        const double kap = val[2], g1 = val[3], g2 = val[4];
+        const double det = (1.0 - kap) * (1.0 - kap) - g1 * g1 - g2 * g2;
+        o[2 * a.plane] = (float)kap;
+        o[3 * a.plane] = (float)g1;
+        o[4 * a.plane] = (float)g2;
+        o[5 * a.plane] = (float)(1.0 / det);
+      }
     }
   }
 }
@@ -926,7 +962,7 @@ constexpr double KF = 3.0, KF_H = 3.5, KC = 2.5, KC_H = 3.0;
 constexpr double TILE_COST = 4000.0, NODE_COST = 3.0;
 // densely listed tiles of the repair: from this many nodes, on maps of at
 // least this many nodes and potentials (below, the extra launch costs more
-// than the repair) and at most this many tiles (2.1 KB each)
+// than the repair) and at most this many tiles (2.1 KB each, 5 KB with the Hessian)
 constexpr int DENSE_MIN = 150, DENSE_NODES = 1 << 19, DENSE_N = 64;
 constexpr long long DENSE_TILES = 65536;
 // margins of the repair: interpolation error below 4e-11 of a potential's own
@@ -998,21 +1034,23 @@ FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mo
   if (p.use && mode != FAR_POT && ctx->repair_ratio > 0.0 && nodes >= DENSE_NODES && m->n >= DENSE_N && m->n_light > 0) {
     const long long tiles = (long long)((g->nx + p.ft - 1) / p.ft) * ((g->ny + p.ft - 1) / p.ft);
     p.rep_cap = tiles <= DENSE_TILES ? (int)tiles : 0;
-    p.rep_bytes = ((size_t)p.rep_cap * (sizeof(float2) * 2 * FP * FP + sizeof(int) + (size_t)p.ft * p.ft / 8) + 255) & ~(size_t)255;
+    const size_t h = mode == FAR_HESS;
+    p.rep_bytes = ((size_t)p.rep_cap * (sizeof(float2) * (h ? 5 : 2) * FP * FP + sizeof(int) + (h ? 2 : 1) * (size_t)p.ft * p.ft / 8) + 255) & ~(size_t)255;
     p.bytes += p.rep_bytes;
   }
   return p;
 }
 
-DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, void *mem, int *count) {
+DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, bool hess, void *mem, int *count) {
   DenseRepair d;
   if (!mem || !p.rep_cap) return d;
   d.count = count;
   d.cap = p.rep_cap;
   d.ft = p.ft;
   d.tpr = (g->nx + p.ft - 1) / p.ft;
+  d.nv = hess ? 5 : 2;
   d.val = (float2 *)mem;
-  d.tile = (int *)(d.val + (size_t)p.rep_cap * 2 * FP * FP);
+  d.tile = (int *)(d.val + (size_t)p.rep_cap * d.nv * FP * FP);
   d.mask = (unsigned *)(d.tile + p.rep_cap);
   const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
   const double R = std::sqrt(2.0) * 0.5 * (p.ft - 1) * std::max(dx, dy);
@@ -1040,10 +1078,10 @@ int launch_far_repair(const Model *m, const lens_grid *g, const DenseRepair &den
   a.dense = dense;
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
-  if (dense.ft == 32)
-    k_far_repair<32><<<4 * nsm, FR_THREADS, 0, st>>>(a);
-  else
-    k_far_repair<64><<<4 * nsm, FR_THREADS, 0, st>>>(a);
+  const bool hess = dense.nv == 5;
+  auto kern = dense.ft == 32 ? (hess ? k_far_repair<32, true> : k_far_repair<32, false>)
+                             : (hess ? k_far_repair<64, true> : k_far_repair<64, false>);
+  kern<<<4 * nsm, FR_THREADS, 0, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "dense map repair launch: %s", cudaGetErrorString(e));
   return LENS_OK;

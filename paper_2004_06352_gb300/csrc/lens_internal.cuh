@@ -398,9 +398,10 @@ constexpr float REPAIR_STRONG_BQ = 4.f;  // b q above which a potential takes th
 struct DenseRepair {
   int *count = nullptr;      // tiles (may exceed cap: the rest are listed node by node)
   int cap = 0, ft = 0, tpr = 0;
-  int *tile = nullptr;       // [cap] tile index
-  unsigned *mask = nullptr;  // [cap][ft * ft / 32] nodes to recompute, row-major
-  float2 *val = nullptr;     // [cap][2][FAR_P * FAR_P] the far potentials' deflection at the nodes
+  int nv = 0;                // values per node: 2 (deflection) or 5 (and kappa, gamma1, gamma2)
+  int *tile = nullptr;       // [cap] tile index; bit 31: all nv values (else the deflection alone)
+  unsigned *mask = nullptr;  // [cap][2 or 1][ft * ft / 32] nodes to recompute (deflection alone, all planes), row-major
+  float2 *val = nullptr;     // [cap][nv][FAR_P * FAR_P] the far potentials' values at the nodes
   float thr = 0.f, thr_h = 0.f;  // squared psi beyond which a potential is far
   float xi[FAR_P];           // the nodes, in grid steps about the tile's centre
 };
@@ -415,7 +416,7 @@ int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mod
                    int row0, int rows, double repair, int *rep_count, int *rep_list, const DenseRepair &dense,
                    const double *beta, cudaStream_t st);
 // the plan's DenseRepair arrays at mem, counting in *count; cap = 0 when mem is NULL
-DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, void *mem, int *count);
+DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, bool hess, void *mem, int *count);
 // the listed nodes of the dense tiles, after the far potentials' values
 int launch_far_repair(const Model *m, const lens_grid *g, const DenseRepair &dense, double dls, void *out, int row0,
                       int rows, int device, cudaStream_t st);

@@ -490,8 +490,8 @@ constexpr int REP_WARPS = 8, REP_THREADS = 32 * REP_WARPS, REP_CH = 32;  // pote
 // Each lane sums its terms in double-float and converts once (adding every
 // term in FP64 takes 20 FP64-pipe operations per term with the Hessian).
 // After the listed nodes come the interpolation nodes of the densely listed
-// tiles (lens_far.cu): there the far potentials' deflection goes to
-// dense.val.
+// tiles (lens_far.cu): there the far potentials' deflection (and Hessian)
+// goes to dense.val.
 template <bool HESS>
 __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) {
   __shared__ float2 s_rdf[RECDF][REP_CH];
@@ -504,12 +504,13 @@ __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) 
     const bool have = e < all, node = e >= total;  // node: an interpolation node
     const int entry = have && !node ? a.list[e] : 0;
     const int o = entry & 0x7fffffff;
-    const bool full = HESS && entry < 0;  // warp-uniform
     const int slot = node ? (e - total) / NODES : 0, q = node ? (e - total) % NODES : 0;
+    const int dense_tile = have && node ? a.dense.tile[slot] : 0;
+    const bool full = HESS && (node ? dense_tile : entry) < 0;  // warp-uniform
     double X, Y;
     df Cx = {0.f, 0.f}, Cy = {0.f, 0.f};
     if (have && node) {
-      const int tile = a.dense.tile[slot];
+      const int tile = dense_tile & 0x7fffffff;
       Cx = tile_centre(a.xmin, (double)(tile % a.dense.tpr * a.dense.ft), a.dense.ft, a.dx);
       Cy = tile_centre(a.ymin, (double)(a.row0 + tile / a.dense.tpr * a.dense.ft), a.dense.ft, a.dy);
       X = df_to_double(Cx) + a.dense.xi[q % FAR_P] * a.dx;
@@ -545,9 +546,10 @@ __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) 
       for (int off = 16; off; off >>= 1) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], off);
     if (have && lane == 0 && node) {
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
+      for (int c = 0; c < (HESS ? 5 : 2); ++c) {
+        if (c >= 2 && !full) break;
         const df v = df_from_double(acc[c]);
-        a.dense.val[((size_t)slot * 2 + c) * NODES + q] = make_float2(v.hi, v.lo);
+        a.dense.val[((size_t)slot * a.dense.nv + c) * NODES + q] = make_float2(v.hi, v.lo);
       }
     } else if (have && lane == 0) {
       a.out[o] = (float)(a.dls * acc[0]);
@@ -714,7 +716,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
   constexpr int KPG = LENS_KP_GRAD, KPH = LENS_KP_HESS;
   DenseRepair dense;
   if (far) {
-    if (repair && dense_mem) dense = dense_repair(g, *far, dense_mem, a.rep_count + 1);
+    if (repair && dense_mem) dense = dense_repair(g, *far, hess, dense_mem, a.rep_count + 1);
     const int rc = launch_far_map(m, g, *far, hess, far_mem, dls, out, row0, rows, a.repair, a.rep_count, a.rep_list,
                                   dense, nullptr, st);
     if (rc) return rc;
