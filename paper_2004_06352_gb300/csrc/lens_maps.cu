@@ -22,7 +22,7 @@
 //   - Potentials at or above the FP64 threshold (cluster-scale halos) are
 //     evaluated in FP64; the final sum, scaling by D_ls/D_s and the derived
 //     kappa/gamma/mu are formed in FP64 per point and stored as FP32.
-// LENS_FP64 kernel: one point per thread, every potential in FP64.
+// LENS_FP64 kernels: one point per thread, every potential in FP64.
 #include <algorithm>
 #include <climits>
 #include <type_traits>
@@ -566,36 +566,206 @@ __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) 
   }
 }
 
-template <int MODE>
-__global__ void __launch_bounds__(256) k_map_fp64(const double *__restrict__ all64, int n, double xmin, double ymin,
-                                                  double dx, double dy, int nx, int row0, double dls,
-                                                  double *__restrict__ out, long long plane, int tau = 0,
-                                                  double bx = 0.0, double by = 0.0) {
-  constexpr bool HESS = MODE == MAP_HESS;
-  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (p >= plane) return;
-  const int i = (int)(p % nx), j = (int)(p / nx);
-  const double X = xmin + i * dx, Y = ymin + (row0 + j) * dy;
-  if constexpr (MODE == MAP_POT) {
-    double PHI = 0;
-    for (int h = 0; h < n; ++h) PHI += pot64(all64 + (size_t)h * REC64, X, Y);
-    const double phi = dls * PHI;
-    out[p] = phi;
-    if (tau) out[plane + p] = 0.5 * ((X - bx) * (X - bx) + (Y - by) * (Y - by)) - phi;
-    return;
+// LENS_FP64 deflection and Hessian maps.  Bound: the FP64 pipe (2 lanes per
+// SM and clock), so the evaluation is written for the fewest FP64 operations
+// (78 per pair of node and dPIE for the deflection instead of 105, more where
+// the arctangents need their reduction):
+//   - the record's products are formed once per potential and CTA, 32
+//     potentials at a time in shared memory;
+//   - reciprocals and roots take one cubic step on the MUFU seed (its error
+//     of ~2^-20 cubed) instead of two Newton steps;
+//   - the arctangents' reductions act on numerator and denominator before the
+//     division (atan(n/d) = pi/2 - atan(d/n) and = atan(c) + atan((n - c d) /
+//     (d + c n)), atanh likewise), so lanes inside and outside the
+//     interpolants' range share one division and one polynomial; which of
+//     them a lane needs is decided in FP32 from the doubles' bits.
+// 64-thread CTAs: 256^2 nodes are 1024 CTAs, 6.7 per SM; of 256 threads, 1.7.
+enum Rec64M : int {
+  M_X0 = 0, M_Y0, M_C, M_S, M_Q2, M_KC, M_KT, M_SC, M_ST, M_Q2SC, M_Q2ST, M_U2,
+  M_FDS, M_FDK, M_FQ2DS, M_BF,  // f dS, f q^2 dS sS, f q^2 dS, b q / f with f = u (1 for the series kind)
+  M_KIND, M_B,
+  M_DC0, M_DT0, M_U2SC2, M_U2ST2, M_HC, M_HS, M_HB  // (1 + q^2) s^2, u^2 s^2; b q / 2 times cos, sin 2 theta; b q / 2
+};
+constexpr int REC64M = 25, F64_CH = 32, F64_THREADS = 64;
+
+__device__ __forceinline__ double rcp64c(double b) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(b));
+  const double e = fma(-b, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// 1 / sqrt(a), and sqrt(a) itself
+__device__ __forceinline__ double rsqrt64c(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-a * y, y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+__device__ __forceinline__ double sqrt64c(double a) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double t = a * y, e = fma(-t, y, 1.0);
+  return fma(t * e, fma(0.375, e, 0.5), t);
+}
+// v > 0 over 2^k in FP32, from its bits; k as the exponent field of a double
+// (values beyond 2^+-100 are clamped)
+__device__ __forceinline__ float scaled_float(double v, int k) {
+  const int h = min(max(__double2hiint(v) - k + (1023 << 20), 923 << 20), 1123 << 20);
+  return __int_as_float(((h - (896 << 20)) << 3) | (int)((unsigned)__double2loint(v) >> 29));
+}
+// (p + e) c with one rounding, (p, e) an unevaluated sum, and the exact
+// product of two doubles as one: a constant's error would be every node's.
+struct Prod64 {
+  double p, e;
+};
+__device__ __forceinline__ Prod64 prod64(double a, double b) {
+  const double p = a * b;
+  return {p, fma(a, b, -p)};
+}
+__device__ __forceinline__ Prod64 prod64(Prod64 a, double c) {
+  const double p = a.p * c;
+  return {p, fma(a.p, c, -p) + a.e * c};
+}
+// b atan(n / d) and b atanh(n / d), d > 0 (|n| < d for atanh)
+__device__ __forceinline__ double atan_ratio64(double n, double d, double b) {
+  const double p = fabs(n);
+  const int k = __double2hiint(d) & 0x7ff00000;
+  const float fp = scaled_float(p, k), fd = scaled_float(d, k);
+  const bool inv = fp > fd;
+  double P = inv ? d : p, Q = inv ? p : d, base = 0.0;
+  if (fminf(fp, fd) > 0.4f * fmaxf(fp, fd)) {
+    const double t = fma(-0.6875, Q, P);
+    Q = fma(0.6875, P, Q);
+    P = t;
+    base = ATAN_11_16;
   }
+  const double v = P * rcp64c(Q);
+  double r = fma(v, atan_over_w64(v * v), base);
+  if (inv) r = (PI_2_HI - r) + PI_2_LO;
+  return b * copysign(r, n);
+}
+__device__ __forceinline__ double atanh_ratio64(double n, double d, double b) {
+  const double p = fabs(n);
+  const int k = __double2hiint(d) & 0x7ff00000;
+  const float fp = scaled_float(p, k), fd = scaled_float(d, k);
+  double P = p, Q = d, base = 0.0;
+  if (fp > 0.4f * fd) {
+    const double m = d - p;
+    const int kk = m > 0.0 ? __float2int_rn(0.625f * (__logf(fd + fp) - __logf(scaled_float(m, k)))) : ATANH_K + 1;
+    if (kk > ATANH_K) return b * atanh(n / d);  // |n / d| >= 1 or within 1e-15 of it
+    const int q = kk < 1 ? 1 : kk;
+    const double c = ATANH_C[q];
+    P = fma(-c, d, p);
+    Q = fma(-c, p, d);
+    base = ATANH_A[q];
+  }
+  const double v = P * rcp64c(Q);
+  return b * copysign(fma(v, atanh_over_w64(v * v), base), n);
+}
+
+template <bool HESS>
+__global__ void __launch_bounds__(F64_THREADS) k_map_fp64(const double *__restrict__ all64, int n, double xmin,
+                                                          double ymin, double dx, double dy, int nx, int row0,
+                                                          double dls, double *__restrict__ out, long long plane) {
+  __shared__ double s_r[F64_CH][REC64M];
+  const long long p = (long long)blockIdx.x * F64_THREADS + threadIdx.x;
+  const long long q = p < plane ? p : plane - 1;  // (past the end: the last node again, not stored)
+  const int i = (int)(q % nx), j = (int)(q / nx);
+  const double X = xmin + i * dx, Y = ymin + (row0 + j) * dy;
   double AX = 0, AY = 0, KA = 0, G1 = 0, G2 = 0;
-  for (int h = 0; h < n; ++h) {
-    double ax, ay, kk = 0, q1 = 0, q2 = 0;
-    eval64<HESS>(all64 + (size_t)h * REC64, X, Y, ax, ay, kk, q1, q2);
-    AX += ax;
-    AY += ay;
-    if (HESS) {
-      KA += kk;
-      G1 += q1;
-      G2 += q2;
+  for (int h0 = 0; h0 < n; h0 += F64_CH) {
+    const int cnt = min(F64_CH, n - h0);
+    __syncthreads();  // the previous chunk has been used
+    if (threadIdx.x < cnt) {
+      const double *r = all64 + (size_t)(h0 + threadIdx.x) * REC64;
+      double *m = s_r[threadIdx.x];
+      const double q2 = r[D_Q2], u2 = r[D_U2], sc = r[D_SC], st = r[D_ST], bq = r[D_BQ], dS = r[D_DS];
+      const double f = r[D_KIND] == K64_DPIE ? r[D_U] : 1.0;
+      m[M_X0] = r[D_X0];
+      m[M_Y0] = r[D_Y0];
+      m[M_C] = r[D_C];
+      m[M_S] = r[D_S];
+      m[M_Q2] = q2;
+      auto sum = [](Prod64 v) { return v.p + v.e; };
+      m[M_KC] = sum(prod64(prod64(q2, sc), sc));
+      m[M_KT] = sum(prod64(prod64(q2, st), st));
+      m[M_SC] = sc;
+      m[M_ST] = st;
+      m[M_Q2SC] = q2 * sc;
+      m[M_Q2ST] = q2 * st;
+      m[M_U2] = u2;
+      m[M_FDS] = f * dS;
+      m[M_FQ2DS] = sum(prod64(prod64(f, q2), dS));
+      m[M_FDK] = sum(prod64(prod64(prod64(f, q2), dS), r[D_SS]));
+      m[M_BF] = bq / f;
+      m[M_KIND] = r[D_KIND];
+      m[M_B] = r[D_B];
+      if (HESS) {
+        m[M_DC0] = (1.0 + q2) * sc * sc;
+        m[M_DT0] = (1.0 + q2) * st * st;
+        m[M_U2SC2] = u2 * sc * sc;
+        m[M_U2ST2] = u2 * st * st;
+        m[M_HB] = 0.5 * bq;
+        m[M_HC] = 0.5 * bq * r[D_C2T];
+        m[M_HS] = 0.5 * bq * r[D_S2T];
+      }
+    }
+    __syncthreads();
+    for (int h = 0; h < cnt; ++h) {
+      const double *r = s_r[h];
+      const int kind = (int)r[M_KIND];
+      if (kind != K64_DPIE && kind != K64_DPIE_SERIES) {
+        double ax, ay, kk = 0, q1 = 0, q2 = 0;
+        eval64<HESS>(all64 + (size_t)(h0 + h) * REC64, X, Y, ax, ay, kk, q1, q2);
+        AX += ax;
+        AY += ay;
+        KA += kk;
+        G1 += q1;
+        G2 += q2;
+        continue;
+      }
+      const double c = r[M_C], s = r[M_S], q2 = r[M_Q2], u2 = r[M_U2], sc = r[M_SC], st = r[M_ST];
+      const double dX = X - r[M_X0], dY = Y - r[M_Y0];
+      const double x = fma(s, dY, c * dX), y = fma(c, dY, -(s * dX));
+      const double x2 = x * x, y2 = y * y, R = fma(q2, x2, y2);
+      double psc, pst, ic = 0, it = 0;
+      if (HESS) {
+        const double pc2 = R + r[M_KC], pt2 = R + r[M_KT];
+        ic = rsqrt64c(pc2);
+        it = rsqrt64c(pt2);
+        psc = pc2 * ic;
+        pst = pt2 * it;
+      } else {
+        psc = sqrt64c(R + r[M_KC]);
+        pst = sqrt64c(R + r[M_KT]);
+      }
+      const double Sp = psc + pst;
+      const double nx_ = x * fma(r[M_FDS], Sp, r[M_FDK]), ny_ = y * fma(r[M_FQ2DS], Sp, r[M_FDK]);
+      const double dx_ = Sp * fma(psc + sc, pst + st, u2 * x2);
+      const double dy_ = Sp * fma(-u2, y2, (psc + r[M_Q2SC]) * (pst + r[M_Q2ST]));
+      double axp, ayp;
+      if (kind == K64_DPIE) {  // b q / u times atan, atanh of u Z
+        axp = atan_ratio64(nx_, dx_, r[M_BF]);
+        ayp = atanh_ratio64(ny_, dy_, r[M_BF]);
+      } else {
+        const double Zx = nx_ * rcp64c(dx_), Zy = ny_ * rcp64c(dy_), wx = u2 * Zx * Zx, wy = u2 * Zy * Zy;
+        axp = r[M_BF] * Zx * (1.0 - wx / 3.0 + wx * wx / 5.0);
+        ayp = r[M_BF] * Zy * (1.0 + wy / 3.0 + wy * wy / 5.0);
+      }
+      AX += fma(c, axp, -(s * ayp));
+      AY += fma(s, axp, c * ayp);
+      if (HESS) {
+        const double r2 = x2 + y2, ymx = y2 - x2;
+        const double fc = ic * rcp64c(fma(2.0 * sc, psc, r[M_DC0]) + r2), ft = it * rcp64c(fma(2.0 * st, pst, r[M_DT0]) + r2);
+        // over b q / 2
+        const double g1p = fc * (ymx - r[M_U2SC2]) - ft * (ymx - r[M_U2ST2]), g2p = -2.0 * (fc - ft) * (x * y);
+        KA += r[M_HB] * (ic - it);
+        G1 += fma(r[M_HC], g1p, -(r[M_HS] * g2p));
+        G2 += fma(r[M_HS], g1p, r[M_HC] * g2p);
+      }
     }
   }
+  if (p >= plane) return;
   out[p] = dls * AX;
   out[plane + p] = dls * AY;
   if (HESS) {
@@ -605,6 +775,21 @@ __global__ void __launch_bounds__(256) k_map_fp64(const double *__restrict__ all
     out[4 * plane + p] = g2;
     out[5 * plane + p] = 1.0 / ((1.0 - kap) * (1.0 - kap) - g1 * g1 - g2 * g2);
   }
+}
+
+// LENS_FP64 potential maps.
+__global__ void __launch_bounds__(256) k_pot_fp64(const double *__restrict__ all64, int n, double xmin, double ymin,
+                                                  double dx, double dy, int nx, double dls, double *__restrict__ out,
+                                                  long long plane, int tau, double bx, double by) {
+  const long long p = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (p >= plane) return;
+  const int i = (int)(p % nx), j = (int)(p / nx);
+  const double X = xmin + i * dx, Y = ymin + j * dy;
+  double PHI = 0;
+  for (int h = 0; h < n; ++h) PHI += pot64(all64 + (size_t)h * REC64, X, Y);
+  const double phi = dls * PHI;
+  out[p] = phi;
+  if (tau) out[plane + p] = 0.5 * ((X - bx) * (X - bx) + (Y - by) * (Y - by)) - phi;
 }
 
 // The bounded-wait failure path on its own: one thread waits on an mbarrier
@@ -769,13 +954,9 @@ int launch_map_fp64(lens_ctx *ctx, const Model *m, const lens_grid *g, double dl
   if (rows < 0) rows = g->ny - row0;
   const long long plane = (long long)g->nx * rows;
   const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
-  const unsigned blocks = (unsigned)((plane + 255) / 256);
-  if (hess)
-    k_map_fp64<MAP_HESS><<<blocks, 256, 0, st>>>(m->all64, m->n, g->xmin, g->ymin, dx, dy, g->nx, row0, dls,
-                                              (double *)out, plane);
-  else
-    k_map_fp64<MAP_GRAD><<<blocks, 256, 0, st>>>(m->all64, m->n, g->xmin, g->ymin, dx, dy, g->nx, row0, dls,
-                                               (double *)out, plane);
+  const unsigned blocks = (unsigned)((plane + F64_THREADS - 1) / F64_THREADS);
+  auto kern = hess ? k_map_fp64<true> : k_map_fp64<false>;
+  kern<<<blocks, F64_THREADS, 0, st>>>(m->all64, m->n, g->xmin, g->ymin, dx, dy, g->nx, row0, dls, (double *)out, plane);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "FP64 map kernel launch: %s", cudaGetErrorString(e));
   return LENS_OK;
@@ -788,9 +969,8 @@ int launch_pot_map(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls
   const long long plane = (long long)g->nx * rows;
   if (precision == LENS_FP64) {
     const unsigned blocks = (unsigned)((plane + 255) / 256);
-    k_map_fp64<MAP_POT><<<blocks, 256, 0, st>>>(m->all64, m->n, g->xmin, g->ymin, dx, dy, g->nx, 0, dls,
-                                                 (double *)out, plane, beta != nullptr, beta ? beta[0] : 0.0,
-                                                 beta ? beta[1] : 0.0);
+    k_pot_fp64<<<blocks, 256, 0, st>>>(m->all64, m->n, g->xmin, g->ymin, dx, dy, g->nx, dls, (double *)out, plane,
+                                       beta != nullptr, beta ? beta[0] : 0.0, beta ? beta[1] : 0.0);
   } else {
     FarPlan plan = plan_far(ctx, m, g, 2);
     CallScratch far(ctx, st);  // the coarse level's values
