@@ -43,7 +43,7 @@ namespace {
 
 constexpr int FP = FAR_P;  // interpolation nodes per axis of a fine tile
 constexpr int CP = 12;   // a coarse tile's
-constexpr int FF_THREADS = 256, FF_WARPS = FF_THREADS / 32;
+constexpr int CO_THREADS = 256;  // coarse kernel
 constexpr int FF_CH = 64;            // potentials per staged chunk
 constexpr int REC_STRIDE4 = REC32 / 4 + 1;  // float4 slots per staged record (the pad spreads the records a warp reads)
 constexpr int FF_SUB = 16;           // partial sums folded every FF_SUB potentials
@@ -56,6 +56,9 @@ enum FarMode : int { FAR_GRAD = 0, FAR_HESS = 1, FAR_POT = 2 };
 __host__ __device__ constexpr int nval(int mode) { return mode == FAR_HESS ? 5 : mode == FAR_GRAD ? 2 : 1; }
 __host__ __device__ constexpr int ncmp(int mode) { return nval(mode) + (mode == FAR_POT ? 0 : 1); }
 __host__ __device__ constexpr int ncmp2(int mode) { return (ncmp(mode) + 1) / 2; }
+
+// CTAs per SM of the fine kernel with 128 or 256 threads (launch_far_map)
+__host__ __device__ constexpr int fi_blocks(int mode, int th) { return th == 256 ? 2 : mode == FAR_GRAD ? 5 : 4; }
 
 // Chebyshev nodes of a fine tile of FT x FT map nodes (FT = 32 or 64), in
 // units of 1/64 grid step about its centre, and of the coarse tile in units
@@ -248,10 +251,11 @@ struct Sums {
 
 // Potential idx of the list (FP32) into staging slot h: its record, and the
 // tile centre's offset from its centre as hi/lo pairs.
+template <int TH>
 __device__ __forceinline__ void stage_chunk(const FarArgs &a, const unsigned short *list, int cnt, df Tx, df Ty,
                                             float4 *s_rec, float4 *s_off) {
   const float4 *g_rec = reinterpret_cast<const float4 *>(a.rec32);
-  for (int q = threadIdx.x; q < cnt * (REC32 / 4); q += FF_THREADS)
+  for (int q = threadIdx.x; q < cnt * (REC32 / 4); q += TH)
     s_rec[(q >> 3) * REC_STRIDE4 + (q & 7)] = __ldg(g_rec + (size_t)list[q >> 3] * (REC32 / 4) + (q & 7));
   if (threadIdx.x < cnt) {
     const float4 c = __ldg(a.cen32 + list[threadIdx.x]);
@@ -264,11 +268,12 @@ __device__ __forceinline__ void stage_chunk(const FarArgs &a, const unsigned sho
 // the tile or near, and list the far ones then the near ones, each in index
 // order.  s_far / s_near: nw words each.  cnt: far FP32, far cluster-scale,
 // near FP32, near cluster-scale.  Ends synchronised.
+template <int TH>
 __device__ __forceinline__ void classify(const FarArgs &a, const unsigned *in, df Tx, df Ty, float thr, float thr_h,
                                          unsigned *s_far, unsigned *s_near, unsigned short *s_list, int *s_cnt) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float4 *g_rec = reinterpret_cast<const float4 *>(a.rec32);
-  for (int w = warp; w < a.nw; w += FF_WARPS) {
+  for (int w = warp; w < a.nw; w += (TH / 32)) {
     const bool hv = w >= a.nwl;
     const int i = (hv ? w - a.nwl : w) * 32 + lane;
     bool mine = i < (hv ? a.n_heavy : a.n_light);
@@ -317,7 +322,7 @@ __device__ __forceinline__ void classify(const FarArgs &a, const unsigned *in, d
     }
   }
   __syncthreads();
-  for (int w = warp; w < 2 * a.nw; w += FF_WARPS) {
+  for (int w = warp; w < 2 * a.nw; w += (TH / 32)) {
     const int wi = w < a.nw ? w : w - a.nw;
     const unsigned m = w < a.nw ? s_far[wi] : s_near[wi];
     const int i = (wi >= a.nwl ? wi - a.nwl : wi) * 32 + lane;
@@ -334,11 +339,11 @@ __device__ __forceinline__ float slope8(float v) { return __int_as_float(__float
 // double-float (node = y index * P + x index).  Ends synchronised.
 // kb: the FP32 potentials' largest |kappa|, |gamma1|, |gamma2| at the nodes
 // (HESS), added to what is there.
-template <int MODE, int P>
+template <int MODE, int P, int TH>
 __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short *list, int n_far, int n_far_h,
                                           df Tx, df Ty, const float2 *s_nx, const float2 *s_ny, float4 *s_rec,
                                           float4 *s_off, float2 *s_part, float2 *s_val, float *s_kb) {
-  constexpr int NODES = P * P, PAIRS = NODES / 2, SPLITS = FF_THREADS / PAIRS, NC = ncmp(MODE), NV = nval(MODE);
+  constexpr int NODES = P * P, PAIRS = NODES / 2, SPLITS = TH / PAIRS, NC = ncmp(MODE), NV = nval(MODE);
   const int tid = threadIdx.x, split = tid / PAIRS, pr = tid % PAIRS, ix = pr % P, jy = 2 * (pr / P);
   const bool active = split < SPLITS;
   Sums<MODE> S;
@@ -347,7 +352,7 @@ __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short
   for (int c0 = 0; c0 < n_far; c0 += FF_CH) {
     const int cnt = min(FF_CH, n_far - c0);
     if (c0) __syncthreads();  // the previous chunk has been used
-    stage_chunk(a, list + c0, cnt, Tx, Ty, s_rec, s_off);
+    stage_chunk<TH>(a, list + c0, cnt, Tx, Ty, s_rec, s_off);
     __syncthreads();
     if (active)
       S.sweep(s_rec, s_off, split, cnt, SPLITS, ox, make_float2(y0.x, y1.x), make_float2(y0.y, y1.y));
@@ -366,7 +371,7 @@ __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short
     }
   }
   __syncthreads();
-  for (int q = tid; q < NODES * NC; q += FF_THREADS) {
+  for (int q = tid; q < NODES * NC; q += TH) {
     df v = {s_part[q].x, s_part[q].y};
     for (int s = 1; s < SPLITS; ++s) {
       const float2 t = s_part[(size_t)s * NODES * NC + q];
@@ -379,7 +384,7 @@ __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short
   }
   __syncthreads();
   if (n_far_h > 0) {
-    for (int node = tid; node < NODES; node += FF_THREADS) {
+    for (int node = tid; node < NODES; node += TH) {
       const float2 nx = s_nx[node % P], ny = s_ny[node / P];
       const df X = df_add(Tx, df{nx.x, nx.y}), Y = df_add(Ty, df{ny.x, ny.y});
       df sum[5] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
@@ -408,8 +413,8 @@ __device__ __forceinline__ float4 plane_of(const float2 *v, float span) {
 }
 
 template <int MODE>
-__global__ void __launch_bounds__(FF_THREADS, 2) k_far_coarse(const FarArgs a) {
-  constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), SPLITS = FF_THREADS / (NODES / 2);
+__global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
+  constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), SPLITS = CO_THREADS / (NODES / 2);
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);
   float4 *s_off = s_rec + FF_CH * REC_STRIDE4;
@@ -435,13 +440,13 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_coarse(const FarArgs a) {
     s_ny[tid] = make_float2(oy.hi, oy.lo);
   }
   if (tid < 4) s_kb[tid] = 0.f;
-  classify(a, nullptr, Tx, Ty, a.thr_c, a.thr_ch, s_far, s_near, s_list, s_cnt);
-  for (int w = tid; w < a.nw; w += FF_THREADS) a.cmask[(size_t)tile * a.nw + w] = s_near[w];
-  node_sums<MODE, CP>(a, s_list, s_cnt[0], s_cnt[1], Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
+  classify<CO_THREADS>(a, nullptr, Tx, Ty, a.thr_c, a.thr_ch, s_far, s_near, s_list, s_cnt);
+  for (int w = tid; w < a.nw; w += CO_THREADS) a.cmask[(size_t)tile * a.nw + w] = s_near[w];
+  node_sums<MODE, CP, CO_THREADS>(a, s_list, s_cnt[0], s_cnt[1], Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
   if (tid < NV) s_plane[tid] = plane_of<CP>(s_val + tid * NODES, (D_ZC[0] - D_ZC[CP - 1]) * (float)half);
   __syncthreads();
   float *o = a.cval + (size_t)tile * coarse_floats(MODE);
-  for (int q = tid; q < NODES * NC; q += FF_THREADS) {
+  for (int q = tid; q < NODES * NC; q += CO_THREADS) {
     const int c = q / NODES, node = q % NODES;
     const float2 v = s_val[q];
     float r = v.x;
@@ -466,10 +471,10 @@ __device__ __forceinline__ float rcp_dff(float hi, float lo) {
   return fabsf(e) < 1e-3f ? fmaf(r, e, r) : 1.f / hi;
 }
 
-template <int MODE, int FT>
-__global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
+template <int MODE, int FT, int FI_THREADS>
+__global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far_map(const FarArgs a) {
   constexpr bool HESS = MODE == FAR_HESS, POT = MODE == FAR_POT;
-  constexpr int NODES = FP * FP, NC = ncmp(MODE), NV = nval(MODE), NC2 = ncmp2(MODE), SPLITS = FF_THREADS / (NODES / 2);
+  constexpr int NODES = FP * FP, NC = ncmp(MODE), NV = nval(MODE), NC2 = ncmp2(MODE), SPLITS = FI_THREADS / (NODES / 2);
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);                      // [FF_CH][REC_STRIDE4]
   float4 *s_off = s_rec + FF_CH * REC_STRIDE4;                            // [FF_CH]
@@ -494,32 +499,33 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   const int i0 = blockIdx.x * FT, j0 = a.row0 + blockIdx.y * FT;  // grid column and row of the tile's first node
   // the few FP64 operations once per tile
   constexpr double HALF = 0.5 * (FT - 1);
-  if (tid < 2) {
-    const df t = df_from_double(tid == 0 ? a.xmin + (i0 + HALF) * a.dx : a.ymin + (j0 + HALF) * a.dy);
-    reinterpret_cast<float2 *>(&s_T)[tid] = make_float2(t.hi, t.lo);
-  } else if (tid >= 32 && tid < 32 + 2 * FP) {
-    const int k = (tid - 32) % FP;
-    const df o = df_from_double(fine_table<FT>().xi[k] * (tid < 32 + FP ? a.dx : a.dy));
-    (tid < 32 + FP ? s_nx : s_ny)[k] = make_float2(o.hi, o.lo);
-  } else if (tid >= 64 && tid < 64 + 2 * FT) {
-    const int k = (tid - 64) % FT;
-    const df o = df_from_double((k - HALF) * (tid < 64 + FT ? a.dx : a.dy));
-    (tid < 64 + FT ? s_cx : s_ry)[k] = make_float2(o.hi, o.lo);
-    if (POT && a.tau) {
-      const double d = tid < 64 + FT ? a.xmin + (i0 + k) * a.dx - a.bx : a.ymin + (j0 + k) * a.dy - a.by;
-      s_tau[POT && tid >= 64 + FT][POT ? k : 0] = 0.5 * d * d;
+  for (int q = tid; q < 2 + 2 * FP + 2 * FT; q += FI_THREADS) {
+    if (q < 2) {
+      const df t = df_from_double(q == 0 ? a.xmin + (i0 + HALF) * a.dx : a.ymin + (j0 + HALF) * a.dy);
+      reinterpret_cast<float2 *>(&s_T)[q] = make_float2(t.hi, t.lo);
+    } else if (q < 2 + 2 * FP) {
+      const int k = (q - 2) % FP;
+      const df o = df_from_double(fine_table<FT>().xi[k] * (q < 2 + FP ? a.dx : a.dy));
+      (q < 2 + FP ? s_nx : s_ny)[k] = make_float2(o.hi, o.lo);
+      s_xi[k] = fine_table<FT>().xi[k];
+    } else {
+      const int e = q - 2 - 2 * FP, k = e % FT;
+      const df o = df_from_double((k - HALF) * (e < FT ? a.dx : a.dy));
+      (e < FT ? s_cx : s_ry)[k] = make_float2(o.hi, o.lo);
+      if (POT && a.tau) {
+        const double d = e < FT ? a.xmin + (i0 + k) * a.dx - a.bx : a.ymin + (j0 + k) * a.dy - a.by;
+        s_tau[POT && e >= FT][POT ? k : 0] = 0.5 * d * d;
+      }
     }
-  } else if (tid < 6) {
-    s_kb[tid - 2] = 0.f;
   }
-  if (tid >= 256 - FP) s_xi[tid - (256 - FP)] = fine_table<FT>().xi[tid - (256 - FP)];
-  for (int q = tid; q < FT * FP; q += FF_THREADS) s_L[q / FP][q % FP] = (&fine_table<FT>().w[0][0])[q];
+  if (tid < 4) s_kb[tid] = 0.f;
+  for (int q = tid; q < FT * FP; q += FI_THREADS) s_L[q / FP][q % FP] = (&fine_table<FT>().w[0][0])[q];
   __syncthreads();
   const df Tx = {s_T.x, s_T.y}, Ty = {s_T.z, s_T.w};
   const int ctile = a.ct ? (j0 / a.ct) * a.nct + i0 / a.ct : 0;
-  classify(a, a.ct ? a.cmask + (size_t)ctile * a.nw : nullptr, Tx, Ty, a.thr_f, a.thr_fh, s_far, s_near, s_list, s_cnt);
+  classify<FI_THREADS>(a, a.ct ? a.cmask + (size_t)ctile * a.nw : nullptr, Tx, Ty, a.thr_f, a.thr_fh, s_far, s_near, s_list, s_cnt);
   const int n_far = s_cnt[0], n_far_h = s_cnt[1], n_near = s_cnt[2], n_near_h = s_cnt[3];
-  node_sums<MODE, FP>(a, s_list, n_far, n_far_h, Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
+  node_sums<MODE, FP, FI_THREADS>(a, s_list, n_far, n_far_h, Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
   if (a.ct) {
     // the coarse tile's interpolant at this tile's nodes: rows of the tensor
     // product, then columns; its plane (exact products) in double-float
@@ -528,9 +534,9 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     const float *W = coarse_weights<FT>(sub);
     const float *Wx = W + cx * FP * CP, *Wy = W + cy * FP * CP;
     float *s_t1 = s_tmp + NC * CP * CP;
-    for (int q = tid; q < NC * CP * CP; q += FF_THREADS) s_tmp[q] = cv[q];
+    for (int q = tid; q < NC * CP * CP; q += FI_THREADS) s_tmp[q] = cv[q];
     __syncthreads();
-    for (int q = tid; q < NC * CP * FP; q += FF_THREADS) {  // (c, coarse row, fine column)
+    for (int q = tid; q < NC * CP * FP; q += FI_THREADS) {  // (c, coarse row, fine column)
       const int i = q % FP, cr = q / FP;
       const float *f = s_tmp + cr * CP;
       float v = 0.f;
@@ -540,7 +546,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     }
     __syncthreads();
     const float bx0 = FT * (cx + 0.5f) - 0.5f * a.ct, by0 = FT * (cy + 0.5f) - 0.5f * a.ct;
-    for (int q = tid; q < NC * NODES; q += FF_THREADS) {
+    for (int q = tid; q < NC * NODES; q += FI_THREADS) {
       const int c = q / NODES, node = q % NODES, i = node % FP, j = node / FP;
       float v = 0.f;
 #pragma unroll
@@ -560,7 +566,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   }
   if (tid < NV) s_plane[tid] = plane_of<FP>(s_val + tid * NODES, s_xi[0] - s_xi[FP - 1]);
   __syncthreads();
-  for (int q = tid; q < NC * NODES; q += FF_THREADS) {
+  for (int q = tid; q < NC * NODES; q += FI_THREADS) {
     const int c = q / NODES, node = q % NODES;
     const float2 v = s_val[q];
     float r = v.x;
@@ -576,7 +582,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   __syncthreads();
   // coefficients of every row pair: the remainders interpolated in y at the
   // tile's rows, one float4 = two values at two rows
-  for (int q = tid; q < (FT / 2) * FP * NC2 * 2; q += FF_THREADS) {
+  for (int q = tid; q < (FT / 2) * FP * NC2 * 2; q += FI_THREADS) {
     const int c = q % (2 * NC2), i = q / (2 * NC2) % FP, rp = q / (2 * NC2 * FP);
     float u = 0.f, v = 0.f;
     if (c < NC) {
@@ -590,10 +596,10 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
     reinterpret_cast<float2 *>(s_c)[q] = make_float2(u, v);
   }
   // the near potentials and the interpolant at the map nodes: lane = column,
-  // a warp takes row pairs warp, warp + FF_WARPS
+  // a warp takes row pairs warp, warp + (FI_THREADS / 32)
   bool staged = false;
 #pragma unroll 1
-  for (int task = warp; task < (FT / 2) * (FT / 32); task += FF_WARPS) {
+  for (int task = warp; task < (FT / 2) * (FT / 32); task += (FI_THREADS / 32)) {
     const int rp = task % (FT / 2), m = task / (FT / 2) * 32 + lane, i = i0 + m;
     const float mx = m - (float)HALF;
     const float2 ox = s_cx[m], r0 = s_ry[2 * rp], r1 = s_ry[2 * rp + 1];
@@ -604,7 +610,7 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
       const int cnt = min(FF_CH, n_near - c0);
       if (n_near > FF_CH || !staged) {
         __syncthreads();
-        stage_chunk(a, s_list + n_far + n_far_h + c0, cnt, Tx, Ty, s_rec, s_off);
+        stage_chunk<FI_THREADS>(a, s_list + n_far + n_far_h + c0, cnt, Tx, Ty, s_rec, s_off);
         __syncthreads();
         staged = true;
       }
@@ -786,13 +792,13 @@ __global__ void __launch_bounds__(FF_THREADS, 2) k_far_map(const FarArgs a) {
   const int nl = s_to[0], slot = s_to[1];
   const bool full = s_to[2] != 0, list_h = slot < 0 || !full;
   if (slot >= 0)
-    for (int w = tid; w < NW; w += FF_THREADS) {
+    for (int w = tid; w < NW; w += FI_THREADS) {
       unsigned *m = a.dense.mask + (size_t)slot * (HESS ? 2 : 1) * NW + w;
       m[0] = s_m[w];
       if (HESS) m[NW] = full ? s_mh[HESS ? w : 0] : 0u;
     }
   if (nl)
-    for (int w = warp; w < 2 * NW; w += FF_WARPS) {
+    for (int w = warp; w < 2 * NW; w += (FI_THREADS / 32)) {
       const int wi = w % NW;
       const unsigned mask = w < NW ? (HESS && list_h ? s_mh[HESS ? wi : 0] : 0u) : slot < 0 ? s_m[wi] : 0u;
       const int j = blockIdx.y * FT + wi / (FT / 32), i = i0 + wi % (FT / 32) * 32 + lane;
@@ -941,9 +947,9 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
 }
 
 // ft = 0: the coarse kernel
-size_t far_smem(int mode, int ft, int nw, int n) {
+size_t far_smem(int mode, int ft, int nw, int n, int threads = 256) {
   const bool coarse = ft == 0;
-  const int nodes = coarse ? CP * CP : FP * FP, splits = FF_THREADS / (nodes / 2), nc = ncmp(mode);
+  const int nodes = coarse ? CP * CP : FP * FP, splits = threads / (nodes / 2), nc = ncmp(mode);
   size_t b = sizeof(float4) * (FF_CH * REC_STRIDE4 + FF_CH);
   if (!coarse) b += sizeof(float4) * (ft / 2) * FP * ncmp2(mode);
   // the partial sums' space also holds the coarse tile's values (fine kernel)
@@ -1130,22 +1136,37 @@ static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, in
 
 template <int MODE>
 static int coarse_launch(const FarArgs &a, const FarPlan &p, int n, cudaStream_t st) {
-  const size_t smem = far_smem(MODE, 0, a.nw, n);
+  const size_t smem = far_smem(MODE, 0, a.nw, n, CO_THREADS);
   cudaFuncSetAttribute(k_far_coarse<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_far_coarse<MODE><<<dim3(p.nct, p.ncr), FF_THREADS, smem, st>>>(a);
+  k_far_coarse<MODE><<<dim3(p.nct, p.ncr), CO_THREADS, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "coarse map level launch: %s", cudaGetErrorString(e));
   return LENS_OK;
 }
 
-template <int MODE, int FT>
+template <int MODE, int FT, int TH>
 static int fine_launch(const FarArgs &a, int n, cudaStream_t st) {
-  const size_t smem = far_smem(MODE, FT, a.nw, n);
-  cudaFuncSetAttribute(k_far_map<MODE, FT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  k_far_map<MODE, FT><<<dim3((a.nx + FT - 1) / FT, (a.ny + FT - 1) / FT), FF_THREADS, smem, st>>>(a);
+  const size_t smem = far_smem(MODE, FT, a.nw, n, TH);
+  cudaFuncSetAttribute(k_far_map<MODE, FT, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_far_map<MODE, FT, TH><<<dim3((a.nx + FT - 1) / FT, (a.ny + FT - 1) / FT), TH, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "interpolated map launch: %s", cudaGetErrorString(e));
   return LENS_OK;
+}
+
+// 128 threads where there are many tiles (small CTAs overlap each other's
+// phases), 256 where the longest tile shows.  Both, whole map (256 / 128):
+// Hessian x 1000, 256 tiles 422 / 627 us, 1024 tiles 654 / 700, 2304 tiles 651
+// / 667, 4096 tiles 824 / 798; deflection x 200, 2304 tiles 197 / 181, 2304 of
+// 64 x 64 299 / 323, 4096 tiles 250 / 210, 6241 (5000^2 x 217) 524 / 451.
+// The potential's FP64 terms want the 256 (0.266 against 0.279 ms).
+// Counted over the whole map, also where a band of it is launched: the split of
+// the node sums, and with it the last bits, is then the same.
+constexpr int FI_TILES = 3072;
+template <int MODE, int FT>
+static int fine_threads(const FarArgs &a, const lens_grid *g, int n, cudaStream_t st) {
+  const long long tiles = (long long)((g->nx + FT - 1) / FT) * ((g->ny + FT - 1) / FT);
+  return tiles >= FI_TILES ? fine_launch<MODE, FT, 128>(a, n, st) : fine_launch<MODE, FT, 256>(a, n, st);
 }
 
 int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st) {
@@ -1175,11 +1196,11 @@ int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mod
     a.tau = beta != nullptr;
     a.bx = beta ? beta[0] : 0.0;
     a.by = beta ? beta[1] : 0.0;
-    return p.ft == 32 ? fine_launch<FAR_POT, 32>(a, m->n, st) : fine_launch<FAR_POT, 64>(a, m->n, st);
+    return p.ft == 32 ? fine_launch<FAR_POT, 32, 256>(a, m->n, st) : fine_launch<FAR_POT, 64, 256>(a, m->n, st);
   }
   a.out = (float *)out;
-  if (mode == FAR_HESS) return p.ft == 32 ? fine_launch<FAR_HESS, 32>(a, m->n, st) : fine_launch<FAR_HESS, 64>(a, m->n, st);
-  return p.ft == 32 ? fine_launch<FAR_GRAD, 32>(a, m->n, st) : fine_launch<FAR_GRAD, 64>(a, m->n, st);
+  if (mode == FAR_HESS) return p.ft == 32 ? fine_threads<FAR_HESS, 32>(a, g, m->n, st) : fine_threads<FAR_HESS, 64>(a, g, m->n, st);
+  return p.ft == 32 ? fine_threads<FAR_GRAD, 32>(a, g, m->n, st) : fine_threads<FAR_GRAD, 64>(a, g, m->n, st);
 }
 
 }  // namespace lens
