@@ -807,13 +807,14 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
     }
 }
 
-// The listed nodes of the densely listed tiles: a CTA takes 128 of a tile's
-// nodes, one per thread; the near potentials (those the interpolation nodes
-// left out) one by one in double-float, their records staged, then the far
-// ones' deflection interpolated in double-float (weights and values as
-// pairs: the FP32 weights' 6e-8 of a far sum of tens of arcsec would show
-// where the deflection is near zero).  8192^2 x 2000: the repair spends its
-// time on 100 instead of up to 4096 evaluations of every potential per tile.
+// The listed nodes of the densely listed tiles: a CTA takes some of a tile's
+// nodes, FR_LANES lanes each (launch_far_repair); the near potentials (those
+// the interpolation nodes left out) in double-float, dealt to the lanes, their
+// records staged, then the far ones' values interpolated in double-float
+// (weights and values as pairs: the FP32 weights' 6e-8 of a far sum of tens of
+// arcsec would show where the deflection is near zero).  8192^2 x 2000: the
+// repair spends its time on 100 instead of up to 4096 evaluations of every
+// potential per tile.  Bound: latency on small maps, else issue (74 %).
 constexpr int FR_THREADS = 128;
 struct FarRepairArgs {
   const float2 *recdf;
@@ -827,9 +828,10 @@ struct FarRepairArgs {
   DenseRepair dense;
 };
 
-template <int FT, bool HESS>
+template <int FT, bool HESS, int FR_LANES>
 __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a) {
-  constexpr int NW = FT * FT / 32, PARTS = FT * FT / FR_THREADS, NODES = FP * FP, NV = HESS ? 5 : 2, NM = HESS ? 2 : 1;
+  constexpr int FR_NODES = FR_THREADS / FR_LANES;
+  constexpr int NW = FT * FT / 32, PARTS = FT * FT / FR_NODES, NODES = FP * FP, NV = HESS ? 5 : 2, NM = HESS ? 2 : 1;
   __shared__ unsigned s_w[NW], s_wh[HESS ? NW : 1];
   __shared__ int s_pos[NW + 1], s_near[FR_THREADS], s_nn[FR_THREADS / 32];
   __shared__ float2 s_val[NV][NODES];
@@ -837,7 +839,9 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nh = min(*a.dense.count, a.dense.cap);
   for (long long item = blockIdx.x; item < (long long)nh * PARTS; item += gridDim.x) {
-    const int slot = (int)(item / PARTS), part = (int)(item % PARTS);
+    // part by part: the tiles' last parts, often empty, come last (tile by tile
+    // a CTA's items all had the same part number: 5000^2 x 1500 9.93 ms, so 9.39)
+    const int slot = (int)(item % nh), part = (int)(item / nh);
     __syncthreads();  // the previous item's shared data has been used
     const int entry = a.dense.tile[slot], tile = entry & 0x7fffffff;
     const bool full = HESS && entry < 0;  // the tile's Hessian values are there too
@@ -866,10 +870,11 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
     }
     __syncthreads();
     const int listed = s_pos[NW];
-    if (part * FR_THREADS >= listed) continue;  // uniform over the CTA
-    // this thread's node: the (part * 128 + tid)-th listed one
-    const int rank = min(part * FR_THREADS + tid, listed - 1);
-    const bool mine = part * FR_THREADS + tid < listed;
+    if (part * FR_NODES >= listed) continue;  // uniform over the CTA
+    // this lane group's node
+    const int want = part * FR_NODES + tid / FR_LANES, sub = tid % FR_LANES;
+    const int rank = min(want, listed - 1);
+    const bool mine = want < listed && sub == 0;
     int lo = 0, hi = NW;  // s_pos[lo] <= rank < s_pos[hi]
     while (hi - lo > 1) {
       const int mid = (lo + hi) / 2;
@@ -903,21 +908,28 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
       __syncthreads();
       for (int q = tid; q < RECDF * nn; q += FR_THREADS) s_rdf[q / nn][q % nn] = a.recdf[(size_t)(q / nn) * a.n + s_near[q % nn]];
       __syncthreads();
-      for (int k = 0; k < nn; ++k)
+      for (int k = sub; k < nn; k += FR_LANES)
         if (HESS && full)
           add_potential_dfs<true>(&s_rdf[0][k], FR_THREADS, a.all64 + (size_t)s_near[k] * REC64, X, Y, Xd, Yd, sum);
         else
           add_potential_dfs<false>(&s_rdf[0][k], FR_THREADS, a.all64 + (size_t)s_near[k] * REC64, X, Y, Xd, Yd, sum);
     }
-    // the far potentials: rows of the tensor product, then the column
+    // the lanes' sums (every lane gets the same bits)
+#pragma unroll
+    for (int c = 0; c < NV; ++c)
+#pragma unroll
+      for (int o = 1; o < FR_LANES; o <<= 1)
+        sum[c] = df_add(sum[c], df{__shfl_xor_sync(0xffffffffu, sum[c].hi, o), __shfl_xor_sync(0xffffffffu, sum[c].lo, o)});
+    // the far potentials: rows of the tensor product (spread over the lanes),
+    // then the column
     const FineTab<FT> &t = fine_table<FT>();
     double val[NV];
 #pragma unroll
     for (int c = 0; c < NV; ++c) {
       if (c >= 2 && !full) break;
-      df v = sum[c];
+      df v = {0.f, 0.f};
 #pragma unroll 1
-      for (int j = 0; j < FP; ++j) {
+      for (int j = sub; j < FP; j += FR_LANES) {
         df r = {0.f, 0.f};
 #pragma unroll
         for (int i = 0; i < FP; ++i) {
@@ -926,7 +938,10 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
         }
         v = df_add(v, df_mul(df{t.w[jr][j], t.wlo[jr][j]}, r));
       }
-      val[c] = a.dls * df_to_double(v);
+#pragma unroll
+      for (int o = 1; o < FR_LANES; o <<= 1)
+        v = df_add(v, df{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+      val[c] = a.dls * df_to_double(df_add(v, sum[c]));
     }
     float *o = a.out + (long long)(j0 + jr) * a.nx + i0 + ic;
     if (mine) {
@@ -1085,8 +1100,16 @@ int launch_far_repair(const Model *m, const lens_grid *g, const DenseRepair &den
   int nsm = 0;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, device);
   const bool hess = dense.nv == 5;
-  auto kern = dense.ft == 32 ? (hess ? k_far_repair<32, true> : k_far_repair<32, false>)
-                             : (hess ? k_far_repair<64, true> : k_far_repair<64, false>);
+  // Lanes per node: the near potentials of one node are a long chain, and a map
+  // of few nodes has few listed ones to fill the chip with; more lanes repeat
+  // the search for the near potentials more often.  Whole Hessian map with 1 /
+  // 2 / 4 lanes: 768^2 x 1000 705 / 595 / 556 us, 1024^2 x 300 298 / 278 / 266,
+  // 1536^2 x 500 439 / 423 / 422, 2048^2 x 1000 795 / 780 / 800; 64 x 64 tiles,
+  // 8192^2 x 2000 7.83 / 8.13 ms.  By the whole map, so that bands keep its bits.
+  const bool few = (long long)g->nx * g->ny < 1 << 21;
+  auto kern = dense.ft == 64 ? (hess ? k_far_repair<64, true, 1> : k_far_repair<64, false, 1>)
+              : few          ? (hess ? k_far_repair<32, true, 4> : k_far_repair<32, false, 4>)
+                             : (hess ? k_far_repair<32, true, 2> : k_far_repair<32, false, 2>);
   kern<<<4 * nsm, FR_THREADS, 0, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "dense map repair launch: %s", cudaGetErrorString(e));
