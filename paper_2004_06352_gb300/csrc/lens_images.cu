@@ -4,15 +4,18 @@
 // Per batch of parameter sets, six launches on the caller's stream:
 //   1. k_img_sources  per set: back-trace the constraints in FP64 and form
 //                     each source's barycentre (the source estimate).
-//   2. k_img_search   per (grid tile, set): deflection at the tile's nodes =
-//                     cached static part + the two varying potentials (FP32);
-//                     for each distance ratio the nodes are mapped to the
-//                     source plane, the sources inside the tile's footprint
-//                     (bounding box of its mapped nodes) are listed, and both
-//                     triangles of every cell are tested against that list
-//                     (bounding box, then barycentric weights with a small
-//                     tolerance so that a source on a shared edge is never
-//                     lost); every hit is appended to the set's buffer.
+//   2. k_img_search   per (128 x 64 cells, set): blocks of 8 x 8 cells whose
+//                     image in the source plane (a linear model with a bound
+//                     on its remainder, static part prepared with the grid)
+//                     can hold no source are left out; for the others the
+//                     deflection at the nodes = cached static part + the two
+//                     varying potentials (FP32); for each distance ratio the
+//                     nodes are mapped to the source plane, the sources inside
+//                     their bounding box are found, and both triangles of
+//                     every cell are tested against those (bounding box, then
+//                     barycentric weights with a small tolerance so that a
+//                     source on a shared edge is never lost); every hit is
+//                     appended to the set's buffer.
 //   3. k_img_newton   one group of RF_G threads per candidate: the hit
 //                     triangle is subdivided up to SUBDIV_LEVELS times
 //                     (keeping the sub-triangle that best contains the source;
@@ -62,25 +65,13 @@ constexpr float BARY_TOL = 1e-3f;
 constexpr int SUBDIV_LEVELS = LENS_SUBDIV_LEVELS;
 constexpr double SUBDIV_TOL = 1e-3;  // refinement stops when the source is this far outside every sub-triangle
 constexpr double LOCAL_CELLS = 2.0;  // a root must lie this many cell sizes from its triangle
-// search tile: CT_X x CT_Y cells per CTA of SEARCH_THREADS threads, each
-// thread CPT cells of one column; ratio groups tested SEARCH_GCH at a time
-#ifndef LENS_SEARCH_CT_Y
-#define LENS_SEARCH_CT_Y 64  // 4 cells per thread: faster than 32 (4 %), 16 (6 %) and 8 (fewer barrier-separated phases per cell)
-#endif
-constexpr int CT_X = 32, CT_Y = LENS_SEARCH_CT_Y, NX_T = CT_X + 1, NY_T = CT_Y + 1;
-constexpr int SEARCH_THREADS = 256, SEARCH_WARPS = SEARCH_THREADS / 32, SEARCH_GCH = SEARCH_WARPS;
-constexpr int CPT = CT_X * CT_Y / SEARCH_THREADS;  // cells per thread
-static_assert(CPT >= 1 && CT_X * CT_Y == CPT * SEARCH_THREADS, "whole cells per thread");
-// Sub-tile pre-filter (LENS_SEARCH_SUBTILE): warp w's cells are the tile's
-// cell rows w SUB_R .. w SUB_R + SUB_R - 1 (lane = column), and only the
-// sources inside that sub-tile's own footprint are tested against them
-// (1024^2 grid, 1000-potential model: 0.30 M instead of 1.13 M cell tests
-// per parameter set).
-#ifndef LENS_SEARCH_SUBTILE
-#define LENS_SEARCH_SUBTILE 1
-#endif
-constexpr int SUB_R = CT_Y / SEARCH_WARPS;
-static_assert(CT_X == 32 && SUB_R == CPT, "a warp's sub-tile: 32 columns x CPT rows");
+// Search: blocks of BL x BL cells; a CTA takes SB_X x SB_Y of them, a thread
+// each to cull, then a warp each.  Positions are relative to the origins of
+// TL_X x TL_Y cells.
+constexpr int BL = 8, BN = BL + 1, SB_X = 16, SB_Y = 8;
+constexpr int SEARCH_THREADS = SB_X * SB_Y, SEARCH_WARPS = SEARCH_THREADS / 32;
+constexpr int TL_X = 32, TL_Y = 64, NTL_X = SB_X * BL / TL_X, NTL = NTL_X * (SB_Y * BL / TL_Y);
+static_assert(BL * BL == 64 && SB_X * BL % TL_X == 0 && SB_Y * BL % TL_Y == 0, "two cells per lane; whole tiles");
 // candidate status; the failures say which stage rejected it
 constexpr int ST_PENDING = 0, ST_NEWTON = 1, ST_FINAL = 2, ST_FAILED = -1, ST_FAR = -2, ST_NO_POLISH = -3;
 
@@ -251,43 +242,15 @@ struct SearchArgs {
   const int32_t *grp_off, *grp_src;
   const float *grp_r32;  // ratio of each group, FP32
   int ng;
+  const float4 *plane;   // per block: grid_planes' model of the static deflection; NULL: no culling
+  int nbx, nby;          // blocks
 };
 
-#if !LENS_SEARCH_SUBTILE
-__device__ __forceinline__ void tri_test(float2 A, float2 Bv, float2 Cv, float2 tA, float2 tB, float2 tC,
-                                         const float2 *s_src, const int *list, int nlist, float tiny, int *cnt,
-                                         Hit *hits, int cell) {
-  const float lox = fminf(A.x, fminf(Bv.x, Cv.x)), hix = fmaxf(A.x, fmaxf(Bv.x, Cv.x));
-  const float loy = fminf(A.y, fminf(Bv.y, Cv.y)), hiy = fmaxf(A.y, fmaxf(Bv.y, Cv.y));
-  const float padx = BARY_TOL * (hix - lox) + 1e-6f, pady = BARY_TOL * (hiy - loy) + 1e-6f;
-  const float e1x = Bv.x - A.x, e1y = Bv.y - A.y, e2x = Cv.x - A.x, e2y = Cv.y - A.y;
-  const float area2 = e1x * e2y - e1y * e2x;
-  if (!(fabsf(area2) > tiny)) return;
-  const float inv = 1.f / area2;
-  for (int k = 0; k < nlist; ++k) {
-    const int src = list[k];
-    const float2 P = s_src[src];
-    if (P.x < lox - padx || P.x > hix + padx || P.y < loy - pady || P.y > hiy + pady) continue;
-    const float px = P.x - A.x, py = P.y - A.y;
-    const float wb = (px * e2y - py * e2x) * inv, wc = (e1x * py - e1y * px) * inv, wa = 1.f - wb - wc;
-    if (wa < -BARY_TOL || wb < -BARY_TOL || wc < -BARY_TOL) continue;
-    const int slot = atomicAdd(cnt, 1);
-    if (slot < IMG_CAP) {
-      Hit *h = hits + slot;
-      h->src = src;
-      h->cx = (tA.x + tB.x + tC.x) * (1.f / 3.f);
-      h->cy = (tA.y + tB.y + tC.y) * (1.f / 3.f);
-      h->cell = cell;
-      h->status = ST_PENDING;
-    }
-  }
-}
-
-#else
-// The same for the list entries whose bits are set in mask (entry k: bit k).
+// Triangle A, B, C of the source plane against the sources whose bits are set
+// in mask (bit k: s_src[k], source s_id[k]).
 __device__ __forceinline__ void tri_test_mask(float2 A, float2 Bv, float2 Cv, float2 tA, float2 tB, float2 tC,
-                                              const float2 *s_src, const int *list, unsigned mask, float tiny,
-                                              int *cnt, Hit *hits, int cell) {
+                                              const float2 *s_src, const unsigned short *s_id, unsigned mask,
+                                              float tiny, int *cnt, Hit *hits, int cell) {
   const float lox = fminf(A.x, fminf(Bv.x, Cv.x)), hix = fmaxf(A.x, fmaxf(Bv.x, Cv.x));
   const float loy = fminf(A.y, fminf(Bv.y, Cv.y)), hiy = fmaxf(A.y, fmaxf(Bv.y, Cv.y));
   const float padx = BARY_TOL * (hix - lox) + 1e-6f, pady = BARY_TOL * (hiy - loy) + 1e-6f;
@@ -296,8 +259,8 @@ __device__ __forceinline__ void tri_test_mask(float2 A, float2 Bv, float2 Cv, fl
   if (!(fabsf(area2) > tiny)) return;
   const float inv = 1.f / area2;
   for (unsigned mm = mask; mm; mm &= mm - 1u) {
-    const int src = list[__ffs(mm) - 1];
-    const float2 P = s_src[src];
+    const int k = __ffs(mm) - 1;
+    const float2 P = s_src[k];
     if (P.x < lox - padx || P.x > hix + padx || P.y < loy - pady || P.y > hiy + pady) continue;
     const float px = P.x - A.x, py = P.y - A.y;
     const float wb = (px * e2y - py * e2x) * inv, wc = (e1x * py - e1y * px) * inv, wa = 1.f - wb - wc;
@@ -305,7 +268,7 @@ __device__ __forceinline__ void tri_test_mask(float2 A, float2 Bv, float2 Cv, fl
     const int slot = atomicAdd(cnt, 1);
     if (slot < IMG_CAP) {
       Hit *h = hits + slot;
-      h->src = src;
+      h->src = s_id[k];
       h->cx = (tA.x + tB.x + tC.x) * (1.f / 3.f);
       h->cy = (tA.y + tB.y + tC.y) * (1.f / 3.f);
       h->cell = cell;
@@ -313,7 +276,6 @@ __device__ __forceinline__ void tri_test_mask(float2 A, float2 Bv, float2 Cv, fl
     }
   }
 }
-#endif
 
 // Order-preserving map of floats to signed ints (and back: it is its own
 // inverse), so that integer warp min/max reductions apply to floats.
@@ -323,190 +285,261 @@ __device__ __forceinline__ int f2ord(float f) {
 }
 __device__ __forceinline__ float ord2f(int i) { return __int_as_float(i ^ ((i >> 31) & 0x7fffffff)); }
 
-#ifndef LENS_SEARCH_PAIRED
-#define LENS_SEARCH_PAIRED 0  // 1: two nodes per paired evaluation of the varying potentials (measured 1 % slower)
-#endif
-#ifndef LENS_SEARCH_MINB
-#define LENS_SEARCH_MINB 4  // resident CTAs per SM the search is compiled for (64 registers: 4 % faster than 1, no spills; 5 spills)
-#endif
-__global__ void __launch_bounds__(SEARCH_THREADS, LENS_SEARCH_MINB) k_img_search(const SetArgs a, const SearchArgs g) {
+// Model of the static deflection over each block of BL x BL cells: plane[2 b]
+// = {ax, ay, dax/dx, dax/dy}, plane[2 b + 1] = {day/dx, day/dy, ex, ey}, so
+// that at every node of block b the deflection differs from the plane through
+// the block's centre by ex, ey at most.  A warp per block.
+__global__ void __launch_bounds__(256) k_grid_planes(const float *ax, const float *ay, int nx, int ny, float dx, float dy,
+                                                     int nbx, int nby, float4 *plane) {
+  const int lane = threadIdx.x & 31;
+  const long long nb = (long long)nbx * nby;
+  for (long long b = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); b < nb; b += (long long)gridDim.x * 8) {
+    const int i0 = (int)(b % nbx) * BL, j0 = (int)(b / nbx) * BL;
+    const int w = min(BL, nx - 1 - i0), h = min(BL, ny - 1 - j0);
+    auto at = [&](const float *f, int i, int j) { return f[(size_t)(j0 + j) * nx + i0 + i]; };
+    float g[2][2], lo[2], hi[2], big = 0.f;
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const float *f = c ? ay : ax;
+      const float f00 = at(f, 0, 0), f10 = at(f, w, 0), f01 = at(f, 0, h), f11 = at(f, w, h);
+      g[c][0] = 0.5f * ((f10 - f00) + (f11 - f01)) / (w * dx);
+      g[c][1] = 0.5f * ((f01 - f00) + (f11 - f10)) / (h * dy);
+      lo[c] = INFINITY;
+      hi[c] = -INFINITY;
+      for (int n = lane; n < (w + 1) * (h + 1); n += 32) {
+        const int i = n % (w + 1), j = n / (w + 1);
+        const float v = at(f, i, j);
+        const float d = v - (g[c][0] * ((i - 0.5f * w) * dx) + g[c][1] * ((j - 0.5f * h) * dy));
+        lo[c] = fminf(lo[c], d);
+        hi[c] = fmaxf(hi[c], d);
+        big = fmaxf(big, fabsf(v));
+        if (!(fabsf(d) < INFINITY)) big = INFINITY;  // (fminf and fmaxf drop NaN)
+      }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        lo[c] = fminf(lo[c], __shfl_xor_sync(0xffffffffu, lo[c], o));
+        hi[c] = fmaxf(hi[c], __shfl_xor_sync(0xffffffffu, hi[c], o));
+      }
+    }
+    if (lane == 0) {
+      const float pad = 2e-6f * big;  // the FP32 operations above
+      plane[2 * b] = make_float4(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), g[0][0], g[0][1]);
+      plane[2 * b + 1] = make_float4(g[1][0], g[1][1], 0.5f * (hi[0] - lo[0]) + pad, 0.5f * (hi[1] - lo[1]) + pad);
+    }
+  }
+}
+
+// The ratio groups (bit q & 31) with a source that the block may image: its
+// nodes' image in the source plane lies in the box of the linear model
+//   beta = X - r (a + J (X - Xc)) -+ r e,
+// a and J the static plane's plus the varying potentials' deflection and
+// Hessian at the block's centre.  The varying potentials' remainder over the
+// block's half-diagonal rho: a dPIE (or SIS, point mass) at distance d whose
+// iso-density axis ratio is q varies with its elliptical radius, which changes
+// by at most rho / q; for q d > 4 rho its third derivatives there are at most
+// (4/3)^4 times a few |H| / (q d) (|H| = kappa + |gamma| falls no faster than
+// d^-2 and third derivatives no faster than |H| / d times the power), so
+// |remainder| <= 8 |H| rho^2 / (q d) holds with room; nearer blocks are never
+// left out, nor are those with any value not finite.
+__device__ __forceinline__ unsigned live_groups(const SearchArgs &g, const float (*s_rec)[REC32], float4 p0, float4 p1,
+                                                const float2 *off, float2 T, float ox, float oy, float hx, float hy,
+                                                const float2 *s_src, const float4 &box) {
+  const float rho2 = hx * hx + hy * hy;
+  float ax = p0.x, ay = p0.y, xx = p0.z, xy = p0.w, yx = p1.x, yy = p1.y, ex = p1.z, ey = p1.w;
+#pragma unroll 1
+  for (int v = 0; v < 2; ++v) {
+    const float4 *r4 = reinterpret_cast<const float4 *>(s_rec[v]);
+    Acc<true, 1> acc;
+    acc.zero();
+    const float dX = off[v].x + ox, dY[1] = {off[v].y + oy};
+    const float q2 = __float_as_int(s_rec[v][R_KIND]) >= K32_SIS ? 1.f : s_rec[v][R_Q2];
+    const float qd2 = q2 * (dX * dX + dY[0] * dY[0]);
+    if (!(qd2 > 16.f * rho2)) return ~0u;
+    eval32_any<true, 1, true>(r4, dX, dY, acc);
+    const float k = acc.k[0], g1 = acc.g1[0], g2 = acc.g2[0];
+    const float rem = 8.f * (fabsf(k) + sqrtf(g1 * g1 + g2 * g2)) * rho2 * rsqrtf(qd2);
+    ax += acc.ax[0];
+    ay += acc.ay[0];
+    xx += k + g1;
+    xy += g2;
+    yx += g2;
+    yy += k - g1;
+    ex += rem;
+    ey += rem;
+  }
+  const float X = T.x + ox, Y = T.y + oy;
+  unsigned live = 0;
+  for (int q = 0; q < g.ng; ++q) {
+    const float r = g.grp_r32[q], cx = X - r * ax, cy = Y - r * ay;
+    float bx = fabsf(1.f - r * xx) * hx + fabsf(r * xy) * hy + fabsf(r) * ex;
+    float by = fabsf(r * yx) * hx + fabsf(1.f - r * yy) * hy + fabsf(r) * ey;
+    // the tests' tolerances, and FP32 rounding of nodes and model
+    bx += 4.f * BARY_TOL * bx + 1e-5f * (1.f + fabsf(X) + hx + fabsf(r * ax));
+    by += 4.f * BARY_TOL * by + 1e-5f * (1.f + fabsf(Y) + hy + fabsf(r * ay));
+    if (cx - bx > box.y || cx + bx < box.x || cy - by > box.w || cy + by < box.z) continue;  // beside every source
+    for (int k = g.grp_off[q]; k < g.grp_off[q + 1]; ++k) {
+      const float2 P = s_src[k];
+      if (!(fabsf(P.x - cx) > bx) && !(fabsf(P.y - cy) > by)) {
+        live |= 1u << (q & 31);
+        break;
+      }
+    }
+  }
+  return live;
+}
+
+// Bound: issue (76 %).  100 sources have images in few of the 8 x 8 blocks, so
+// a warp evaluates 81 nodes for those alone: 256 sets of the 1000-potential
+// model on 1024^2 cells 0.90 ms, 7.7e8 warp instructions; every node of every
+// 32 x 64 cells, as it was, 3.69 ms, 3.6e9.  CTAs of 128 threads at 64
+// registers; 256 threads, or 3 to 10 CTAs per SM, within 1 % (smaller ones
+// spread few sets over more SMs).
+__global__ void __launch_bounds__(SEARCH_THREADS, 8) k_img_search(const SetArgs a, const SearchArgs g) {
   __shared__ __align__(16) float s_rec[2][REC32];
-  __shared__ float2 s_off[2];  // tile origin minus each varying potential's centre
-  __shared__ float s_T[2];     // tile origin
-  __shared__ float2 s_al[NX_T * NY_T];
-  __shared__ float2 s_src[MAX_SRC];
-  __shared__ float s_box[SEARCH_GCH][4][SEARCH_WARPS];
-  __shared__ int s_list[MAX_SRC];  // group q's sources inside the footprint, from s_list[grp_off[q]]
-  __shared__ int s_nlist[SEARCH_GCH];
+  __shared__ float2 s_T[NTL], s_off[NTL][2];  // tile origins; the same minus each varying potential's centre
+  __shared__ float2 s_src[MAX_SRC];           // sources by group
+  __shared__ unsigned short s_id[MAX_SRC];
+  __shared__ float4 s_box;                    // of all sources: x from, to, y from, to
+  __shared__ float2 s_al[SEARCH_WARPS][BN * BN];
+  __shared__ unsigned s_grp[SEARCH_THREADS];
+  __shared__ unsigned short s_live[SEARCH_THREADS];
+  __shared__ int s_n, s_next;
   const int b = blockIdx.z;
   if (!a.s.valid[b]) return;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int i0 = blockIdx.x * CT_X, j0 = blockIdx.y * CT_Y;
-  // positions in FP32 relative to the tile origin (the search only decides
+  // positions in FP32 relative to the tile origins (the search only decides
   // which triangles seed a candidate; the refinement is exact); the few FP64
   // operations are done once per CTA
   const VarRecs &var = a.s.var[b];
-  if (tid < 2) {
-    const double T = tid == 0 ? g.xmin + i0 * g.dx : g.ymin + j0 * g.dy;
-    s_T[tid] = (float)T;
-    const double Tx = g.xmin + i0 * g.dx, Ty = g.ymin + j0 * g.dy;
-    s_off[tid] = make_float2((float)(Tx - ((double)var.cen[tid][0] + (double)var.cen[tid][2])),
-                             (float)(Ty - ((double)var.cen[tid][1] + (double)var.cen[tid][3])));
+  if (tid < NTL) {
+    const double Tx = g.xmin + (double)((int)blockIdx.x * SB_X * BL + tid % NTL_X * TL_X) * g.dx;
+    const double Ty = g.ymin + (double)((int)blockIdx.y * SB_Y * BL + tid / NTL_X * TL_Y) * g.dy;
+    s_T[tid] = make_float2((float)Tx, (float)Ty);
+    for (int v = 0; v < 2; ++v)
+      s_off[tid][v] = make_float2((float)(Tx - ((double)var.cen[v][0] + (double)var.cen[v][2])),
+                                  (float)(Ty - ((double)var.cen[v][1] + (double)var.cen[v][3])));
   }
+  if (tid == SEARCH_THREADS - 1) s_n = s_next = 0;
   if (tid < 2 * REC32) s_rec[tid / REC32][tid % REC32] = var.r32[tid / REC32][tid % REC32];
   const float2 *src32 = a.s.src32 + (size_t)b * a.nsrc;
-  for (int i = tid; i < a.nsrc; i += SEARCH_THREADS) s_src[i] = src32[i];
-  __syncthreads();
-  const float fdx = g.fdx, fdy = g.fdy, fTx = s_T[0], fTy = s_T[1];
-#if LENS_SEARCH_PAIRED
-  // the tile's nodes two at a time (n and n + SEARCH_THREADS) on the paired
-  // FP32 path; past the end the second is a copy of the first, not stored
-  for (int n = tid; n < NX_T * NY_T; n += 2 * SEARCH_THREADS) {
-    const int n1 = n + SEARCH_THREADS < NX_T * NY_T ? n + SEARCH_THREADS : n;
-    const int ia = min(i0 + n % NX_T, g.nx - 1), ja = min(j0 + n / NX_T, g.ny - 1);
-    const int ib = min(i0 + n1 % NX_T, g.nx - 1), jb = min(j0 + n1 / NX_T, g.ny - 1);
-    const size_t oa = (size_t)ja * g.nx + ia, ob = (size_t)jb * g.nx + ib;
-    float2 tx = make_float2(g.ax[oa], g.ax[ob]), ty = make_float2(g.ay[oa], g.ay[ob]);
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      const float2 dX2[1] = {make_float2(fmaf((float)(ia - i0), fdx, s_off[v].x), fmaf((float)(ib - i0), fdx, s_off[v].x))};
-      const float2 dY2[1] = {make_float2(fmaf((float)(ja - j0), fdy, s_off[v].y), fmaf((float)(jb - j0), fdy, s_off[v].y))};
-      Acc2<false, 1> acc;
-      acc.zero();
-      eval32x2_any<false, 1, false, true>(reinterpret_cast<const float4 *>(s_rec[v]), dX2, dY2, acc);
-      tx = add2(tx, acc.ax[0]);
-      ty = add2(ty, acc.ay[0]);
-    }
-    s_al[n] = make_float2(tx.x, ty.x);
-    if (n1 != n) s_al[n1] = make_float2(tx.y, ty.y);
+  for (int k = tid; k < a.nsrc; k += SEARCH_THREADS) {
+    const int src = g.grp_src[k];
+    s_src[k] = src32[src];
+    s_id[k] = (unsigned short)src;
   }
-#else
-  for (int n = tid; n < NX_T * NY_T; n += SEARCH_THREADS) {
-    const int li = n % NX_T, lj = n / NX_T;
-    const int ii = min(i0 + li, g.nx - 1), jj = min(j0 + lj, g.ny - 1);
-    const size_t o = (size_t)jj * g.nx + ii;
-    float tx = g.ax[o], ty = g.ay[o];
-#pragma unroll
-    for (int v = 0; v < 2; ++v) {
-      Acc<false, 1> acc;
-      acc.zero();
-      const float dX = fmaf((float)(ii - i0), fdx, s_off[v].x), dY[1] = {fmaf((float)(jj - j0), fdy, s_off[v].y)};
-      eval32_any<false, 1, true>(reinterpret_cast<const float4 *>(s_rec[v]), dX, dY, acc);
-      tx += acc.ax[0];
-      ty += acc.ay[0];
-    }
-    s_al[n] = make_float2(tx, ty);
-  }
-#endif
   __syncthreads();
-#if LENS_SEARCH_SUBTILE
-  const int ci = lane;  // this thread's cells: column ci, rows warp SUB_R .. warp SUB_R + SUB_R - 1
-#else
-  const int ci = tid % CT_X, cj0 = tid / CT_X;  // this thread's cells: column ci, rows cj0, cj0 + CT_Y / CPT, ...
-#endif
+  if (warp == 0) {
+    float lx = INFINITY, hx = -INFINITY, ly = INFINITY, hy = -INFINITY;
+    for (int k = lane; k < a.nsrc; k += 32) {
+      const float2 P = s_src[k];
+      lx = fminf(lx, P.x);
+      hx = fmaxf(hx, P.x);
+      ly = fminf(ly, P.y);
+      hy = fmaxf(hy, P.y);
+    }
+    lx = ord2f(__reduce_min_sync(0xffffffffu, f2ord(lx)));
+    hx = ord2f(__reduce_max_sync(0xffffffffu, f2ord(hx)));
+    ly = ord2f(__reduce_min_sync(0xffffffffu, f2ord(ly)));
+    hy = ord2f(__reduce_max_sync(0xffffffffu, f2ord(hy)));
+    if (lane == 0) s_box = make_float4(lx, hx, ly, hy);
+  }
+  __syncthreads();
+  const float fdx = g.fdx, fdy = g.fdy;
+  {
+    const int bi = tid % SB_X, bj = tid / SB_X, gx = blockIdx.x * SB_X + bi, gy = blockIdx.y * SB_Y + bj;
+    unsigned grp = 0;
+    if (gx < g.nbx && gy < g.nby) {
+      if (g.plane) {
+        const float4 *p = g.plane + 2 * ((size_t)gy * g.nbx + gx);
+        const float w = (float)min(BL, g.nx - 1 - gx * BL), h = (float)min(BL, g.ny - 1 - gy * BL);
+        const int t = bi * BL / TL_X + bj * BL / TL_Y * NTL_X;
+        grp = live_groups(g, s_rec, p[0], p[1], s_off[t], s_T[t], ((float)(bi * BL % TL_X) + 0.5f * w) * fdx,
+                          ((float)(bj * BL % TL_Y) + 0.5f * h) * fdy, 0.5f * w * fdx, 0.5f * h * fdy, s_src, s_box);
+      } else {
+        grp = ~0u;
+      }
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, grp != 0u);
+    int base = 0;
+    if (lane == 0 && m) base = atomicAdd(&s_n, __popc(m));
+    base = __shfl_sync(0xffffffffu, base, 0) + __popc(m & ((1u << lane) - 1u));
+    if (grp) {
+      s_live[base] = (unsigned short)tid;
+      s_grp[base] = grp;
+    }
+  }
+  __syncthreads();
   const float tiny = g.tiny;
   int *cnt = a.s.cnt + b;
   Hit *hits = a.s.hits + (size_t)b * IMG_CAP;
-  for (int q0 = 0; q0 < g.ng; q0 += SEARCH_GCH) {
-    const int nq = min(SEARCH_GCH, g.ng - q0);
-    // the tile's footprint in each ratio's source plane (bounding box of its
-    // nodes): one pass over this thread's nodes for all groups of the chunk,
-    // then one integer min/max reduction per warp and bound
-    float lo[SEARCH_GCH][2], hi[SEARCH_GCH][2];
+  float2 *al = s_al[warp];
+  while (true) {
+    int e = 0;
+    if (lane == 0) e = atomicAdd(&s_next, 1);
+    e = __shfl_sync(0xffffffffu, e, 0);
+    if (e >= s_n) break;
+    const int bi = s_live[e] % SB_X, bj = s_live[e] / SB_X;
+    const unsigned grp = s_grp[e];
+    const int i0 = (blockIdx.x * SB_X + bi) * BL, j0 = (blockIdx.y * SB_Y + bj) * BL;
+    const int t = bi * BL / TL_X + bj * BL / TL_Y * NTL_X, ti = bi * BL % TL_X, tj = bj * BL % TL_Y;  // first node in its tile
+    const float fTx = s_T[t].x, fTy = s_T[t].y;
+    for (int n = lane; n < BN * BN; n += 32) {
+      const int li = min(n % BN, g.nx - 1 - i0), lj = min(n / BN, g.ny - 1 - j0);
+      const size_t o = (size_t)(j0 + lj) * g.nx + i0 + li;
+      float tx = g.ax[o], ty = g.ay[o];
 #pragma unroll
-    for (int qq = 0; qq < SEARCH_GCH; ++qq) lo[qq][0] = lo[qq][1] = INFINITY, hi[qq][0] = hi[qq][1] = -INFINITY;
-#if LENS_SEARCH_SUBTILE
-    // warp w takes node rows w R .. w R + R (its own cells' rows and the row
-    // below), so the bounds it reduces are its sub-tile's footprint
-    for (int k = lane; k < (SUB_R + 1) * NX_T; k += 32) {
-      const int n = warp * SUB_R * NX_T + k;
-#else
-    for (int n = tid; n < NX_T * NY_T; n += SEARCH_THREADS) {
-#endif
-      const int li = n % NX_T, lj = n / NX_T;
-      if (i0 + li >= g.nx || j0 + lj >= g.ny) continue;
-      const float X = fmaf((float)li, fdx, fTx), Y = fmaf((float)lj, fdy, fTy);
-      const float2 al = s_al[n];
-#pragma unroll
-      for (int qq = 0; qq < SEARCH_GCH; ++qq) {
-        if (qq >= nq) break;
-        const float r = g.grp_r32[q0 + qq];
-        const float bx = X - r * al.x, by = Y - r * al.y;
-        lo[qq][0] = fminf(lo[qq][0], bx);
-        hi[qq][0] = fmaxf(hi[qq][0], bx);
-        lo[qq][1] = fminf(lo[qq][1], by);
-        hi[qq][1] = fmaxf(hi[qq][1], by);
+      for (int v = 0; v < 2; ++v) {
+        Acc<false, 1> acc;
+        acc.zero();
+        const float dX = fmaf((float)(ti + li), fdx, s_off[t][v].x), dY[1] = {fmaf((float)(tj + lj), fdy, s_off[t][v].y)};
+        eval32_any<false, 1, true>(reinterpret_cast<const float4 *>(s_rec[v]), dX, dY, acc);
+        tx += acc.ax[0];
+        ty += acc.ay[0];
       }
+      al[n] = make_float2(tx, ty);
     }
-#pragma unroll
-    for (int qq = 0; qq < SEARCH_GCH; ++qq) {
-      if (qq >= nq) break;
-      const int lx = __reduce_min_sync(0xffffffffu, f2ord(lo[qq][0])), hx = __reduce_max_sync(0xffffffffu, f2ord(hi[qq][0]));
-      const int ly = __reduce_min_sync(0xffffffffu, f2ord(lo[qq][1])), hy = __reduce_max_sync(0xffffffffu, f2ord(hi[qq][1]));
-      if (lane == 0) {
-        s_box[qq][0][warp] = ord2f(lx);
-        s_box[qq][1][warp] = ord2f(hx);
-        s_box[qq][2][warp] = ord2f(ly);
-        s_box[qq][3][warp] = ord2f(hy);
+    __syncwarp();
+    for (int q = 0; q < g.ng; ++q) {
+      if (!(grp >> (q & 31) & 1u)) continue;
+      const float r = g.grp_r32[q];
+      // the block's bounding box in this ratio's source plane (nodes past the
+      // grid's end repeat the last ones)
+      float lx = INFINITY, hx = -INFINITY, ly = INFINITY, hy = -INFINITY;
+      for (int n = lane; n < BN * BN; n += 32) {
+        const int li = min(n % BN, g.nx - 1 - i0), lj = min(n / BN, g.ny - 1 - j0);
+        const float bx = fmaf((float)(ti + li), fdx, fTx) - r * al[n].x, by = fmaf((float)(tj + lj), fdy, fTy) - r * al[n].y;
+        lx = fminf(lx, bx);
+        hx = fmaxf(hx, bx);
+        ly = fminf(ly, by);
+        hy = fmaxf(hy, by);
       }
-    }
-    __syncthreads();
-    if (warp < nq) {
-      // warp w: the sources of group q0 + w inside the footprint (+ the test's tolerance)
-      float L = INFINITY, H = -INFINITY, Ly = INFINITY, Hy = -INFINITY;
-      for (int w = 0; w < SEARCH_WARPS; ++w) {
-        L = fminf(L, s_box[warp][0][w]);
-        H = fmaxf(H, s_box[warp][1][w]);
-        Ly = fminf(Ly, s_box[warp][2][w]);
-        Hy = fmaxf(Hy, s_box[warp][3][w]);
-      }
-      const float px = BARY_TOL * (H - L) + 1e-5f, py = BARY_TOL * (Hy - Ly) + 1e-5f;
-      const int g0 = g.grp_off[q0 + warp], g1 = g.grp_off[q0 + warp + 1];
-      int base = 0;
-      for (int k0 = g0; k0 < g1; k0 += 32) {
-        const int k = k0 + lane;
+      lx = ord2f(__reduce_min_sync(0xffffffffu, f2ord(lx)));
+      hx = ord2f(__reduce_max_sync(0xffffffffu, f2ord(hx)));
+      ly = ord2f(__reduce_min_sync(0xffffffffu, f2ord(ly)));
+      hy = ord2f(__reduce_max_sync(0xffffffffu, f2ord(hy)));
+      const float px = BARY_TOL * (hx - lx) + 1e-5f, py = BARY_TOL * (hy - ly) + 1e-5f;
+      const int g1 = g.grp_off[q + 1];
+      for (int k0 = g.grp_off[q]; k0 < g1; k0 += 32) {
         bool in = false;
-        int src = 0;
-        if (k < g1) {
-          src = g.grp_src[k];
-          const float2 P = s_src[src];
-          in = P.x >= L - px && P.x <= H + px && P.y >= Ly - py && P.y <= Hy + py;
-        }
-        const unsigned m = __ballot_sync(0xffffffffu, in);
-        if (in) s_list[g0 + base + __popc(m & ((1u << lane) - 1u))] = src;
-        base += __popc(m);
-      }
-      if (lane == 0) s_nlist[warp] = base;
-    }
-    __syncthreads();
-    for (int qq = 0; qq < nq; ++qq) {
-      const int nlist = s_nlist[qq];
-      if (nlist == 0) continue;
-      const float r = g.grp_r32[q0 + qq];
-      const int *list = s_list + g.grp_off[q0 + qq];
-#if LENS_SEARCH_SUBTILE
-      // the list entries inside this warp's sub-tile footprint (padded as
-      // the tile's, which covers every cell's padding), 32 at a time as bit
-      // masks; a cell's box lies inside its sub-tile's
-      const float sL = s_box[qq][0][warp], sH = s_box[qq][1][warp], sLy = s_box[qq][2][warp], sHy = s_box[qq][3][warp];
-      const float spx = BARY_TOL * (sH - sL) + 1e-5f, spy = BARY_TOL * (sHy - sLy) + 1e-5f;
-      for (int c0 = 0; c0 < nlist; c0 += 32) {
-        bool in = false;
-        if (c0 + lane < nlist) {
-          const float2 P = s_src[list[c0 + lane]];
-          in = P.x >= sL - spx && P.x <= sH + spx && P.y >= sLy - spy && P.y <= sHy + spy;
+        if (k0 + lane < g1) {
+          const float2 P = s_src[k0 + lane];
+          in = P.x >= lx - px && P.x <= hx + px && P.y >= ly - py && P.y <= hy + py;
         }
         const unsigned mask = __ballot_sync(0xffffffffu, in);
         if (mask == 0u) continue;  // uniform over the warp
 #pragma unroll
-        for (int rr = 0; rr < SUB_R; ++rr) {
-          const int cj = warp * SUB_R + rr;
+        for (int rr = 0; rr < 2; ++rr) {
+          const int ci = lane % BL, cj = lane / BL + rr * (BL / 2);
           const int gi = i0 + ci, gj = j0 + cj;
           if (gi >= g.nx - 1 || gj >= g.ny - 1) continue;
-          const float X0 = fmaf((float)ci, fdx, fTx), X1 = fmaf((float)(ci + 1), fdx, fTx);
-          const float Y0 = fmaf((float)cj, fdy, fTy), Y1 = fmaf((float)(cj + 1), fdy, fTy);
-          const int n00 = cj * NX_T + ci;
-          const float2 a00 = s_al[n00], a10 = s_al[n00 + 1], a01 = s_al[n00 + NX_T], a11 = s_al[n00 + NX_T + 1];
+          const float X0 = fmaf((float)(ti + ci), fdx, fTx), X1 = fmaf((float)(ti + ci + 1), fdx, fTx);
+          const float Y0 = fmaf((float)(tj + cj), fdy, fTy), Y1 = fmaf((float)(tj + cj + 1), fdy, fTy);
+          const int n00 = cj * BN + ci;
+          const float2 a00 = al[n00], a10 = al[n00 + 1], a01 = al[n00 + BN], a11 = al[n00 + BN + 1];
           const float2 t00 = make_float2(X0, Y0), t10 = make_float2(X1, Y0), t11 = make_float2(X1, Y1),
                        t01 = make_float2(X0, Y1);
           const float2 b00 = make_float2(X0 - r * a00.x, Y0 - r * a00.y),
@@ -520,50 +553,18 @@ __global__ void __launch_bounds__(SEARCH_THREADS, LENS_SEARCH_MINB) k_img_search
           const float qpx = BARY_TOL * (qhx - qlx) + 1e-6f, qpy = BARY_TOL * (qhy - qly) + 1e-6f;
           bool any = false;
           for (unsigned mm = mask; mm && !any; mm &= mm - 1u) {
-            const float2 P = s_src[list[c0 + __ffs(mm) - 1]];
+            const float2 P = s_src[k0 + __ffs(mm) - 1];
             any = P.x >= qlx - qpx && P.x <= qhx + qpx && P.y >= qly - qpy && P.y <= qhy + qpy;
           }
           if (!any) continue;
           const int cell = 2 * (gj * (g.nx - 1) + gi);
-          tri_test_mask(b00, b10, b11, t00, t10, t11, s_src, list + c0, mask, tiny, cnt, hits, cell);
-          tri_test_mask(b00, b11, b01, t00, t11, t01, s_src, list + c0, mask, tiny, cnt, hits, cell + 1);
+          tri_test_mask(b00, b10, b11, t00, t10, t11, s_src + k0, s_id + k0, mask, tiny, cnt, hits, cell);
+          tri_test_mask(b00, b11, b01, t00, t11, t01, s_src + k0, s_id + k0, mask, tiny, cnt, hits, cell + 1);
         }
+        __syncwarp();
       }
-#else
-#pragma unroll
-      for (int half = 0; half < CPT; ++half) {
-        const int cj = cj0 + half * (CT_Y / CPT);
-        const int gi = i0 + ci, gj = j0 + cj;
-        if (gi >= g.nx - 1 || gj >= g.ny - 1) continue;
-        const float X0 = fmaf((float)ci, fdx, fTx), X1 = fmaf((float)(ci + 1), fdx, fTx);
-        const float Y0 = fmaf((float)cj, fdy, fTy), Y1 = fmaf((float)(cj + 1), fdy, fTy);
-        const int n00 = cj * NX_T + ci;
-        const float2 a00 = s_al[n00], a10 = s_al[n00 + 1], a01 = s_al[n00 + NX_T], a11 = s_al[n00 + NX_T + 1];
-        const float2 t00 = make_float2(X0, Y0), t10 = make_float2(X1, Y0), t11 = make_float2(X1, Y1),
-                     t01 = make_float2(X0, Y1);
-        const float2 b00 = make_float2(X0 - r * a00.x, Y0 - r * a00.y),
-                     b10 = make_float2(X1 - r * a10.x, Y0 - r * a10.y),
-                     b11 = make_float2(X1 - r * a11.x, Y1 - r * a11.y),
-                     b01 = make_float2(X0 - r * a01.x, Y1 - r * a01.y);
-        // the cell's padded bounding box contains both triangles' padded boxes
-        const float qlx = fminf(fminf(b00.x, b10.x), fminf(b11.x, b01.x)),
-                    qhx = fmaxf(fmaxf(b00.x, b10.x), fmaxf(b11.x, b01.x));
-        const float qly = fminf(fminf(b00.y, b10.y), fminf(b11.y, b01.y)),
-                    qhy = fmaxf(fmaxf(b00.y, b10.y), fmaxf(b11.y, b01.y));
-        const float qpx = BARY_TOL * (qhx - qlx) + 1e-6f, qpy = BARY_TOL * (qhy - qly) + 1e-6f;
-        bool any = false;
-        for (int k = 0; k < nlist && !any; ++k) {
-          const float2 P = s_src[list[k]];
-          any = P.x >= qlx - qpx && P.x <= qhx + qpx && P.y >= qly - qpy && P.y <= qhy + qpy;
-        }
-        if (!any) continue;
-        const int cell = 2 * (gj * (g.nx - 1) + gi);
-        tri_test(b00, b10, b11, t00, t10, t11, s_src, list, nlist, tiny, cnt, hits, cell);
-        tri_test(b00, b11, b01, t00, t11, t01, s_src, list, nlist, tiny, cnt, hits, cell + 1);
-      }
-#endif
     }
-    __syncthreads();  // s_box, s_list and s_nlist are rewritten by the next chunk
+    __syncwarp();  // the next block rewrites al
   }
 }
 
@@ -2023,6 +2024,9 @@ int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_
   g.grp_src = c->grp_src;
   g.grp_r32 = c->grp_ratio32;
   g.ng = c->ng;
+  g.plane = (const float4 *)gc->plane;
+  g.nbx = (gc->nx - 1 + BL - 1) / BL;
+  g.nby = (gc->ny - 1 + BL - 1) / BL;
   g.fdx = (float)g.dx;
   g.fdy = (float)g.dy;
   g.tiny = (float)(1e-10 * g.dx * g.dy);
@@ -2039,7 +2043,7 @@ int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_
     a.nimg = c->nimg;
     a.s = bufs(scratch, batch, c->nsrc, lists);
     k_img_sources<<<a.B, SRC_THREADS, src_smem, st>>>(a, c->stat, c->x, c->y, c->ratio, c->src_of, c->img_off);
-    dim3 sg((gc->nx - 1 + CT_X - 1) / CT_X, (gc->ny - 1 + CT_Y - 1) / CT_Y, a.B);
+    dim3 sg((g.nbx + SB_X - 1) / SB_X, (g.nby + SB_Y - 1) / SB_Y, a.B);
     k_img_search<<<sg, SEARCH_THREADS, 0, st>>>(a, g);
     if (LENS_REFINE_LISTS && lists) {
       // step 3 as point lists: the list counters, the initial triangles,
@@ -2086,9 +2090,25 @@ const GridCache *find_grid_cache(const CSet *c, const lens_grid *g) {
   return nullptr;
 }
 
+size_t grid_plane_bytes(int32_t nx, int32_t ny) {
+  return 2 * sizeof(float4) * (size_t)((nx - 1 + BL - 1) / BL) * (size_t)((ny - 1 + BL - 1) / BL);
+}
+
+int launch_grid_planes(const GridCache *gc, cudaStream_t st) {
+  const int nbx = (gc->nx - 1 + BL - 1) / BL, nby = (gc->ny - 1 + BL - 1) / BL;
+  const long long ctas = ((long long)nbx * nby + 7) / 8;
+  k_grid_planes<<<(unsigned)std::min<long long>(ctas, 1 << 20), 256, 0, st>>>(
+      gc->alpha32, gc->alpha32 + (size_t)gc->nx * gc->ny, gc->nx, gc->ny, (float)((gc->xmax - gc->xmin) / (gc->nx - 1)),
+      (float)((gc->ymax - gc->ymin) / (gc->ny - 1)), nbx, nby, (float4 *)gc->plane);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return fail(LENS_ECUDA, "search grid planes launch: %s", cudaGetErrorString(e));
+  return LENS_OK;
+}
+
 // Static deflection of the constraint set's model on grid g (LENS_MIXED map
-// of the static potentials, D_ls/D_s = 1), enqueued on st and kept with the
-// constraint set.
+// of the static potentials, D_ls/D_s = 1) and the search's block planes,
+// enqueued on st and kept with the constraint set; without room for the
+// planes the deflection alone (the search then culls nothing).
 int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st) {
   GridCache n;
   n.xmin = g->xmin;
@@ -2097,13 +2117,22 @@ int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st
   n.ymax = g->ymax;
   n.nx = g->nx;
   n.ny = g->ny;
-  n.bytes = 2 * sizeof(float) * (size_t)g->nx * g->ny;
+  const size_t alpha_bytes = (2 * sizeof(float) * (size_t)g->nx * g->ny + 255) & ~(size_t)255;
+  n.bytes = alpha_bytes + grid_plane_bytes(g->nx, g->ny);
   int rc = dev_alloc(ctx, (void **)&n.alpha32, n.bytes);
-  if (rc) return rc;
+  if (!rc) {
+    n.plane = (float *)((char *)n.alpha32 + alpha_bytes);
+  } else {
+    n.bytes = 2 * sizeof(float) * (size_t)g->nx * g->ny;
+    if ((rc = dev_alloc(ctx, (void **)&n.alpha32, n.bytes))) return rc;
+  }
   if (c->stat_model->n > 0)
     rc = launch_map_mixed(ctx, c->stat_model, g, 1.0, false, n.alpha32, st, 0, -1, false);
   else
-    rc = cudaMemsetAsync(n.alpha32, 0, n.bytes, st) == cudaSuccess ? LENS_OK : fail(LENS_ECUDA, "memset failed");
+    rc = cudaMemsetAsync(n.alpha32, 0, 2 * sizeof(float) * (size_t)g->nx * g->ny, st) == cudaSuccess
+             ? LENS_OK
+             : fail(LENS_ECUDA, "memset failed");
+  if (!rc && n.plane) rc = launch_grid_planes(&n, st);
   if (rc) {
     dev_free(ctx, n.alpha32, n.bytes);
     return rc;

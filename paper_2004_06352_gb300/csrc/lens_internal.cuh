@@ -243,6 +243,7 @@ struct GridCache {
   double xmin, xmax, ymin, ymax;
   int32_t nx, ny;
   float *alpha32 = nullptr;  // [2][ny][nx] deflection of the static potentials, D_ls/D_s = 1 (LENS_MIXED map)
+  float *plane = nullptr;    // the search's model of it per 8 x 8 cells (grid_plane_bytes; same allocation), or NULL
   size_t bytes = 0;
 };
 
@@ -460,6 +461,8 @@ constexpr size_t IMG_SRC_SMEM_MAX = 200 * 1024;
 int check_chi2_image_limits(const CSet *c, const lens_grid *g);
 const GridCache *find_grid_cache(const CSet *c, const lens_grid *g);
 int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st);
+size_t grid_plane_bytes(int32_t nx, int32_t ny);
+int launch_grid_planes(const GridCache *gc, cudaStream_t st);  // gc->alpha32 -> gc->plane
 int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_params, int32_t P,
                    double *d_chi2, int32_t *d_nfound, void *scratch, int32_t batch, cudaStream_t st,
                    double *d_images = nullptr, int32_t img_max = 0, int32_t *d_img_count = nullptr,

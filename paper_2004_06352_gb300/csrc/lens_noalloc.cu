@@ -101,6 +101,12 @@ extern "C" int lens_chi2_image_noalloc(lens_ctx *ctx, lens_cset_t cset, const le
   } else if (cudaMemsetAsync(gc.alpha32, 0, 2 * sizeof(float) * (size_t)grid->nx * grid->ny, st) != cudaSuccess) {
     return fail(LENS_ECUDA, "clearing the static deflection failed");
   }
+  // the search's block planes where there is room for them behind the rest
+  const size_t used = align256(grid_bytes + chi2_image_scratch_bytes(c, batch, lists));
+  if (used + grid_plane_bytes(grid->nx, grid->ny) <= LENS_NOALLOC_SCRATCH_BYTES) {
+    gc.plane = (float *)((char *)base + used);
+    if ((rc = launch_grid_planes(&gc, st))) return rc;
+  }
   return run_chi2_image(ctx, c, &gc, d_params, P, d_chi2, d_nimg_found, (char *)base + grid_bytes, batch, st,
                         nullptr, 0, nullptr, lists);
 }
