@@ -584,7 +584,6 @@ struct NewtonArgs {
   int nx;
   const float *gax, *gay;      // static deflection at the grid nodes [ny][nx] (D_ls/D_s = 1)
   int *err;                    // the context's error word
-  int nsm;                     // SMs
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -1064,24 +1063,22 @@ __device__ __forceinline__ void entry_point(const Bufs &s, int e, double &X, dou
   }
 }
 
-// SPLIT: S groups of PE_THREADS / S threads share the CTA's points, each group
-// takes every S-th static potential, and group k (mod S) finishes the threads'
-// points k.
-template <bool HESS, bool SPLIT>
-__device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, const int *__restrict__ lst, int npts,
-                                         int splits, float (*s_rec)[PE_CH * REC32], float4 (*s_cen)[PE_CH],
-                                         uint64_t *s_bar,
-                                         double (*s_hv)[HESS ? 2 : 4][HESS ? 5 : 2]) {
+template <bool HESS>
+__global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE_MINB_GRAD)
+    k_pts_eval(const SetArgs a, const NewtonArgs n, const int *__restrict__ lst, const int *__restrict__ count) {
   constexpr int KP = HESS ? 2 : 4, NP = KP / 2, NC = HESS ? 5 : 2;
-  const int S = SPLIT ? splits : 1, group = PE_THREADS / S, p0 = blockIdx.x * (pe_points(HESS) / S);
+  __shared__ __align__(128) float s_rec[2][PE_CH * REC32];
+  __shared__ __align__(16) float4 s_cen[2][PE_CH];
+  __shared__ __align__(8) uint64_t s_bar[2];
+  __shared__ double s_hv[PE_THREADS][KP][NC];
+  const int npts = *count, p0 = blockIdx.x * pe_points(HESS);
   if (p0 >= npts) return;  // uniform over the CTA
-  const int tid = threadIdx.x, grp = SPLIT ? tid / group : 0, t = SPLIT ? tid % group : tid;
-  auto mine = [&](int k) { return !SPLIT || k % S == grp; };
+  const int tid = threadIdx.x;
   int ent[KP];
   bool live[KP];
 #pragma unroll
   for (int k = 0; k < KP; ++k) {
-    const int p = p0 + k * group + t;
+    const int p = p0 + k * PE_THREADS + tid;
     live[k] = p < npts;
     ent[k] = lst[live[k] ? p : p0];  // past the end: the tile's first point again, not stored
   }
@@ -1116,7 +1113,6 @@ __device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, 
   auto heavy_pass = [&]() {
 #pragma unroll
     for (int k = 0; k < KP; ++k) {
-      if (!mine(k)) continue;
       double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
       double X, Y;
       entry_point(a.s, ent[k], X, Y);
@@ -1166,13 +1162,11 @@ __device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, 
     const float4 *cens = &s_cen[buf][0];
     auto run = [&](auto kind_tag, int h0, int h1) {
       constexpr int KIND = decltype(kind_tag)::value;
-      for (int hb = h0; hb < h1;) {
-        const int he = min(hb + (PE_SUB - seen) * S, h1);
-        seen += SPLIT ? (he - hb + S - 1) / S : he - hb;
+      for (int h = h0; h < h1;) {
+        const int he = min(h + (PE_SUB - seen), h1);
+        seen += he - h;
 #pragma unroll 2
-        for (; hb < he; hb += S) {
-          const int h = hb + grp;
-          if (SPLIT && h >= he) continue;
+        for (; h < he; ++h) {
           const float4 *r4 = recs + h * (REC32 / 4);
           const float4 c = cens[h];
           float2 dX[NP], dY[NP];
@@ -1210,27 +1204,12 @@ __device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, 
   }
   fold2(tot, cmp, part);
   if (!heavy_first) heavy_pass();
-  // SPLIT: the groups' sums, in FP64, into the records' space
-  double *s_sum = reinterpret_cast<double *>(&s_rec[0][0]);  // [S][group][KP][NC]
-  static_assert(sizeof(double) * PE_THREADS * KP * NC <= sizeof(float) * 2 * PE_CH * REC32, "fits the records' space");
-  if (SPLIT) {
-    __syncthreads();  // the last chunk has been used
-    const float2 *tt[5] = {tot.ax, tot.ay, tot.k, tot.g1, tot.g2};
-    const float2 *cc[5] = {cmp.ax, cmp.ay, cmp.k, cmp.g1, cmp.g2};
-#pragma unroll
-    for (int k = 0; k < KP; ++k)
-#pragma unroll
-      for (int c = 0; c < NC; ++c)
-        s_sum[(tid * KP + k) * NC + c] = (double)part2(tt[c][k >> 1], k & 1) - (double)part2(cc[c][k >> 1], k & 1);
-    __syncthreads();
-  }
 
   // the two varying potentials of each point's parameter set: FP32 in the
   // subdivision (as k_img_newton's sweeps), double-float with FP64 fallback
   // in the Newton steps
 #pragma unroll
   for (int k = 0; k < KP; ++k) {
-    if (!mine(k)) continue;
     const int slot = ent[k] >> 2;
     const VarRecs &var = a.s.var[slot / IMG_CAP];
     double Xk, Yk;
@@ -1240,11 +1219,6 @@ __device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, 
     for (int c = 0; c < 5; ++c) o[c] = c < NC ? s_hv[tid][k][c] : 0.0;
     const float2 *tt[5] = {tot.ax, tot.ay, tot.k, tot.g1, tot.g2};
     const float2 *cc[5] = {cmp.ax, cmp.ay, cmp.k, cmp.g1, cmp.g2};
-    if (SPLIT) {
-      for (int q = 0; q < S; ++q)
-#pragma unroll
-        for (int c = 0; c < NC; ++c) o[c] += s_sum[((q * group + t) * KP + k) * NC + c];
-    } else
 #pragma unroll
     for (int c = 0; c < NC; ++c) o[c] += (double)part2(tt[c][k >> 1], k & 1) - (double)part2(cc[c][k >> 1], k & 1);
     if (!HESS) {
@@ -1294,29 +1268,6 @@ __device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, 
       r.mo[2 * m + 1] = o[1];
     }
   }
-}
-
-// S: doubled while that still leaves the chip room for the CTAs (PE_FILL per
-// SM), so that a short list (few parameter sets, a late Newton round) is not a
-// handful of CTAs each sweeping every potential.  Image-plane chi2, 1000
-// potentials, 1024^2 grid, without / with: 1 set 1678 / 664 us, 4 sets 1830 /
-// 770, 16 sets 2187 / 1235, 100 sets 4274 / 3907, 256 sets 8255 / 8078; 150
-// potentials, 16 sets 621 / 504.
-constexpr int PE_SPLITS = 16, PE_FILL = 4;
-template <bool HESS>
-__global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE_MINB_GRAD)
-    k_pts_eval(const SetArgs a, const NewtonArgs n, const int *__restrict__ lst, const int *__restrict__ count) {
-  __shared__ __align__(128) float s_rec[2][PE_CH * REC32];
-  __shared__ __align__(16) float4 s_cen[2][PE_CH];
-  __shared__ __align__(8) uint64_t s_bar[2];
-  __shared__ double s_hv[PE_THREADS][HESS ? 2 : 4][HESS ? 5 : 2];
-  const int npts = *count, ctas = min((int)gridDim.x, PE_FILL * n.nsm);
-  int S = 1;
-  while (S < PE_SPLITS && (npts + pe_points(HESS) / (2 * S) - 1) / (pe_points(HESS) / (2 * S)) <= ctas) S *= 2;
-  if (S == 1)
-    pts_eval<HESS, false>(a, n, lst, npts, 1, s_rec, s_cen, s_bar, s_hv);
-  else
-    pts_eval<HESS, true>(a, n, lst, npts, S, s_rec, s_cen, s_bar, s_hv);
 }
 
 // The source position, ratio and grid spacing a candidate's decisions use.
@@ -2060,7 +2011,6 @@ int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_
   n.gax = gc->alpha32;
   n.gay = gc->alpha32 + (size_t)gc->nx * gc->ny;
   n.err = ctx->d_err;
-  n.nsm = nsm;
   SearchArgs g;
   g.ax = gc->alpha32;
   g.ay = gc->alpha32 + (size_t)gc->nx * gc->ny;
@@ -2104,8 +2054,8 @@ int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_
         return fail(LENS_ECUDA, "cudaMemsetAsync failed");
       k_ref_init<<<dim3((IMG_CAP + RL_THREADS - 1) / RL_THREADS, a.B), RL_THREADS, 0, st>>>(a, n);
       const size_t N = (size_t)a.B * IMG_CAP;
-      const unsigned gsub = std::max((unsigned)((3 * N + pe_points(false) - 1) / pe_points(false)), (unsigned)(PE_FILL * nsm));
-      const unsigned gnew = std::max((unsigned)((N + pe_points(true) - 1) / pe_points(true)), (unsigned)(PE_FILL * nsm));
+      const unsigned gsub = (unsigned)((3 * N + pe_points(false) - 1) / pe_points(false));
+      const unsigned gnew = (unsigned)((N + pe_points(true) - 1) / pe_points(true));
       for (int lev = 0; lev < SUBDIV_LEVELS; ++lev) {
         k_pts_eval<false><<<gsub, PE_THREADS, 0, st>>>(a, n, a.s.lst + ((lev & 1) ? 3 * N : 0), a.s.lcnt + lev);
         k_ref_level<<<4 * nsm, RL_THREADS, 0, st>>>(a, n, lev);
