@@ -1007,7 +1007,7 @@ int far_words(const Model *m) { return (m->n_light + 31) / 32 + (m->n_heavy + 31
 // one with each coarse level, in evaluations of one FP32 potential (HV of
 // them for a cluster-scale potential in double-float), idle SMs of small
 // grids included.
-FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode, bool coarse_level) {
+FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode) {
   FarPlan p;
   if (m->n > FAR_MAX_N || m->n < 1) return p;
   const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
@@ -1025,7 +1025,7 @@ FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mo
     const double Rf = std::sqrt(2.0) * 0.5 * (ft - 1) * step;
     const double near = light(KF * Rf) + HV * heavy(KF_H * Rf);
     for (int ct = 0; ct <= CT_MAX; ct = ct ? 2 * ct : 2 * ft) {
-      if (ct && (!coarse_level || ct >= 2 * std::max(g->nx, g->ny))) break;
+      if (ct && ct >= 2 * std::max(g->nx, g->ny)) break;
       double mid = m->n_light, mid_h = m->n_heavy, coarse = 0.0;
       if (ct) {
         const double Rc = std::sqrt(2.0) * 0.5 * ct * step;

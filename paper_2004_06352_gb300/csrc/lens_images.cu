@@ -2094,23 +2094,7 @@ size_t grid_plane_bytes(int32_t nx, int32_t ny) {
   return 2 * sizeof(float4) * (size_t)((nx - 1 + BL - 1) / BL) * (size_t)((ny - 1 + BL - 1) / BL);
 }
 
-// Static deflection of the constraint set's model on the grid (LENS_MIXED map
-// of the static potentials without repair, D_ls/D_s = 1) and, where the cache
-// has them, the search's block planes.  Interpolated far potentials without a
-// coarse level: no memory beyond the cache, so that every caller gets the same
-// values (1000-potential model on 1024^2: first call of 256 sets 9.99 -> 8.76
-// ms against the direct kernel, allocation-free call of 12 sets 5.81 -> 4.49).
-int launch_grid_cache(lens_ctx *ctx, const CSet *c, const GridCache *gc, cudaStream_t st) {
-  const lens_grid g = {gc->xmin, gc->xmax, gc->ymin, gc->ymax, gc->nx, gc->ny};
-  if (c->stat_model->n > 0) {
-    const FarPlan plan = plan_far(ctx, c->stat_model, &g, 0, false);
-    const int rc = launch_map_mixed(ctx, c->stat_model, &g, 1.0, false, gc->alpha32, st, 0, -1, false, nullptr,
-                                    plan.use ? &plan : nullptr);
-    if (rc) return rc;
-  } else if (cudaMemsetAsync(gc->alpha32, 0, 2 * sizeof(float) * (size_t)gc->nx * gc->ny, st) != cudaSuccess) {
-    return fail(LENS_ECUDA, "clearing the static deflection failed");
-  }
-  if (!gc->plane) return LENS_OK;
+int launch_grid_planes(const GridCache *gc, cudaStream_t st) {
   const int nbx = (gc->nx - 1 + BL - 1) / BL, nby = (gc->ny - 1 + BL - 1) / BL;
   const long long ctas = ((long long)nbx * nby + 7) / 8;
   k_grid_planes<<<(unsigned)std::min<long long>(ctas, 1 << 20), 256, 0, st>>>(
@@ -2121,9 +2105,10 @@ int launch_grid_cache(lens_ctx *ctx, const CSet *c, const GridCache *gc, cudaStr
   return LENS_OK;
 }
 
-// Static deflection and block planes of grid g, enqueued on st and kept with
-// the constraint set; without room for the planes the deflection alone (the
-// search then leaves nothing out).
+// Static deflection of the constraint set's model on grid g (LENS_MIXED map
+// of the static potentials, D_ls/D_s = 1) and the search's block planes,
+// enqueued on st and kept with the constraint set; without room for the
+// planes the deflection alone (the search then culls nothing).
 int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st) {
   GridCache n;
   n.xmin = g->xmin;
@@ -2141,7 +2126,13 @@ int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st
     n.bytes = 2 * sizeof(float) * (size_t)g->nx * g->ny;
     if ((rc = dev_alloc(ctx, (void **)&n.alpha32, n.bytes))) return rc;
   }
-  rc = launch_grid_cache(ctx, c, &n, st);
+  if (c->stat_model->n > 0)
+    rc = launch_map_mixed(ctx, c->stat_model, g, 1.0, false, n.alpha32, st, 0, -1, false);
+  else
+    rc = cudaMemsetAsync(n.alpha32, 0, 2 * sizeof(float) * (size_t)g->nx * g->ny, st) == cudaSuccess
+             ? LENS_OK
+             : fail(LENS_ECUDA, "memset failed");
+  if (!rc && n.plane) rc = launch_grid_planes(&n, st);
   if (rc) {
     dev_free(ctx, n.alpha32, n.bytes);
     return rc;

@@ -411,8 +411,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
                      const FarPlan *far = nullptr, void *far_mem = nullptr, void *dense_mem = nullptr);
 // modes of the interpolated maps: 0 deflection, 1 deflection + Hessian, 2 potential
 // (rows of a band must be a multiple of the plan's fine tile)
-// coarse_level = false: a plan that needs no memory (without repair)
-FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode, bool coarse_level = true);
+FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode);
 int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st);
 int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, double dls, void *out,
                    int row0, int rows, double repair, int *rep_count, int *rep_list, const DenseRepair &dense,
@@ -463,7 +462,7 @@ int check_chi2_image_limits(const CSet *c, const lens_grid *g);
 const GridCache *find_grid_cache(const CSet *c, const lens_grid *g);
 int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st);
 size_t grid_plane_bytes(int32_t nx, int32_t ny);
-int launch_grid_cache(lens_ctx *ctx, const CSet *c, const GridCache *gc, cudaStream_t st);  // fills alpha32 and plane
+int launch_grid_planes(const GridCache *gc, cudaStream_t st);  // gc->alpha32 -> gc->plane
 int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_params, int32_t P,
                    double *d_chi2, int32_t *d_nfound, void *scratch, int32_t batch, cudaStream_t st,
                    double *d_images = nullptr, int32_t img_max = 0, int32_t *d_img_count = nullptr,

@@ -96,11 +96,17 @@ extern "C" int lens_chi2_image_noalloc(lens_ctx *ctx, lens_cset_t cset, const le
   gc.ny = grid->ny;
   gc.alpha32 = (float *)base;
   gc.bytes = grid_bytes;
+  if (c->stat_model->n > 0) {
+    if ((rc = launch_map_mixed(ctx, c->stat_model, grid, 1.0, false, gc.alpha32, st, 0, -1, false))) return rc;
+  } else if (cudaMemsetAsync(gc.alpha32, 0, 2 * sizeof(float) * (size_t)grid->nx * grid->ny, st) != cudaSuccess) {
+    return fail(LENS_ECUDA, "clearing the static deflection failed");
+  }
   // the search's block planes where there is room for them behind the rest
   const size_t used = align256(grid_bytes + chi2_image_scratch_bytes(c, batch, lists));
-  if (used + grid_plane_bytes(grid->nx, grid->ny) <= LENS_NOALLOC_SCRATCH_BYTES)
+  if (used + grid_plane_bytes(grid->nx, grid->ny) <= LENS_NOALLOC_SCRATCH_BYTES) {
     gc.plane = (float *)((char *)base + used);
-  if ((rc = launch_grid_cache(ctx, c, &gc, st))) return rc;
+    if ((rc = launch_grid_planes(&gc, st))) return rc;
+  }
   return run_chi2_image(ctx, c, &gc, d_params, P, d_chi2, d_nimg_found, (char *)base + grid_bytes, batch, st,
                         nullptr, 0, nullptr, lists);
 }
