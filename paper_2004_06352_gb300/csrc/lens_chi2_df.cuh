@@ -1,5 +1,5 @@
-// The double-float evaluator of the source-plane chi2: dPIE, SIS and point
-// mass at one image, or at two images side by side.
+// The double-float evaluator of the source-plane chi2 and of the image search's
+// Newton steps: dPIE, SIS and point mass at one image, or at two side by side.
 //
 // Its roundings are fixed.  A set with an image next to a critical curve
 // divides by det ~ 1e-5 and smaller, which turns an evaluator's last bits
@@ -8,6 +8,8 @@
 // every shortcut below gives the same bits: FastTwoSum where the larger
 // operand is known, differences that are exact by Sterbenz' lemma, sums with
 // an exact zero left out, constants of a record formed once per record.
+// Newton started next to a fold wanders, so that there too the last bits decide
+// whether a borderline image is found (1 of 10^5 images).
 // (lens_device.cuh's dpie_df takes 40 % fewer operations, with other bits.)
 //
 // F is float (one image) or float2 (two: the paired FP32 instructions round
@@ -244,10 +246,11 @@ __device__ __forceinline__ void record_consts(float2 *r) {
   if (u.hi > 0.f) put(F_BU, d_div(D(F_BQ), u));  // (never used for a circular one)
 }
 
-// One dPIE potential (record r after record_consts<UW>, shared by the images):
+// One dPIE potential (record r after record_consts<UW>, or as it is (RAW, with
+// UW = false); shared by the images):
 // deflection and, if HESS, kappa, gamma1, gamma2 into h[0..2].  Returns the
 // components whose result is finite.
-template <bool HESS, bool UW, class F>
+template <bool HESS, bool UW, class F, bool RAW = false>
 __device__ __forceinline__ unsigned dpie_fixed(const float2 *__restrict__ r, Df<F> X, Df<F> Y, Df<F> &ax, Df<F> &ay,
                                                Df<F> *h) {
   auto ld = [&](int k) {
@@ -262,7 +265,8 @@ __device__ __forceinline__ unsigned dpie_fixed(const float2 *__restrict__ r, Df<
   const Df<F> psc = d_sqrt(d_ss(R, ld(F_KC))), pst = d_sqrt(d_ss(R, ld(F_KT)));
   const Df<F> Sp = d_ss_big(pst, psc);
   const Df<F> sc = ld(F_SC), st = ld(F_ST);
-  const Df<F> numx = d_mul(d_mul(x, ld(F_DS)), d_ss(Sp, ld(F_Q2SS)));
+  const Df<F> dS = RAW ? d_ss(st, d_neg(sc)) : ld(F_DS);
+  const Df<F> numx = d_mul(d_mul(x, dS), d_ss(Sp, ld(F_Q2SS)));
   const Df<F> denx = d_mul(Sp, d_ss(d_mul(d_ss(psc, sc), d_ss(pst, st)), d_mul(u2, x2)));
   const Df<F> Zx = d_div(numx, denx);
   const Df<F> numy = d_mul(d_mul(y, ld(F_Q2DS)), d_ss(Sp, ld(F_SS)));
@@ -303,7 +307,7 @@ __device__ __forceinline__ unsigned dpie_fixed(const float2 *__restrict__ r, Df<
     const Df<F> fc = d_div(one, d_mul(psc, Dc)), ft = d_div(one, d_mul(pst, Dt));
     const Df<F> g1p = d_mul(ld(F_HB), d_sub(d_mul(fc, d_sub(ymx, ld(F_U2SC2))), d_mul(ft, d_sub(ymx, ld(F_U2ST2)))));
     const Df<F> g2p = d_neg(d_mul(d_mul(bq, d_sub(fc, ft)), d_mul(x, y)));
-    h[0] = d_div(ld(F_KTC), d_mul(d_mul(Sp, psc), pst));
+    h[0] = d_div(RAW ? d_mul(ld(F_HB), ld(F_KTC)) : ld(F_KTC), d_mul(d_mul(Sp, psc), pst));
     const Df<F> c2 = ld(F_C2), s2 = ld(F_S2);
     h[1] = d_sub(d_mul(c2, g1p), d_mul(s2, g2p));
     h[2] = d_add(d_mul(s2, g1p), d_mul(c2, g2p));
@@ -333,14 +337,14 @@ __device__ __noinline__ void circ_fixed(float2 x0, float2 y0, float2 bb, bool po
 }
 
 // Any potential: the components whose result holds (the others take FP64).
-template <bool HESS, bool UW, class F>
+template <bool HESS, bool UW, class F, bool RAW = false>
 __device__ __forceinline__ unsigned any_fixed(const float2 *__restrict__ r, Df<F> X, Df<F> Y, Df<F> &ax, Df<F> &ay,
                                               Df<F> *h) {
   if (r[F_U2].x < 0.f) {
     circ_fixed<HESS>(r[F_X0], r[F_Y0], r[F_BQ], r[F_U2].x < -1.5f, X, Y, ax, ay, h);
     return f_all<F>;
   }
-  return dpie_fixed<HESS, UW>(r, X, Y, ax, ay, h);
+  return dpie_fixed<HESS, UW, F, RAW>(r, X, Y, ax, ay, h);
 }
 
 }  // namespace lens

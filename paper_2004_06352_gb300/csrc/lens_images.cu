@@ -39,7 +39,7 @@
 // makes that set's chi2 NaN and sets ERRBIT_CAPACITY.
 #include <type_traits>
 
-#include "lens_device.cuh"
+#include "lens_chi2_df.cuh"
 
 namespace lens {
 namespace {
@@ -188,6 +188,84 @@ struct SetArgs {  // what every kernel needs to know about the batch
 };
 
 // ---------------------------------------------------------------- 1. sources
+// A potential in double-float with the fixed roundings of lens_chi2_df.cuh
+// (false: not finite, FP64 then), and added to acc[0..4] as doubles.
+template <bool HESS>
+__device__ __forceinline__ bool potential_fixed(const float2 *__restrict__ rec, df X, df Y, df &ax, df &ay, df *h) {
+  Df<float> t[5] = {};
+  const unsigned ok =
+      any_fixed<HESS, false, float, true>(rec, Df<float>{X.hi, X.lo}, Df<float>{Y.hi, Y.lo}, t[0], t[1], t + 2);
+  ax = df{t[0].hi, t[0].lo};
+  ay = df{t[1].hi, t[1].lo};
+#pragma unroll
+  for (int q = 0; q < 3; ++q) h[q] = df{t[2 + q].hi, t[2 + q].lo};
+  return ok != 0u;
+}
+template <bool HESS>
+__device__ __forceinline__ void add_potential_fixed(const float2 *__restrict__ rec, const double *__restrict__ r64,
+                                                    double X, double Y, double *acc) {
+  df a[5];
+  double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+  if (potential_fixed<HESS>(rec, df_from_double(X), df_from_double(Y), a[0], a[1], a + 2)) {
+#pragma unroll
+    for (int q = 0; q < (HESS ? 5 : 2); ++q) e[q] = df_to_double(a[q]);
+  } else {
+    eval64_cold<HESS>(r64, X, Y, e);
+  }
+#pragma unroll
+  for (int q = 0; q < (HESS ? 5 : 2); ++q) acc[q] += e[q];
+}
+
+// Back-trace every constraint of one parameter set (Sec. 2.1 Eq. 1):
+// beta_j = theta_j - r alpha(theta_j), alpha = static cache + the two varying
+// potentials in double-float (FP64 where that fails), then each source's
+// barycentre (Sec. 2.2, Fig. 3).  Fills s_beta [nimg][2] and s_bary [nsrc][2].
+// Called by all THREADS threads of the CTA; ends synchronised.
+template <int THREADS>
+__device__ __forceinline__ void backtrace_set(const double *__restrict__ stat, const double *__restrict__ x,
+                                              const double *__restrict__ y, const double *__restrict__ ratio,
+                                              const int32_t *__restrict__ src_of, const int32_t *__restrict__ img_off,
+                                              int nimg, int nsrc, const double *s_rec, const float2 *s_rdf,
+                                              double *s_beta, double *s_bary) {
+  for (int j = threadIdx.x; j < nimg; j += THREADS) {
+    const double X = x[j], Y = y[j];
+    const df Xd = df_from_double(X), Yd = df_from_double(Y);
+    double ax = stat[(size_t)j * 5], ay = stat[(size_t)j * 5 + 1];
+    Df<float> sx = {0.f, 0.f}, sy = {0.f, 0.f};
+#pragma unroll 1
+    for (int v = 0; v < 2; ++v) {
+      df vx, vy, h[3];
+      if (potential_fixed<false>(s_rdf + v * RECDF, Xd, Yd, vx, vy, h)) {
+        sx = d_add(sx, Df<float>{vx.hi, vx.lo});
+        sy = d_add(sy, Df<float>{vy.hi, vy.lo});
+      } else {
+        double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        eval64_cold<false>(s_rec + v * REC64, X, Y, e);
+        ax += e[0];
+        ay += e[1];
+      }
+    }
+    ax += df_to_double(df{sx.hi, sx.lo});
+    ay += df_to_double(df{sy.hi, sy.lo});
+    const double r = ratio[src_of[j]];
+    s_beta[2 * j] = X - r * ax;
+    s_beta[2 * j + 1] = Y - r * ay;
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < nsrc; i += THREADS) {
+    const int b = img_off[i], e = img_off[i + 1];
+    double sx = 0, sy = 0;
+    for (int j = b; j < e; ++j) {
+      sx += s_beta[2 * j];
+      sy += s_beta[2 * j + 1];
+    }
+    const double im = e > b ? 1.0 / (e - b) : 0.0;
+    s_bary[2 * i] = sx * im;
+    s_bary[2 * i + 1] = sy * im;
+  }
+  __syncthreads();
+}
+
 constexpr int SRC_THREADS = 128;
 
 __global__ void __launch_bounds__(SRC_THREADS) k_img_sources(const SetArgs a, const double *__restrict__ stat,
@@ -227,7 +305,7 @@ __global__ void __launch_bounds__(SRC_THREADS) k_img_sources(const SetArgs a, co
   }
   if (!s_ok) return;
   backtrace_set<SRC_THREADS>(stat, x, y, ratio, src_of, img_off, a.nimg, a.nsrc, s_rec, &a.s.var[b].rdf[0][0], s_beta,
-                             nullptr, s_bary);
+                             s_bary);
   for (int i = threadIdx.x; i < 2 * a.nsrc; i += SRC_THREADS) a.s.bary[(size_t)b * a.nsrc * 2 + i] = s_bary[i];
   for (int i = threadIdx.x; i < a.nsrc; i += SRC_THREADS)
     a.s.src32[(size_t)b * a.nsrc + i] = make_float2((float)s_bary[2 * i], (float)s_bary[2 * i + 1]);
@@ -827,10 +905,7 @@ __device__ __forceinline__ void sweep(const NewtonArgs &n, const VarRecs &var, f
         const df X = df_from_double(px[k]), Y = df_from_double(py[k]);
         df ax, ay, h[3];
         bool ok = true;
-        if (rec[F_U2].x < 0.f)
-          circ_df<true>(rec, 1, X, Y, ax, ay, h);
-        else
-          ok = dpie_df<true, true>(rec, 1, X, Y, ax, ay, h);
+        ok = potential_fixed<true>(rec, X, Y, ax, ay, h);
         if (!ok) {
           double e[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
           eval64<true>(var.r64[gl], px[k], py[k], e[0], e[1], e[2], e[3], e[4]);
@@ -1117,7 +1192,7 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
       double X, Y;
       entry_point(a.s, ent[k], X, Y);
       for (int j = 0; j < n.n_heavy; ++j)
-        add_potential_df<HESS>(n.heavydf + (size_t)j * RECDF, 1, n.heavy + (size_t)j * REC64, X, Y, v);
+        add_potential_fixed<HESS>(n.heavydf + (size_t)j * RECDF, n.heavy + (size_t)j * REC64, X, Y, v);
 #pragma unroll
       for (int c = 0; c < NC; ++c) s_hv[tid][k][c] = v[c];
     }
@@ -1239,10 +1314,7 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
         const float2 *rec = var.rdf[v];
         df ax, ay, hh[3];
         bool okv = true;
-        if (rec[F_U2].x < 0.f)
-          circ_df<true>(rec, 1, Xd, Yd, ax, ay, hh);
-        else
-          okv = dpie_df<true, true>(rec, 1, Xd, Yd, ax, ay, hh);
+        okv = potential_fixed<true>(rec, Xd, Yd, ax, ay, hh);
         if (okv) {
           o[0] += df_to_double(ax);
           o[1] += df_to_double(ay);
@@ -1647,7 +1719,7 @@ __global__ void __launch_bounds__(RS_THREADS) k_ref_straggle(const SetArgs a, co
           v[q] = df_to_double(t);
         }
         for (int j = 0; j < n.n_heavy; ++j)  // static cluster-scale potentials (double-float)
-          add_potential_df<true>(n.heavydf + (size_t)j * RECDF, 1, n.heavy + (size_t)j * REC64, X, Y, v);
+          add_potential_fixed<true>(n.heavydf + (size_t)j * RECDF, n.heavy + (size_t)j * REC64, X, Y, v);
         const bool more = newton_step(a, slot, c, v, tx, ty, nit, settled);
         s_pos[g][0] = tx;
         s_pos[g][1] = ty;
