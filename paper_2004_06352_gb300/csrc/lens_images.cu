@@ -662,6 +662,7 @@ struct NewtonArgs {
   int nx;
   const float *gax, *gay;      // static deflection at the grid nodes [ny][nx] (D_ls/D_s = 1)
   int *err;                    // the context's error word
+  int nsm;                     // SMs
 };
 
 __device__ __forceinline__ double warp_sum(double v) {
@@ -1138,22 +1139,39 @@ __device__ __forceinline__ void entry_point(const Bufs &s, int e, double &X, dou
   }
 }
 
+// Shared memory of a CTA of k_pts_eval; part: SPLIT's sums of a chunk's
+// PE_SUB-blocks, per point.
 template <bool HESS>
-__global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE_MINB_GRAD)
-    k_pts_eval(const SetArgs a, const NewtonArgs n, const int *__restrict__ lst, const int *__restrict__ count) {
+struct PtsShared {
+  static constexpr int KP = HESS ? 2 : 4, NC = HESS ? 5 : 2;
+  __align__(128) float rec[2][PE_CH * REC32];
+  __align__(16) float4 cen[2][PE_CH];
+  __align__(8) uint64_t bar[2];
+  double hv[PE_THREADS][KP][NC];
+  float part[PE_CH / PE_SUB][PE_THREADS / 2 * KP][NC];
+};
+// SPLIT: S groups of PE_THREADS / S threads share the CTA's points; of each
+// chunk a group evaluates every S-th block of PE_SUB potentials, and group k
+// (mod S) folds the blocks' sums of the threads' points k in the potentials'
+// order and finishes those points.  The sums are the same to the last bit as
+// with one group (borderline images depend on them).
+template <bool HESS, bool SPLIT>
+__device__ __forceinline__ void pts_eval(const SetArgs &a, const NewtonArgs &n, const int *__restrict__ lst, int npts,
+                                         int splits, PtsShared<HESS> &sh) {
   constexpr int KP = HESS ? 2 : 4, NP = KP / 2, NC = HESS ? 5 : 2;
-  __shared__ __align__(128) float s_rec[2][PE_CH * REC32];
-  __shared__ __align__(16) float4 s_cen[2][PE_CH];
-  __shared__ __align__(8) uint64_t s_bar[2];
-  __shared__ double s_hv[PE_THREADS][KP][NC];
-  const int npts = *count, p0 = blockIdx.x * pe_points(HESS);
+  auto &s_rec = sh.rec;
+  auto &s_cen = sh.cen;
+  auto &s_bar = sh.bar;
+  auto &s_hv = sh.hv;
+  const int S = SPLIT ? splits : 1, group = PE_THREADS / S, p0 = blockIdx.x * (pe_points(HESS) / S);
   if (p0 >= npts) return;  // uniform over the CTA
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, grp = SPLIT ? tid / group : 0, t = SPLIT ? tid % group : tid;
+  auto mine = [&](int k) { return !SPLIT || k % S == grp; };
   int ent[KP];
   bool live[KP];
 #pragma unroll
   for (int k = 0; k < KP; ++k) {
-    const int p = p0 + k * PE_THREADS + tid;
+    const int p = p0 + k * group + t;
     live[k] = p < npts;
     ent[k] = lst[live[k] ? p : p0];  // past the end: the tile's first point again, not stored
   }
@@ -1188,6 +1206,7 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
   auto heavy_pass = [&]() {
 #pragma unroll
     for (int k = 0; k < KP; ++k) {
+      if (!mine(k)) continue;
       double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
       double X, Y;
       entry_point(a.s, ent[k], X, Y);
@@ -1201,9 +1220,15 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
   if (heavy_first) heavy_pass();
 
   Acc2<HESS, NP> tot, cmp, part;
-  tot.zero();
-  cmp.zero();
+  if (!SPLIT) tot.zero();
+  if (!SPLIT) cmp.zero();
   part.zero();
+  float ptot[KP][NC], pcmp[KP][NC], prem[KP][NC];  // SPLIT: the same per point, and the last block's sums
+  if (SPLIT)
+#pragma unroll
+    for (int k = 0; k < KP; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) ptot[k][c] = pcmp[k][c] = prem[k][c] = 0.f;
   const int nl = n.n_light, nch = (nl + PE_CH - 1) / PE_CH;
   if (tid == 0) {
     mbar_init(&s_bar[0], 1);
@@ -1238,7 +1263,7 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
     auto run = [&](auto kind_tag, int h0, int h1) {
       constexpr int KIND = decltype(kind_tag)::value;
       for (int h = h0; h < h1;) {
-        const int he = min(h + (PE_SUB - seen), h1);
+        const int he = SPLIT ? h1 : min(h + (PE_SUB - seen), h1);
         seen += he - h;
 #pragma unroll 2
         for (; h < he; ++h) {
@@ -1257,7 +1282,7 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
           else
             circ32x2<HESS, NP, KIND == K32_POINT, false>(r4, dX, dY, part);
         }
-        if (seen == PE_SUB) {
+        if (!SPLIT && seen == PE_SUB) {
           fold2(tot, cmp, part);
           seen = 0;
         }
@@ -1267,17 +1292,55 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
       h0 = max(n.koff[k] - base, 0);
       h1 = min(n.koff[k + 1] - base, cnt);
     };
-    int h0, h1;
-    seg(K32_DPIE, h0, h1);
-    if (h0 < h1) run(std::integral_constant<int, K32_DPIE>(), h0, h1);
-    seg(K32_DPIE_SERIES, h0, h1);
-    if (h0 < h1) run(std::integral_constant<int, K32_DPIE_SERIES>(), h0, h1);
-    seg(K32_SIS, h0, h1);
-    if (h0 < h1) run(std::integral_constant<int, K32_SIS>(), h0, h1);
-    seg(K32_POINT, h0, h1);
-    if (h0 < h1) run(std::integral_constant<int, K32_POINT>(), h0, h1);
+    // the chunk's potentials from b0 to b1 - 1, kind by kind
+    auto block = [&](int b0, int b1) {
+      int h0, h1;
+      auto kind = [&](auto kind_tag) {
+        seg(decltype(kind_tag)::value, h0, h1);
+        h0 = max(h0, b0);
+        h1 = min(h1, b1);
+        if (h0 < h1) run(kind_tag, h0, h1);
+      };
+      kind(std::integral_constant<int, K32_DPIE>());
+      kind(std::integral_constant<int, K32_DPIE_SERIES>());
+      kind(std::integral_constant<int, K32_SIS>());
+      kind(std::integral_constant<int, K32_POINT>());
+    };
+    if (!SPLIT) {
+      block(0, cnt);
+    } else {
+#pragma unroll 1
+      for (int q = grp; q * PE_SUB < cnt; q += S) {
+        part.zero();
+        block(q * PE_SUB, min(cnt, (q + 1) * PE_SUB));
+        const float2 *pp[5] = {part.ax, part.ay, part.k, part.g1, part.g2};
+#pragma unroll
+        for (int k = 0; k < KP; ++k)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) sh.part[q][k * group + t][c] = part2(pp[c][k >> 1], k & 1);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int k = 0; k < KP; ++k) {
+        if (!mine(k)) continue;
+        for (int q = 0; q * PE_SUB < cnt; ++q)
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            const float v = sh.part[q][k * group + t][c];
+            if ((q + 1) * PE_SUB <= cnt)
+              kahan(ptot[k][c], pcmp[k][c], v);
+            else
+              prem[k][c] = v;
+          }
+      }
+    }
   }
-  fold2(tot, cmp, part);
+  if (!SPLIT) fold2(tot, cmp, part);
+  if (SPLIT)
+#pragma unroll
+    for (int k = 0; k < KP; ++k)
+#pragma unroll
+      for (int c = 0; c < NC; ++c) kahan(ptot[k][c], pcmp[k][c], prem[k][c]);
   if (!heavy_first) heavy_pass();
 
   // the two varying potentials of each point's parameter set: FP32 in the
@@ -1285,6 +1348,7 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
   // in the Newton steps
 #pragma unroll
   for (int k = 0; k < KP; ++k) {
+    if (!mine(k)) continue;
     const int slot = ent[k] >> 2;
     const VarRecs &var = a.s.var[slot / IMG_CAP];
     double Xk, Yk;
@@ -1295,7 +1359,9 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
     const float2 *tt[5] = {tot.ax, tot.ay, tot.k, tot.g1, tot.g2};
     const float2 *cc[5] = {cmp.ax, cmp.ay, cmp.k, cmp.g1, cmp.g2};
 #pragma unroll
-    for (int c = 0; c < NC; ++c) o[c] += (double)part2(tt[c][k >> 1], k & 1) - (double)part2(cc[c][k >> 1], k & 1);
+    for (int c = 0; c < NC; ++c)
+      o[c] += SPLIT ? (double)ptot[k][c] - (double)pcmp[k][c]
+                    : (double)part2(tt[c][k >> 1], k & 1) - (double)part2(cc[c][k >> 1], k & 1);
     if (!HESS) {
 #pragma unroll
       for (int v = 0; v < 2; ++v) {
@@ -1340,6 +1406,27 @@ __global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE
       r.mo[2 * m + 1] = o[1];
     }
   }
+}
+
+// S: doubled while that still leaves the chip room for the CTAs (PE_FILL per
+// SM), so that a short list (few parameter sets, a late Newton round) is not a
+// handful of CTAs each sweeping every potential.  Image-plane chi2, 1000
+// potentials, 1024^2 grid, without / with: 1 set 1717 / 883 us, 4 sets 1869 /
+// 995, 16 sets 2371 / 1555, 100 sets 4334 / 3946, 256 sets 8279 / 8155; 150
+// potentials, 16 sets 644 / 497.  A warp is in one group.
+constexpr int PE_SPLITS = 4, PE_FILL = 4;
+static_assert(PE_THREADS / PE_SPLITS >= 32 && PE_CH % (PE_SUB * PE_SPLITS) == 0, "whole warps and blocks per group");
+template <bool HESS>
+__global__ void __launch_bounds__(PE_THREADS, HESS ? LENS_PE_MINB_HESS : LENS_PE_MINB_GRAD)
+    k_pts_eval(const SetArgs a, const NewtonArgs n, const int *__restrict__ lst, const int *__restrict__ count) {
+  __shared__ PtsShared<HESS> sh;
+  const int npts = *count, ctas = min((int)gridDim.x, PE_FILL * n.nsm);
+  int S = 1;
+  while (S < PE_SPLITS && (npts + pe_points(HESS) / (2 * S) - 1) / (pe_points(HESS) / (2 * S)) <= ctas) S *= 2;
+  if (S == 1)
+    pts_eval<HESS, false>(a, n, lst, npts, 1, sh);
+  else
+    pts_eval<HESS, true>(a, n, lst, npts, S, sh);
 }
 
 // The source position, ratio and grid spacing a candidate's decisions use.
@@ -2083,6 +2170,7 @@ int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_
   n.gax = gc->alpha32;
   n.gay = gc->alpha32 + (size_t)gc->nx * gc->ny;
   n.err = ctx->d_err;
+  n.nsm = nsm;
   SearchArgs g;
   g.ax = gc->alpha32;
   g.ay = gc->alpha32 + (size_t)gc->nx * gc->ny;
@@ -2126,8 +2214,9 @@ int run_chi2_image(lens_ctx *ctx, CSet *c, const GridCache *gc, const double *d_
         return fail(LENS_ECUDA, "cudaMemsetAsync failed");
       k_ref_init<<<dim3((IMG_CAP + RL_THREADS - 1) / RL_THREADS, a.B), RL_THREADS, 0, st>>>(a, n);
       const size_t N = (size_t)a.B * IMG_CAP;
-      const unsigned gsub = (unsigned)((3 * N + pe_points(false) - 1) / pe_points(false));
-      const unsigned gnew = (unsigned)((N + pe_points(true) - 1) / pe_points(true));
+      const unsigned fill = (unsigned)(PE_FILL * nsm);
+      const unsigned gsub = std::max((unsigned)((3 * N + pe_points(false) - 1) / pe_points(false)), fill);
+      const unsigned gnew = std::max((unsigned)((N + pe_points(true) - 1) / pe_points(true)), fill);
       for (int lev = 0; lev < SUBDIV_LEVELS; ++lev) {
         k_pts_eval<false><<<gsub, PE_THREADS, 0, st>>>(a, n, a.s.lst + ((lev & 1) ? 3 * N : 0), a.s.lcnt + lev);
         k_ref_level<<<4 * nsm, RL_THREADS, 0, st>>>(a, n, lev);
