@@ -27,35 +27,30 @@ UNIT = "pair/s"
 MAP_N, N_HALO = 2048, 1000
 L2_FLUSH_BYTES = 256 << 20   # > 129 MB L2, written between timed steps
 
-# FP32-pipe lane operations (FFMA + FADD + FMUL, each paired FFMA2 / FADD2 /
-# FMUL2 counting two) and MUFU (XU pipe) instructions per point-halo pair of
-# the lens arithmetic of the LENS_MIXED Hessian map kernel, from ncu on the
-# 2048^2 x 1000 workload (the counter group of the map kernel's summary
-# under profiles/: 65.0 lane operations per pair, of which 2.0 are the
-# magnitude sum that decides the double-float repair); the compensated-fold
-# overhead (~1 op per pair) is included.
-FP32_OPS_PER_PAIR = 63.0
-MUFU_OPS_PER_PAIR = 6.03
-# every FP32 lane operation of the map call per pair: the kernel's 65.0 and
-# the double-float repair kernel's 1.27 (same capture)
-CALL_FP32_OPS_PER_PAIR = 66.3
-# the same count for the potential-map kernel (ncu, same workload)
-POT_FP32_OPS_PER_PAIR = 48.9
-# DRAM bytes (read + write) of one launch of that kernel on that workload,
-# from the same ncu capture; the 100.7 MB of output are partly still in L2
-# when the kernel ends
-MAP_TRAFFIC_BYTES = 352000 + 39027968
+# FP32-pipe lane operations and MUFU (XU pipe) operations that one
+# LENS_MIXED map call of the 2048^2 x 1000 workload executes: per kernel the
+# pipe's busy fraction x elapsed cycles x lanes, from ncu, summed over the
+# call's kernels (summary under profiles/).  Far potentials are interpolated
+# over tiles, so the executed work is far below nodes x potentials x the
+# ~63 operations of one evaluation, and the fractions below are of what runs.
+MAP_FP32_OPS = 1.27e10   # coarse level 3.07e9, fine tiles 7.50e9, repair 1.36e9 + 0.77e9
+MAP_MUFU_OPS = 3.64e8
+POT_FP32_OPS = 7.75e9    # the potential map's two kernels
+MAP_KERNELS = 4          # launched per Hessian map: coarse level, fine tiles, two repairs
+# DRAM bytes (read + write) of those four launches, from the same capture; the
+# 100.7 MB of output are partly still in L2 when the last kernel ends
+MAP_TRAFFIC_BYTES = 43000000
 SMS, FP32_LANES, MUFU_LANES = 152, 128, 16
 # FP64 FMA lanes per SM and clock (measured on this GPU: 1/64 of the FP32 rate)
 FP64_LANES = 2
-# Thread operations per model of the batched chi2 legs (ncu instruction
-# counters on the 1000-potential model, 372 images; summary under profiles/):
-# FP32 = FFMA + FADD + FMUL, FP64 = DFMA + DADD + DMUL, MUFU = XU pipe.
+# Pipe operations per model of the batched chi2 legs, counted the same way
+# (1000-potential model, 372 images; the FP64 pipe's share includes the
+# float/double conversions).
 # Source-plane chi2, 4096 sets (k_chi2_source):
-CHI2_SRC_OPS = {"fp32": 1.276e6, "fp64": 1.658e4, "mufu": 1.168e4}
+CHI2_SRC_OPS = {"fp32": 1.59e6, "fp64": 2.49e4, "mufu": 5.5e3}
 # Image-plane chi2, 1024^2 grid, 256 sets (k_img_sources + search + the
 # refinement's point-list kernels + dedup + polish + chi2, per model):
-CHI2_IMG_OPS = {"fp32": 1.014e9, "fp64": 1.20e6, "mufu": 5.67e7}
+CHI2_IMG_OPS = {"fp32": 7.28e8, "fp64": 2.14e6, "mufu": 1.41e7}
 
 
 def hbm_peak_gbs():
@@ -381,20 +376,11 @@ def main():
         return
     f_max = (clocks.get("sm_max_mhz") or 2070.0) * 1e6
     roof = {"bound": "alu", "unit": "Top/s", "traffic": MAP_TRAFFIC_BYTES}
-    if FP32_OPS_PER_PAIR:
-        ach = FP32_OPS_PER_PAIR * pairs / (ms * 1e-3) / 1e12
-        peak = SMS * FP32_LANES * f_max / 1e12
-        roof.update({"achieved": ach, "peak": peak, "frac": ach / peak,
-                     "ops_per_pair": FP32_OPS_PER_PAIR, "pipe": "fp32 (FFMA/FADD/FMUL lanes)"})
-        # the FP32 pipe's use by the whole call (magnitude sum and repair too)
-        roof["call_ops_per_pair"] = CALL_FP32_OPS_PER_PAIR
-        roof["call_frac"] = CALL_FP32_OPS_PER_PAIR * pairs / (ms * 1e-3) / 1e12 / peak
-        if MUFU_OPS_PER_PAIR:
-            mach = MUFU_OPS_PER_PAIR * pairs / (ms * 1e-3) / 1e12
-            roof["mufu"] = {"achieved": mach, "peak": SMS * MUFU_LANES * f_max / 1e12,
-                            "frac": mach / (SMS * MUFU_LANES * f_max / 1e12)}
-    else:
-        roof.update({"achieved": None, "peak": SMS * FP32_LANES * f_max / 1e12, "frac": None})
+    ach, peak = MAP_FP32_OPS / (ms * 1e-3) / 1e12, SMS * FP32_LANES * f_max / 1e12
+    roof.update({"achieved": ach, "peak": peak, "frac": ach / peak, "ops_per_call": MAP_FP32_OPS,
+                 "pipe": "fp32 (FFMA/FADD/FMUL lanes), operations executed by the call's kernels"})
+    mach, mpeak = MAP_MUFU_OPS / (ms * 1e-3) / 1e12, SMS * MUFU_LANES * f_max / 1e12
+    roof["mufu"] = {"achieved": mach, "peak": mpeak, "frac": mach / mpeak}
     # the map's DRAM traffic against the measured copy bandwidth (the output
     # planes are written once; the kernel is nowhere near this bound)
     hbm_peak, hbm_src = hbm_peak_gbs()
@@ -404,14 +390,14 @@ def main():
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32", "data": "synthetic",
-            "config": {"workload": "hessian_map 2048x2048 grid x 1000 dPIE potentials (2 cluster FP64 + 998 "
+            "config": {"workload": "hessian_map 2048x2048 grid x 1000 dPIE potentials (2 cluster double-float + 998 "
                                    "members FP32), LENS_MIXED, outputs alpha_x, alpha_y, kappa, gamma1, gamma2, mu",
                        "l2": "256 MB buffer written between timed steps", "parallelism": f"replicas x{ws}"},
             "e2e": {"value": ws * pairs / (e2e_t * 1e-3), "unit": UNIT,
                     "h2d_bytes_per_step": h2d_bytes, "d2h_bytes_per_step": 6 * MAP_N * MAP_N * 4},
-            # per timed step one map kernel and one repair kernel (the
-            # repair launches whatever the length of its list)
-            "gpu_launches": 2 * args.steps, "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
+            # per timed step the coarse level, the fine tiles and the two
+            # repair kernels (launched whatever the length of their lists)
+            "gpu_launches": MAP_KERNELS * args.steps, "roofline": roof, "cpu_baseline": cpu, "clocks": clocks,
             "wall_s_timed": wall, "extra": extra}
     print(json.dumps(line), flush=True)
     ctx.close()
@@ -481,9 +467,8 @@ def extra_legs(ctx, api, I, torch, dev, m, g, mid, stream, errs, out):
     except Exception as e:
         errs["potential_map"] = {"error": str(e)}
     ex["potential_map_mixed"] = {"ms": t, "pair_per_s": pairs / (t * 1e-3),
-                                 "ops_per_pair": POT_FP32_OPS_PER_PAIR,
-                                 "fp32_frac": POT_FP32_OPS_PER_PAIR * pairs / (t * 1e-3)
-                                 / (SMS * FP32_LANES * 2.07e9) if POT_FP32_OPS_PER_PAIR else None,
+                                 "ops_per_call": POT_FP32_OPS,
+                                 "fp32_frac": POT_FP32_OPS / (t * 1e-3) / (SMS * FP32_LANES * 2.07e9),
                                  "workload": "potential + Fermat surface, 2048^2 x 1000, LENS_MIXED"}
     del outp
     # the same map with the members' cut radii at 45" (L/L*)^1/2 instead of

@@ -136,10 +136,10 @@ int lens_destroy(lens_ctx *ctx);
 
 /* Potentials with b0 >= threshold_b0 are evaluated in FP64 by LENS_MIXED
  * maps (default 5 arcsec) -- in double-float on the FP32 pipe instead (about
- * 1e-13 relative, FP64 where that fails) by the deflection and Hessian maps
- * of a model with fewer than 400 other potentials per such potential, where
- * the FP64 unit (1/64 of the FP32 rate) would set the pace.  Applies to
- * models uploaded afterwards. */
+ * 1e-13 relative, FP64 where that fails) by the interpolated deflection and
+ * Hessian maps, and by the direct ones of a model with fewer than 400 other
+ * potentials per such potential, where the FP64 unit (1/64 of the FP32 rate)
+ * would set the pace.  Applies to models uploaded afterwards. */
 int lens_set_fp64_threshold(lens_ctx *ctx, double threshold_b0);
 
 /* LENS_MIXED deflection and Hessian maps: where the deflection at a node is
@@ -154,6 +154,9 @@ int lens_set_fp64_threshold(lens_ctx *ctx, double threshold_b0);
  * repaired nodes the measured error then stays below 0.83 of 1e-6 |alpha|
  * (the FP32 error never exceeded 1.32e-7 of the sum on the models measured);
  * r = 0 turns the repair off.
+ * (Where far potentials are interpolated over a tile, so is their part of the
+ * sum; many listed nodes of one tile share an interpolation of the far
+ * potentials in double-float.)
  * The list is working memory of the call (4 bytes per grid point, stream
  * ordered).  LENS_EINVAL for r < 0 or not finite. */
 int lens_set_repair_ratio(lens_ctx *ctx, double r);
@@ -180,6 +183,12 @@ int lens_model_upload(lens_ctx *ctx, const lens_halo *h, int32_t n, lens_model_t
 int lens_model_release(lens_ctx *ctx, lens_model_t model);
 
 /* ------------------------------------------------------------------- maps */
+
+/* LENS_MIXED maps evaluate a potential at every node of the tiles near it and
+ * interpolate it over the tiles far from it where that is cheaper; errors are
+ * those of evaluating every pair.  The interpolation's working memory (stream
+ * ordered; about 20 MB for a 2048 x 2048 Hessian map) is optional: without it every pair is
+ * evaluated. */
 
 /* Deflection map (Sec. 4.1, Eq. 10; lens equation Sec. 2.1 Eq. 1):
  * d_out holds 2 planes [2][ny][nx] -- alpha_x, alpha_y -- of float
@@ -356,8 +365,10 @@ int lens_chi2_autotune(lens_ctx *ctx, lens_cset_t cset, const double *d_params, 
  * context's error flag, which the next lens_wait reports as LENS_ECAPACITY
  * (and clears).  At most 1024 sources per constraint set (LENS_EINVAL
  * beyond, nothing launched).  The first call on a (constraint set, grid)
- * pair computes and keeps the static potentials' deflection on the grid;
- * each call's candidate buffers are working memory allocated and freed in
+ * pair computes and keeps the static potentials' deflection on the grid (8
+ * bytes per node) and a model of it per 8 x 8 cells (0.5 bytes per node;
+ * without room for it the search is slower, with the same result); each
+ * call's candidate buffers are working memory allocated and freed in
  * stream order on `stream`. */
 int lens_chi2_image(lens_ctx *ctx, lens_cset_t cset, const lens_grid *grid, const double *d_params, int32_t P,
                     double *d_chi2, int32_t *d_nimg_found, void *stream);
@@ -387,7 +398,8 @@ int lens_find_images(lens_ctx *ctx, lens_cset_t cset, const lens_grid *grid, con
  *     call rewrites everything it reads.  Calls whose work overlaps on the
  *     GPU (different streams, or different contexts on one device) race.
  *   - LENS_EINVAL, with a message, when the grid's static deflection
- *     (8 bytes per node) plus the buffers of one parameter set do not fit. */
+ *     (8 bytes per node) plus the buffers of one parameter set do not fit.
+ *     (The search's model of it is used where it fits as well.) */
 #define LENS_NOALLOC_SCRATCH_BYTES (16u << 20)
 int lens_chi2_image_noalloc(lens_ctx *ctx, lens_cset_t cset, const lens_grid *grid, const double *d_params,
                             int32_t P, double *d_chi2, int32_t *d_nimg_found, void *stream);

@@ -18,8 +18,8 @@
 // every model.
 //
 // The two varying potentials are evaluated in double-float (FP32 pipe,
-// ~1e-13 relative), FP64 only where that fails; the static cache itself is
-// FP64.
+// ~1e-13 relative; lens_chi2_df.cuh), two images side by side per thread, FP64
+// only where that fails; the static cache itself is FP64.
 #include "lens_chi2_df.cuh"
 
 namespace lens {

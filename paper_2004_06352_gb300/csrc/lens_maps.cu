@@ -2,7 +2,10 @@
 // (Sec. 2.4, Eqs. 7-9; magnification Sec. 2.1, Eqs. 4-5) over a rectangular
 // grid with inclusive corners.
 //
-// LENS_MIXED kernel (the hot path):
+// LENS_MIXED: maps whose far potentials are worth interpolating are computed by
+// lens_far.cu; here the direct kernel (every potential at every node: small
+// models and grids, no memory for the interpolation, the image search's grid)
+// and the repair of both.  The direct kernel:
 //   - CTA = 128 threads = 4 warps over a 32 x (4 KP) point tile; lane l owns
 //     column i0 + l, warp w owns rows j0 + w KP .. + KP-1, so every store of
 //     one row is 32 consecutive elements (one 128-byte segment per warp).
