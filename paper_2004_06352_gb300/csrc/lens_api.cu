@@ -610,20 +610,35 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   const size_t esize = precision == LENS_FP64 ? 8 : 4;
   if ((uintptr_t)h_out % esize) return fail(LENS_EINVAL, "h_out must be aligned to its element size");
   const int planes = hess ? 6 : 2, nx = grid->nx, ny = grid->ny;
-  // about 8 bands, each a whole number of tiles
   FarPlan plan;
   if (precision == LENS_MIXED) plan = plan_far(ctx, m, grid, hess);
   const int tile = plan.use ? plan.ft : map_tile_rows(hess);
-  int rows = (ny + 7) / 8;
-  rows = std::max(tile, (rows + tile - 1) / tile * tile);
-  const size_t band_bytes = (size_t)rows * nx * planes * esize;
+  // Bands, each a whole number of tiles.  A band costs launches and underfilled
+  // kernels (~20 us), fewer bands leave more of the copy (192 GB/s) after the
+  // last kernel; two overlap nothing (both streams end together).  Time with
+  // 1 / 3 / 6 / 8 bands: 256^2 Hessian (1.6 MB) 88 / 112 / 172 / 201 us, 600^2
+  // deflection (2.9 MB) 160 / 175 / 227 / 265, 1601 x 1203 (15 MB) 478 / 412 /
+  // 517 / 592, 2048^2 Hessian (101 MB) 1285 / 1203 / 1276 / 1336, 5000^2
+  // deflection (200 MB) 1525 / 1419 / 1300 / 1372, 4096^2 Hessian (403 MB) 2926
+  // / 2800 / 2444 / 2463.  A context with a memory budget, or without
+  // room for the larger bands' buffers (they are kept): 8 of them.
+  auto band_rows = [&](int bands) { return std::max(tile, ((ny + bands - 1) / bands + tile - 1) / tile * tile); };
+  const size_t row_bytes = (size_t)nx * planes * esize, map_bytes = row_bytes * ny;
+  int rows = band_rows(ctx->budget ? 8 : map_bytes <= (8u << 20) ? 1 : map_bytes <= (128u << 20) ? 3 : 6);
+  size_t band_bytes = rows * row_bytes;
   if (ctx->band_bytes < 2 * band_bytes) {
     if (ctx->band) {
       dev_free(ctx, ctx->band, ctx->band_bytes);  // after the bands in flight have left
       ctx->band = nullptr;
       ctx->band_bytes = 0;
     }
-    if ((rc = dev_alloc(ctx, &ctx->band, 2 * band_bytes))) return rc;
+    rc = dev_alloc(ctx, &ctx->band, 2 * band_bytes);
+    if (rc && rows > band_rows(8)) {
+      rows = band_rows(8);
+      band_bytes = rows * row_bytes;
+      rc = dev_alloc(ctx, &ctx->band, 2 * band_bytes);
+    }
+    if (rc) return rc;
     ctx->band_bytes = 2 * band_bytes;
   }
   if (!ctx->pipe_cp) {
