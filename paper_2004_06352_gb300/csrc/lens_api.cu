@@ -656,6 +656,20 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   for (int k = 0; k < 2; ++k) LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[k], ctx->pipe_start, 0));
   // the interpolated form's coarse level, of the whole grid, before the bands
   CallScratch far(ctx, ctx->pipe_cs[0]);
+  // freed on the first band stream once the second has left it too, also
+  // where a band fails after others were launched
+  struct FreeAfterBands {
+    lens_ctx *ctx;
+    CallScratch &far;
+    ~FreeAfterBands() { now(); }
+    void now() {
+      if (!far.p) return;
+      if (cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[1]) != cudaSuccess ||
+          cudaStreamWaitEvent(ctx->pipe_cs[0], ctx->pipe_start, 0) != cudaSuccess)
+        cudaStreamSynchronize(ctx->pipe_cs[1]);
+      far.release();
+    }
+  } free_far{ctx, far};
   const size_t far_bytes = plan.bytes + plan.rep_bytes;  // the dense tiles' arrays for each band stream
   if (plan.use && far_bytes) {
     const bool room = !ctx->budget || ctx->used + far_bytes + map_repair_bytes(grid, rows) <= ctx->budget;
@@ -690,9 +704,7 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   for (int k = 0; k < 2; ++k) LENS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->pipe_copied[k], 0));
   if (far.p) {
     // the coarse level goes once both band streams have read it; st joins
-    LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[1]));
-    LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[0], ctx->pipe_start, 0));
-    far.release();
+    free_far.now();
     LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[0]));
     LENS_CUDA_TRY(cudaStreamWaitEvent(st, ctx->pipe_start, 0));
   }
