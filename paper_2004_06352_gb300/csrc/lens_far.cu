@@ -43,8 +43,17 @@ namespace {
 
 constexpr int FP = FAR_P;  // interpolation nodes per axis of a fine tile
 constexpr int CP = 12;   // a coarse tile's
-constexpr int CO_THREADS = 256;  // coarse kernel
+// Coarse kernel: its few CTAs (256 for 2048^2 x 1000) are one wave bound by the
+// latency of each thread's chain of potentials, so 5 threads share a node pair's
+// potentials (256 threads are 3, of which 40 threads idle; 448 are 6 and spill).
+// Whole map with 256 / 288 / 384 / 448 threads: Hessian 2048^2 x 1000 719 / 714 /
+// 710 / 721 us, deflection 5000^2 x 217 439 / 435 / 425 / 425, potential 1537 x
+// 1021 x 500 258 / 254 / 247 / 247.
+constexpr int CO_THREADS = 384;
 constexpr int FF_CH = 64;            // potentials per staged chunk
+// the coarse kernel's: with 64 / 128 / 256 the Hessian map above took 714 / 702 /
+// 712 us on another GPU (fewer waits for records against shared memory for L1)
+constexpr int CO_CH = 128;
 constexpr int REC_STRIDE4 = REC32 / 4 + 1;  // float4 slots per staged record (the pad spreads the records a warp reads)
 constexpr int FF_SUB = 16;           // partial sums folded every FF_SUB potentials
 constexpr double DET_TERM_ERR = 2e-7, DET_REPAIR_ABS = 1e-5;  // as in lens_maps.cu
@@ -339,7 +348,7 @@ __device__ __forceinline__ float slope8(float v) { return __int_as_float(__float
 // double-float (node = y index * P + x index).  Ends synchronised.
 // kb: the FP32 potentials' largest |kappa|, |gamma1|, |gamma2| at the nodes
 // (HESS), added to what is there.
-template <int MODE, int P, int TH>
+template <int MODE, int P, int TH, int CH>
 __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short *list, int n_far, int n_far_h,
                                           df Tx, df Ty, const float2 *s_nx, const float2 *s_ny, float4 *s_rec,
                                           float4 *s_off, float2 *s_part, float2 *s_val, float *s_kb) {
@@ -349,8 +358,9 @@ __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short
   Sums<MODE> S;
   S.zero();
   const float2 ox = s_nx[ix], y0 = s_ny[jy], y1 = s_ny[jy + 1];
-  for (int c0 = 0; c0 < n_far; c0 += FF_CH) {
-    const int cnt = min(FF_CH, n_far - c0);
+  static_assert(CH <= TH, "stage_chunk: one offset per thread");
+  for (int c0 = 0; c0 < n_far; c0 += CH) {
+    const int cnt = min(CH, n_far - c0);
     if (c0) __syncthreads();  // the previous chunk has been used
     stage_chunk<TH>(a, list + c0, cnt, Tx, Ty, s_rec, s_off);
     __syncthreads();
@@ -417,8 +427,8 @@ __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
   constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), SPLITS = CO_THREADS / (NODES / 2);
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);
-  float4 *s_off = s_rec + FF_CH * REC_STRIDE4;
-  float2 *s_part = reinterpret_cast<float2 *>(s_off + FF_CH);
+  float4 *s_off = s_rec + CO_CH * REC_STRIDE4;
+  float2 *s_part = reinterpret_cast<float2 *>(s_off + CO_CH);
   float2 *s_val = s_part + SPLITS * NODES * NC;
   unsigned *s_far = reinterpret_cast<unsigned *>(s_val + NODES * NC);
   unsigned *s_near = s_far + a.nw;
@@ -442,7 +452,7 @@ __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
   if (tid < 4) s_kb[tid] = 0.f;
   classify<CO_THREADS>(a, nullptr, Tx, Ty, a.thr_c, a.thr_ch, s_far, s_near, s_list, s_cnt);
   for (int w = tid; w < a.nw; w += CO_THREADS) a.cmask[(size_t)tile * a.nw + w] = s_near[w];
-  node_sums<MODE, CP, CO_THREADS>(a, s_list, s_cnt[0], s_cnt[1], Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
+  node_sums<MODE, CP, CO_THREADS, CO_CH>(a, s_list, s_cnt[0], s_cnt[1], Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
   if (tid < NV) s_plane[tid] = plane_of<CP>(s_val + tid * NODES, (D_ZC[0] - D_ZC[CP - 1]) * (float)half);
   __syncthreads();
   float *o = a.cval + (size_t)tile * coarse_floats(MODE);
@@ -525,7 +535,7 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
   const int ctile = a.ct ? (j0 / a.ct) * a.nct + i0 / a.ct : 0;
   classify<FI_THREADS>(a, a.ct ? a.cmask + (size_t)ctile * a.nw : nullptr, Tx, Ty, a.thr_f, a.thr_fh, s_far, s_near, s_list, s_cnt);
   const int n_far = s_cnt[0], n_far_h = s_cnt[1], n_near = s_cnt[2], n_near_h = s_cnt[3];
-  node_sums<MODE, FP, FI_THREADS>(a, s_list, n_far, n_far_h, Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
+  node_sums<MODE, FP, FI_THREADS, FF_CH>(a, s_list, n_far, n_far_h, Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
   if (a.ct) {
     // the coarse tile's interpolant at this tile's nodes: rows of the tensor
     // product, then columns; its plane (exact products) in double-float
@@ -965,7 +975,7 @@ __global__ void __launch_bounds__(FR_THREADS) k_far_repair(const FarRepairArgs a
 size_t far_smem(int mode, int ft, int nw, int n, int threads = 256) {
   const bool coarse = ft == 0;
   const int nodes = coarse ? CP * CP : FP * FP, splits = threads / (nodes / 2), nc = ncmp(mode);
-  size_t b = sizeof(float4) * (FF_CH * REC_STRIDE4 + FF_CH);
+  size_t b = sizeof(float4) * (size_t)(coarse ? CO_CH : FF_CH) * (REC_STRIDE4 + 1);
   if (!coarse) b += sizeof(float4) * (ft / 2) * FP * ncmp2(mode);
   // the partial sums' space also holds the coarse tile's values (fine kernel)
   const size_t part = std::max(sizeof(float2) * splits * nodes * nc, coarse ? 0 : sizeof(float) * nc * (CP * CP + CP * FP));
