@@ -66,8 +66,8 @@ __host__ __device__ constexpr int nval(int mode) { return mode == FAR_HESS ? 5 :
 __host__ __device__ constexpr int ncmp(int mode) { return nval(mode) + (mode == FAR_POT ? 0 : 1); }
 __host__ __device__ constexpr int ncmp2(int mode) { return (ncmp(mode) + 1) / 2; }
 
-// CTAs per SM of the fine kernel with 128 or 256 threads (launch_far_map)
-__host__ __device__ constexpr int fi_blocks(int mode, int th) { return th == 256 ? 2 : mode == FAR_GRAD ? 5 : 4; }
+// CTAs per SM of the fine kernel with 128, 256 or 512 threads (launch_far_map)
+__host__ __device__ constexpr int fi_blocks(int mode, int th) { return th == 512 ? 1 : th == 256 ? 2 : mode == FAR_GRAD ? 5 : 4; }
 
 // Chebyshev nodes of a fine tile of FT x FT map nodes (FT = 32 or 64), in
 // units of 1/64 grid step about its centre, and of the coarse tile in units
@@ -1193,13 +1193,24 @@ static int fine_launch(const FarArgs &a, int n, cudaStream_t st) {
 // / 667, 4096 tiles 824 / 798; deflection x 200, 2304 tiles 197 / 181, 2304 of
 // 64 x 64 299 / 323, 4096 tiles 250 / 210, 6241 (5000^2 x 217) 524 / 451.
 // The potential's FP64 terms want the 256 (0.266 against 0.279 ms).
+// 512 threads (one CTA per SM) where not every SM has two tiles: a tile is a
+// chain of phases, and twice the threads shorten it.  256 / 512 threads, us:
+// Hessian x 1000, 100 tiles 480 / 355, 196 tiles 395 / 299, 256 tiles 396 / 331;
+// x 300, 175 / 135, 147 / 115, 145 / 129; deflection x 300, 256 tiles 122 / 104;
+// potential x 1000, 256 tiles 389 / 294.  With 10 potentials there is little to
+// share: Hessian, 196 tiles 40.2 / 36.5, 256 tiles 40.3 / 42.9 (60 potentials
+// 60.5 / 59.7), hence the lower line there.
 // Counted over the whole map, also where a band of it is launched: the split of
 // the node sums, and with it the last bits, is then the same.
-constexpr int FI_TILES = 3072;
+constexpr int FI_TILES = 3072, FI_FEW = 304, FI_FEW_SMALL = 200, FI_SMALL = 32;
 template <int MODE, int FT>
 static int fine_threads(const FarArgs &a, const lens_grid *g, int n, cudaStream_t st) {
   const long long tiles = (long long)((g->nx + FT - 1) / FT) * ((g->ny + FT - 1) / FT);
-  return tiles >= FI_TILES ? fine_launch<MODE, FT, 128>(a, n, st) : fine_launch<MODE, FT, 256>(a, n, st);
+  if constexpr (MODE != FAR_POT)
+    if (tiles >= FI_TILES) return fine_launch<MODE, FT, 128>(a, n, st);
+  if constexpr (FT == 32)
+    if (tiles <= (MODE != FAR_POT && n < FI_SMALL ? FI_FEW_SMALL : FI_FEW)) return fine_launch<MODE, FT, 512>(a, n, st);
+  return fine_launch<MODE, FT, 256>(a, n, st);
 }
 
 int launch_far_coarse(const Model *m, const lens_grid *g, const FarPlan &p, int mode, void *mem, cudaStream_t st) {
@@ -1229,7 +1240,7 @@ int launch_far_map(const Model *m, const lens_grid *g, const FarPlan &p, int mod
     a.tau = beta != nullptr;
     a.bx = beta ? beta[0] : 0.0;
     a.by = beta ? beta[1] : 0.0;
-    return p.ft == 32 ? fine_launch<FAR_POT, 32, 256>(a, m->n, st) : fine_launch<FAR_POT, 64, 256>(a, m->n, st);
+    return p.ft == 32 ? fine_threads<FAR_POT, 32>(a, g, m->n, st) : fine_threads<FAR_POT, 64>(a, g, m->n, st);
   }
   a.out = (float *)out;
   if (mode == FAR_HESS) return p.ft == 32 ? fine_threads<FAR_HESS, 32>(a, g, m->n, st) : fine_threads<FAR_HESS, 64>(a, g, m->n, st);

@@ -26,6 +26,9 @@ CASES = [
     # most nodes recomputed in double-float, deflection and all planes (dense tiles of the repair)
     (860, 650, 25.0, lambda: I.cfg2_model(seed=12, n_members=700, rcut_star=45.0)),
     (2100, 1900, 25.0, lambda: I.cfg2_model(seed=13, n_members=300, rcut_star=45.0)),
+    # few tiles and few potentials; few tiles and several chunks of potentials at a tile's nodes
+    (448, 440, 100.0, lambda: I.cfg2_model(seed=14, n_members=8)),
+    (385, 383, 60.0, lambda: I.cfg2_model(seed=15, n_members=1100)),
 ]
 
 
