@@ -286,6 +286,17 @@ int build_model(lens_ctx *ctx, const lens_halo *h, int32_t n, Model **out) {
   double iq = 0.0;
   for (int32_t i : light) iq += h[i].type == LENS_DPIE ? (1.0 + h[i].eps) / (1.0 - h[i].eps) : 1.0;
   m->invq_light = light.empty() ? 1.0 : iq / (double)light.size();
+  double scales = 0.0, squares = 0.0;
+  size_t round_light = 0;
+  for (int32_t i : light) {
+    const double s = h[i].type == LENS_DPIE ? h[i].b0 * h[i].rcut : 0.0;
+    round_light += h[i].type != LENS_DPIE;
+    scales += s;
+    squares += s * s;
+  }
+  for (int32_t i : heavy) scales += h[i].type == LENS_DPIE ? h[i].b0 * h[i].rcut : 0.0;
+  // (SIS and point mass have no scale of their own: most of them, no estimate)
+  m->pot_light = light.empty() ? 0.0 : scales > 0.0 && 2 * round_light <= light.size() ? std::sqrt(squares) / scales : 1.0;
   for (int32_t i : heavy) {
     const bool d = h[i].type == LENS_DPIE;
     m->heavy_shape.push_back({d ? (1.0 - h[i].eps) / (1.0 + h[i].eps) : 1.0, d ? h[i].rcore * (1.0 + h[i].eps) : 0.0});

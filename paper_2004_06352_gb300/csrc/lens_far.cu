@@ -999,6 +999,11 @@ constexpr long long DENSE_TILES = 65536;
 // margins of the repair: interpolation error below 4e-11 of a potential's own
 // deflection at the edge of its far region (4e-14 for the strong ones)
 constexpr double KR = 5.0, KR_H = 8.0;
+// Potential maps are stored in double, so the FP32 terms' rounding, which
+// differs between the two forms, shows in them: by 0.5e-10 to 7.3e-10 of the
+// map where Model::pot_light is below this (50 models of 60 to 2000 potentials;
+// 8.3e-10 to 6.4e-9 from 0.003 on).  Beyond, the direct kernel keeps its values.
+constexpr double POT_LIGHT = 0.0025;
 constexpr int FAR_MAX_N = 16384;  // potentials (two bytes each of shared memory)
 
 // Fraction of the map's nodes within psi < r of a potential of axis ratio q
@@ -1020,6 +1025,7 @@ int far_words(const Model *m) { return (m->n_light + 31) / 32 + (m->n_heavy + 31
 FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode) {
   FarPlan p;
   if (m->n > FAR_MAX_N || m->n < 1) return p;
+  if (mode == FAR_POT && m->pot_light > POT_LIGHT) return p;
   const double dx = (g->xmax - g->xmin) / (g->nx - 1), dy = (g->ymax - g->ymin) / (g->ny - 1);
   const double area = (g->xmax - g->xmin) * (g->ymax - g->ymin), nodes = (double)g->nx * g->ny;
   const double HV = mode == FAR_HESS ? 20.0 : 10.0, step = std::max(dx, dy);

@@ -237,6 +237,9 @@ struct Model {
   // and core of each cluster-scale one
   double invq_light = 1.0;
   std::vector<std::pair<double, double>> heavy_shape;
+  // size of the FP32 potentials' rounding in the lensing potential: root of
+  // their squared scales b0 r_cut over the sum of all scales
+  double pot_light = 0.0;
 };
 
 struct GridCache {
