@@ -153,10 +153,13 @@ int lens_set_fp64_threshold(lens_ctx *ctx, double threshold_b0);
  * rewritten.  r = LENS_REPAIR_RATIO_DEFAULT = 0.16 by default: outside the
  * repaired nodes the measured error then stays below 0.83 of 1e-6 |alpha|
  * (the FP32 error never exceeded 1.32e-7 of the sum on the models measured);
- * r = 0 turns the repair off.
- * (Where far potentials are interpolated over a tile, so is their part of the
- * sum; many listed nodes of one tile share an interpolation of the far
- * potentials in double-float.)
+ * r = 0 turns this repair off.
+ * Where far potentials are interpolated over a tile, so is their part of the
+ * sum, and the largest remainders that the tile interpolates in FP32 (their
+ * rounding is at most 8.6e-7 of them) join it as the root of both squares:
+ * whatever r is, and in models without FP32 potentials.
+ * Many listed nodes of one tile share an interpolation of the far potentials
+ * in double-float.
  * The list is working memory of the call (4 bytes per grid point, stream
  * ordered).  LENS_EINVAL for r < 0 or not finite. */
 int lens_set_repair_ratio(lens_ctx *ctx, double r);
@@ -185,10 +188,10 @@ int lens_model_release(lens_ctx *ctx, lens_model_t model);
 /* ------------------------------------------------------------------- maps */
 
 /* LENS_MIXED maps evaluate a potential at every node of the tiles near it and
- * interpolate it over the tiles far from it where that is cheaper; errors are
- * those of evaluating every pair.  The interpolation's working memory (stream
- * ordered; about 20 MB for a 2048 x 2048 Hessian map) is optional: without it every pair is
- * evaluated. */
+ * interpolate it over the tiles far from it where that is cheaper, within the
+ * same error bounds as evaluating every pair.  The interpolation's working
+ * memory (stream ordered; about 20 MB for a 2048 x 2048 Hessian map) is
+ * optional: without it every pair is evaluated. */
 
 /* Deflection map (Sec. 4.1, Eq. 10; lens equation Sec. 2.1 Eq. 1):
  * d_out holds 2 planes [2][ny][nx] -- alpha_x, alpha_y -- of float

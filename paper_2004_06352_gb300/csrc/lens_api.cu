@@ -566,10 +566,14 @@ static int map_common(lens_ctx *ctx, lens_model_t model, const lens_grid *grid, 
   StreamMark mark(ctx, st);
   if (precision == LENS_MIXED) {
     FarPlan plan = plan_far(ctx, m, grid, hess);
-    // the repair list first: without it there is no map, without room for
-    // the coarse level's values there is the direct kernel
+    // the repair list first: without it there is no map (or only the direct
+    // kernel, where that lists nothing), without room for the coarse level's
+    // values there is the direct kernel
     CallScratch list(ctx, st), far(ctx, st);
-    if (plan.use && ctx->repair_ratio > 0.0 && m->n_light > 0 && (rc = list.alloc(map_repair_bytes(grid)))) return rc;
+    if (plan.use && (rc = list.alloc(map_repair_bytes(grid)))) {
+      if (map_needs_list(ctx, m)) return rc;
+      plan = FarPlan();
+    }
     if (plan.use && plan.bytes && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
     if (plan.use && (rc = launch_far_coarse(m, grid, plan, hess, far.p, st))) return rc;
     return launch_map_mixed(ctx, m, grid, dls_ds, hess, d_out, st, 0, -1, true, list.p, plan.use ? &plan : nullptr,
@@ -682,11 +686,11 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
     }
   } free_far{ctx, far};
   const size_t far_bytes = plan.bytes + plan.rep_bytes;  // the dense tiles' arrays for each band stream
-  if (plan.use && far_bytes) {
+  if (plan.use) {
     const bool room = !ctx->budget || ctx->used + far_bytes + map_repair_bytes(grid, rows) <= ctx->budget;
     if (!room || far.alloc(far_bytes) != LENS_OK) {
       plan = FarPlan();  // no room beside the bands' repair lists: the direct kernel, whose tiles divide the bands too
-    } else {
+    } else if (far_bytes) {
       if ((rc = launch_far_coarse(m, grid, plan, hess, far.p, ctx->pipe_cs[0]))) return rc;
       LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[0]));
       LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[1], ctx->pipe_start, 0));

@@ -33,6 +33,17 @@
 // plus the remainder plus the near sum in double-float, scaled by D_ls/D_s
 // and rounded once.  The magnitude sum that decides the double-float repair
 // is interpolated as well (a few percent off where a far term changes sign).
+// It stands for the FP32 terms' rounding, not for that of the remainders,
+// which the cluster-scale potentials' deflections feed as well: where those
+// cancel, that rounding shows (2e-7 to 7e-7 arcsec between two b0 = 30"
+// clusters, 7 times the 1e-6 |alpha| bound).  Per tile it is at most 14.4
+// 2^-24 = 8.6e-7 of the largest remainder of the coarse plus that of the fine
+// interpolation (restated on the CPU: 1 to 3 random cluster-scale terms beyond
+// the margins, 16000 tiles of every size, every map node; rms 3 2^-24).  It is
+// independent of the FP32 terms' rounding, so a node is listed where |alpha| is
+// below the root of (ratio x magnitude sum)^2 + (those two remainders)^2 -- also
+// in a model without FP32 potentials and with the FP32 terms' repair off.  (The
+// plain sum lists a sixth more nodes of 8192^2 x 2000: 8.8 instead of 7.8 ms.)
 #include <algorithm>
 #include <cmath>
 
@@ -163,20 +174,21 @@ struct FarArgs {
   float thr_c, thr_ch, thr_f, thr_fh;  // squared psi beyond which a potential is far: coarse / fine, FP32 / cluster-scale
   // coarse level: tile (0, 0) covers the grid's first nodes
   int ct, nct;       // nodes a side (0: no coarse level), tiles per row
-  float *cval;       // per coarse tile: remainders [ncmp][CP * CP], planes [nval][4], light kappa and gamma bounds [4]
+  float *cval;       // per coarse tile: remainders [ncmp][CP * CP], planes [nval][4], s_kb [KB]
   unsigned *cmask;   // per coarse tile: nw words, bit set = left to the fine level
   float *out;
   double *out64;
   long long plane;
   int tau;
   double bx, by;
-  float repair_f;    // 2 * ratio, 0: no repair
-  int *rep_count, *rep_list;
+  float repair_f;    // 2 * ratio, 0: only the remainders' part of the repair
+  int *rep_count, *rep_list;  // NULL: no repair
   DenseRepair dense;
   int dense_min;     // listed nodes from which a tile is dense
 };
 
-__host__ __device__ constexpr int coarse_floats(int mode) { return ncmp(mode) * CP * CP + nval(mode) * 4 + 4; }
+constexpr int KB = 6;  // a tile's s_kb (repair_bound)
+__host__ __device__ constexpr int coarse_floats(int mode) { return ncmp(mode) * CP * CP + nval(mode) * 4 + KB; }
 
 // Is the potential far from a tile centred at (dx, dy) from it?
 __device__ __forceinline__ bool far32(const float4 *r4, float dX, float dY, float thr) {
@@ -340,6 +352,12 @@ __device__ __forceinline__ void classify(const FarArgs &a, const unsigned *in, d
   __syncthreads();
 }
 
+// det's error, 2 |1 - kappa| d kappa + 2 |gamma| d gamma, in units of 2
+// DET_TERM_ERR: above DET_LIST a node's planes are all recomputed.  A
+// remainder's rounding (below 5 DET_TERM_ERR of it) adds to the FP32 terms' as
+// the root of both squares, like the deflection's.
+constexpr float REM_TERM = 5.f, DET_LIST = (float)(DET_REPAIR_ABS / (2.0 * DET_TERM_ERR));
+
 // Slope with 8 significant bits: its products with node offsets (up to 15
 // bits) are exact in FP32.
 __device__ __forceinline__ float slope8(float v) { return __int_as_float(__float_as_int(v) & 0xffff0000); }
@@ -422,6 +440,22 @@ __device__ __forceinline__ float4 plane_of(const float2 *v, float span) {
                      slope8((v[m].x - v[(P - 1) * P + m].x) / span), 0.f);
 }
 
+// Entry `lane` of a tile's s_kb, for the repair (one warp): the far FP32
+// potentials' largest |kappa|, |gamma1|, |gamma2| (kb), then the largest
+// remainders of the deflection, of kappa and of gamma; the remainder of value c
+// at a node is f[(c NODES + node) stride].
+template <int MODE, int NODES>
+__device__ __forceinline__ float repair_bound(const float *kb, const float *f, int stride, int lane) {
+  float rm[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int c = 0; c < nval(MODE); ++c) {
+    for (int node = lane; node < NODES; node += 32) rm[c] = fmaxf(rm[c], fabsf(f[(c * NODES + node) * stride]));
+    rm[c] = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(rm[c])));
+  }
+  if (lane < 3) return kb[lane];
+  return lane == 3 ? fmaxf(rm[0], rm[1]) : lane == 4 ? rm[2] : sqrtf(fmaf(rm[3], rm[3], rm[4] * rm[4]));
+}
+
 template <int MODE>
 __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
   constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), SPLITS = CO_THREADS / (NODES / 2);
@@ -434,7 +468,7 @@ __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
   unsigned *s_near = s_far + a.nw;
   unsigned short *s_list = reinterpret_cast<unsigned short *>(s_near + 3 * a.nw);
   __shared__ float2 s_nx[CP], s_ny[CP];
-  __shared__ float s_kb[4];
+  __shared__ float s_kb[KB];
   __shared__ float4 s_plane[NV];
   __shared__ int s_cnt[4];
   const int tid = threadIdx.x, tile = blockIdx.y * a.nct + blockIdx.x;
@@ -449,7 +483,7 @@ __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
     s_nx[tid] = make_float2(ox.hi, ox.lo);
     s_ny[tid] = make_float2(oy.hi, oy.lo);
   }
-  if (tid < 4) s_kb[tid] = 0.f;
+  if (tid < KB) s_kb[tid] = 0.f;
   classify<CO_THREADS>(a, nullptr, Tx, Ty, a.thr_c, a.thr_ch, s_far, s_near, s_list, s_cnt);
   for (int w = tid; w < a.nw; w += CO_THREADS) a.cmask[(size_t)tile * a.nw + w] = s_near[w];
   node_sums<MODE, CP, CO_THREADS, CO_CH>(a, s_list, s_cnt[0], s_cnt[1], Tx, Ty, s_nx, s_ny, s_rec, s_off, s_part, s_val, s_kb);
@@ -467,11 +501,17 @@ __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
       d = df_sub(d, df{p.y * zx, 0.f});
       d = df_sub(d, df{p.z * zy, 0.f});
       r = d.hi + d.lo;
+      s_val[q].x = r;
     }
     o[q] = r;
   }
   if (tid < NV * 4) o[NC * NODES + tid] = reinterpret_cast<const float *>(s_plane)[tid];
-  if (tid < 4) o[NC * NODES + NV * 4 + tid] = s_kb[tid];
+  if (MODE == FAR_POT) return;
+  __syncthreads();
+  if (tid < 32) {
+    const float b = repair_bound<MODE, NODES>(s_kb, reinterpret_cast<const float *>(s_val), 2, tid);
+    if (tid < KB) o[NC * NODES + NV * 4 + tid] = b;
+  }
 }
 
 // 1 / (hi + lo), one Newton step on the MUFU reciprocal
@@ -502,7 +542,7 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
   __shared__ float4 s_T;                 // the centre, hi/lo
   __shared__ unsigned s_m[FT * FT / 32], s_mh[HESS ? FT * FT / 32 : 1];  // nodes to recompute: deflection alone / all planes
   __shared__ double s_tau[POT ? 2 : 1][POT ? FT : 1];  // half the squared offsets from beta
-  __shared__ float s_kb[4];
+  __shared__ float s_kb[KB];  // for the repair: repair_bound (here and of the coarse tile), [3] squared
   __shared__ float4 s_plane[NV];
   __shared__ int s_cnt[4];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -528,7 +568,7 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
       }
     }
   }
-  if (tid < 4) s_kb[tid] = 0.f;
+  if (tid < KB) s_kb[tid] = 0.f;
   for (int q = tid; q < FT * FP; q += FI_THREADS) s_L[q / FP][q % FP] = (&fine_table<FT>().w[0][0])[q];
   __syncthreads();
   const df Tx = {s_T.x, s_T.y}, Ty = {s_T.z, s_T.w};
@@ -571,7 +611,6 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
       }
       s_val[q] = make_float2(d.hi, d.lo);
     }
-    if (HESS && tid < 3) s_kb[tid] += cv[NC * CP * CP + NV * 4 + tid];
     __syncthreads();
   }
   if (tid < NV) s_plane[tid] = plane_of<FP>(s_val + tid * NODES, s_xi[0] - s_xi[FP - 1]);
@@ -590,6 +629,13 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
     s_rem[q] = r;
   }
   __syncthreads();
+  if (!POT && warp == 0) {
+    float b = repair_bound<MODE, NODES>(s_kb, s_rem, 1, lane);
+    if (lane < KB) {
+      if (a.ct) b += a.cval[(size_t)ctile * coarse_floats(MODE) + NC * CP * CP + NV * 4 + lane];
+      s_kb[lane] = lane == 3 ? b * b : b;
+    }
+  }
   // coefficients of every row pair: the remainders interpolated in y at the
   // tile's rows, one float4 = two values at two rows
   for (int q = tid; q < (FT / 2) * FP * NC2 * 2; q += FI_THREADS) {
@@ -694,20 +740,22 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
       const float dh = a.dls_h, dl = a.dls_l;
       // which nodes the double-float repair recomputes (see k_map_mixed);
       // the far potentials' kappa and gamma enter by their bounds on the tile
-      if (a.repair_f > 0.f) {
+      if (a.rep_count) {
         bool rep[2], rep_h[2] = {false, false};
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
           const bool in = i < a.nx && jl + h < a.ny;
           const float mg = a.repair_f * (part2(v[NV], h) + S.mag(h)), fx = part2(vh[0], h), fy = part2(vh[1], h);
-          rep[h] = in && fmaf(fx, fx, fy * fy) < mg * mg;
+          rep[h] = in && fmaf(fx, fx, fy * fy) < fmaf(mg, mg, s_kb[3]);
           if (HESS) {
             const float kl = dh * (fabsf(S.value(2, h).hi) + s_kb[0]);
             const float g1l = dh * (fabsf(S.value(3, h).hi) + s_kb[1]), g2l = dh * (fabsf(S.value(4, h).hi) + s_kb[2]);
             const float kap = dh * part2(vh[NV > 2 ? 2 : 0], h), g1 = dh * part2(vh[NV > 3 ? 3 : 0], h),
                         g2 = dh * part2(vh[NV > 4 ? 4 : 0], h);
             const float gm = sqrtf(fmaf(g1, g1, g2 * g2)), gl = sqrtf(fmaf(g1l, g1l, g2l * g2l));
-            rep_h[h] = in && (float)(2.0 * DET_TERM_ERR) * (fabsf(1.f - kap) * kl + gm * (kl + gl)) > (float)DET_REPAIR_ABS;
+            const float om = fabsf(1.f - kap), e1 = a.repair_f > 0.f ? fmaf(om, kl, gm * (kl + gl)) : 0.f;
+            const float e2 = REM_TERM * dh * fmaf(om, s_kb[4], gm * s_kb[5]);
+            rep_h[h] = in && fmaf(e1, e1, e2 * e2) > DET_LIST * DET_LIST;
           }
         }
 #pragma unroll
@@ -753,7 +801,7 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
       }
     }
   }
-  if (POT || !(a.repair_f > 0.f)) return;
+  if (POT || !a.rep_count) return;
   // the nodes to recompute: a tile with many of them goes to the dense tiles
   // (all planes' nodes with it where they are many), the others' to the list
   constexpr int NW = FT * FT / 32;

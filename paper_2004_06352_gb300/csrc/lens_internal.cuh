@@ -425,6 +425,7 @@ DenseRepair dense_repair(const lens_grid *g, const FarPlan &p, bool hess, void *
 int launch_far_repair(const Model *m, const lens_grid *g, const DenseRepair &dense, double dls, void *out, int row0,
                       int rows, int device, cudaStream_t st);
 size_t map_repair_bytes(const lens_grid *g, int rows = -1);
+bool map_needs_list(const lens_ctx *ctx, const Model *m);  // the FP32 terms' repair is on: no map without its list
 int launch_map_fp64(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, bool hess, void *out,
                     cudaStream_t st, int row0 = 0, int rows = -1);
 int map_tile_rows(bool hess);  // rows per CTA tile of the mixed map kernel

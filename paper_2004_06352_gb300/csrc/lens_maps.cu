@@ -851,6 +851,7 @@ int map_tile_rows(bool hess) { return map_threads(hess) / 32 * (hess ? LENS_KP_H
 
 // the list after the counts of listed nodes and of densely listed tiles
 constexpr int REP_HEADER = 4;
+bool map_needs_list(const lens_ctx *ctx, const Model *m) { return ctx->repair_ratio > 0.0 && m->n_light > 0; }
 size_t map_repair_bytes(const lens_grid *g, int rows) {
   return sizeof(int) * ((size_t)g->nx * (size_t)(rows < 0 ? g->ny : rows) + REP_HEADER);
 }
@@ -861,16 +862,19 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
   if (rows < 0) rows = g->ny - row0;
   const long long nodes = (long long)g->nx * rows;
   if (nodes > INT32_MAX) return fail(LENS_EINVAL, "map launch of more than 2^31 points");
-  repair = repair && ctx->repair_ratio > 0.0 && m->n_light > 0;
+  const bool fp32_repair = repair && map_needs_list(ctx, m);
+  repair = fp32_repair || far;  // (the interpolated form's remainders: lens_far.cu)
   CallScratch rs(ctx, st);  // repair list: the counts and up to one entry per node
-  if (repair) {
-    if (repair_mem) {
-      rs.p = nullptr;  // the caller's memory (the request loop's arena)
-    } else {
-      int rc = rs.alloc(map_repair_bytes(g, rows));
-      if (rc) return rc;
-      repair_mem = rs.p;
+  if (repair && !repair_mem) {  // (else the caller's memory: the request loop's arena)
+    const int rc = rs.alloc(map_repair_bytes(g, rows));
+    if (rc && fp32_repair) return rc;
+    repair_mem = rs.p;
+    if (rc) {  // the direct kernel needs none
+      far = nullptr;
+      repair = false;
     }
+  }
+  if (repair) {
     if (cudaMemsetAsync(repair_mem, 0, REP_HEADER * sizeof(int), st) != cudaSuccess)
       return fail(LENS_ECUDA, "cudaMemsetAsync failed");
   }
@@ -897,7 +901,7 @@ int launch_map_mixed(lens_ctx *ctx, const Model *m, const lens_grid *g, double d
   a.tau = 0;
   a.bx = a.by = 0.0;
   a.out64 = nullptr;
-  a.repair = repair ? ctx->repair_ratio : 0.0;
+  a.repair = fp32_repair ? ctx->repair_ratio : 0.0;
   a.repair_f = (float)(2.0 * a.repair);
   a.rep_count = repair ? (int *)repair_mem : nullptr;
   a.rep_list = repair ? (int *)repair_mem + REP_HEADER : nullptr;
