@@ -1221,10 +1221,21 @@ static FarArgs far_args(const Model *m, const lens_grid *g, const FarPlan &p, in
   return a;
 }
 
+// A kernel's shared memory limit: what the largest model takes, whatever this
+// call's takes.  It belongs to the kernel on the device, not to the context, and
+// another context's thread may be between setting it and launching.
+template <typename K>
+static int far_limit(K kern, int mode, int ft, int threads) {
+  const size_t most = far_smem(mode, ft, FAR_MAX_N / 32 + 1, FAR_MAX_N, threads);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+  return e == cudaSuccess ? LENS_OK : fail(LENS_ECUDA, "interpolated map's shared memory: %s", cudaGetErrorString(e));
+}
+
 template <int MODE>
 static int coarse_launch(const FarArgs &a, const FarPlan &p, int n, cudaStream_t st) {
   const size_t smem = far_smem(MODE, 0, a.nw, n, CO_THREADS);
-  cudaFuncSetAttribute(k_far_coarse<MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int rc = far_limit(k_far_coarse<MODE>, MODE, 0, CO_THREADS);
+  if (rc) return rc;
   k_far_coarse<MODE><<<dim3(p.nct, p.ncr), CO_THREADS, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "coarse map level launch: %s", cudaGetErrorString(e));
@@ -1234,7 +1245,8 @@ static int coarse_launch(const FarArgs &a, const FarPlan &p, int n, cudaStream_t
 template <int MODE, int FT, int TH>
 static int fine_launch(const FarArgs &a, int n, cudaStream_t st) {
   const size_t smem = far_smem(MODE, FT, a.nw, n, TH);
-  cudaFuncSetAttribute(k_far_map<MODE, FT, TH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const int rc = far_limit(k_far_map<MODE, FT, TH>, MODE, FT, TH);
+  if (rc) return rc;
   k_far_map<MODE, FT, TH><<<dim3((a.nx + FT - 1) / FT, (a.ny + FT - 1) / FT), TH, smem, st>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "interpolated map launch: %s", cudaGetErrorString(e));
