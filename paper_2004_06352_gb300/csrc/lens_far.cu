@@ -44,6 +44,10 @@
 // below the root of (ratio x magnitude sum)^2 + (those two remainders)^2 -- also
 // in a model without FP32 potentials and with the FP32 terms' repair off.  (The
 // plain sum lists a sixth more nodes of 8192^2 x 2000: 8.8 instead of 7.8 ms.)
+// A potential map is stored in double and its cluster-scale terms are FP64, so
+// its remainders (tens of arcsec^2) are interpolated as pairs, weights and all
+// (in FP32 they left 1.5e-5 arcsec^2 where the members leave none; now 3e-9.
+// 1537 x 1021 x 500 potentials 263 -> 269 us).
 #include <algorithm>
 #include <cmath>
 
@@ -76,6 +80,8 @@ enum FarMode : int { FAR_GRAD = 0, FAR_HESS = 1, FAR_POT = 2 };
 __host__ __device__ constexpr int nval(int mode) { return mode == FAR_HESS ? 5 : mode == FAR_GRAD ? 2 : 1; }
 __host__ __device__ constexpr int ncmp(int mode) { return nval(mode) + (mode == FAR_POT ? 0 : 1); }
 __host__ __device__ constexpr int ncmp2(int mode) { return (ncmp(mode) + 1) / 2; }
+// floats per remainder: a pair for the potential (hi values, then lo)
+__host__ __device__ constexpr int nrem(int mode) { return mode == FAR_POT ? 2 : 1; }
 
 // CTAs per SM of the fine kernel with 128, 256 or 512 threads (launch_far_map)
 __host__ __device__ constexpr int fi_blocks(int mode, int th) { return th == 512 ? 1 : th == 256 ? 2 : mode == FAR_GRAD ? 5 : 4; }
@@ -123,7 +129,7 @@ __device__ const FineTab<64> D_FINE64 = fine_tab<64>();
 // axis, node i, coarse node k
 template <int SUBT>
 struct CoarseTab {
-  float w[SUBT][FP][CP];
+  float w[SUBT][FP][CP], wlo[SUBT][FP][CP];  // (wlo: the potential's)
 };
 template <int FT, int SUBT>
 constexpr CoarseTab<SUBT> coarse_tab() {
@@ -137,6 +143,7 @@ constexpr CoarseTab<SUBT> coarse_tab() {
         for (int l = 0; l < CP; ++l)
           if (l != k) v *= (x - ZC512[l]) / (double)(ZC512[k] - ZC512[l]);
         t.w[c][i][k] = (float)v;
+        t.wlo[c][i][k] = (float)(v - (double)t.w[c][i][k]);
       }
   return t;
 }
@@ -150,6 +157,7 @@ template <>
 __device__ __forceinline__ const FineTab<32> &fine_table<32>() { return D_FINE32; }
 template <>
 __device__ __forceinline__ const FineTab<64> &fine_table<64>() { return D_FINE64; }
+// CoarseTab::w of the table with `sub` fine tiles per axis (wlo follows it)
 template <int FT>
 __device__ __forceinline__ const float *coarse_weights(int sub) {
   if (FT == 32)
@@ -174,7 +182,7 @@ struct FarArgs {
   float thr_c, thr_ch, thr_f, thr_fh;  // squared psi beyond which a potential is far: coarse / fine, FP32 / cluster-scale
   // coarse level: tile (0, 0) covers the grid's first nodes
   int ct, nct;       // nodes a side (0: no coarse level), tiles per row
-  float *cval;       // per coarse tile: remainders [ncmp][CP * CP], planes [nval][4], s_kb [KB]
+  float *cval;       // per coarse tile: remainders [nrem][ncmp][CP * CP], planes [nval][4], s_kb [KB]
   unsigned *cmask;   // per coarse tile: nw words, bit set = left to the fine level
   float *out;
   double *out64;
@@ -188,7 +196,7 @@ struct FarArgs {
 };
 
 constexpr int KB = 6;  // a tile's s_kb (repair_bound)
-__host__ __device__ constexpr int coarse_floats(int mode) { return ncmp(mode) * CP * CP + nval(mode) * 4 + KB; }
+__host__ __device__ constexpr int coarse_floats(int mode) { return nrem(mode) * ncmp(mode) * CP * CP + nval(mode) * 4 + KB; }
 
 // Is the potential far from a tile centred at (dx, dy) from it?
 __device__ __forceinline__ bool far32(const float4 *r4, float dX, float dY, float thr) {
@@ -431,6 +439,14 @@ __device__ __forceinline__ void node_sums(const FarArgs &a, const unsigned short
   }
 }
 
+// acc + (w + wlo) (f + flo), pairs
+__device__ __forceinline__ df fma_pair(float w, float wlo, float f, float flo, df acc) {
+  const float p = __fmul_rn(w, f);
+  const float e = fmaf(wlo, f, fmaf(w, flo, fmaf(w, f, -p)));
+  const df s = two_sum(acc.hi, p);
+  return {s.hi, acc.lo + (s.lo + e)};
+}
+
 // Plane of value c: the middle node's value and slopes (per grid step)
 // between the outermost nodes of the middle row and column.
 template <int P>
@@ -458,7 +474,7 @@ __device__ __forceinline__ float repair_bound(const float *kb, const float *f, i
 
 template <int MODE>
 __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
-  constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), SPLITS = CO_THREADS / (NODES / 2);
+  constexpr int NODES = CP * CP, NC = ncmp(MODE), NV = nval(MODE), NR = nrem(MODE) * NC, SPLITS = CO_THREADS / (NODES / 2);
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);
   float4 *s_off = s_rec + CO_CH * REC_STRIDE4;
@@ -502,15 +518,16 @@ __global__ void __launch_bounds__(CO_THREADS, 2) k_far_coarse(const FarArgs a) {
       d = df_sub(d, df{p.z * zy, 0.f});
       r = d.hi + d.lo;
       s_val[q].x = r;
+      if (MODE == FAR_POT) o[NC * NODES + q] = (d.hi - r) + d.lo;
     }
     o[q] = r;
   }
-  if (tid < NV * 4) o[NC * NODES + tid] = reinterpret_cast<const float *>(s_plane)[tid];
+  if (tid < NV * 4) o[NR * NODES + tid] = reinterpret_cast<const float *>(s_plane)[tid];
   if (MODE == FAR_POT) return;
   __syncthreads();
   if (tid < 32) {
     const float b = repair_bound<MODE, NODES>(s_kb, reinterpret_cast<const float *>(s_val), 2, tid);
-    if (tid < KB) o[NC * NODES + NV * 4 + tid] = b;
+    if (tid < KB) o[NR * NODES + NV * 4 + tid] = b;
   }
 }
 
@@ -525,6 +542,7 @@ template <int MODE, int FT, int FI_THREADS>
 __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far_map(const FarArgs a) {
   constexpr bool HESS = MODE == FAR_HESS, POT = MODE == FAR_POT;
   constexpr int NODES = FP * FP, NC = ncmp(MODE), NV = nval(MODE), NC2 = ncmp2(MODE), SPLITS = FI_THREADS / (NODES / 2);
+  constexpr int NR = nrem(MODE) * NC, CV_PLANE = NR * CP * CP;  // floats of a coarse tile's values before its planes
   extern __shared__ __align__(16) unsigned char s_dyn[];
   float4 *s_rec = reinterpret_cast<float4 *>(s_dyn);                      // [FF_CH][REC_STRIDE4]
   float4 *s_off = s_rec + FF_CH * REC_STRIDE4;                            // [FF_CH]
@@ -534,11 +552,12 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
   unsigned *s_far = reinterpret_cast<unsigned *>(s_val + NODES * NC);
   unsigned *s_near = s_far + a.nw;
   unsigned short *s_list = reinterpret_cast<unsigned short *>(s_near + 3 * a.nw);
-  float *s_tmp = reinterpret_cast<float *>(s_part);  // coarse level: [NC][CP * CP] values, [NC][FP][CP] (after node_sums)
-  float *s_rem = s_tmp;                              // then the remainders [NC][NODES]
+  float *s_tmp = reinterpret_cast<float *>(s_part);  // coarse level: [NR][CP * CP] values, [NR][FP][CP] (after node_sums)
+  float *s_rem = s_tmp;                              // then the remainders [NR][NODES]
   __shared__ float2 s_nx[FP], s_ny[FP];
   __shared__ float2 s_cx[FT], s_ry[FT];  // offsets of the tile's columns and rows from its centre, hi/lo
   __shared__ float s_L[FT][FP + 1], s_xi[FP];  // (odd stride: lanes read a column each)
+  __shared__ float s_Ll[POT ? FT : 1][FP + 1];
   __shared__ float4 s_T;                 // the centre, hi/lo
   __shared__ unsigned s_m[FT * FT / 32], s_mh[HESS ? FT * FT / 32 : 1];  // nodes to recompute: deflection alone / all planes
   __shared__ double s_tau[POT ? 2 : 1][POT ? FT : 1];  // half the squared offsets from beta
@@ -569,7 +588,10 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
     }
   }
   if (tid < KB) s_kb[tid] = 0.f;
-  for (int q = tid; q < FT * FP; q += FI_THREADS) s_L[q / FP][q % FP] = (&fine_table<FT>().w[0][0])[q];
+  for (int q = tid; q < FT * FP; q += FI_THREADS) {
+    s_L[q / FP][q % FP] = (&fine_table<FT>().w[0][0])[q];
+    if (POT) s_Ll[POT ? q / FP : 0][q % FP] = (&fine_table<FT>().wlo[0][0])[q];
+  }
   __syncthreads();
   const df Tx = {s_T.x, s_T.y}, Ty = {s_T.z, s_T.w};
   const int ctile = a.ct ? (j0 / a.ct) * a.nct + i0 / a.ct : 0;
@@ -583,28 +605,44 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
     const int sub = a.ct / FT, cx = (i0 % a.ct) / FT, cy = (j0 % a.ct) / FT;
     const float *W = coarse_weights<FT>(sub);
     const float *Wx = W + cx * FP * CP, *Wy = W + cy * FP * CP;
-    float *s_t1 = s_tmp + NC * CP * CP;
-    for (int q = tid; q < NC * CP * CP; q += FI_THREADS) s_tmp[q] = cv[q];
+    const int wlo = sub * FP * CP;  // from a weight to its low part
+    float *s_t1 = s_tmp + NR * CP * CP;
+    for (int q = tid; q < NR * CP * CP; q += FI_THREADS) s_tmp[q] = cv[q];
     __syncthreads();
     for (int q = tid; q < NC * CP * FP; q += FI_THREADS) {  // (c, coarse row, fine column)
       const int i = q % FP, cr = q / FP;
       const float *f = s_tmp + cr * CP;
-      float v = 0.f;
+      if constexpr (POT) {
+        df v = {0.f, 0.f};
 #pragma unroll
-      for (int k = 0; k < CP; ++k) v = fmaf(Wx[i * CP + k], f[k], v);
-      s_t1[q] = v;
+        for (int k = 0; k < CP; ++k) v = fma_pair(Wx[i * CP + k], Wx[wlo + i * CP + k], f[k], f[NC * CP * CP + k], v);
+        v = fast_two_sum(v.hi, v.lo);
+        s_t1[q] = v.hi;
+        s_t1[NC * CP * FP + q] = v.lo;
+      } else {
+        float v = 0.f;
+#pragma unroll
+        for (int k = 0; k < CP; ++k) v = fmaf(Wx[i * CP + k], f[k], v);
+        s_t1[q] = v;
+      }
     }
     __syncthreads();
     const float bx0 = FT * (cx + 0.5f) - 0.5f * a.ct, by0 = FT * (cy + 0.5f) - 0.5f * a.ct;
     for (int q = tid; q < NC * NODES; q += FI_THREADS) {
       const int c = q / NODES, node = q % NODES, i = node % FP, j = node / FP;
-      float v = 0.f;
+      df v = {0.f, 0.f};
 #pragma unroll
-      for (int k = 0; k < CP; ++k) v = fmaf(Wy[j * CP + k], s_t1[(c * CP + k) * FP + i], v);
+      for (int k = 0; k < CP; ++k) {
+        const float *f = s_t1 + (c * CP + k) * FP + i;
+        if constexpr (POT)
+          v = fma_pair(Wy[j * CP + k], Wy[wlo + j * CP + k], f[0], f[NC * CP * FP], v);
+        else
+          v.hi = fmaf(Wy[j * CP + k], f[0], v.hi);
+      }
       df d = {s_val[q].x, s_val[q].y};
-      d = df_add(d, df{v, 0.f});
+      d = df_add(d, v);
       if (c < NV) {
-        const float *p = cv + NC * CP * CP + c * 4;
+        const float *p = cv + CV_PLANE + c * 4;
         d = df_add(d, df{p[0], 0.f});
         d = df_add(d, df{p[1] * (bx0 + s_xi[i]), 0.f});
         d = df_add(d, df{p[2] * (by0 + s_xi[j]), 0.f});
@@ -625,6 +663,7 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
       d = df_sub(d, df{p.y * s_xi[node % FP], 0.f});
       d = df_sub(d, df{p.z * s_xi[node / FP], 0.f});
       r = d.hi + d.lo;
+      if (POT) s_rem[NC * NODES + q] = (d.hi - r) + d.lo;
     }
     s_rem[q] = r;
   }
@@ -632,7 +671,7 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
   if (!POT && warp == 0) {
     float b = repair_bound<MODE, NODES>(s_kb, s_rem, 1, lane);
     if (lane < KB) {
-      if (a.ct) b += a.cval[(size_t)ctile * coarse_floats(MODE) + NC * CP * CP + NV * 4 + lane];
+      if (a.ct) b += a.cval[(size_t)ctile * coarse_floats(MODE) + CV_PLANE + NV * 4 + lane];
       s_kb[lane] = lane == 3 ? b * b : b;
     }
   }
@@ -641,7 +680,19 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
   for (int q = tid; q < (FT / 2) * FP * NC2 * 2; q += FI_THREADS) {
     const int c = q % (2 * NC2), i = q / (2 * NC2) % FP, rp = q / (2 * NC2 * FP);
     float u = 0.f, v = 0.f;
-    if (c < NC) {
+    if constexpr (POT) {  // c = 1: the low parts
+      df x = {0.f, 0.f}, y = {0.f, 0.f};
+#pragma unroll
+      for (int j = 0; j < FP; ++j) {
+        const float f = s_rem[j * FP + i], g = s_rem[NODES + j * FP + i];
+        x = fma_pair(s_L[2 * rp][j], s_Ll[POT ? 2 * rp : 0][j], f, g, x);
+        y = fma_pair(s_L[2 * rp + 1][j], s_Ll[POT ? 2 * rp + 1 : 0][j], f, g, y);
+      }
+      x = fast_two_sum(x.hi, x.lo);
+      y = fast_two_sum(y.hi, y.lo);
+      u = c ? x.lo : x.hi;
+      v = c ? y.lo : y.hi;
+    } else if (c < NC) {
 #pragma unroll
       for (int j = 0; j < FP; ++j) {
         const float f = s_rem[c * NODES + j * FP + i];
@@ -682,6 +733,14 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
 #pragma unroll
       for (int c = 0; c < NC2; ++c) {
         const float4 t = s_c[(rp * FP + k) * NC2 + c];
+        if constexpr (POT) {  // v[0], v[1]: hi and lo sums of pairs
+          const float2 f = make_float2(t.x, t.y), p = mul2(L, f);
+          const float2 e = fma2(dup2(s_Ll[POT ? m : 0][k]), f, fma2(L, make_float2(t.z, t.w), fma2(L, f, neg2(p))));
+          const df2 r = two_sum2(v[0], p);
+          v[0] = r.hi;
+          v[1] = add2(v[1], add2(r.lo, e));
+          continue;
+        }
         v[2 * c] = fma2(L, make_float2(t.x, t.y), v[2 * c]);
         v[2 * c + 1] = fma2(L, make_float2(t.z, t.w), v[2 * c + 1]);
       }
@@ -697,8 +756,12 @@ __global__ void __launch_bounds__(FI_THREADS, fi_blocks(MODE, FI_THREADS)) k_far
       const df n0 = S.value(c, 0), n1 = S.value(c, 1);
       const df2 z = two_sum2(y.hi, make_float2(n0.hi, n1.hi));
       float2 lo = add2(add2(y.lo, dup2(x.lo)), add2(z.lo, make_float2(n0.lo, n1.lo)));
-      lo = add2(lo, v[c]);
-      const df2 r = two_sum2(z.hi, lo);
+      df2 w = {z.hi, v[c]};
+      if constexpr (POT) {
+        w = two_sum2(z.hi, v[0]);
+        w.lo = add2(w.lo, v[1]);
+      }
+      const df2 r = two_sum2(w.hi, add2(lo, w.lo));
       vh[c] = r.hi;
       vl[c] = r.lo;
     }
@@ -1026,7 +1089,7 @@ size_t far_smem(int mode, int ft, int nw, int n, int threads = 256) {
   size_t b = sizeof(float4) * (size_t)(coarse ? CO_CH : FF_CH) * (REC_STRIDE4 + 1);
   if (!coarse) b += sizeof(float4) * (ft / 2) * FP * ncmp2(mode);
   // the partial sums' space also holds the coarse tile's values (fine kernel)
-  const size_t part = std::max(sizeof(float2) * splits * nodes * nc, coarse ? 0 : sizeof(float) * nc * (CP * CP + CP * FP));
+  const size_t part = std::max(sizeof(float2) * splits * nodes * nc, coarse ? 0 : sizeof(float) * nrem(mode) * nc * (CP * CP + CP * FP));
   b += (part + 15) / 16 * 16 + sizeof(float2) * nodes * nc;
   b += sizeof(unsigned) * 4 * (size_t)nw + sizeof(unsigned short) * (size_t)n;
   return (b + 15) / 16 * 16;
