@@ -347,11 +347,14 @@ int lens_chi2_source_nocache(lens_ctx *ctx, lens_cset_t cset, const double *d_pa
                              double *d_chi2, void *stream);
 
 /* Autotuner of lens_chi2_source's launch shape (threads per CTA x CTAs per
- * SM, 8 candidates) for this constraint set: runs each candidate on d_params
- * (DEVICE [P][14]) into d_chi2 (DEVICE [P]) on `stream`, times it (best of
- * 3 after a warm-up), and keeps the fastest for every later lens_chi2_source
- * call on the set.  Synchronous.  *chosen (may be NULL) = threads*100 +
- * CTAs-per-SM cap (0 = no cap); *best_ms (may be NULL) its time. */
+ * SM, 8 candidates) for this constraint set: runs the untuned rule and each
+ * candidate on d_params (DEVICE [P][14]) into d_chi2 (DEVICE [P]) on
+ * `stream`, times it (best of 3 after a warm-up), and keeps the fastest
+ * candidate for every later lens_chi2_source call on the set, or the untuned
+ * rule (whose shape follows each call's P and variant) where no candidate is
+ * 2 % faster.  Synchronous.  *chosen (may be NULL) = threads*100 +
+ * CTAs-per-SM cap (0 = no cap) of the fastest candidate; *best_ms (may be
+ * NULL) the time of what is kept. */
 int lens_chi2_autotune(lens_ctx *ctx, lens_cset_t cset, const double *d_params, int32_t P, double *d_chi2,
                        void *stream, int32_t *chosen, float *best_ms);
 
