@@ -9,8 +9,8 @@
 //               (2) admits queued requests onto free slots while the arena
 //               can hold their device buffers (inputs, outputs, scratch),
 //               shortest expected work first with ageing: each request's
-//               rank is its expected GPU time (from the measured rates of
-//               its kernels) minus the time it has waited, so a large map
+//               rank is its expected time (from the measured rates of its
+//               kernels and of the result's copy) minus the time it has waited, so a large map
 //               waits at most about its own run time behind smaller work.
 //               A request that does not fit is skipped so others can start;
 //               once the first-ranked request has been skipped MAX_SKIPS
@@ -89,23 +89,26 @@ struct Req {
   int32_t batch = 0;
   FarPlan far;  // maps: the interpolated form's plan, its coarse level after the repair list
   double t_submit = 0, t_admit = 0;
-  double cost_ms = 0;  // expected GPU time
+  double cost_ms = 0;  // expected time
   int skips = 0;
 };
 
-// Expected GPU time of a request from the rates measured on GB300 (2048^2 x
-// 1000 maps: 3.1e11 Hessian / 4.6e11 deflection / 3.5e9 FP64 point-potential
-// pairs per s; source-plane chi2: 2.8e9 image evaluations per s; image-plane
-// chi2: 1.3e10 grid cells x sets per s).  Only the order matters.
-double expected_ms(const lens_request &r, int32_t n_potentials, int32_t nimg) {
-  const double cells = (double)r.grid.nx * r.grid.ny;
+// Expected time of a request from the rates measured on GB300, kernels and
+// result copy (192 GB/s).  Interpolated maps by their plan's cost: 1.2e8 to
+// 3.6e8 of its units per ms over grids of 512^2 to 8192^2 and 10 to 2000
+// potentials.  Direct maps 4.2e8 (Hessian, 2048^2 x 1000 in 10 ms) or 6.3e8
+// point-potential pairs per ms, FP64 4.5e6 or 5.5e6; source-plane chi2 5.1e6
+// image evaluations (4096 x 372 in 0.30 ms); image-plane chi2 3.3e7 grid cells
+// x sets (256 x 1024^2 in 8.2 ms).  Only the order matters.
+double expected_ms(const lens_request &r, const FarPlan &far, int32_t n_potentials, int32_t nimg, size_t out_bytes) {
+  const double cells = (double)r.grid.nx * r.grid.ny, copy = (double)out_bytes / 1.92e8;
   if (r.kind == LENS_REQ_MAP) {
     const double pairs = cells * n_potentials;
-    if (r.precision == LENS_FP64) return pairs / 3.5e6;
-    return pairs / (r.hessian ? 3.1e8 : 4.6e8);
+    if (r.precision == LENS_FP64) return copy + pairs / (r.hessian ? 4.5e6 : 5.5e6);
+    return copy + (far.use ? far.cost * cells / 1.7e8 : pairs / (r.hessian ? 4.2e8 : 6.3e8));
   }
-  if (r.kind == LENS_REQ_CHI2_SOURCE) return (double)r.P * nimg / 2.8e6;
-  return (double)r.P * cells / 1.3e7;
+  if (r.kind == LENS_REQ_CHI2_SOURCE) return copy + (double)r.P * nimg / 5.1e6;
+  return copy + (double)r.P * cells / 3.3e7;
 }
 
 struct Slot {
@@ -274,10 +277,10 @@ int lens_server_submit(lens_server *s, const lens_request *r, int64_t *ticket) {
   }
   if (!rc) {
     if (r->kind == LENS_REQ_MAP) {
-      q->cost_ms = expected_ms(*r, find_model(ctx, r->handle)->n, 0);
+      q->cost_ms = expected_ms(*r, q->far, find_model(ctx, r->handle)->n, 0, q->out_bytes);
     } else {
       const CSet *c = find_cset(ctx, r->handle);
-      q->cost_ms = expected_ms(*r, 0, c->nimg);
+      q->cost_ms = expected_ms(*r, q->far, 0, c->nimg, q->out_bytes);
     }
     q->total = up(q->out_bytes) + up(q->in_bytes) + up(q->scratch_bytes);
     if (q->total > s->pool_bytes)
