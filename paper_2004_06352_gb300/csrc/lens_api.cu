@@ -627,7 +627,7 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   const int planes = hess ? 6 : 2, nx = grid->nx, ny = grid->ny;
   FarPlan plan;
   if (precision == LENS_MIXED) plan = plan_far(ctx, m, grid, hess);
-  const int tile = plan.use ? plan.ft : map_tile_rows(hess);
+  int tile = plan.use ? plan.ft : map_tile_rows(hess);
   // Bands, each a whole number of tiles.  A band costs launches and underfilled
   // kernels (~20 us), fewer bands leave more of the copy (192 GB/s) after the
   // last kernel; two overlap nothing (both streams end together).  Time with
@@ -641,6 +641,16 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
   const size_t row_bytes = (size_t)nx * planes * esize, map_bytes = row_bytes * ny;
   int rows = band_rows(ctx->budget ? 8 : map_bytes <= (8u << 20) ? 1 : map_bytes <= (128u << 20) ? 3 : 6);
   size_t band_bytes = rows * row_bytes;
+  if (ctx->budget && plan.use) {
+    // the direct kernel's tiles make lower bands: they where only those fit
+    const size_t used = ctx->used - std::min(ctx->used, ctx->band_bytes + ctx->cached_bytes);
+    if (used + std::max(ctx->band_bytes, 2 * band_bytes) + map_repair_bytes(grid, rows) > ctx->budget) {
+      plan = FarPlan();
+      tile = map_tile_rows(hess);
+      rows = band_rows(8);
+      band_bytes = rows * row_bytes;
+    }
+  }
   if (ctx->band_bytes < 2 * band_bytes) {
     if (ctx->band) {
       dev_free(ctx, ctx->band, ctx->band_bytes);  // after the bands in flight have left
