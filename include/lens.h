@@ -191,7 +191,11 @@ int lens_model_release(lens_ctx *ctx, lens_model_t model);
  * interpolate it over the tiles far from it where that is cheaper, within the
  * same error bounds as evaluating every pair.  The interpolation's working
  * memory (stream ordered; about 20 MB for a 2048 x 2048 Hessian map) is
- * optional: without it every pair is evaluated. */
+ * optional: without room for the part that shares the repair of many listed
+ * nodes of a tile (2.1 KB per 32 x 32 or 64 x 64 tile, 5 KB with the Hessian)
+ * they are recomputed one by one, without room for the rest, or for a model of
+ * more than 16384 potentials, every pair is evaluated.  Maps of more than
+ * 65536 tiles do without the shared repair. */
 
 /* Deflection map (Sec. 4.1, Eq. 10; lens equation Sec. 2.1 Eq. 1):
  * d_out holds 2 planes [2][ny][nx] -- alpha_x, alpha_y -- of float

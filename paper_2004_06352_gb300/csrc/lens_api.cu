@@ -574,7 +574,10 @@ static int map_common(lens_ctx *ctx, lens_model_t model, const lens_grid *grid, 
       if (map_needs_list(ctx, m)) return rc;
       plan = FarPlan();
     }
-    if (plan.use && plan.bytes && far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
+    if (plan.use && far.alloc(plan.bytes) != LENS_OK) {
+      plan.drop_dense();
+      if (far.alloc(plan.bytes) != LENS_OK) plan = FarPlan();  // no room: the direct kernel
+    }
     if (plan.use && (rc = launch_far_coarse(m, grid, plan, hess, far.p, st))) return rc;
     return launch_map_mixed(ctx, m, grid, dls_ds, hess, d_out, st, 0, -1, true, list.p, plan.use ? &plan : nullptr,
                             far.p, plan.rep_bytes ? (char *)far.p + plan.bytes - plan.rep_bytes : nullptr);
@@ -695,12 +698,17 @@ static int map_host_common(lens_ctx *ctx, lens_model_t model, const lens_grid *g
       far.release();
     }
   } free_far{ctx, far};
-  const size_t far_bytes = plan.bytes + plan.rep_bytes;  // the dense tiles' arrays for each band stream
+  // (beside the bands' repair lists; the dense tiles' arrays for each band stream)
+  auto room = [&]() {
+    const size_t n = plan.bytes + plan.rep_bytes;
+    return (!ctx->budget || ctx->used + n + map_repair_bytes(grid, rows) <= ctx->budget) && far.alloc(n) == LENS_OK;
+  };
+  if (plan.use && !room()) {
+    plan.drop_dense();
+    if (!room()) plan = FarPlan();  // the direct kernel, whose tiles divide the bands too
+  }
   if (plan.use) {
-    const bool room = !ctx->budget || ctx->used + far_bytes + map_repair_bytes(grid, rows) <= ctx->budget;
-    if (!room || far.alloc(far_bytes) != LENS_OK) {
-      plan = FarPlan();  // no room beside the bands' repair lists: the direct kernel, whose tiles divide the bands too
-    } else if (far_bytes) {
+    if (far.p) {
       if ((rc = launch_far_coarse(m, grid, plan, hess, far.p, ctx->pipe_cs[0]))) return rc;
       LENS_CUDA_TRY(cudaEventRecord(ctx->pipe_start, ctx->pipe_cs[0]));
       LENS_CUDA_TRY(cudaStreamWaitEvent(ctx->pipe_cs[1], ctx->pipe_start, 0));

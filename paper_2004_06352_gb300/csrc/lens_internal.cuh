@@ -393,6 +393,11 @@ struct FarPlan {
   // DenseRepair arrays, which lie at byte `bytes - rep_bytes` of the plan's memory
   int rep_cap = 0;
   size_t rep_bytes = 0;
+  void drop_dense() {  // without room for those arrays: every node is listed
+    bytes -= rep_bytes;
+    rep_bytes = 0;
+    rep_cap = 0;
+  }
 };
 // Tiles of the interpolated maps in which so many nodes are to be recomputed
 // in double-float that the far potentials are evaluated at the tile's FAR_P x

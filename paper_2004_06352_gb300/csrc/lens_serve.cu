@@ -242,9 +242,10 @@ int lens_server_submit(lens_server *s, const lens_request *r, int64_t *ticket) {
     if (!rc && r->precision == LENS_MIXED) {
       q->scratch_bytes = map_repair_bytes(&r->grid);
       q->far = plan_far(ctx, find_model(ctx, r->handle), &r->grid, r->hessian != 0);
-      const size_t with = up(q->scratch_bytes) + up(q->far.bytes);
-      if (up(q->out_bytes) + with <= s->pool_bytes)
-        q->scratch_bytes = with;
+      const size_t need = up(q->out_bytes) + up(q->scratch_bytes);
+      if (need + up(q->far.bytes) > s->pool_bytes) q->far.drop_dense();
+      if (need + up(q->far.bytes) <= s->pool_bytes)
+        q->scratch_bytes = up(q->scratch_bytes) + up(q->far.bytes);
       else if (q->far.bytes)
         q->far = FarPlan();  // only the direct kernel fits the pool
     }

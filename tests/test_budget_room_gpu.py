@@ -32,3 +32,27 @@ def test_streamed_map_in_small_bands(lens):
         ctx.wait()
     dev = dev.cpu()
     assert float((host - dev).abs().max()) <= 2e-6 * float(dev.abs().max())
+
+
+@pytest.mark.parametrize("host", [False, True])
+def test_interpolated_without_dense_repair(lens, host):
+    """Room for the coarse level but not for the dense repair's arrays: still
+    the interpolated form (the same bits but at repaired nodes)."""
+    m, g = I.cfg2_model(seed=10, n_members=400), I.grid(1024)
+    out, ref = torch.empty((2, 1024, 1024), pin_memory=True), torch.empty((2, 1024, 1024), device=DEV)
+    used = uploaded(lens, m)
+    with lens.Context(0) as ctx:
+        ctx.grad_map(ctx.model_upload(m), g, 1.0, lens.LENS_MIXED, ref)
+        ctx.wait()
+    room = (2 << 20) + (2 * 8 * 128 * 1024 + 4 * 128 * 1024 if host else 4 * 1024 * 1024) + 4096
+    with lens.Context(0, mem_budget_bytes=used + room) as ctx:
+        mid = ctx.model_upload(m)
+        if host:
+            ctx.grad_map_host(mid, g, 1.0, lens.LENS_MIXED, out)
+        else:
+            d = torch.empty((2, 1024, 1024), device=DEV)
+            ctx.grad_map(mid, g, 1.0, lens.LENS_MIXED, d)
+            out = d
+        ctx.wait()
+    same = (out.cpu() == ref.cpu()).double().mean()
+    assert same > 0.99, float(same)
