@@ -376,8 +376,9 @@ int lens_chi2_autotune(lens_ctx *ctx, lens_cset_t cset, const double *d_params, 
  * (and clears).  At most 1024 sources per constraint set (LENS_EINVAL
  * beyond, nothing launched).  The first call on a (constraint set, grid)
  * pair computes and keeps the static potentials' deflection on the grid (8
- * bytes per node) and a model of it per 8 x 8 cells (0.5 bytes per node;
- * without room for it the search is slower, with the same result); each
+ * bytes per node) and a model of it per 8 x 8 cells (0.5 bytes per node; in a
+ * context with a memory budget each call's working memory instead; without
+ * room for it the search is slower, with the same result); each
  * call's candidate buffers are working memory allocated and freed in
  * stream order on `stream`. */
 int lens_chi2_image(lens_ctx *ctx, lens_cset_t cset, const lens_grid *grid, const double *d_params, int32_t P,

@@ -2268,8 +2268,10 @@ int launch_grid_planes(const GridCache *gc, cudaStream_t st) {
 
 // Static deflection of the constraint set's model on grid g (LENS_MIXED map
 // of the static potentials, D_ls/D_s = 1) and the search's block planes,
-// enqueued on st and kept with the constraint set; without room for the
-// planes the deflection alone (the search then culls nothing).
+// enqueued on st and kept with the constraint set; the deflection alone
+// without room for the planes, and under a memory budget, where they are
+// working memory of the calls (a grid, or the last call's buffers, may need
+// what they take).
 int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st) {
   GridCache n;
   n.xmin = g->xmin;
@@ -2280,7 +2282,7 @@ int build_grid_cache(lens_ctx *ctx, CSet *c, const lens_grid *g, cudaStream_t st
   n.ny = g->ny;
   const size_t alpha_bytes = (2 * sizeof(float) * (size_t)g->nx * g->ny + 255) & ~(size_t)255;
   n.bytes = alpha_bytes + grid_plane_bytes(g->nx, g->ny);
-  int rc = dev_alloc(ctx, (void **)&n.alpha32, n.bytes);
+  int rc = ctx->budget ? LENS_ENOMEM : dev_alloc(ctx, (void **)&n.alpha32, n.bytes);
   if (!rc) {
     n.plane = (float *)((char *)n.alpha32 + alpha_bytes);
   } else {
@@ -2325,8 +2327,15 @@ int launch_chi2_image(lens_ctx *ctx, const Model *m, CSet *c, const lens_grid *g
   }
   const int32_t batch = std::min<int32_t>(IMG_BATCH, P);
   CallScratch scratch(ctx, st);  // this call's candidate buffers, on its own stream
-  const int rc = scratch.alloc(chi2_image_scratch_bytes(c, batch));
+  int rc = scratch.alloc(chi2_image_scratch_bytes(c, batch));
   if (rc) return rc;
+  GridCache with = *gc;  // the planes of this call where they are not kept
+  CallScratch planes(ctx, st);
+  if (!gc->plane && planes.alloc(grid_plane_bytes(g->nx, g->ny)) == LENS_OK) {
+    with.plane = (float *)planes.p;
+    if ((rc = launch_grid_planes(&with, st))) return rc;
+    gc = &with;
+  }
   return run_chi2_image(ctx, c, gc, d_params, P, d_chi2, d_nfound, scratch.p, batch, st, d_images, img_max,
                         d_img_count);
 }

@@ -86,6 +86,7 @@ struct Req {
   lens_request r{};
   std::vector<double> params;
   size_t out_bytes = 0, in_bytes = 0, scratch_bytes = 0, total = 0, off = 0;
+  size_t plane_off = 0;  // image-plane chi2: the search's planes in the scratch (0: the grid's own)
   int32_t batch = 0;
   FarPlan far;  // maps: the interpolated form's plan, its coarse level after the repair list
   double t_submit = 0, t_admit = 0;
@@ -167,8 +168,13 @@ static int launch_req(lens_server *s, Slot &sl, Req *q) {
     } else {
       const GridCache *gc = find_grid_cache(c, &r.grid);
       if (!gc) return fail(LENS_ENOTFOUND, "grid cache missing");
-      void *scratch = base + up(q->out_bytes) + up(q->in_bytes);
-      rc = run_chi2_image(ctx, c, gc, d_params, r.P, (double *)base, nullptr, scratch, q->batch, st);
+      char *scratch = base + up(q->out_bytes) + up(q->in_bytes);
+      GridCache with = *gc;
+      if (q->plane_off) {
+        with.plane = (float *)(scratch + q->plane_off);
+        rc = launch_grid_planes(&with, st);
+      }
+      if (!rc) rc = run_chi2_image(ctx, c, &with, d_params, r.P, (double *)base, nullptr, scratch, q->batch, st);
     }
   }
   if (rc) return rc;
@@ -271,6 +277,13 @@ int lens_server_submit(lens_server *s, const lens_request *r, int64_t *ticket) {
         }
         q->batch = std::min<int32_t>(r->P, 16);
         q->scratch_bytes = chi2_image_scratch_bytes(c, q->batch);
+        // the search's planes of the grid after them, where they are not kept with it
+        const GridCache *gc = rc ? nullptr : find_grid_cache(c, &r->grid);
+        const size_t with = up(q->scratch_bytes) + up(grid_plane_bytes(r->grid.nx, r->grid.ny));
+        if (gc && !gc->plane && up(q->out_bytes) + up(q->in_bytes) + with <= s->pool_bytes) {
+          q->plane_off = up(q->scratch_bytes);
+          q->scratch_bytes = with;
+        }
       }
     }
   } else {

@@ -56,3 +56,31 @@ def test_interpolated_without_dense_repair(lens, host):
         ctx.wait()
     same = (out.cpu() == ref.cpu()).double().mean()
     assert same > 0.99, float(same)
+
+
+def test_image_search_keeps_the_grid_alone(lens):
+    """Under a budget the search's model of a grid is working memory: a grid
+    costs its 8 bytes per node, and the results are the same."""
+    m, cons = I.cfg2_model(n_members=40), I.random_constraints(8, seed=9, field=30)
+    g, P = I.grid(500), 3
+    p = torch.tensor(I.perturbed_params(m, (0, 1), P, seed=2), device=DEV)
+    res = []
+    for budget in (0, 1 << 30):
+        with lens.Context(0, mem_budget_bytes=budget) as ctx:
+            cs = ctx.cset_create(ctx.model_upload(m), cons, (0, 1))
+            chi2, found = torch.empty(P, dtype=torch.float64, device=DEV), torch.empty((P, 8), dtype=torch.int32, device=DEV)
+            used = ctx.mem_used()
+            ctx.chi2_image(cs, g, p, P, chi2, found)
+            ctx.wait()
+            kept = ctx.mem_used() - used
+            if budget:
+                assert kept <= 8 * 500 * 500 + 256, kept
+                srv = lens.Server(ctx, slots=1, pool_bytes=64 << 20)
+                r = torch.empty(P, dtype=torch.float64, pin_memory=True)
+                srv.submit_chi2_image(cs, g, p.cpu().numpy(), r)
+                while not srv.progress():
+                    pass
+                srv.close()
+                assert torch.equal(r, chi2.cpu())
+            res.append((chi2.cpu(), found.cpu()))
+    assert torch.equal(res[0][0], res[1][0]) and torch.equal(res[0][1], res[1][1])
