@@ -490,6 +490,9 @@ int lens_selftest_wait(lens_ctx *ctx, int32_t polls, void *stream);
  * normal values), d_out (device, [4][n]) receives rcp, 1/x, rsqrt, CUDA
  * rsqrt.  Asynchronous on `stream`. */
 int lens_selftest_math(lens_ctx *ctx, const double *d_x, int32_t n, double *d_out, void *stream);
+/* The same for those of the LENS_FP64 maps (one third-order step): d_out
+ * [3][n] receives 1/x, 1/sqrt(x), sqrt(x). */
+int lens_selftest_math_maps(lens_ctx *ctx, const double *d_x, int32_t n, double *d_out, void *stream);
 
 /* Wait until all work enqueued on `stream` has finished, polling without
  * blocking the thread for more than timeout_ms (>= 0) milliseconds.

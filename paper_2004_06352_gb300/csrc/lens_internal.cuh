@@ -438,7 +438,7 @@ int map_tile_rows(bool hess);  // rows per CTA tile of the mixed map kernel
 int launch_pot_map(lens_ctx *ctx, const Model *m, const lens_grid *g, double dls, int32_t precision,
                    const double *beta, void *out, cudaStream_t st);  // (LENS_MIXED: interpolated where that is cheaper)
 int launch_wait_selftest(lens_ctx *ctx, unsigned polls, cudaStream_t st);
-int launch_math_selftest(const double *x, int n, double *out, cudaStream_t st);
+int launch_math_selftest(const double *x, int n, double *out, bool maps, cudaStream_t st);
 int launch_mcmc_step(lens_ctx *ctx, const Model *m, const CSet *c, double *d_params, double *d_chi2, int32_t W,
                      const double *d_sigma, double temperature, unsigned long long seed, unsigned long long step,
                      int32_t variant, int32_t np, double *d_scratch, int32_t *d_accepted, cudaStream_t st,

@@ -575,8 +575,11 @@ __global__ void __launch_bounds__(REP_THREADS) k_map_repair(const RepairArgs a) 
 // the arctangents need their reduction):
 //   - the record's products are formed once per potential and CTA, 32
 //     potentials at a time in shared memory;
-//   - reciprocals and roots take one cubic step on the MUFU seed (its error
-//     of ~2^-20 cubed) instead of two Newton steps;
+//   - reciprocals and roots take one third-order step on the MUFU seed (its
+//     error of ~2^-20 cubed) instead of two Newton steps: Householder's
+//     iteration of order 2 ("The Numerical Treatment of a Single Nonlinear
+//     Equation", 1970), i.e. with e = 1 - b y the series 1/b = y (1 + e + e^2 +
+//     ..) and with e = 1 - a y^2 a^-1/2 = y (1 + e/2 + 3 e^2/8 + ..) up to e^2;
 //   - the arctangents' reductions act on numerator and denominator before the
 //     division (atan(n/d) = pi/2 - atan(d/n) and = atan(c) + atan((n - c d) /
 //     (d + c n)), atanh likewise), so lanes inside and outside the
@@ -819,10 +822,20 @@ __global__ void k_math_selftest(const double *__restrict__ x, int n, double *__r
   out[3 * n + i] = rsqrt(v);
 }
 
+// The FP64 maps' own: out[0..2][i] = rcp64c, rsqrt64c, sqrt64c.
+__global__ void k_math_selftest_maps(const double *__restrict__ x, int n, double *__restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const double v = x[i];
+  out[i] = rcp64c(v);
+  out[n + i] = rsqrt64c(v);
+  out[2 * n + i] = sqrt64c(v);
+}
+
 }  // namespace
 
-int launch_math_selftest(const double *x, int n, double *out, cudaStream_t st) {
-  if (n > 0) k_math_selftest<<<(n + 255) / 256, 256, 0, st>>>(x, n, out);
+int launch_math_selftest(const double *x, int n, double *out, bool maps, cudaStream_t st) {
+  if (n > 0) (maps ? k_math_selftest_maps : k_math_selftest)<<<(n + 255) / 256, 256, 0, st>>>(x, n, out);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(LENS_ECUDA, "self-test launch: %s", cudaGetErrorString(e));
   return LENS_OK;
