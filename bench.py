@@ -33,9 +33,9 @@ L2_FLUSH_BYTES = 256 << 20   # > 129 MB L2, written between timed steps
 # call's kernels (summary under profiles/).  Far potentials are interpolated
 # over tiles, so the executed work is far below nodes x potentials x the
 # ~63 operations of one evaluation, and the fractions below are of what runs.
-MAP_FP32_OPS = 1.27e10   # coarse level 3.07e9, fine tiles 7.50e9, repair 1.36e9 + 0.77e9
-MAP_MUFU_OPS = 3.64e8
-POT_FP32_OPS = 7.75e9    # the potential map's two kernels
+MAP_FP32_OPS = 1.28e10   # coarse level 3.28e9, fine tiles 7.52e9, repair 1.35e9 + 0.65e9
+MAP_MUFU_OPS = 3.72e8
+POT_FP32_OPS = 2.29e11   # the potential map: every pair (this model's members outweigh what is interpolated)
 MAP_KERNELS = 4          # launched per Hessian map: coarse level, fine tiles, two repairs
 # DRAM bytes (read + write) of those four launches, from the same capture; the
 # 100.7 MB of output are partly still in L2 when the last kernel ends

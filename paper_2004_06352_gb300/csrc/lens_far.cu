@@ -1110,10 +1110,13 @@ constexpr long long DENSE_TILES = 65536;
 // margins of the repair: interpolation error below 4e-11 of a potential's own
 // deflection at the edge of its far region (4e-14 for the strong ones)
 constexpr double KR = 5.0, KR_H = 8.0;
-// Potential maps are stored in double, so the FP32 terms' rounding, which
-// differs between the two forms, shows in them: by 0.5e-10 to 7.3e-10 of the
-// map where Model::pot_light is below this (50 models of 60 to 2000 potentials;
-// 8.3e-10 to 6.4e-9 from 0.003 on).  Beyond, the direct kernel keeps its values.
+// Potential maps are stored in double, so the FP32 terms' rounding shows in
+// them.  Both forms are as far from 64 bits, but they round differently: they
+// differ by 0.5e-10 to 7.3e-10 of the map where Model::pot_light is below this
+// (50 models of 60 to 2000 potentials; 8.3e-10 to 6.4e-9 from 0.003 on).  Which
+// form a grid takes depends on its size and on the memory at hand, and a map is
+// not to move with that by more than 1e-9 of itself: beyond, every size takes
+// the direct kernel (2048^2 x 1000, 0.00303: 8 ms; interpolated 0.52).
 constexpr double POT_LIGHT = 0.0025;
 constexpr int FAR_MAX_N = 16384;  // potentials (two bytes each of shared memory)
 
@@ -1132,7 +1135,8 @@ int far_words(const Model *m) { return (m->n_light + 31) / 32 + (m->n_heavy + 31
 // Expected cost per map node of the direct kernel and of the interpolated
 // one with each coarse level, in evaluations of one FP32 potential (HV of
 // them for a cluster-scale potential in double-float), idle SMs of small
-// grids included.
+// grids included (152 SMs: 4 CTAs of the direct kernel, 1 of the coarse or 2 of
+// the fine one each).
 FarPlan plan_far(const lens_ctx *ctx, const Model *m, const lens_grid *g, int mode) {
   FarPlan p;
   if (m->n > FAR_MAX_N || m->n < 1) return p;
