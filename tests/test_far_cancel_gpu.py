@@ -32,14 +32,11 @@ CASES = [  # model, nodes a side, hessian
     (lambda: I.cfg2_model(seed=8, n_members=0), 4096, True), (lambda: I.cfg2_model(seed=4, n_members=8), 1024, True)]
 
 
-@pytest.mark.parametrize("ratio", [None, 0.0])
-@pytest.mark.parametrize("k", range(len(CASES)))
+# (with the repair of the FP32 terms off: the models without any)
+@pytest.mark.parametrize("k,ratio", [(k, None) for k in range(len(CASES))] + [(k, 0.0) for k in (3, 4, 5, 6)])
 def test_zero_of_cluster_deflection(lens, k, ratio):
     make, n, hess = CASES[k]
     m, g = make(), I.grid(n)
-    light = (m[:, 7] < 5.0).any()
-    if ratio == 0.0 and light:
-        pytest.skip("without the repair the FP32 members' own rounding stays")
     with lens.Context(0) as ctx:
         if ratio is not None:
             ctx.set_repair_ratio(ratio)
